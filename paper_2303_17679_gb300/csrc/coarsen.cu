@@ -32,10 +32,10 @@
 //              8-byte load, with no dependent gather.
 //   cst[C]   = {cw[C], status[C]}: cluster weight and status (the node's
 //              sub-round while it is unclustered, -1 once clustered).
-//   imeta[j] = {first pin, rated size or 0, Q20 term} of the net of
-//              incidence j, and lnode[x] = {u, ioff[u], ioff[u+1], c(u)} for
-//              every listed node: a node's walk reads its own record, then one
-//              record per incident net.
+//   imeta[j] = {first pin, pins to visit, Q20 term} of an incident net; a
+//              node's records with pins to visit sit at [ioff[u], rend[u]), and
+//              lnode[x] = {u, ioff[u], rend[u], c(u)} for every listed node:
+//              a node's walk reads its own record, then one record per net.
 // Nodes are bucketed per level by class and sub-round.  With W(u) = sum of
 // |e| over u's rated nets (the pins its rating visits) and D = min(W(u), n)
 // (a bound on its distinct candidates), a team accumulates u's ratings in a
@@ -97,9 +97,9 @@ enum { CW_MOVES = 0, CW_TOUCHED = 1, CW_SLOTS = 2, CW_CURSOR = 3, CW_WORDS = 8 }
 // work counters
 enum { ST_PINS = 0, ST_INCID = 1, ST_NODES = 2, ST_WORDS = 4 };
 
-// Per incidence (aligned with inets): the first pin position of its net,
-// the net's size when it is rated (2 <= |e| <= T), else 0, and its Q20 term
-// (0 when not rated).
+// Of an incidence (u, e): the first pin position to visit, the number of pins
+// to visit (the net's size, or u's range in it on grouped levels, when it is
+// rated, 2 <= |e| <= T, else 0) and the Q20 term of the net (0 when not rated).
 struct __align__(16) IncMeta {
   int32_t start, eff;
   unsigned long long r;
@@ -122,10 +122,10 @@ struct RateArgs {
   const int32_t* comm;
   const int32_t* pcomm;
   const unsigned long long* rterm;  // Q20 net term of every rated net, 0 otherwise
-  // hypergraph levels: the metadata of the net of every incidence (aligned
-  // with inets), so a walk reads one record per incident net
+  // hypergraph levels: the metadata of every node's nets with pins to visit,
+  // from ioff[u] on, so a walk reads one record per such net
   const IncMeta* imeta;
-  // {u, ioff[u], ioff[u + 1], c(u)} of every listed node: lnode is aligned
+  // {u, ioff[u], rend[u], c(u)} of every listed node: lnode is aligned
   // with list (this class and sub-round), lsplit with the split nodes
   const int4* lnode;
   const int4* lsplit;
@@ -1062,8 +1062,8 @@ __device__ __forceinline__ int rate_class(int64_t W, int32_t n, bool dense_block
   return 4;
 }
 
-// W(u) (pins of rated nets, or rated incident edges on graph levels) of every
-// node, and the largest bound on a node's rating (sum of its net terms),
+// W(u) (pins its rating visits: the ranges of its rated nets, or its rated
+// incident edges on graph levels) of every node, and the largest bound on a node's rating (sum of its net terms),
 // which decides the value width.
 // floor(w(e) * 2^20 / (|e| - 1)) for the rated nets (2 <= |e| <= T), else 0;
 // at least 1 for a rated net since |e| - 1 < 2^20.
@@ -1078,10 +1078,179 @@ __global__ void k_net_terms(const int32_t* __restrict__ eoff, const int32_t* __r
   }
 }
 
-// IncMeta of every incidence of a hypergraph level.
-__global__ void k_inc_meta(const int32_t* __restrict__ inets, const int32_t* __restrict__ eoff,
+// ------------------------------------------------ grouped pin order
+
+// A pin visit is wasted when the pin's cluster can never take u: it lies in
+// another community, or cw[C] + c(u) > c_max.  Cluster weights only grow
+// within a level and cw[C] >= c(v) for every member v, so the pins v with
+// c(v) + c(u) > c_max are known before the first sub-round.  On levels where
+// such pins abound the pins of every rated net of at most GROUP_NET pins are
+// therefore sorted by (community, weight bucket) once per level, and an
+// incidence (u, e) walks only the pins of u's community whose bucket does not
+// exceed that of c_max - c(u); the exact tests stay in the walk.  The range
+// holds all members of every admissible cluster (each is in u's community
+// and weighs at most c_max - c(u)), so the cluster's first position, the one
+// that carries its word, lies in it.
+// Coarse levels: most clusters are too heavy to pair up (of the 440M pin
+// visits of a level of 1571 nodes and 5.07M pins, 407M failed the weight test
+// and none passed).  With communities: 99 % of the visits of a 1.35M-pin
+// input were pins of other communities.  Measured (GB300, with the records
+// compacted by k_node_work): coarsening of a 4e6-node large-net input at
+// k = 64, 215 -> 143 ms (its levels of 377k nodes and fewer 36.5 -> 23.9,
+// 41.2 -> 13.6, 25.3 -> 10.6 ms); with communities on the 1.35M-pin input
+// 34.2 -> 16.2 ms; the sort takes 0.15 ms per level of 5M pins and 1 ms per
+// level of 31M.
+constexpr int GROUP_IDX_BITS = 10;
+constexpr int GROUP_NET = 1 << GROUP_IDX_BITS;
+constexpr int GROUP_W_BITS = 8;
+constexpr uint32_t GROUP_W_MASK = (1u << GROUP_W_BITS) - 1;
+constexpr uint32_t GROUP_COMM_MASK = (1u << (32 - GROUP_IDX_BITS - GROUP_W_BITS)) - 1;
+constexpr int GROUP_WARPS = 8;
+// Levels without communities are grouped when at least GROUP_HEAVY_NUM /
+// GROUP_HEAVY_DEN of their incidences belong to nodes of more than c_max / 2
+// (two of these never share a cluster): below that the sort and the range
+// searches (0.35-0.6 ms per 5M pins) cost more than the visits they save.
+constexpr unsigned long long GROUP_HEAVY_NUM = 1, GROUP_HEAVY_DEN = 4;
+
+// Monotone in c >= 1: exact below 16, then three mantissa bits (at most 231).
+__device__ __forceinline__ uint32_t weight_bucket(int32_t c) {
+  if (c < 16) return (uint32_t)c;
+  const int e = 31 - __clz(c);
+  return (uint32_t)(((e - 3) << 3) + (c >> (e - 3)));
+}
+
+// Group key of a pin: low bits of its community, then its weight bucket.
+__device__ __forceinline__ uint32_t group_key(int32_t comm, int32_t c) {
+  return (((uint32_t)comm & GROUP_COMM_MASK) << GROUP_W_BITS) | weight_bucket(c);
+}
+
+// Incidences of the nodes of more than c_max / 2.
+__global__ void k_heavy_pins(const int32_t* __restrict__ c, const int32_t* __restrict__ ioff,
+                             int32_t n, int32_t c_max, unsigned long long* __restrict__ heavy) {
+  unsigned long long h = 0;
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+       u += (int64_t)gridDim.x * blockDim.x)
+    if (2ll * c[u] > (long long)c_max) h += (unsigned long long)(ioff[u + 1] - ioff[u]);
+  const unsigned long long v[1] = {h};
+  block_add_counters(heavy, v);
+}
+
+__device__ __forceinline__ bool level_grouped(const unsigned long long* heavy, int64_t p,
+                                              bool comm) {
+  return comm || GROUP_HEAVY_DEN * *heavy >= GROUP_HEAVY_NUM * (unsigned long long)p;
+}
+
+// Sorts the sz <= 32 R pins of one net by group key with the warp: a bitonic
+// network over {key, index in the net} words held R per lane (in-thread swaps
+// below R, lane shuffles above).  The order of equal keys does not matter.
+template <int R>
+__device__ __forceinline__ void group_sort(int32_t b, int32_t sz, const int32_t* __restrict__ pins,
+                                           const int32_t* __restrict__ c,
+                                           const int32_t* __restrict__ comm,
+                                           int32_t* __restrict__ gpins,
+                                           int32_t* __restrict__ qnew,
+                                           uint32_t* __restrict__ gkey) {
+  const int lane = lane_id();
+  uint32_t v[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int32_t i = r * 32 + lane;
+    v[r] = ~0u;
+    if (i < sz) {
+      const int32_t x = pins[b + i];
+      v[r] = (group_key(comm ? comm[x] : 0, c[x]) << GROUP_IDX_BITS) | (uint32_t)i;
+    }
+  }
+#pragma unroll 1
+  for (int kk = 2; kk <= 32 * R; kk <<= 1) {
+#pragma unroll 1
+    for (int j = kk >> 1; j >= R; j >>= 1) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = lane * R + r;
+        const uint32_t y = __shfl_xor_sync(FULL, v[r], j / R);
+        const bool keep_min = ((i & kk) == 0) == ((i & j) == 0);
+        v[r] = keep_min ? min(v[r], y) : max(v[r], y);
+      }
+    }
+#pragma unroll
+    for (int j = R / 2; j > 0; j >>= 1) {
+      if (j >= kk) continue;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if ((r ^ j) > r) {
+          const bool up = ((lane * R + r) & kk) == 0;
+          const uint32_t lo = min(v[r], v[r ^ j]), hi = max(v[r], v[r ^ j]);
+          v[r] = up ? lo : hi;
+          v[r ^ j] = up ? hi : lo;
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int32_t i = lane * R + r;
+    if (i < sz) {
+      const int32_t from = b + (int32_t)(v[r] & (GROUP_NET - 1));
+      gpins[b + i] = pins[from];
+      gkey[b + i] = v[r] >> GROUP_IDX_BITS;
+      qnew[from] = b + i;
+    }
+  }
+}
+
+// One warp per net: gpins = the grouped pin order, qnew[q] = new position of
+// pin position q, gkey = group key per new position.  Unrated nets and nets
+// of more than GROUP_NET pins keep their order.
+__global__ void __launch_bounds__(GROUP_WARPS * 32)
+k_group_nets(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins, int32_t m, int T,
+             const int32_t* __restrict__ c, const int32_t* __restrict__ comm, int64_t p,
+             const unsigned long long* __restrict__ heavy, int32_t* __restrict__ gpins,
+             int32_t* __restrict__ qnew, uint32_t* __restrict__ gkey) {
+  if (!level_grouped(heavy, p, comm != nullptr)) return;
+  for (int64_t e = (int64_t)blockIdx.x * GROUP_WARPS + warp_in_block(); e < m;
+       e += (int64_t)gridDim.x * GROUP_WARPS) {
+    const int32_t b = eoff[e], sz = eoff[e + 1] - b;
+    if (sz < 2 || sz > T || sz > GROUP_NET) {
+      for (int32_t q = b + lane_id(); q < b + sz; q += 32) {
+        gpins[q] = pins[q];
+        qnew[q] = q;
+      }
+    } else if (sz <= 32) {
+      group_sort<1>(b, sz, pins, c, comm, gpins, qnew, gkey);
+    } else if (sz <= 128) {
+      group_sort<4>(b, sz, pins, c, comm, gpins, qnew, gkey);
+    } else if (sz <= 512) {
+      group_sort<16>(b, sz, pins, c, comm, gpins, qnew, gkey);
+    } else {
+      group_sort<32>(b, sz, pins, c, comm, gpins, qnew, gkey);
+    }
+  }
+}
+
+// First index of gkey[lo, hi) that is >= key (hi if none).
+__device__ __forceinline__ int32_t group_lower(const uint32_t* __restrict__ gkey, int32_t lo,
+                                               int32_t hi, uint32_t key) {
+  while (lo < hi) {
+    const int32_t mid = (lo + hi) >> 1;
+    if (gkey[mid] < key) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// IncMeta of every incidence of a hypergraph level; on grouped levels the
+// range of u's possible candidates in the net, and jpin[j] = the incidence's
+// pin position in the grouped order.
+__global__ void k_inc_meta(const int32_t* __restrict__ inets, const int32_t* __restrict__ ipin,
+                           const int32_t* __restrict__ eoff,
                            const unsigned long long* __restrict__ rterm, int64_t p,
+                           const int32_t* __restrict__ c, int32_t c_max, bool comm,
+                           const unsigned long long* __restrict__ heavy,
+                           const int32_t* __restrict__ gpins, const int32_t* __restrict__ qnew,
+                           const uint32_t* __restrict__ gkey, int32_t* __restrict__ jpin,
                            IncMeta* __restrict__ imeta) {
+  const bool grouped = level_grouped(heavy, p, comm);
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p;
        j += (int64_t)gridDim.x * blockDim.x) {
     const int32_t e = inets[j];
@@ -1090,44 +1259,86 @@ __global__ void k_inc_meta(const int32_t* __restrict__ inets, const int32_t* __r
     x.start = eoff[e];
     x.eff = r != 0 ? eoff[e + 1] - x.start : 0;
     x.r = r;
+    if (grouped) {
+      const int32_t qn = qnew[ipin[j]];
+      jpin[j] = qn;
+      if (x.eff != 0 && x.eff <= GROUP_NET) {
+        const int32_t end = x.start + x.eff, left = c_max - c[gpins[qn]];
+        x.eff = 0;
+        if (left > 0) {
+          const uint32_t key = gkey[qn], base = key & ~GROUP_W_MASK, top = weight_bucket(left);
+          if (comm) x.start = group_lower(gkey, x.start, qn, base);
+          x.eff = group_lower(gkey, x.start, end, base + top + 1) - x.start;
+          // a range holding u alone has no candidate
+          if (x.eff == 1 && (key & GROUP_W_MASK) <= top) x.eff = 0;
+        }
+      }
+    }
     imeta[j] = x;
   }
 }
 
-// {u, ioff[u], ioff[u + 1], c(u)} of every listed node.
+// {u, ioff[u], rend[u], c(u)} of every listed node.
 __global__ void k_list_nodes(const int32_t* __restrict__ list, int32_t cnt,
-                             const int32_t* __restrict__ ioff, const int32_t* __restrict__ c,
-                             int4* __restrict__ lnode) {
+                             const int32_t* __restrict__ ioff, const int32_t* __restrict__ rend,
+                             const int32_t* __restrict__ c, int4* __restrict__ lnode) {
   for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < cnt; x += gridDim.x * blockDim.x) {
     const int32_t u = list[x];
-    lnode[x] = make_int4(u, ioff[u], ioff[u + 1], c[u]);
+    lnode[x] = make_int4(u, ioff[u], rend[u], c[u]);
   }
 }
 
-// One warp per node, lanes over its incident nets.
+// One warp per node, lanes over its incident nets.  Hypergraph levels: over
+// their records, and the records that hold a visit are moved to the front of
+// the node's range (rend[u] = their end), so the walks never load the records
+// of unrated nets or of nets without a candidate (on large-net inputs most
+// incidences are of unrated nets; on grouped coarse levels a node of thousands
+// of nets may have a handful left).  Visits bound the records a walk loads.
 __global__ void k_node_work(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
-                            const int32_t* __restrict__ eoff,
+                            IncMeta* __restrict__ imeta,
                             const unsigned long long* __restrict__ rterm, int32_t n, bool graph,
-                            int32_t* __restrict__ wof, unsigned long long* __restrict__ max_r) {
+                            int32_t* __restrict__ wof, int32_t* __restrict__ rend,
+                            unsigned long long* __restrict__ max_r) {
   unsigned long long lr = 0;
+  const int lane = lane_id();
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
     long long W = 0;
     unsigned long long R = 0;
-    for (int32_t j = ioff[u] + lane_id(); j < ioff[u + 1]; j += 32) {
-      const int32_t e = inets[j];
-      const unsigned long long r = rterm[e];
-      if (r != 0) {
-        W += graph ? 1 : eoff[e + 1] - eoff[e];  // a graph visits the other endpoint only
+    const int32_t beg = ioff[u], end = ioff[u + 1];
+    int32_t out = beg;
+    if (graph) {
+      for (int32_t j = beg + lane; j < end; j += 32) {
+        const unsigned long long r = rterm[inets[j]];
+        W += r != 0;  // a graph visits the other endpoint only
         R += r;
+      }
+      out = end;
+    } else {
+      for (int32_t j0 = beg; j0 < end; j0 += 32) {
+        const int32_t j = j0 + lane;
+        IncMeta x{0, 0, 0};
+        if (j < end) x = imeta[j];
+        const unsigned live = __ballot_sync(FULL, x.eff != 0);
+        if (x.eff != 0) {
+          W += x.eff;
+          R += x.r;
+          // never past the records this warp has read
+          const int32_t to = out + __popc(live & ((1u << lane) - 1u));
+          if (to != j) imeta[to] = x;
+        }
+        out += __popc(live);
       }
     }
     W = warp_sum(W);
     R = warp_sum(R);
     lr = R > lr ? R : lr;
-    if (lane_id() == 0) wof[u] = W > 0x7fffffff ? 0x7fffffff : (int32_t)W;
+    if (lane == 0) {
+      wof[u] = W > 0x7fffffff ? 0x7fffffff : (int32_t)W;
+      rend[u] = out;
+    }
   }
-  if (lane_id() == 0 && lr) atomicMax(max_r, lr);
+  if (lane == 0 && lr) atomicMax(max_r, lr);
 }
 
 // key = class * S + sub-round of every node with W(u) > 0, and the counts.
@@ -1176,14 +1387,14 @@ __global__ void k_node_scatter(const int32_t* __restrict__ key_of, int32_t n, in
 //   else P = ceil(D / part_d) shared-memory parts when P <= PART_MAX (no
 //   global table);
 //   else a global hash table of a power of two >= 2 D + 2 slots, with items.
-__global__ void k_split_sizes(const int32_t* __restrict__ split, int32_t nsplit,
-                              const int32_t* __restrict__ ioff, const int32_t* __restrict__ wof,
+__global__ void k_split_sizes(const int4* __restrict__ lsplit, int32_t nsplit,
+                              const int32_t* __restrict__ wof,
                               int32_t n, int32_t part_d, int32_t* __restrict__ items,
                               int32_t* __restrict__ parts, int32_t* __restrict__ cap,
                               int8_t* __restrict__ dense) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nsplit; i += gridDim.x * blockDim.x) {
-    const int32_t u = split[i];
-    const int32_t deg = ioff[u + 1] - ioff[u];
+    const int4 nd = lsplit[i];
+    const int32_t u = nd.x, deg = nd.z - nd.y;
     const bool d = n <= SPLIT_DENSE_MAX && (int64_t)n <= 2 * (int64_t)wof[u];
     const int32_t D = min(wof[u], n);
     const int32_t P = d ? 0 : (D + part_d - 1) / part_d;
@@ -1520,7 +1731,7 @@ k_posmap_pass(const int4* __restrict__ lnode, const int32_t* __restrict__ lpre,
         const int32_t u = nd.x;
         const int32_t C = rep[u];
         const int32_t j = nd.y + (x - s_pre[a]);
-        if (j >= nd.z) {
+        if (x >= s_pre[a + 1]) {
           dev_fail(status, DEV_CAPACITY);  // the tile outran its staged nodes
         } else if (C == u) {
           // not joined
@@ -1825,7 +2036,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   kfill.alloc(&cx.alloc, (size_t)nkeys);
   words.alloc(&cx.alloc, (size_t)S * CW_WORDS);
   clusters.alloc(&cx.alloc, 1);
-  max_r.alloc(&cx.alloc, 1);
+  max_r.alloc(&cx.alloc, 2);  // largest possible rating, incidences of heavy nodes
   stats.alloc(&cx.alloc, (size_t)ST_WORDS * NCLASS);
   rinfo.alloc(&cx.alloc, L.graph ? 1 : (size_t)std::max<int64_t>(L.p, 1));
   HG_CUDA(cudaMemsetAsync(gw.p, 0, gw.bytes(), cx.stream));
@@ -1841,15 +2052,6 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   // (net, cluster) map
   const bool records = L.p > 0 && !L.graph;
   DBuf<int32_t> tiles;
-  if (records) {
-    tiles.alloc(&cx.alloc, (size_t)num_pin_tiles(L.p) + 1);
-    build_tile_index(cx, L.eoff.p, L.m, L.p, tiles.p);
-    k_rinfo_init<<<grid_for(num_pin_tiles(L.p), 1, cx.num_sms, 8), PIN_TILE_THREADS, 0,
-                   cx.stream>>>(L.eoff.p, L.pins.p, tiles.p, L.m, L.p, P.T, rinfo.p);
-    check_launch("rinfo_init");
-    if (cx.launches) *cx.launches += 1;
-  }
-
   const int g_nodes = grid_for(n, 256, cx.num_sms, 4);
   k_init_cluster<<<g_nodes, 256, 0, cx.stream>>>(L.c.p, n, P.seed, P.level, S, L.rep.p, cst.p,
                                                  slot_of.p);
@@ -1861,10 +2063,55 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
                                                                           P.T, rterm.p);
     check_launch("net_terms");
   }
+  // hypergraph levels: the grouped pin order (where it pays, decided on the
+  // device) and the net record of every incidence
+  DBuf<IncMeta> imeta;
+  DBuf<int32_t> gpins, jpin, rend;
+  rend.alloc(&cx.alloc, ncap);
+  if (records) {
+    DBuf<int32_t> qnew;
+    DBuf<uint32_t> gkey;
+    gpins.alloc(&cx.alloc, (size_t)L.p);
+    jpin.alloc(&cx.alloc, (size_t)L.p);
+    qnew.alloc(&cx.alloc, (size_t)L.p);
+    gkey.alloc(&cx.alloc, (size_t)L.p);
+    imeta.alloc(&cx.alloc, (size_t)L.p);
+    k_heavy_pins<<<g_nodes, 256, 0, cx.stream>>>(L.c.p, L.ioff.p, n, P.c_max, max_r.p + 1);
+    check_launch("heavy_pins");
+    k_group_nets<<<grid_for(L.m, GROUP_WARPS, cx.num_sms, 16), GROUP_WARPS * 32, 0, cx.stream>>>(
+        L.eoff.p, L.pins.p, L.m, P.T, L.c.p, L.comm.p, L.p, max_r.p + 1, gpins.p, qnew.p, gkey.p);
+    check_launch("group_nets");
+    k_inc_meta<<<grid_for(L.p, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
+        L.inets.p, L.ipin.p, L.eoff.p, rterm.p, L.p, L.c.p, P.c_max, L.comm.p != nullptr,
+        max_r.p + 1, gpins.p, qnew.p, gkey.p, jpin.p, imeta.p);
+    check_launch("inc_meta");
+    if (cx.launches) *cx.launches += 3;
+  }
   k_node_work<<<grid_for(n, 8, cx.num_sms, 16), 256, 0, cx.stream>>>(
-      L.ioff.p, L.inets.p, L.eoff.p, rterm.p, n, L.graph, wof.p, max_r.p);
+      L.ioff.p, L.inets.p, imeta.p, rterm.p, n, L.graph, wof.p, rend.p, max_r.p);
   check_launch("node_work");
-  const unsigned long long hmax_r = (unsigned long long)read_i64(cx, (const int64_t*)max_r.p);
+  unsigned long long hmax[2];
+  wait_stream(cx);
+  HG_CUDA(cudaMemcpyAsync(hmax, max_r.p, sizeof(hmax), cudaMemcpyDeviceToHost, cx.stream));
+  check_status(cx);
+  const unsigned long long hmax_r = hmax[0];
+  // the pins and pin positions the rating and the map work on
+  const bool grouped =
+      records && (L.comm.p || GROUP_HEAVY_DEN * hmax[1] >= GROUP_HEAVY_NUM * (unsigned long long)L.p);
+  const int32_t* rpins = grouped ? gpins.p : L.pins.p;
+  const int32_t* rpos = grouped ? jpin.p : L.ipin.p;
+  if (!grouped) {
+    gpins.release();
+    jpin.release();
+  }
+  if (records) {
+    tiles.alloc(&cx.alloc, (size_t)num_pin_tiles(L.p) + 1);
+    build_tile_index(cx, L.eoff.p, L.m, L.p, tiles.p);
+    k_rinfo_init<<<grid_for(num_pin_tiles(L.p), 1, cx.num_sms, 8), PIN_TILE_THREADS, 0,
+                   cx.stream>>>(L.eoff.p, rpins, tiles.p, L.m, L.p, P.T, rinfo.p);
+    check_launch("rinfo_init");
+    if (cx.launches) *cx.launches += 1;
+  }
   // 32-bit rating words when no node's total rating can reach 2^31; block
   // tables are direct-indexed when one value and one used-list entry per
   // node of the level fit the shared-memory budget
@@ -1886,22 +2133,13 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   check_status(cx);
   std::vector<int32_t> hoff(nkeys + 1, 0);
   for (int i = 0; i < nkeys; ++i) hoff[i + 1] = hoff[i] + hcount[i];
-  // per listed node {u, ioff[u], ioff[u + 1], c(u)}, and on hypergraph
-  // levels the net metadata of every incidence, for the rating walks
+  // per listed node {u, ioff[u], rend[u], c(u)}, for the rating walks
   DBuf<int4> lnode;
   lnode.alloc(&cx.alloc, (size_t)std::max<int32_t>(hoff[nkeys], 1));
   if (hoff[nkeys] > 0) {
     k_list_nodes<<<grid_for(hoff[nkeys], 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
-        list.p, hoff[nkeys], L.ioff.p, L.c.p, lnode.p);
+        list.p, hoff[nkeys], L.ioff.p, rend.p, L.c.p, lnode.p);
     check_launch("list_nodes");
-    if (cx.launches) *cx.launches += 1;
-  }
-  DBuf<IncMeta> imeta;
-  if (!L.graph && L.p > 0) {
-    imeta.alloc(&cx.alloc, (size_t)L.p);
-    k_inc_meta<<<grid_for(L.p, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(L.inets.p, L.eoff.p,
-                                                                         rterm.p, L.p, imeta.p);
-    check_launch("inc_meta");
     if (cx.launches) *cx.launches += 1;
   }
 
@@ -1935,7 +2173,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
     HG_CUDA(cudaMemsetAsync(sp.tnused.p, 0, sp.tnused.bytes(), cx.stream));
     const int gs = grid_for(nsplit, 256, cx.num_sms, 4);
     k_split_sizes<<<gs, 256, 0, cx.stream>>>(
-        sp.split, nsplit, L.ioff.p, wof.p, n, narrow ? PartCfg<uint32_t>::D : PartCfg<unsigned long long>::D,
+        lnode.p + split_base, nsplit, wof.p, n, narrow ? PartCfg<uint32_t>::D : PartCfg<unsigned long long>::D,
         items.p, parts.p, cap32.p, sp.tab_dense.p);
     check_launch("split_sizes");
     scan_exclusive_i32(cx, items.p, sp.item_off.p, nsplit, sp.item_off.p + nsplit);
@@ -2022,7 +2260,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
       check_launch("tile_node");
     }
     k_posmap_init<<<grid_for(num_pin_tiles(L.p), 1, cx.num_sms, 8), PIN_TILE_THREADS, 0,
-                    cx.stream>>>(L.eoff.p, L.pins.p, tiles.p, L.m, L.p, P.T, pm, cx.d_status);
+                    cx.stream>>>(L.eoff.p, rpins, tiles.p, L.m, L.p, P.T, pm, cx.d_status);
     check_launch("posmap_init");
     if (cx.launches) *cx.launches += 1 + 2 * (nlisted > 0);
   }
@@ -2040,7 +2278,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   DBuf<int32_t> pcomm;
   if (L.comm.p && !L.graph && L.p > 0) {
     pcomm.alloc(&cx.alloc, (size_t)L.p);
-    k_pin_comm<<<grid_for(L.p, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(L.pins.p, L.p, L.comm.p,
+    k_pin_comm<<<grid_for(L.p, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(rpins, L.p, L.comm.p,
                                                                          pcomm.p);
     check_launch("pin_comm");
     if (cx.launches) *cx.launches += 1;
@@ -2119,11 +2357,11 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
       }
       const int g = cx.num_sms * 8;
       k_posmap_pass<true><<<g, POS_TILE, 0, lx.stream>>>(
-          lnode.p, lpre.p, tile_node.p, hoff[nkeys], R, L.rep.p, L.inets.p, L.ipin.p, L.eoff.p,
+          lnode.p, lpre.p, tile_node.p, hoff[nkeys], R, L.rep.p, L.inets.p, rpos, L.eoff.p,
           P.T, pm, jslot.p, reinterpret_cast<int32_t*>(rinfo.p), cx.d_status);
       check_launch("posmap_join");
       k_posmap_pass<false><<<g, POS_TILE, 0, lx.stream>>>(
-          lnode.p, lpre.p, tile_node.p, hoff[nkeys], R, L.rep.p, L.inets.p, L.ipin.p, L.eoff.p,
+          lnode.p, lpre.p, tile_node.p, hoff[nkeys], R, L.rep.p, L.inets.p, rpos, L.eoff.p,
           P.T, pm, jslot.p, reinterpret_cast<int32_t*>(rinfo.p), cx.d_status);
       check_launch("posmap_fix");
       if (cx.launches) *cx.launches += 2;
