@@ -82,10 +82,10 @@ constexpr int32_t D_QUAD = 2048;
 constexpr int32_t D_BLOCK = 4096;
 constexpr int32_t TEAM_W = 65536;        // largest W of a node rated by one eight-warp team
 constexpr int32_t DENSE_W = 32768;       // largest W of a direct-indexed block node
+constexpr int32_t TEAM_RECORDS = 4096;   // most records of a node rated by one team or block
 constexpr int32_t SPLIT_DENSE_MAX = 65536;
 constexpr int SPLIT_WARPS = 8;
 constexpr int PART_THREADS = 1024;
-constexpr int PART_TEAMS = 1;
 // part blocks: see PartCfg (table slots and distinct candidates per part)
 constexpr int32_t PART_MAX = 8;          // more parts: the node uses a global hash table
 constexpr int ARGMAX_THREADS = 256;
@@ -398,17 +398,24 @@ __device__ __forceinline__ int32_t graph_walk(const RateArgs& A, int32_t lo, int
   return wt == 0 ? hi - lo : 0;
 }
 
-// Adds one group of (up to) 32 consecutive incident nets of u, starting at
-// position g0 of I(u), through `add`.  Nets of at least 32 rated pins are
-// walked one at a time with the lanes over their pins; the smaller nets of
-// the group are walked together over their flattened pins.  A team of TW
-// warps shares the group: the chunks of 32 * ILP visits are numbered on
-// from `run` (the chunks the team has walked before, for this node) and warp
-// wt takes those whose number is wt modulo TW, so the team stays balanced
-// across groups; `run` is advanced past the group's chunks.  Returns the
-// group's pin visits in warp 0 (0 in the other warps, so the team counts each
-// visit once).
-// Per lane: first pin, rated size (0 if the net is not rated) and Q20 term of
+// Adds one group of (up to) 32 consecutive records of u (one per lane)
+// through `add`: the lanes walk the group's visits flattened, 32 * ILP of
+// them at a time.  A visit's record is the number of records that end at or
+// before it: one ballot counts those that end before the 32 visits at hand,
+// and the ends that fall among them are collected as bits of one word (a
+// warp-wide OR), so a lane counts the bits up to its own position.  Bound by
+// instruction issue and L2 latency: a binary search through five dependent
+// shuffles per visit, and one pass of every warp of a team over each net of
+// 32 pins or more, cost more instructions than the visits themselves (1e6
+// Zipf coarsening 76.8 -> 70.6 ms without them).  Every record holds a visit (k_node_work), so the ends are
+// distinct.
+// A team of TW warps (a power of two) shares the group: the chunks of
+// 32 * ILP visits are numbered on from `run` (the chunks the team has walked
+// before, for this node) and warp wt takes those whose number is wt modulo
+// TW, so the team stays balanced across groups; `run` is advanced past the
+// group's chunks.  Returns the group's pin visits in warp 0 (0 in the other
+// warps, so the team counts each visit once).
+// Per lane: first pin to visit, pins to visit (0: no record) and Q20 term of
 // one incident net.
 template <typename VT>
 struct NetMeta {
@@ -416,8 +423,7 @@ struct NetMeta {
   VT r;
 };
 
-// The metadata of incidence j (-1: none): the first pin position of its net,
-// the net's size if it is rated (else 0) and its Q20 term.
+// The record at j (-1: none).
 template <typename VT>
 __device__ __forceinline__ NetMeta<VT> inc_meta(const RateArgs& A, int32_t j) {
   NetMeta<VT> m{0, 0, (VT)0};
@@ -435,60 +441,47 @@ __device__ __forceinline__ int32_t walk_group(const NetMeta<VT>& m, int wt, int 
                                               Visit& visit_batch) {
   constexpr int32_t CH = 32 * ILP;
   const int lane = lane_id();
-  const int32_t start = m.start, eff = m.eff;
+  const int32_t eff = m.eff;
   const VT r = m.r;
-  // big nets, one at a time
-  unsigned big = __ballot_sync(FULL, eff >= 32);
-  int32_t visits = 0;
-  while (big) {
-    const int j = __ffs(big) - 1;
-    big &= big - 1;
-    const int32_t st = __shfl_sync(FULL, start, j);
-    const int32_t sz = __shfl_sync(FULL, eff, j);
-    const VT rj = __shfl_sync(FULL, r, j);
-    const int32_t first = ((wt - run) % TW + TW) % TW;  // this warp's first chunk of the net
-    run += (sz + CH - 1) / CH;
-    for (int32_t q0 = CH * first; q0 < sz; q0 += CH * TW) {
-      int32_t q[ILP];
-      VT rr[ILP];
-#pragma unroll
-      for (int k = 0; k < ILP; ++k) {
-        const int32_t qq = q0 + 32 * k + lane;
-        q[k] = qq < sz ? st + qq : -1;
-        rr[k] = rj;
-      }
-      visit_batch(q, rr);
-    }
-    visits += sz;
-  }
-  // small nets together
-  const int32_t small = eff < 32 ? eff : 0;
-  const int32_t incl = warp_inclusive_scan(small);
+  const int32_t incl = warp_inclusive_scan(eff);
   const int32_t Z = __shfl_sync(FULL, incl, 31);
-  const int32_t first = ((wt - run) % TW + TW) % TW;
+  const int32_t off = m.start - (incl - eff);  // visit f of this record is at off + f
+  const unsigned upto = (2u << lane) - 1u;     // bits 0 .. lane
+  const int32_t first = (wt - run) & (TW - 1);
   run += (Z + CH - 1) / CH;
   for (int32_t f0 = CH * first; f0 < Z; f0 += CH * TW) {
     int32_t q[ILP];
     VT rr[ILP];
 #pragma unroll
     for (int k = 0; k < ILP; ++k) {
-      const int32_t f = f0 + 32 * k + lane;
-      int j = 0;
-#pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const int32_t probe = __shfl_sync(FULL, incl, j + step - 1);
-        if (probe <= f) j += step;
-      }
-      j = j > 31 ? 31 : j;
-      const int32_t incl_j = __shfl_sync(FULL, incl, j);
-      const int32_t eff_j = __shfl_sync(FULL, small, j);
-      const int32_t start_j = __shfl_sync(FULL, start, j);
+      const int32_t F = f0 + 32 * k;
+      const int32_t d = incl - F;
+      const int before = __popc(__ballot_sync(FULL, d <= 0));
+      const unsigned ends = __reduce_or_sync(FULL, eff > 0 && d > 0 && d < 32 ? 1u << d : 0u);
+      const int j = min(before + __popc(ends & upto), 31);
+      const int32_t off_j = __shfl_sync(FULL, off, j);
       rr[k] = __shfl_sync(FULL, r, j);
-      q[k] = f < Z ? start_j + f - (incl_j - eff_j) : -1;
+      q[k] = F + lane < Z ? off_j + F + lane : -1;
     }
     visit_batch(q, rr);
   }
-  return wt == 0 ? visits + Z : 0;
+  return wt == 0 ? Z : 0;
+}
+
+// How a team of TW warps walks a node's records: a node of at least
+// OWN_GROUPS groups of 32 records per warp gives each warp its own groups (a
+// warp then loads and scans only those); nodes of fewer records share every
+// group chunk by chunk, which balances them whatever their net sizes.
+constexpr int32_t OWN_GROUPS = 4;
+struct TeamWalk {
+  int32_t first, step;
+  int wt, TW;
+};
+__device__ __forceinline__ TeamWalk team_walk(const RateArgs& A, int32_t beg, int32_t end, int wt,
+                                              int TW) {
+  if (TW > 1 && !A.graph && end - beg >= OWN_GROUPS * 32 * TW)
+    return TeamWalk{beg + 32 * wt, 32 * TW, 0, 1};
+  return TeamWalk{beg, 32, wt, TW};
 }
 
 template <typename VT, int ILP, typename Visit>
@@ -626,7 +619,8 @@ __global__ void __launch_bounds__(TW * 32 * TEAMS, 1024 / (TW * 32 * TEAMS)) k_r
     // next node once every thread has read this one
     int32_t* nused = &s_nused[team][it & 1];
     int32_t run = 0;
-    visits += rate_groups<VT, TEAM_ILP>(A, u, cu, beg, end, 32, wt, TW, run,
+    const TeamWalk tw = team_walk(A, beg, end, wt, TW);
+    visits += rate_groups<VT, TEAM_ILP>(A, u, cu, tw.first, end, tw.step, tw.wt, tw.TW, run,
                                         each_visit<VT, TEAM_ILP>([&](int32_t C, VT r) HG_INLINE {
                                 const int32_t sl = tab.add(C, r);
                                 if (sl >= 0) used[atomicAdd(nused, 1)] = sl;
@@ -699,7 +693,8 @@ __global__ void __launch_bounds__(256, 4) k_rate_dense(RateArgs A) {
     // node once every thread has read this one
     int32_t* nused = &s_nused[it & 1];
     int32_t run = 0;
-    visits += rate_groups<VT, DENSE_ILP>(A, u, cu, beg, end, 32, wv, nw, run,
+    const TeamWalk tw = team_walk(A, beg, end, wv, nw);
+    visits += rate_groups<VT, DENSE_ILP>(A, u, cu, tw.first, end, tw.step, tw.wt, tw.TW, run,
                                          each_visit<VT, DENSE_ILP>([&](int32_t C, VT r) HG_INLINE {
                                 // every term is >= 1, so a zero before the add
                                 // marks the first touch
@@ -866,7 +861,7 @@ k_rate_part(RateArgs A, const int32_t* __restrict__ split, const int32_t* __rest
             VT* __restrict__ res_v, int32_t* __restrict__ res_c) {
   using H = typename PartCfg<VT>::Hash;
   constexpr uint32_t PART_SLOTS = PartCfg<VT>::SLOTS;
-  constexpr int NW = PART_THREADS / 32, TW = NW / PART_TEAMS;
+  constexpr int NW = PART_THREADS / 32;
   constexpr uint32_t CAP = PartCfg<VT>::CAP;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ VT s_rv[NW];
@@ -878,7 +873,7 @@ k_rate_part(RateArgs A, const int32_t* __restrict__ split, const int32_t* __rest
   for (uint32_t x = threadIdx.x; x < PART_SLOTS; x += blockDim.x) tab.init(x);
   if (threadIdx.x == 0) s_nused[0] = s_nused[1] = 0;
   __syncthreads();
-  const int wv = warp_in_block(), team = wv / TW, wt = wv % TW;
+  const int wv = warp_in_block();
   int64_t visits = 0, incid = 0, nodes = 0;
   int it = 0;
   for (int32_t t = part_lo + blockIdx.x; t < part_hi; t += gridDim.x) {
@@ -911,8 +906,9 @@ k_rate_part(RateArgs A, const int32_t* __restrict__ split, const int32_t* __rest
       }
     };
     int32_t run = 0;
-    const int64_t v = rate_groups_raw<VT, PART_ILP>(A, beg + 32 * team, end, 32 * PART_TEAMS, wt, TW, run,
-                                          visit);
+    const TeamWalk tw = team_walk(A, beg, end, wv, NW);
+    const int64_t v =
+        rate_groups_raw<VT, PART_ILP>(A, tw.first, end, tw.step, tw.wt, tw.TW, run, visit);
     if (k == 0) visits += v;
     __syncthreads();
     const int32_t nu = *nused;
@@ -1050,12 +1046,13 @@ k_rate_split_argmax(RateArgs A, const int32_t* __restrict__ split, int32_t lo, i
 //     eight warps, 4096-slot hash          D <= 2048, W <= 65536 (other levels)
 //   3 sixteen warps, 8192-slot hash        D <= 4096, W <= 65536 (other levels)
 //   4 split over the grid                  the rest
-__device__ __forceinline__ int rate_class(int64_t W, int32_t n, bool dense_block, RateCuts cut) {
+__device__ __forceinline__ int rate_class(int64_t W, int32_t records, int32_t n, bool dense_block,
+                                          RateCuts cut) {
   const int64_t D = W < n ? W : n;  // bound on the distinct candidate clusters
   if (D <= cut.warp) return 0;
-  if (dense_block && W <= DENSE_W) return 2;
+  if (dense_block && W <= DENSE_W && records <= TEAM_RECORDS) return 2;
   if (D <= cut.pair) return 1;
-  if (!dense_block && W <= TEAM_W) {
+  if (!dense_block && W <= TEAM_W && records <= TEAM_RECORDS) {
     if (D <= cut.quad) return 2;
     if (D <= cut.block) return 3;
   }
@@ -1342,7 +1339,8 @@ __global__ void k_node_work(const int32_t* __restrict__ ioff, const int32_t* __r
 }
 
 // key = class * S + sub-round of every node with W(u) > 0, and the counts.
-__global__ void k_node_classify(const int32_t* __restrict__ wof, int32_t n, uint64_t seed,
+__global__ void k_node_classify(const int32_t* __restrict__ wof, const int32_t* __restrict__ ioff,
+                                const int32_t* __restrict__ rend, int32_t n, uint64_t seed,
                                 int level, int S, bool dense_block, RateCuts cut,
                                 int32_t* __restrict__ key_of, int32_t* __restrict__ kcount) {
   for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
@@ -1350,7 +1348,7 @@ __global__ void k_node_classify(const int32_t* __restrict__ wof, int32_t n, uint
     const int32_t W = wof[u];
     int32_t key = -1;
     if (W > 0) {
-      key = rate_class(W, n, dense_block, cut) * S +
+      key = rate_class(W, rend[u] - ioff[u], n, dense_block, cut) * S +
             subround_of_node_cluster(seed, level, (int)u, S);
       atomicAdd(&kcount[key], 1);
     }
@@ -2118,7 +2116,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   const bool narrow = hmax_r < (1ull << 31);
   const size_t vbytes = narrow ? 4 : 8;
   const bool dense_block = (size_t)n * (vbytes + 4) <= SMEM_BUDGET;
-  k_node_classify<<<g_nodes, 256, 0, cx.stream>>>(wof.p, n, P.seed, P.level, S, dense_block,
+  k_node_classify<<<g_nodes, 256, 0, cx.stream>>>(wof.p, L.ioff.p, rend.p, n, P.seed, P.level, S, dense_block,
                                                    P.cuts, key_of.p, kcount.p);
   check_launch("node_classify");
   k_node_scatter<<<g_nodes, 256, nkeys * sizeof(int32_t), cx.stream>>>(key_of.p, n, nkeys,
