@@ -93,7 +93,8 @@ typedef struct {
    * <= 2048, default 2048), sixteen warps (rate_block_max_d, <= 4096,
    * default 4096), else the grid-split path.  In label propagation, nodes
    * with more than lp_block_min_deg incident nets (default 64, <= 2^20) are
-   * evaluated by a block of sixteen warps, the others by one warp. */
+   * evaluated by whole warps, one per 128 to 1024 of their nets, the others by
+   * groups of eight lanes. */
   int32_t rate_warp_max_d;
   int32_t rate_pair_max_d;
   int32_t rate_quad_max_d;
@@ -141,13 +142,13 @@ typedef struct {
   int64_t lp_nodes;           /* nodes evaluated by the gain kernels */
   int64_t lp_gain_launches;
   double ms_rating_kernels;   /* sum of rating kernel durations (timing on) */
-  double ms_lp_gain_kernels;  /* best-move kernel duration (timing flag 2; inside a captured
-                                 pass the two parallel branches count once) */
+  double ms_lp_gain_kernels;  /* best-move phases incl. the pass's node lists (timing flag 2;
+                                 device clock of one block, barriers included) */
   double ms_rating_refresh;   /* per-sub-round refresh of the deduplicated pin clusters */
   double ms_rating_class[8];  /* rating kernel time per node class (timing flag 2) */
   int64_t rating_visits_class[8]; /* pin visits per node class */
-  double ms_lp_select_kernels; /* bucketing and pair selection duration (timing flag 2) */
-  double ms_lp_apply_kernels;  /* move application duration (timing flag 2) */
+  double ms_lp_select_kernels; /* pair selection phases (timing flag 2) */
+  double ms_lp_apply_kernels;  /* move application phases (timing flag 2) */
   int64_t lp_moved_incidences; /* incident nets of the moved nodes */
   int64_t lp_passes;           /* label-propagation passes run */
   int64_t timing_failures;     /* kernel-timing event pairs that could not be read */

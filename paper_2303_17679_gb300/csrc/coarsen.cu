@@ -1095,8 +1095,8 @@ __global__ void k_net_terms(const int32_t* __restrict__ eoff, const int32_t* __r
 // compacted by k_node_work): coarsening of a 4e6-node large-net input at
 // k = 64, 215 -> 143 ms (its levels of 377k nodes and fewer 36.5 -> 23.9,
 // 41.2 -> 13.6, 25.3 -> 10.6 ms); with communities on the 1.35M-pin input
-// 34.2 -> 16.2 ms; the sort takes 0.15 ms per level of 5M pins and 1 ms per
-// level of 31M.
+// 34.2 -> 16.2 ms; the sort and the range searches take 0.65 ms
+// on a level of 5M pins.
 constexpr int GROUP_IDX_BITS = 10;
 constexpr int GROUP_NET = 1 << GROUP_IDX_BITS;
 constexpr int GROUP_W_BITS = 8;
@@ -1106,7 +1106,7 @@ constexpr int GROUP_WARPS = 8;
 // Levels without communities are grouped when at least GROUP_HEAVY_NUM /
 // GROUP_HEAVY_DEN of their incidences belong to nodes of more than c_max / 2
 // (two of these never share a cluster): below that the sort and the range
-// searches (0.35-0.6 ms per 5M pins) cost more than the visits they save.
+// searches cost more than the visits they save.
 constexpr unsigned long long GROUP_HEAVY_NUM = 1, GROUP_HEAVY_DEN = 4;
 
 // Monotone in c >= 1: exact below 16, then three mantissa bits (at most 231).

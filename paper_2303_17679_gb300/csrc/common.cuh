@@ -65,12 +65,18 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
   return z ^ (z >> 31);
 }
 
+// x mod S, without the 64-bit division (some 70 instructions) for powers of
+// two such as the default 16.
+__host__ __device__ __forceinline__ int subround_mod(uint64_t x, int S) {
+  return (S & (S - 1)) == 0 ? (int)(x & (uint64_t)(S - 1)) : (int)(x % (uint64_t)S);
+}
+
 // Sub-round of node u in clustering round `level` (Sec. 11: nodes are split
 // into sub-rounds by a hash of the seed, the level and the node id).
 __host__ __device__ __forceinline__ int subround_of_node_cluster(uint64_t seed, int level, int u,
                                                                  int S) {
   const uint64_t x = seed ^ ((uint64_t)(uint32_t)level << 32) ^ (uint64_t)(uint32_t)u;
-  return (int)(mix64(x) % (uint64_t)S);
+  return subround_mod(mix64(x), S);
 }
 
 // Sub-round of node u in label-propagation pass `pass` of level `level`.
@@ -78,7 +84,7 @@ __host__ __device__ __forceinline__ int subround_of_node_lp(uint64_t seed, int l
                                                             int u, int S) {
   const uint64_t x = seed ^ ((uint64_t)(uint32_t)level << 32) ^
                      ((uint64_t)(uint32_t)(pass + 1) << 48) ^ (uint64_t)(uint32_t)u;
-  return (int)(mix64(x) % (uint64_t)S);
+  return subround_mod(mix64(x), S);
 }
 
 // ------------------------------------------------------------- warp utils
@@ -385,6 +391,18 @@ struct RefineCounters {
          ms_gain_kernels = 0, ms_select_kernels = 0, ms_apply_kernels = 0;
 };
 
+// Pin counts Phi, connectivity sets Lambda and block weights of a partition.
+struct PinState {
+  DBuf<int32_t> phi;
+  DBuf<unsigned long long> lam;
+  DBuf<long long> bw;
+  DBuf<int32_t> tiles;
+};
+
+// counts == false (graph levels in label propagation): block weights only.
+void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, PinState& st,
+                     bool counts);
+
 void project_partition(const Ctx& cx, const Level& fine, const int32_t* coarse_part,
                        int32_t* fine_part);
 
@@ -412,6 +430,7 @@ struct LPResult {
 void recalculate_gains(const Ctx& cx, const Level& L, int k, const int32_t* part, int32_t l,
                        const int32_t* nodes, const int32_t* targets, int64_t* gains);
 
+// Label propagation (lp.cu).
 LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, int eps_ppm,
                          int max_passes, int S, uint64_t seed, int64_t total_node_weight,
                          int lp_block_deg, int32_t* part, RefineCounters& rc);
