@@ -1,0 +1,75 @@
+// Barrier of all blocks of a persistent kernel.
+#pragma once
+
+#include "common.cuh"
+
+namespace hgk {
+
+constexpr int SPIN_LIMIT = 1 << 24;  // polls of one grid barrier (seconds)
+
+// cluster: the blocks are one thread-block cluster (hardware barrier, 0.35 to
+// 0.5 us); else they were launched cooperatively and count arrivals in
+// `counter` (zero at the launch; 1.4 us over 152 blocks).  `gen` counts the
+// barriers passed.  Returns false when a grid barrier gave up: the status
+// word is set and every thread of the block returns from the kernel.
+__device__ __forceinline__ bool grid_sync(bool cluster, unsigned* counter, int32_t* status,
+                                          unsigned& gen) {
+  if (cluster) {
+    __threadfence();
+    asm volatile(
+        "barrier.cluster.arrive.release.aligned;\n"
+        "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  }
+  ++gen;
+  __syncthreads();
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned target = gen * gridDim.x;
+    atomicAdd(counter, 1u);
+    int polls = 0;
+    unsigned v;
+    do {
+      asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+    } while ((int)(v - target) < 0 && ++polls < SPIN_LIMIT);
+    ok = (int)(v - target) >= 0;
+    if (!ok) dev_fail(status, DEV_TIMEOUT);
+    __threadfence();
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Launches a kernel of `blocks` blocks that meets at grid_sync: one cluster
+// when cluster is set (1, 2, 4, 8 or 16 blocks), else cooperatively.
+template <typename K, typename... Args>
+void launch_persistent(const Ctx& cx, K kernel, int blocks, int threads, size_t smem, bool cluster,
+                       Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = cx.stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cluster) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)blocks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
+  HG_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
+  if (cx.launches) *cx.launches += 1;
+}
+
+}  // namespace hgk

@@ -28,7 +28,7 @@
 #include <climits>
 #include <mutex>
 
-#include "common.cuh"
+#include "gridsync.cuh"
 
 namespace hgk {
 
@@ -44,7 +44,6 @@ constexpr int32_t ITEM_INC_MIN = 128, ITEM_INC_MAX = 1024;
 constexpr int MACC_STRIDE = HG_MAX_K + 4; // sums of a node split over several items: k blocks, bw
 constexpr int RANK_MAX = 1024;            // directions of up to this many moves: rank sort
 constexpr int MAX_PAIRS = HG_MAX_K * (HG_MAX_K - 1) / 2;
-constexpr int SPIN_LIMIT = 1 << 24;       // polls of one grid barrier (seconds)
 
 // ------------------------------------------------ packed net records (a11)
 
@@ -141,39 +140,8 @@ __device__ __forceinline__ unsigned long long sel_key(int32_t g, int32_t u) {
   return ((unsigned long long)(uint32_t)(0x7fffffff - g) << 32) | (unsigned)u;
 }
 
-__device__ __forceinline__ unsigned long long now_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Barrier of all blocks; false when a grid barrier gave up (then every
-// thread of the block returns).  `gen` counts the barriers passed.
 __device__ __forceinline__ bool lp_sync(const LpArgs& A, unsigned& gen) {
-  if (A.cluster) {
-    __threadfence();
-    asm volatile(
-        "barrier.cluster.arrive.release.aligned;\n"
-        "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    return true;
-  }
-  ++gen;
-  __syncthreads();
-  bool ok = true;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned target = gen * gridDim.x;
-    atomicAdd(A.barrier, 1u);
-    int polls = 0;
-    unsigned v;
-    do {
-      asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(A.barrier) : "memory");
-    } while ((int)(v - target) < 0 && ++polls < SPIN_LIMIT);
-    ok = (int)(v - target) >= 0;
-    if (!ok) dev_fail(A.status, DEV_TIMEOUT);
-    __threadfence();
-  }
-  return __syncthreads_and(ok) != 0;
+  return grid_sync(A.cluster, A.barrier, A.status, gen);
 }
 
 // ------------------------------------------------- sub-round lists
@@ -1139,35 +1107,21 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
   const size_t bytes = lp_smem_bytes(k);
   const int64_t need = std::max<int64_t>(
       {nodes_sr / (LP_WARPS * NG) + 1, inc_sr / (LP_THREADS * 8) + 1, (int64_t)k * (k - 1) / 256 + 1});
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr[1];
-  cfg.blockDim = dim3(LP_THREADS);
-  cfg.dynamicSmemBytes = bytes;
-  cfg.stream = cx.stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (need <= CLUSTER_MAX) {
-    int c = 1;
-    while (c < need) c <<= 1;
-    A.cluster = true;
-    cfg.gridDim = dim3(c);
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = c;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+  int blocks = 1;
+  A.cluster = need <= CLUSTER_MAX;
+  if (A.cluster) {
+    while (blocks < need) blocks <<= 1;
   } else {
-    A.cluster = false;
     int per_sm = 0;
     HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
         &per_sm, reinterpret_cast<const void*>(kernel), LP_THREADS, bytes));
     if (per_sm < 1) throw HgError(HG_ERR_CUDA, "label propagation does not fit an SM");
+    // a handle that shares the GPU with others (it sleeps while it waits) takes
+    // no more blocks than its work fills
     const int64_t most = (int64_t)cx.num_sms * std::min(per_sm, 2);
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>(need <= cx.num_sms ? cx.num_sms : most, most));
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
+    blocks = (int)(cx.sync_event ? std::min(need, most) : need <= cx.num_sms ? cx.num_sms : most);
   }
-  HG_CUDA(cudaLaunchKernelEx(&cfg, kernel, A));
-  if (cx.launches) *cx.launches += 1;
+  launch_persistent(cx, kernel, blocks, LP_THREADS, bytes, A.cluster, A);
   unsigned long long hres[LR_WORDS];
   wait_stream(cx);
   HG_CUDA(cudaMemcpyAsync(hres, A.res, sizeof(hres), cudaMemcpyDeviceToHost, cx.stream));
