@@ -300,6 +300,8 @@ void scan_exclusive_i32(const Ctx& cx, const int32_t* in, int32_t* out, int64_t 
 // Same with int64 output.
 void scan_exclusive_i32_to_i64(const Ctx& cx, const int32_t* in, int64_t* out, int64_t n,
                                int64_t* d_total);
+void scan_exclusive_i64(const Ctx& cx, const int64_t* in, int64_t* out, int64_t n,
+                        int64_t* d_total);
 
 // Copies a device scalar to the host (synchronizes the stream) and checks
 // the device status word.

@@ -23,12 +23,18 @@
 //
 // Layout per level: CSR with int64 offsets, int32 neighbours, int64 weights,
 // int64 self-loop weights, degrees k and volumes.  Per round the vertices
-// are listed by (sub-round, class): class 0 (degree <= LV_SMALL) is decided
-// by one warp per vertex with a shared-memory table of its neighbouring
-// clusters; class 1 inserts its edges into per-vertex tables in global
-// memory with one thread per edge over the whole grid, then one block per
-// vertex takes the best entry.  Aggregation uses the same global tables, one
-// per coarse vertex.
+// are listed by (sub-round, class): vertices of at most 8 (32) edges are decided
+// by a group of eight lanes (a warp) that holds one edge per lane and sums the
+// edges of a cluster by exchanging them; up to LV_SMALL edges by one warp with
+// a shared-memory table of the neighbouring clusters; the rest insert their
+// edges into per-vertex tables in global memory with one thread per edge over
+// the whole grid, then one block per vertex takes the best entry.  Aggregation
+// uses the same global tables, one per coarse vertex.
+// What bounds it: 16 dependent sub-rounds of gathers per round, some 25 rounds.
+// Most vertices have a handful of edges (a table of 512 slots, cleared and
+// scanned per vertex, cost more than they did), and the host reads only the
+// class boundaries of a round (copying the table offsets of all vertices took
+// over a millisecond per round).
 #include <algorithm>
 #include <mutex>
 
@@ -40,7 +46,10 @@ namespace {
 
 constexpr int LV_ROUNDS = 5;
 constexpr int LV_LEVELS = 32;
-constexpr int LV_SMALL = 256;          // class 0: degree <= LV_SMALL
+constexpr int LV_CLASSES = 4;
+constexpr int LV_GROUP = 8;            // class 0: degree <= 8, eight lanes per vertex
+constexpr int LV_LANES = 32;           // class 1: degree <= 32, a warp per vertex
+constexpr int LV_SMALL = 256;          // class 2: degree <= 256, a warp and a shared table
 constexpr int LV_SLOTS = 2 * LV_SMALL;  // shared slots per warp (load <= 1/2)
 constexpr int LV_WARPS = 8;
 constexpr int LV_ARGMAX_THREADS = 256;
@@ -52,7 +61,7 @@ __device__ __forceinline__ int subround_louvain(uint64_t seed, int level, int ro
                                                 int S) {
   const uint64_t x = seed ^ (1ull << 62) ^ ((uint64_t)(uint32_t)level << 32) ^
                      ((uint64_t)(uint32_t)(round + 1) << 48) ^ (uint64_t)(uint32_t)i;
-  return (int)(mix64(x) % (uint64_t)S);
+  return subround_mod(mix64(x), S);
 }
 
 // ------------------------------------------------------------ level 0
@@ -113,18 +122,19 @@ __global__ void k_lv_init(int64_t V, const long long* __restrict__ k, int32_t* _
 
 // ------------------------------------------------------------ lists
 
-// key = sub-round * 2 + class of every vertex with at least one edge.
+// key = sub-round * LV_CLASSES + class of every vertex with at least one edge.
 __device__ __forceinline__ int lv_key(const long long* off, uint64_t seed, int level, int round,
                                       int64_t i, int S) {
   const long long deg = off[i + 1] - off[i];
   if (deg == 0) return -1;  // no neighbouring cluster: never moves
-  return subround_louvain(seed, level, round, i, S) * 2 + (deg > LV_SMALL ? 1 : 0);
+  const int cls = deg <= LV_GROUP ? 0 : deg <= LV_LANES ? 1 : deg <= LV_SMALL ? 2 : 3;
+  return subround_louvain(seed, level, round, i, S) * LV_CLASSES + cls;
 }
 
 __global__ void k_lv_count(const long long* __restrict__ off, int64_t V, uint64_t seed, int level,
                            int round, int S, int32_t* __restrict__ cnt) {
   extern __shared__ int32_t s_cnt[];
-  for (int i = threadIdx.x; i < 2 * S; i += blockDim.x) s_cnt[i] = 0;
+  for (int i = threadIdx.x; i < LV_CLASSES * S; i += blockDim.x) s_cnt[i] = 0;
   __syncthreads();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -132,7 +142,7 @@ __global__ void k_lv_count(const long long* __restrict__ off, int64_t V, uint64_
     if (key >= 0) atomicAdd(&s_cnt[key], 1);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 2 * S; i += blockDim.x)
+  for (int i = threadIdx.x; i < LV_CLASSES * S; i += blockDim.x)
     if (s_cnt[i]) atomicAdd(&cnt[i], s_cnt[i]);
 }
 
@@ -151,21 +161,37 @@ __global__ void k_lv_scatter(const long long* __restrict__ off, int64_t V, uint6
   }
 }
 
-// Degrees and global table sizes (power of two >= 2 deg + 2) along a list.
-__global__ void k_lv_list_sizes(const int32_t* __restrict__ list, int32_t cnt,
-                                const long long* __restrict__ off, int32_t* __restrict__ deg,
-                                int32_t* __restrict__ tsize) {
-  for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < cnt; x += gridDim.x * blockDim.x) {
-    const int32_t i = list[x];
-    const int32_t d = (int32_t)(off[i + 1] - off[i]);
-    deg[x] = d;
-    if (tsize) {
-      // at most 2^30 slots: a larger vertex fills its table, which the
-      // insertion reports as a full table
-      int64_t c = 4;
-      while (c < 2 * (int64_t)d + 2 && c < (1ll << 30)) c <<= 1;
-      tsize[x] = (int32_t)c;
+// Degrees and global table sizes (power of two >= 2 deg + 2) of the vertices
+// that need a table along the list of *listed <= cap vertices (zeros after it
+// and for the others).
+__global__ void k_lv_list_sizes(const int32_t* __restrict__ list, const int32_t* __restrict__ listed,
+                                int32_t cap, const long long* __restrict__ off,
+                                int32_t* __restrict__ deg, int32_t* __restrict__ tsize) {
+  const int32_t cnt = *listed;
+  for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < cap; x += gridDim.x * blockDim.x) {
+    int32_t d = 0, t = 0;
+    if (x < cnt) {
+      const int32_t i = list[x];
+      d = (int32_t)(off[i + 1] - off[i]);
+      if (d > LV_SMALL) {
+        // at most 2^30 slots: a larger vertex fills its table, which the
+        // insertion reports as a full table
+        int64_t c = 4;
+        while (c < 2 * (int64_t)d + 2 && c < (1ll << 30)) c <<= 1;
+        t = (int32_t)c;
+      }
     }
+    deg[x] = d;
+    tsize[x] = t;
+  }
+}
+
+// The class boundaries of a round and the table offsets there.
+__global__ void k_lv_bounds(const int32_t* __restrict__ koff, int nkeys,
+                            const long long* __restrict__ toff, long long* __restrict__ out) {
+  for (int i = threadIdx.x; i <= nkeys; i += blockDim.x) {
+    out[i] = koff[i];
+    out[nkeys + 1 + i] = toff[koff[i]];
   }
 }
 
@@ -244,7 +270,62 @@ __device__ __forceinline__ void lv_emit(const LvArgs& A, int32_t i, long long ki
   }
 }
 
-// Class 0: one warp per vertex, shared table of LV_SLOTS entries.
+// Classes 0 and 1: G lanes per vertex of at most G edges, one edge per lane.
+// Every lane sums the edges of its own cluster (equal lanes hold equal
+// candidates); the groups of a warp stay in step.
+template <int G>
+__global__ void __launch_bounds__(LV_WARPS * 32) k_lv_lanes(LvArgs A, int32_t lo, int32_t hi) {
+  constexpr int PER = 32 / G;
+  const int lane = lane_id(), sub = lane % G, grp = lane / G;
+  const int32_t stride = gridDim.x * LV_WARPS * PER;
+  for (int32_t x0 = lo + (blockIdx.x * LV_WARPS + warp_in_block()) * PER; x0 < hi; x0 += stride) {
+    const int32_t x = x0 + grp;
+    const bool on = x < hi;
+    const int32_t i = on ? A.list[x] : 0;
+    const long long b = on ? A.off[i] : 0;
+    const int d = on ? (int)(A.off[i + 1] - b) : 0;
+    int32_t C = -1;
+    long long w = 0;
+    if (sub < d) {
+      C = A.cl[A.adj[b + sub]];
+      w = A.aw[b + sub];
+    }
+    const int32_t own = on ? A.cl[i] : -1;
+    const long long ki = on ? A.k[i] : 0;
+    const long long vol = C >= 0 ? A.vol[C] : 0;
+    const int steps = __reduce_max_sync(FULL, (unsigned)d);
+    long long kic = 0;
+    for (int t = 0; t < steps; ++t) {
+      const int32_t Ct = __shfl_sync(FULL, C, grp * G + t);
+      const long long wt = __shfl_sync(FULL, w, grp * G + t);
+      if (Ct == C) kic += wt;
+    }
+    Cand best{0, -1};
+    if (C >= 0 && C != own) best = Cand{(i128)A.W2 * kic - (i128)ki * vol, C};
+    long long kia = C >= 0 && C == own ? kic : 0;  // the same in every lane of the own cluster
+#pragma unroll
+    for (int s = G / 2; s > 0; s >>= 1) {
+      cand_better(best, shfl_cand(best, s));
+      const long long o = __shfl_xor_sync(FULL, kia, s);
+      kia = o > kia ? o : kia;
+    }
+    bool moves = false;
+    if (on && sub == 0 && best.c >= 0)
+      moves = best.s > (i128)A.W2 * kia - (i128)ki * (A.vol[own] - ki);
+    const unsigned who = __ballot_sync(FULL, moves);
+    if (who) {
+      int32_t slot = 0;
+      if (lane == 0) slot = atomicAdd(&A.words[0], __popc(who));
+      slot = __shfl_sync(FULL, slot, 0) + __popc(who & ((1u << lane) - 1u));
+      if (moves) {
+        A.mv_v[slot] = i;
+        A.mv_to[slot] = best.c;
+      }
+    }
+  }
+}
+
+// Class 2: one warp per vertex, shared table of LV_SLOTS entries.
 __global__ void __launch_bounds__(LV_WARPS * 32) k_lv_small(LvArgs A, int32_t lo, int32_t hi) {
   __shared__ int32_t s_key[LV_WARPS][LV_SLOTS];
   __shared__ long long s_val[LV_WARPS][LV_SLOTS];
@@ -287,7 +368,7 @@ __global__ void __launch_bounds__(LV_WARPS * 32) k_lv_small(LvArgs A, int32_t lo
   }
 }
 
-// Class 1, step 1: one thread per edge of the listed vertices [lo, hi):
+// Class 3, step 1: one thread per edge of the listed vertices [lo, hi):
 // lpre = exclusive prefix of their degrees along the list, toff = offsets of
 // their global tables (relative to tbase).
 __global__ void k_lv_big_insert(LvArgs A, int32_t lo, int32_t hi, const long long* __restrict__ lpre,
@@ -312,7 +393,7 @@ __global__ void k_lv_big_insert(LvArgs A, int32_t lo, int32_t hi, const long lon
   }
 }
 
-// Class 1, step 2: one block per listed vertex, best entry of its table
+// Class 3, step 2: one block per listed vertex, best entry of its table
 // (cleared on the way for the next sub-round).
 __global__ void __launch_bounds__(LV_ARGMAX_THREADS)
 k_lv_big_argmax(LvArgs A, int32_t lo, int32_t hi, const long long* __restrict__ toff,
@@ -385,99 +466,92 @@ __global__ void k_lv_used(const int32_t* __restrict__ cl, int64_t V, int32_t* __
     flag[cl[i]] = 1;
 }
 
-// cv[i] = coarse vertex of i; member counts per coarse vertex.
+// cv[i] = coarse vertex of i; per coarse vertex the sum of its members' degrees
+// in the edge lists (a bound on its coarse degree) and of their self-loop
+// weights.
 __global__ void k_lv_coarse_of(const int32_t* __restrict__ cl, const int32_t* __restrict__ cid,
-                               int64_t V, int32_t* __restrict__ cv, int32_t* __restrict__ mcnt) {
+                               int64_t V, const long long* __restrict__ off,
+                               const long long* __restrict__ self, int32_t* __restrict__ cv,
+                               long long* __restrict__ bound, long long* __restrict__ self2) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t c = cid[cl[i]];
     cv[i] = c;
-    atomicAdd(&mcnt[c], 1);
+    const long long d = off[i + 1] - off[i], sl = self[i];
+    if (d) atomic_add_i64(&bound[c], d);
+    if (sl) atomic_add_i64(&self2[c], sl);
   }
 }
 
-__global__ void k_lv_members(const int32_t* __restrict__ cv, int64_t V,
-                             const int32_t* __restrict__ moff, int32_t* __restrict__ mfill,
-                             int32_t* __restrict__ members) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t c = cv[i];
-    members[moff[c] + atomicAdd(&mfill[c], 1)] = (int32_t)i;
-  }
-}
-
-// Per coarse vertex: the sum of its members' degrees in the edge lists (a
-// bound on its coarse degree) and of their self-loop weights.
-__global__ void k_lv_coarse_bounds(const int32_t* __restrict__ members, const int32_t* __restrict__ moff,
-                                   int32_t V2, const long long* __restrict__ off,
-                                   const long long* __restrict__ self,
-                                   long long* __restrict__ bound, long long* __restrict__ self2) {
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < V2; c += nw) {
-    long long d = 0, sl = 0;
-    for (int32_t x = moff[c] + lane_id(); x < moff[c + 1]; x += 32) {
-      const int32_t i = members[x];
-      d += off[i + 1] - off[i];
-      sl += self[i];
-    }
-    d = warp_sum(d);
-    sl = warp_sum(sl);
-    if (lane_id() == 0) {
-      bound[c] = d;
-      self2[c] = sl;
-    }
-  }
-}
-
+// Table sizes (powers of two >= 2 bound + 2) and the largest.
 __global__ void k_lv_table_sizes(const long long* __restrict__ bound, int32_t V2,
-                                 long long* __restrict__ tsz) {
+                                 int64_t* __restrict__ tsz, unsigned long long* __restrict__ most) {
+  unsigned long long mx = 0;
   for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < V2; c += gridDim.x * blockDim.x) {
     long long s = 4;
     while (s < 2 * bound[c] + 2) s <<= 1;
     tsz[c] = s;
+    mx = (unsigned long long)s > mx ? (unsigned long long)s : mx;
   }
+  mx = warp_max(mx);
+  if (lane_id() == 0 && mx) atomicMax(most, mx);
 }
 
-// One thread per member edge (in member order; mpre = exclusive prefix of
-// the members' degrees): an edge to another coarse vertex is added to the
-// coarse vertex's table, an edge inside it to its internal weight.
-__global__ void k_lv_agg_insert(const int32_t* __restrict__ members, const long long* __restrict__ mpre,
-                                int64_t V, const int32_t* __restrict__ cv,
+// The largest x in [lo, hi] with first[x] <= y (first non-decreasing).
+template <typename I>
+__device__ __forceinline__ I owner_in(const long long* first, I lo, I hi, long long y) {
+  while (lo < hi) {
+    const I mid = lo + (hi - lo + 1) / 2;
+    if (first[mid] <= y) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// Positions [t0, t1) of a tile and the range of owners that can hold them: two
+// searches per block of LV_TILE positions instead of one per position (19
+// dependent loads each).
+constexpr int LV_TILE = 2048;
+struct OwnerTile {
+  long long t0, t1;
+  int64_t lo, hi;
+};
+__device__ __forceinline__ OwnerTile owner_tile(const long long* first, int64_t owners,
+                                                long long tile, long long total, int64_t* s_own) {
+  OwnerTile o;
+  o.t0 = tile * LV_TILE;
+  o.t1 = o.t0 + LV_TILE < total ? o.t0 + LV_TILE : total;
+  __syncthreads();
+  if (threadIdx.x < 2)
+    s_own[threadIdx.x] = owner_in<int64_t>(first, 0, owners - 1, threadIdx.x ? o.t1 - 1 : o.t0);
+  __syncthreads();
+  o.lo = s_own[0];
+  o.hi = s_own[1];
+  return o;
+}
+
+// One thread per edge: an edge to another coarse vertex is added to the coarse
+// vertex's table, an edge inside it to its internal weight.
+__global__ void k_lv_agg_insert(int64_t V, long long E, const int32_t* __restrict__ cv,
                                 const long long* __restrict__ off, const int32_t* __restrict__ adj,
                                 const long long* __restrict__ aw, const long long* __restrict__ toff,
                                 int32_t* __restrict__ tkey, long long* __restrict__ tval,
                                 long long* __restrict__ internal, int32_t* status) {
-  const long long total = mpre[V];
-  for (long long y = (long long)blockIdx.x * blockDim.x + threadIdx.x; y < total;
-       y += (long long)gridDim.x * blockDim.x) {
-    int64_t a = 0, b = V - 1;  // largest x with mpre[x] <= y
-    while (a < b) {
-      const int64_t mid = (a + b + 1) >> 1;
-      if (mpre[mid] <= y) a = mid;
-      else b = mid - 1;
-    }
-    const int32_t i = members[a];
-    const long long q = off[i] + (y - mpre[a]);
-    const int32_t ci = cv[i], cj = cv[adj[q]];
-    if (ci == cj) {
-      atomic_add_i64(&internal[ci], aw[q]);
-    } else {
-      const long long tb = toff[ci];
-      const uint32_t mask = (uint32_t)(toff[ci + 1] - tb) - 1;
-      if (!table_add(tkey + tb, tval + tb, mask, cj, aw[q])) dev_fail(status, DEV_HASH_FULL);
+  __shared__ int64_t s_own[2];
+  for (long long tile = blockIdx.x; tile * LV_TILE < E; tile += gridDim.x) {
+    const OwnerTile o = owner_tile(off, V, tile, E, s_own);
+    for (long long q = o.t0 + threadIdx.x; q < o.t1; q += blockDim.x) {
+      const int64_t i = owner_in<int64_t>(off, o.lo, o.hi, q);
+      const int32_t ci = cv[i], cj = cv[adj[q]];
+      if (ci == cj) {
+        atomic_add_i64(&internal[ci], aw[q]);
+      } else {
+        const long long tb = toff[ci];
+        const uint32_t mask = (uint32_t)(toff[ci + 1] - tb) - 1;
+        if (!table_add(tkey + tb, tval + tb, mask, cj, aw[q])) dev_fail(status, DEV_HASH_FULL);
+      }
     }
   }
-}
-
-// The coarse vertex owning table slot s: the largest c with toff[c] <= s.
-__device__ __forceinline__ int32_t table_owner(const long long* toff, int32_t V2, long long s) {
-  int32_t a = 0, b = V2 - 1;
-  while (a < b) {
-    const int32_t mid = (a + b + 1) >> 1;
-    if (toff[mid] <= s) a = mid;
-    else b = mid - 1;
-  }
-  return a;
 }
 
 // Distinct neighbours of every coarse vertex: one thread per table slot over
@@ -485,14 +559,16 @@ __device__ __forceinline__ int32_t table_owner(const long long* toff, int32_t V2
 // count for the same coarse vertex share one atomic.
 __global__ void k_lv_agg_count(const long long* __restrict__ toff, int32_t V2,
                                const int32_t* __restrict__ tkey, int32_t* __restrict__ deg2) {
+  __shared__ int64_t s_own[2];
   const long long total = toff[V2];
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long b = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < total;
-       b += stride) {
-    const long long s = b + lane_id();
-    const bool used = s < total && tkey[s] != LV_EMPTY;
-    const int32_t c = used ? table_owner(toff, V2, s) : -1;
-    warp_claim_slot(deg2, c, __ballot_sync(FULL, used));
+  for (long long tile = blockIdx.x; tile * LV_TILE < total; tile += gridDim.x) {
+    const OwnerTile o = owner_tile(toff, V2, tile, total, s_own);
+    for (long long b = o.t0 + (threadIdx.x & ~31); b < o.t1; b += blockDim.x) {
+      const long long s = b + lane_id();
+      const bool used = s < o.t1 && tkey[s] != LV_EMPTY;
+      const int32_t c = used ? (int32_t)owner_in<int64_t>(toff, o.lo, o.hi, s) : -1;
+      warp_claim_slot(deg2, c, __ballot_sync(FULL, used));
+    }
   }
 }
 
@@ -503,19 +579,21 @@ __global__ void k_lv_agg_write(const long long* __restrict__ toff, int32_t V2,
                                const int32_t* __restrict__ tkey, const long long* __restrict__ tval,
                                const long long* __restrict__ off2, int32_t* __restrict__ adj2,
                                long long* __restrict__ aw2, int32_t* __restrict__ fill) {
+  __shared__ int64_t s_own[2];
   const long long total = toff[V2];
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long b = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < total;
-       b += stride) {
-    const long long s = b + lane_id();
-    const int32_t key = s < total ? tkey[s] : LV_EMPTY;
-    const bool used = key != LV_EMPTY;
-    const int32_t c = used ? table_owner(toff, V2, s) : -1;
-    const int32_t slot = warp_claim_slot(fill, c, __ballot_sync(FULL, used));
-    if (used) {
-      const long long pos = off2[c] + slot;
-      adj2[pos] = key;
-      aw2[pos] = tval[s];
+  for (long long tile = blockIdx.x; tile * LV_TILE < total; tile += gridDim.x) {
+    const OwnerTile o = owner_tile(toff, V2, tile, total, s_own);
+    for (long long b = o.t0 + (threadIdx.x & ~31); b < o.t1; b += blockDim.x) {
+      const long long s = b + lane_id();
+      const int32_t key = s < o.t1 ? tkey[s] : LV_EMPTY;
+      const bool used = key != LV_EMPTY;
+      const int32_t c = used ? (int32_t)owner_in<int64_t>(toff, o.lo, o.hi, s) : -1;
+      const int32_t slot = warp_claim_slot(fill, c, __ballot_sync(FULL, used));
+      if (used) {
+        const long long pos = off2[c] + slot;
+        adj2[pos] = key;
+        aw2[pos] = tval[s];
+      }
     }
   }
 }
@@ -564,7 +642,7 @@ void lv_aggregate(const Ctx& cx, const LvGraph& g, const int32_t* cl, LvGraph& o
                   DBuf<int32_t>& cv) {
   const int64_t V = g.V;
   const int gV = grid_for(V, 256, cx.num_sms, 8);
-  DBuf<int32_t> flag, cid, mcnt, moff, mfill, members;
+  DBuf<int32_t> flag, cid;
   flag.alloc(&cx.alloc, (size_t)V + 1);
   cid.alloc(&cx.alloc, (size_t)V + 1);
   HG_CUDA(cudaMemsetAsync(flag.p, 0, flag.bytes(), cx.stream));
@@ -573,67 +651,49 @@ void lv_aggregate(const Ctx& cx, const LvGraph& g, const int32_t* cl, LvGraph& o
   scan_exclusive_i32(cx, flag.p, cid.p, V, cid.p + V);
   const int32_t V2 = read_i32(cx, cid.p + V);
   cv.alloc(&cx.alloc, (size_t)V);
-  mcnt.alloc(&cx.alloc, (size_t)V2 + 1);
-  moff.alloc(&cx.alloc, (size_t)V2 + 1);
-  mfill.alloc(&cx.alloc, (size_t)V2 + 1);
-  members.alloc(&cx.alloc, (size_t)V);
-  HG_CUDA(cudaMemsetAsync(mcnt.p, 0, mcnt.bytes(), cx.stream));
-  HG_CUDA(cudaMemsetAsync(mfill.p, 0, mfill.bytes(), cx.stream));
-  k_lv_coarse_of<<<gV, 256, 0, cx.stream>>>(cl, cid.p, V, cv.p, mcnt.p);
-  check_launch("lv_coarse_of");
-  scan_exclusive_i32(cx, mcnt.p, moff.p, V2, moff.p + V2);
-  k_lv_members<<<gV, 256, 0, cx.stream>>>(cv.p, V, moff.p, mfill.p, members.p);
-  check_launch("lv_members");
-  // member degrees along the member list, table offsets per coarse vertex
-  DBuf<int32_t> mdeg;
-  DBuf<long long> mpre, bound, tsz, toff, internal;
-  mdeg.alloc(&cx.alloc, (size_t)V + 1);
-  mpre.alloc(&cx.alloc, (size_t)V + 1);
-  k_lv_list_sizes<<<gV, 256, 0, cx.stream>>>(members.p, (int32_t)V, g.off.p, mdeg.p, nullptr);
-  check_launch("lv_member_degrees");
-  scan_exclusive_i32_to_i64(cx, mdeg.p, reinterpret_cast<int64_t*>(mpre.p), V,
-                            reinterpret_cast<int64_t*>(mpre.p) + V);
+  DBuf<long long> bound, tsz, toff, internal;
+  DBuf<unsigned long long> most;
   bound.alloc(&cx.alloc, (size_t)V2 + 1);
   tsz.alloc(&cx.alloc, (size_t)V2 + 1);
   toff.alloc(&cx.alloc, (size_t)V2 + 1);
   internal.alloc(&cx.alloc, (size_t)V2 + 1);
+  most.alloc(&cx.alloc, 1);
   out.self.alloc(&cx.alloc, (size_t)V2 + 1);
+  HG_CUDA(cudaMemsetAsync(bound.p, 0, bound.bytes(), cx.stream));
+  HG_CUDA(cudaMemsetAsync(out.self.p, 0, out.self.bytes(), cx.stream));
   HG_CUDA(cudaMemsetAsync(internal.p, 0, internal.bytes(), cx.stream));
-  const int gC = grid_for(V2, 8, cx.num_sms, 16);
-  k_lv_coarse_bounds<<<gC, 256, 0, cx.stream>>>(members.p, moff.p, V2, g.off.p, g.self.p, bound.p,
-                                              out.self.p);
-  check_launch("lv_coarse_bounds");
-  k_lv_table_sizes<<<grid_for(V2, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(bound.p, V2, tsz.p);
+  HG_CUDA(cudaMemsetAsync(most.p, 0, most.bytes(), cx.stream));
+  k_lv_coarse_of<<<gV, 256, 0, cx.stream>>>(cl, cid.p, V, g.off.p, g.self.p, cv.p, bound.p,
+                                            out.self.p);
+  check_launch("lv_coarse_of");
+  k_lv_table_sizes<<<grid_for(V2, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
+      bound.p, V2, reinterpret_cast<int64_t*>(tsz.p), most.p);
   check_launch("lv_table_sizes");
-  std::vector<long long> htsz((size_t)V2);
-  HG_CUDA(cudaMemcpyAsync(htsz.data(), tsz.p, sizeof(long long) * (size_t)V2,
-                          cudaMemcpyDeviceToHost, cx.stream));
+  scan_exclusive_i64(cx, reinterpret_cast<const int64_t*>(tsz.p),
+                     reinterpret_cast<int64_t*>(toff.p), V2,
+                     reinterpret_cast<int64_t*>(toff.p) + V2);
+  long long tslots = 0;
+  unsigned long long hmost = 0;
   wait_stream(cx);
+  HG_CUDA(cudaMemcpyAsync(&tslots, toff.p + V2, sizeof(tslots), cudaMemcpyDeviceToHost, cx.stream));
+  HG_CUDA(cudaMemcpyAsync(&hmost, most.p, sizeof(hmost), cudaMemcpyDeviceToHost, cx.stream));
   check_status(cx);
-  std::vector<long long> htoff((size_t)V2 + 1, 0);
-  for (int32_t c = 0; c < V2; ++c) {
-    if (htsz[c] > (1ll << 31)) throw HgError(HG_ERR_UNSUPPORTED, "coarse vertex degree too large");
-    htoff[c + 1] = htoff[c] + htsz[c];
-  }
-  HG_CUDA(cudaMemcpyAsync(toff.p, htoff.data(), sizeof(long long) * ((size_t)V2 + 1),
-                          cudaMemcpyHostToDevice, cx.stream));
-  const long long tslots = htoff[V2];
+  if (hmost > (1ull << 31)) throw HgError(HG_ERR_UNSUPPORTED, "coarse vertex degree too large");
   DBuf<int32_t> tkey;
   DBuf<long long> tval;
   tkey.alloc(&cx.alloc, (size_t)std::max<long long>(tslots, 1));
   tval.alloc(&cx.alloc, (size_t)std::max<long long>(tslots, 1));
   HG_CUDA(cudaMemsetAsync(tkey.p, 0xff, tkey.bytes(), cx.stream));
   HG_CUDA(cudaMemsetAsync(tval.p, 0, tval.bytes(), cx.stream));
-  k_lv_agg_insert<<<grid_for(g.E, 256, cx.num_sms, 16), 256, 0, cx.stream>>>(
-      members.p, mpre.p, V, cv.p, g.off.p, g.adj.p, g.aw.p, toff.p, tkey.p, tval.p, internal.p,
-      cx.d_status);
+  k_lv_agg_insert<<<grid_for(g.E, LV_TILE, cx.num_sms, 8), 256, 0, cx.stream>>>(
+      V, g.E, cv.p, g.off.p, g.adj.p, g.aw.p, toff.p, tkey.p, tval.p, internal.p, cx.d_status);
   check_launch("lv_agg_insert");
   DBuf<int32_t> deg2, fill2;
   deg2.alloc(&cx.alloc, (size_t)V2 + 1);
   fill2.alloc(&cx.alloc, (size_t)V2 + 1);
   HG_CUDA(cudaMemsetAsync(fill2.p, 0, fill2.bytes(), cx.stream));
   HG_CUDA(cudaMemsetAsync(deg2.p, 0, deg2.bytes(), cx.stream));
-  const int gT = grid_for(tslots, 256, cx.num_sms, 8);
+  const int gT = grid_for(tslots, LV_TILE, cx.num_sms, 8);
   k_lv_agg_count<<<gT, 256, 0, cx.stream>>>(toff.p, V2, tkey.p, deg2.p);
   check_launch("lv_agg_count");
   out.V = V2;
@@ -664,7 +724,7 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   DBuf<int32_t> cnt, fill, koff, list, mv_v, mv_to, words, ldeg, tsize;
   DBuf<long long> lpre, toff;
   DBuf<unsigned long long> moved;
-  const int nkeys = 2 * S;
+  const int nkeys = LV_CLASSES * S;
   cnt.alloc(&cx.alloc, (size_t)nkeys);
   fill.alloc(&cx.alloc, (size_t)nkeys);
   koff.alloc(&cx.alloc, (size_t)nkeys + 1);
@@ -677,6 +737,8 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   lpre.alloc(&cx.alloc, (size_t)V + 1);
   toff.alloc(&cx.alloc, (size_t)V + 1);
   moved.alloc(&cx.alloc, 1);
+  DBuf<long long> bounds;
+  bounds.alloc(&cx.alloc, 2 * ((size_t)nkeys + 1));
   DBuf<int32_t> tkey;
   DBuf<long long> tval;
   size_t tcap = 0;
@@ -705,29 +767,26 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
     k_lv_scatter<<<gV, 256, 0, cx.stream>>>(g.off.p, V, seed, level, round, S, koff.p, fill.p,
                                             list.p);
     check_launch("lv_scatter");
-    std::vector<int32_t> hkoff((size_t)nkeys + 1);
-    HG_CUDA(cudaMemcpyAsync(hkoff.data(), koff.p, sizeof(int32_t) * hkoff.size(),
-                            cudaMemcpyDeviceToHost, cx.stream));
+    // degrees and table sizes along the list, class-3 tables per sub-round
+    k_lv_list_sizes<<<gV, 256, 0, cx.stream>>>(list.p, koff.p + nkeys, (int32_t)V, g.off.p, ldeg.p,
+                                               tsize.p);
+    check_launch("lv_list_sizes");
+    scan_exclusive_i32_to_i64(cx, ldeg.p, reinterpret_cast<int64_t*>(lpre.p), V,
+                              reinterpret_cast<int64_t*>(lpre.p) + V);
+    scan_exclusive_i32_to_i64(cx, tsize.p, reinterpret_cast<int64_t*>(toff.p), V,
+                              reinterpret_cast<int64_t*>(toff.p) + V);
+    k_lv_bounds<<<1, 256, 0, cx.stream>>>(koff.p, nkeys, toff.p, bounds.p);
+    check_launch("lv_bounds");
+    std::vector<long long> hb(2 * ((size_t)nkeys + 1));
     wait_stream(cx);
+    HG_CUDA(cudaMemcpyAsync(hb.data(), bounds.p, sizeof(long long) * hb.size(),
+                            cudaMemcpyDeviceToHost, cx.stream));
     check_status(cx);
-    const int32_t listed = hkoff[nkeys];
-    // degrees and table sizes along the list; class-1 tables per sub-round
-    if (listed > 0) {
-      k_lv_list_sizes<<<grid_for(listed, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
-          list.p, listed, g.off.p, ldeg.p, tsize.p);
-      check_launch("lv_list_sizes");
-    }
-    scan_exclusive_i32_to_i64(cx, ldeg.p, reinterpret_cast<int64_t*>(lpre.p), listed,
-                              reinterpret_cast<int64_t*>(lpre.p) + listed);
-    scan_exclusive_i32_to_i64(cx, tsize.p, reinterpret_cast<int64_t*>(toff.p), listed,
-                              reinterpret_cast<int64_t*>(toff.p) + listed);
-    std::vector<long long> htoff((size_t)listed + 1);
-    HG_CUDA(cudaMemcpyAsync(htoff.data(), toff.p, sizeof(long long) * htoff.size(),
-                            cudaMemcpyDeviceToHost, cx.stream));
-    wait_stream(cx);
+    const long long* hkoff = hb.data();
+    const long long* htoff = hb.data() + nkeys + 1;
     size_t need = 1;
     for (int s = 0; s < S; ++s)
-      need = std::max<size_t>(need, (size_t)(htoff[hkoff[2 * s + 2]] - htoff[hkoff[2 * s + 1]]));
+      need = std::max<size_t>(need, (size_t)(htoff[LV_CLASSES * s + 4] - htoff[LV_CLASSES * s + 3]));
     if (need > tcap) {
       tkey.alloc(&cx.alloc, need);
       tval.alloc(&cx.alloc, need);
@@ -737,19 +796,33 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
     }
     for (int s = 0; s < S; ++s) {
       A.words = words.p + 4 * s;
-      const int32_t lo0 = hkoff[2 * s], hi0 = hkoff[2 * s + 1], hi1 = hkoff[2 * s + 2];
-      if (hi0 > lo0) {
-        k_lv_small<<<grid_for(hi0 - lo0, LV_WARPS, cx.num_sms, 8), LV_WARPS * 32, 0, cx.stream>>>(
-            A, lo0, hi0);
+      int32_t at[LV_CLASSES + 1];
+      for (int c = 0; c <= LV_CLASSES; ++c) at[c] = (int32_t)hkoff[LV_CLASSES * s + c];
+      if (at[1] > at[0]) {
+        k_lv_lanes<LV_GROUP><<<grid_for(at[1] - at[0], LV_WARPS * (32 / LV_GROUP), cx.num_sms, 8),
+                               LV_WARPS * 32, 0, cx.stream>>>(A, at[0], at[1]);
+        check_launch("lv_lanes");
+        lc.launches += 1;
+      }
+      if (at[2] > at[1]) {
+        k_lv_lanes<LV_LANES><<<grid_for(at[2] - at[1], LV_WARPS, cx.num_sms, 8), LV_WARPS * 32, 0,
+                               cx.stream>>>(A, at[1], at[2]);
+        check_launch("lv_lanes");
+        lc.launches += 1;
+      }
+      if (at[3] > at[2]) {
+        k_lv_small<<<grid_for(at[3] - at[2], LV_WARPS, cx.num_sms, 8), LV_WARPS * 32, 0,
+                     cx.stream>>>(A, at[2], at[3]);
         check_launch("lv_small");
         lc.launches += 1;
       }
-      if (hi1 > hi0) {
-        k_lv_big_insert<<<cx.num_sms * 8, 256, 0, cx.stream>>>(A, hi0, hi1, lpre.p, toff.p,
-                                                               htoff[hi0], tsize.p, tkey.p, tval.p);
+      if (at[4] > at[3]) {
+        const long long tbase = htoff[LV_CLASSES * s + 3];
+        k_lv_big_insert<<<cx.num_sms * 8, 256, 0, cx.stream>>>(A, at[3], at[4], lpre.p, toff.p,
+                                                               tbase, tsize.p, tkey.p, tval.p);
         check_launch("lv_big_insert");
-        k_lv_big_argmax<<<grid_for(hi1 - hi0, 1, cx.num_sms, 8), LV_ARGMAX_THREADS, 0,
-                          cx.stream>>>(A, hi0, hi1, toff.p, htoff[hi0], tsize.p, tkey.p, tval.p);
+        k_lv_big_argmax<<<grid_for(at[4] - at[3], 1, cx.num_sms, 8), LV_ARGMAX_THREADS, 0,
+                          cx.stream>>>(A, at[3], at[4], toff.p, tbase, tsize.p, tkey.p, tval.p);
         check_launch("lv_big_argmax");
         lc.launches += 2;
       }

@@ -26,8 +26,8 @@ int64_t now_ns() {
 
 // Device bytes a job may hold at its peak: the level hierarchy (about eight
 // times the input's pins, net and node arrays on a Zipf(2.2) n = m = 1e6 input), the
-// clustering temporaries of the finest level (pin-cluster map: 12 bytes per
-// slot, 4 slots per pin), Phi (m x k int32) and Lambda, plus a fixed margin.
+// clustering temporaries of the finest level (records, net metadata and grouped
+// pins: under 64 bytes per pin), Phi (m x k int32) and Lambda, plus a fixed margin.
 int64_t estimate_bytes(const hg_job& j, int64_t p) {
   const int64_t n = j.n, m = j.m, k = j.k;
   return 8 * (12 * p + 16 * m + 24 * n) + 64 * p + 4 * m * k + 8 * m + (32ll << 20);

