@@ -626,9 +626,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
       L.ioff.p, L.inets.p, imeta.p, rterm.p, n, L.graph, wof.p, rend.p, max_r.p);
   check_launch("node_work");
   unsigned long long hmax[3];
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(hmax, max_r.p, sizeof(hmax), cudaMemcpyDeviceToHost, cx.stream));
-  check_status(cx);
+  read_back(cx, hmax, max_r.p, sizeof(hmax));
   const unsigned long long hmax_r = hmax[0];
   // the pins the rating works on
   const bool grouped =
@@ -660,10 +658,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   if (cx.launches) *cx.launches += 5;
 
   std::vector<int32_t> hcount(nkeys);
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(hcount.data(), kcount.p, sizeof(int32_t) * nkeys, cudaMemcpyDeviceToHost,
-                          cx.stream));
-  check_status(cx);
+  read_back(cx, hcount.data(), kcount.p, sizeof(int32_t) * nkeys);
   std::vector<int32_t> hoff(nkeys + 1, 0);
   for (int i = 0; i < nkeys; ++i) hoff[i + 1] = hoff[i] + hcount[i];
   // per listed node {u, ioff[u], rend[u], c(u)}, for the rating walks
@@ -876,9 +871,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   HG_CUDA(cudaMemcpy2DAsync(cw_out.p, sizeof(int32_t), cst.p, sizeof(int2), sizeof(int32_t),
                             (size_t)n, cudaMemcpyDeviceToDevice, cx.stream));
   unsigned long long hs[ST_TOTAL];
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, cx.stream));
-  check_status(cx);
+  read_back(cx, hs, stats.p, sizeof(hs));
   for (int c = 0; c < NCLASS; ++c) {
     const unsigned long long* h = hs + c * ST_WORDS;
     cc.rating_pin_visits += (int64_t)h[ST_PINS];

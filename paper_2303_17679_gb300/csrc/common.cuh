@@ -302,9 +302,14 @@ void scan_exclusive_i32_to_i64(const Ctx& cx, const int32_t* in, int64_t* out, i
                                int64_t* d_total);
 void scan_exclusive_i64(const Ctx& cx, const int64_t* in, int64_t* out, int64_t n,
                         int64_t* d_total);
+void scan_exclusive_i64(const Ctx& cx, const int64_t* in, int64_t* out, int64_t n,
+                        int64_t* d_total);
 
-// Copies a device scalar to the host (synchronizes the stream) and checks
-// the device status word.
+// Copies `bytes` of device memory to the host once the stream's work is done
+// (synchronizes the stream) and checks the device status word; read_status
+// returns the status instead.
+void read_back(const Ctx& cx, void* dst, const void* src, size_t bytes);
+int32_t read_status(const Ctx& cx, void* dst, const void* src, size_t bytes);
 int32_t read_i32(const Ctx& cx, const int32_t* d);
 int64_t read_i64(const Ctx& cx, const int64_t* d);
 void check_status(const Ctx& cx);

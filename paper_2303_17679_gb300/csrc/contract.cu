@@ -441,9 +441,7 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
   k_classify_nets<<<gm, 256, 0, cx.stream>>>(L.eoff.p, m, lists.p, counts.p);
   check_launch("classify_nets");
   int32_t hc[4];
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(hc, counts.p, sizeof(hc), cudaMemcpyDeviceToHost, cx.stream));
-  check_status(cx);
+  read_back(cx, hc, counts.p, sizeof(hc));
   if (hc[0])
     k_remap_small<<<grid_for(hc[0], 128, cx.num_sms, 16), 128, 0, cx.stream>>>(
         lists.p, hc[0], L.eoff.p, L.pins.p, L.map.p, fingerprint_bits, tpins.p, tsize.p, fp.p);
@@ -520,9 +518,7 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
   scan_exclusive_i32(cx, kflag.p, newid.p, m, d_tot.p);      // keep flag -> new id
   scan_exclusive_i32(cx, ksize.p, ksize.p, m, d_tot.p + 1);  // kept size -> coarse offset
   int32_t tot[2];
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(tot, d_tot.p, sizeof(tot), cudaMemcpyDeviceToHost, cx.stream));
-  check_status(cx);
+  read_back(cx, tot, d_tot.p, sizeof(tot));
   out.m = tot[0];
   out.p = tot[1];
   out.eoff.alloc(&cx.alloc, (size_t)out.m + 1);

@@ -1123,9 +1123,7 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
   }
   launch_persistent(cx, kernel, blocks, LP_THREADS, bytes, A.cluster, A);
   unsigned long long hres[LR_WORDS];
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(hres, A.res, sizeof(hres), cudaMemcpyDeviceToHost, cx.stream));
-  check_status(cx);
+  read_back(cx, hres, A.res, sizeof(hres));
   res.passes = (int)hres[LR_PASSES];
   res.moves = (int64_t)hres[LR_MOVES];
   res.objective = (int64_t)hres[LR_OBJECTIVE];

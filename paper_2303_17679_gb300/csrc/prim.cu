@@ -1,6 +1,7 @@
 // Data-parallel primitives: exclusive prefix sums, fills, scalar readback.
 // The prefix sums are the "parallel prefix sum operations" the contraction
 // algorithm relies on (Sec. 4.2), written here without CUB.
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -215,36 +216,76 @@ void wait_stream(const Ctx& cx) {
   }
 }
 
-void check_status(const Ctx& cx) {
-  wait_stream(cx);
-  int32_t st = 0;
-  HG_CUDA(cudaMemcpyAsync(&st, cx.d_status, sizeof(st), cudaMemcpyDeviceToHost, cx.stream));
-  HG_CUDA(cudaStreamSynchronize(cx.stream));
-  if (st != DEV_OK) {
-    int32_t zero = 0;
-    cudaMemcpy(cx.d_status, &zero, sizeof(zero), cudaMemcpyHostToDevice);
-    switch (st) {
-      case DEV_TIMEOUT: throw HgError(HG_ERR_TIMEOUT, "a bounded device wait gave up");
-      case DEV_BAD_INPUT: throw HgError(HG_ERR_INVALID, "device-side input validation failed");
-      case DEV_HASH_FULL: throw HgError(HG_ERR_CUDA, "internal: hash table full");
-      default: throw HgError(HG_ERR_CUDA, "internal: device capacity exceeded");
-    }
+namespace {
+
+// Page-locked words of the calling thread that readbacks go through: copies to
+// them are queued behind the kernels like any other work, so a readback costs
+// one wait (a copy to pageable memory waits for the stream by itself, and one
+// more for the status word).  Freed when the thread ends.
+constexpr size_t STAGE_BYTES = 4096;
+
+struct Stage {
+  unsigned char* p = nullptr;
+  ~Stage() {
+    if (p) cudaFreeHost(p);
+  }
+};
+
+unsigned char* stage() {
+  thread_local Stage s;
+  if (!s.p) {
+    void* q = nullptr;
+    HG_CUDA(cudaHostAlloc(&q, STAGE_BYTES, cudaHostAllocPortable));
+    s.p = static_cast<unsigned char*>(q);
+  }
+  return s.p;
+}
+
+void throw_status(const Ctx& cx, int32_t st) {
+  if (st == DEV_OK) return;
+  int32_t zero = 0;
+  cudaMemcpy(cx.d_status, &zero, sizeof(zero), cudaMemcpyHostToDevice);
+  switch (st) {
+    case DEV_TIMEOUT: throw HgError(HG_ERR_TIMEOUT, "a bounded device wait gave up");
+    case DEV_BAD_INPUT: throw HgError(HG_ERR_INVALID, "device-side input validation failed");
+    case DEV_HASH_FULL: throw HgError(HG_ERR_CUDA, "internal: hash table full");
+    default: throw HgError(HG_ERR_CUDA, "internal: device capacity exceeded");
   }
 }
 
+}  // namespace
+
+int32_t read_status(const Ctx& cx, void* dst, const void* src, size_t bytes) {
+  unsigned char* st = stage();
+  const bool staged = bytes + 16 <= STAGE_BYTES;
+  HG_CUDA(cudaMemcpyAsync(st, cx.d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, cx.stream));
+  if (bytes > 0 && staged)
+    HG_CUDA(cudaMemcpyAsync(st + 16, src, bytes, cudaMemcpyDeviceToHost, cx.stream));
+  wait_stream(cx);
+  if (bytes > 0 && staged) {
+    std::memcpy(dst, st + 16, bytes);
+  } else if (bytes > 0) {
+    HG_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, cx.stream));
+    HG_CUDA(cudaStreamSynchronize(cx.stream));
+  }
+  return *reinterpret_cast<const int32_t*>(st);
+}
+
+void read_back(const Ctx& cx, void* dst, const void* src, size_t bytes) {
+  throw_status(cx, read_status(cx, dst, src, bytes));
+}
+
+void check_status(const Ctx& cx) { read_back(cx, nullptr, nullptr, 0); }
+
 int32_t read_i32(const Ctx& cx, const int32_t* d) {
   int32_t v = 0;
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(&v, d, sizeof(v), cudaMemcpyDeviceToHost, cx.stream));
-  check_status(cx);
+  read_back(cx, &v, d, sizeof(v));
   return v;
 }
 
 int64_t read_i64(const Ctx& cx, const int64_t* d) {
   int64_t v = 0;
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(&v, d, sizeof(v), cudaMemcpyDeviceToHost, cx.stream));
-  check_status(cx);
+  read_back(cx, &v, d, sizeof(v));
   return v;
 }
 

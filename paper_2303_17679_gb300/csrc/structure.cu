@@ -255,8 +255,7 @@ bool level_is_graph(const Ctx& cx, const Level& L) {
   check_launch("net_size_range");
   if (cx.launches) *cx.launches += 1;
   int32_t h[2];
-  HG_CUDA(cudaMemcpyAsync(h, range.p, sizeof(h), cudaMemcpyDeviceToHost, cx.stream));
-  HG_CUDA(cudaStreamSynchronize(cx.stream));
+  read_back(cx, h, range.p, sizeof(h));
   return h[0] == 2 && h[1] == 2;
 }
 
@@ -339,11 +338,7 @@ bool distinct_pins(const Ctx& cx, const Level& L) {
                                                   cx.d_status);
     check_launch("distinct_big");
   }
-  int32_t st = 0;
-  wait_stream(cx);
-  HG_CUDA(cudaMemcpyAsync(&st, cx.d_status, sizeof(st), cudaMemcpyDeviceToHost, cx.stream));
-  HG_CUDA(cudaStreamSynchronize(cx.stream));
-  if (st != DEV_OK) {
+  if (read_status(cx, nullptr, nullptr, 0) != DEV_OK) {
     int32_t zero = 0;
     HG_CUDA(cudaMemcpy(cx.d_status, &zero, sizeof(zero), cudaMemcpyHostToDevice));
     return false;
@@ -358,10 +353,7 @@ bool validate_pins_device(const Ctx& cx, const Level& L) {
     k_validate_pins<<<grid_for(L.p, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(L.pins.p, L.p, L.n,
                                                                              cx.d_status);
     check_launch("validate_pins");
-    int32_t st = 0;
-    HG_CUDA(cudaMemcpyAsync(&st, cx.d_status, sizeof(st), cudaMemcpyDeviceToHost, cx.stream));
-    HG_CUDA(cudaStreamSynchronize(cx.stream));
-    if (st != DEV_OK) {
+    if (read_status(cx, nullptr, nullptr, 0) != DEV_OK) {
       int32_t zero = 0;
       HG_CUDA(cudaMemcpy(cx.d_status, &zero, sizeof(zero), cudaMemcpyHostToDevice));
       return false;
@@ -389,11 +381,7 @@ bool validate_level_device(const Ctx& cx, const Level& L, int64_t* total_node_w,
                                                                            cx.d_status, sums.p);
   check_launch("validate_nodes");
   unsigned long long h[2] = {0, 0};
-  HG_CUDA(cudaMemcpyAsync(h, sums.p, sizeof(h), cudaMemcpyDeviceToHost, cx.stream));
-  int32_t st = 0;
-  HG_CUDA(cudaMemcpyAsync(&st, cx.d_status, sizeof(st), cudaMemcpyDeviceToHost, cx.stream));
-  HG_CUDA(cudaStreamSynchronize(cx.stream));
-  if (st != DEV_OK) {
+  if (read_status(cx, h, sums.p, sizeof(h)) != DEV_OK) {
     int32_t zero = 0;
     HG_CUDA(cudaMemcpy(cx.d_status, &zero, sizeof(zero), cudaMemcpyHostToDevice));
     return false;
