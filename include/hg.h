@@ -274,8 +274,8 @@ int hg_gain_table(hg_t* h, int32_t level, int32_t k, const int32_t* part, int64_
 /* Moves move_nodes[i] to move_targets[i] for all i at once (every node at
  * most once, each target in [0, k) and not the node's block), updating
  * `part` in place and the gain table (benefit, penalty: the table of `part`
- * on entry, as hg_gain_table writes it) with the update rules of Sec. 6.2
- * applied concurrently; afterwards the benefits of the moved nodes are
+ * on entry, as hg_gain_table writes it) by what the update rules of Sec. 6.2
+ * add up to over all moves; afterwards the benefits of the moved nodes are
  * recomputed (Sec. 6.2, "Benefit Peculiarities"), so the table equals
  * hg_gain_table of the new partition.  Same arguments and errors as
  * hg_gain_table plus those of hg_recalculate_gains for the moves (nothing

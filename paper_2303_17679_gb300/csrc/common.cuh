@@ -302,8 +302,6 @@ void scan_exclusive_i32_to_i64(const Ctx& cx, const int32_t* in, int64_t* out, i
                                int64_t* d_total);
 void scan_exclusive_i64(const Ctx& cx, const int64_t* in, int64_t* out, int64_t n,
                         int64_t* d_total);
-void scan_exclusive_i64(const Ctx& cx, const int64_t* in, int64_t* out, int64_t n,
-                        int64_t* d_total);
 
 // Copies `bytes` of device memory to the host once the stream's work is done
 // (synchronizes the stream) and checks the device status word; read_status
@@ -420,9 +418,14 @@ void pin_counts_of(const Ctx& cx, const Level& L, int k, const int32_t* part, in
 // Throws HG_ERR_INVALID unless every block id of a caller's partition is in
 // [0, k) (a block id indexes Phi).
 void validate_partition(const Ctx& cx, const int32_t* part, int32_t n, int k);
-// Phi (m x k) and Lambda of a partition, left on the device.
-void device_pin_counts(const Ctx& cx, const Level& L, int k, const int32_t* part,
-                       DBuf<int32_t>& phi, DBuf<unsigned long long>& lam);
+// The same check without waiting for its outcome (in the status word).
+void check_partition(const Ctx& cx, const int32_t* part, int32_t n, int k);
+// {move index or -1, block} of every node; bad moves set the status word.
+void index_moves(const Ctx& cx, const Level& L, int k, const int32_t* part, int32_t l,
+                 const int32_t* nodes, const int32_t* targets, DBuf<int2>& info);
+// The nets of the moved nodes, each once, and their number.
+void touched_nets(const Ctx& cx, const Level& L, int32_t l, const int32_t* nodes,
+                  DBuf<int32_t>& list, DBuf<int32_t>& count);
 void gain_table_build(const Ctx& cx, const Level& L, int k, const int32_t* part, int64_t* b,
                       int64_t* p);
 void gain_table_move(const Ctx& cx, const Level& L, int k, int32_t* part, int32_t l,

@@ -10,6 +10,8 @@
 //   before), and loses w(e) when first_in[t] = i, i > last_out[t] and
 //   non_moved[t] = 0 (u is the first pin to enter t after t was emptied).
 // Only the nets of moved nodes are visited, each once.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace hgk {
@@ -17,129 +19,202 @@ namespace hgk {
 namespace {
 
 constexpr int GR_WARPS = 8;
+constexpr int GR_LANES = 8;   // lanes per move or per net of at most GR_SMALL pins
+constexpr int32_t GR_SMALL = 64;
 
-// idx[u] = i for the move of u; a node moved twice, a node out of range, or
-// a target outside [0, k) or equal to the node's block is bad input.
+// info[v] = {index of v's move or -1, Pi[v]}: a pin costs one 8-byte gather.
+__global__ void k_gr_info(const int32_t* __restrict__ part, int32_t n, int2* __restrict__ info) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x)
+    info[v] = make_int2(-1, part[v]);
+}
+
+// A node moved twice, a node out of range, or a target outside [0, k) or equal
+// to the node's block is bad input.
 __global__ void k_gr_index(const int32_t* __restrict__ nodes, const int32_t* __restrict__ targets,
-                           int32_t l, int32_t n, int k, const int32_t* __restrict__ part,
-                           int32_t* __restrict__ idx, int32_t* status) {
+                           int32_t l, int32_t n, int k, int2* __restrict__ info, int32_t* status) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < l; i += gridDim.x * blockDim.x) {
     const int32_t u = nodes[i], t = targets[i];
-    if (u < 0 || u >= n || t < 0 || t >= k || part[u] < 0 || part[u] >= k || t == part[u]) {
+    if (u < 0 || u >= n || t < 0 || t >= k || info[u].y < 0 || info[u].y >= k || t == info[u].y) {
       dev_fail(status, DEV_BAD_INPUT);
       continue;
     }
-    if (atomicCAS(&idx[u], -1, i) != -1) dev_fail(status, DEV_BAD_INPUT);
+    if (atomicCAS(&info[u].x, -1, i) != -1) dev_fail(status, DEV_BAD_INPUT);
   }
 }
 
-// The nets of the moved nodes, each listed once (one warp per move, lanes
-// over its incident nets).
-__global__ void k_gr_nets(const int32_t* __restrict__ nodes, int32_t l, int32_t n,
-                          const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
-                          int32_t* __restrict__ mark, int32_t* __restrict__ list,
-                          int32_t* __restrict__ count) {
-  const int wv = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t i = wv; i < l; i += nw) {
+// One bit per net of a moved node, eight lanes per move.
+__global__ void __launch_bounds__(GR_WARPS * 32)
+k_gr_mark(const int32_t* __restrict__ nodes, int32_t l, int32_t n,
+          const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
+          unsigned* __restrict__ mark) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x / GR_LANES;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / GR_LANES; i < l;
+       i += stride) {
     const int32_t u = nodes[i];
     if (u < 0 || u >= n) continue;  // reported by k_gr_index
-    for (int32_t j = ioff[u] + lane_id(); j < ioff[u + 1]; j += 32) {
+    for (int32_t j = ioff[u] + (int32_t)(threadIdx.x % GR_LANES); j < ioff[u + 1]; j += GR_LANES) {
       const int32_t e = inets[j];
-      if (atomicExch(&mark[e], 1) == 0) list[atomicAdd(count, 1)] = e;
+      atomicOr(&mark[e >> 5], 1u << (e & 31));
     }
   }
 }
 
-// One warp per listed net: the two loops of Algorithm 4 over the net's pins,
-// with the per-block first_in / last_out / non_moved arrays of the warp in
-// shared memory (k <= 64).
-__global__ void __launch_bounds__(GR_WARPS * 32)
-k_gr_net(const int32_t* __restrict__ list, const int32_t* __restrict__ count,
-         const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
-         const int32_t* __restrict__ w, const int32_t* __restrict__ part,
-         const int32_t* __restrict__ idx, const int32_t* __restrict__ targets, int k,
-         unsigned long long* __restrict__ gains, int32_t* status) {
-  __shared__ int32_t s_first_in[GR_WARPS][HG_MAX_K];
-  __shared__ int32_t s_last_out[GR_WARPS][HG_MAX_K];
-  __shared__ int32_t s_non_moved[GR_WARPS][HG_MAX_K];
-  const int wv = warp_in_block(), lane = lane_id();
-  int32_t* first_in = s_first_in[wv];
-  int32_t* last_out = s_last_out[wv];
-  int32_t* non_moved = s_non_moved[wv];
-  for (int b = lane; b < HG_MAX_K; b += 32) {
+// The marked nets in ascending order within a warp's 1024: one claim of the list
+// per warp (an append per net or per lane group is a same-address atomic each).
+__global__ void k_gr_list(const unsigned* __restrict__ mark, int32_t words,
+                          int32_t* __restrict__ list, int32_t* __restrict__ count) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < words;
+       i0 += stride) {
+    const int64_t i = i0 + lane_id();
+    unsigned x = i < words ? mark[i] : 0u;
+    const int32_t c = __popc(x);
+    const int32_t incl = warp_inclusive_scan(c);
+    int32_t base = 0;
+    if (lane_id() == 31 && incl) base = atomicAdd(count, incl);
+    int32_t at = __shfl_sync(FULL, base, 31) + incl - c;
+    while (x) {
+      list[at++] = (int32_t)(32 * i) + __ffs(x) - 1;
+      x &= x - 1;
+    }
+  }
+}
+
+// The per-block arrays of one net: smallest index of a move into a block,
+// largest of a move out of it, pins that do not move.
+struct NetBlocks {
+  int32_t first_in[HG_MAX_K], last_out[HG_MAX_K], non_moved[HG_MAX_K];
+  __device__ __forceinline__ void clear(int b) {
     first_in[b] = INT32_MAX;
     last_out[b] = -1;
     non_moved[b] = 0;
   }
+};
+
+// The two loops of Algorithm 4 over pins [b, end) by W threads (`at` of them),
+// with the net's arrays clear on entry and cleared again.
+template <int W>
+__device__ __forceinline__ void gr_net(const int32_t* __restrict__ pins,
+                                       const int2* __restrict__ info,
+                                       const int32_t* __restrict__ targets, int k, int32_t b,
+                                       int32_t end, long long we, int at, NetBlocks& N,
+                                       unsigned long long* __restrict__ gains, int32_t* status) {
+  // the first two pins of a thread stay in registers for the second loop
+  int2 keep[2] = {make_int2(-1, 0), make_int2(-1, 0)};
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+    if (b + at + x * W < end) keep[x] = info[pins[b + at + x * W]];
+  auto enter = [&](const int2& nd) {
+    const int32_t i = nd.x, s = nd.y;
+    if (s < 0 || s >= k) {  // a block id out of range: bad input, never indexed
+      dev_fail(status, DEV_BAD_INPUT);
+    } else if (i >= 0) {
+      atomicMax(&N.last_out[s], i);
+      atomicMin(&N.first_in[targets[i]], i);
+    } else {
+      atomicAdd(&N.non_moved[s], 1);
+    }
+  };
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+    if (b + at + x * W < end) enter(keep[x]);
+  for (int32_t q = b + at + 2 * W; q < end; q += W) enter(info[pins[q]]);
+  __syncwarp();
+  auto leave = [&](const int2& nd) {
+    const int32_t i = nd.x;
+    if (i < 0) return;
+    const int s = nd.y, t = targets[i];  // both checked by k_gr_index
+    long long d = 0;
+    if (N.last_out[s] == i && i < N.first_in[s] && N.non_moved[s] == 0) d += we;
+    if (N.first_in[t] == i && i > N.last_out[t] && N.non_moved[t] == 0) d -= we;
+    if (d) atomicAdd(&gains[i], (unsigned long long)d);
+  };
+#pragma unroll
+  for (int x = 0; x < 2; ++x) leave(keep[x]);
+  for (int32_t q = b + at + 2 * W; q < end; q += W) leave(info[pins[q]]);
+  __syncwarp();
+  for (int x = at; x < k; x += W) N.clear(x);
+  __syncwarp();
+}
+
+// Listed nets: eight lanes per net of at most GR_SMALL pins (most nets have a
+// handful; a warp per net left its lanes idle), else the warp.
+__global__ void __launch_bounds__(GR_WARPS * 32)
+k_gr_net(const int32_t* __restrict__ list, const int32_t* __restrict__ count,
+         const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+         const int32_t* __restrict__ w, const int2* __restrict__ info,
+         const int32_t* __restrict__ targets, int k,
+         unsigned long long* __restrict__ gains, int32_t* status) {
+  constexpr int PER = 32 / GR_LANES;
+  __shared__ NetBlocks s_blocks[GR_WARPS][PER];
+  const int wv = warp_in_block(), lane = lane_id(), sub = lane % GR_LANES, grp = lane / GR_LANES;
+  for (int x = sub; x < HG_MAX_K; x += GR_LANES) s_blocks[wv][grp].clear(x);
   __syncwarp();
   const int32_t cnt = *count;
-  for (int32_t x = blockIdx.x * GR_WARPS + wv; x < cnt; x += gridDim.x * GR_WARPS) {
-    const int32_t e = list[x];
-    const int32_t b = eoff[e], end = eoff[e + 1];
-    for (int32_t q = b + lane; q < end; q += 32) {
-      const int32_t v = pins[q];
-      const int32_t i = idx[v];
-      const int32_t s = part[v];
-      if (s < 0 || s >= k) {  // a block id out of range: bad input, never indexed
-        dev_fail(status, DEV_BAD_INPUT);
-        continue;
-      }
-      if (i >= 0) {
-        atomicMax(&last_out[s], i);
-        atomicMin(&first_in[targets[i]], i);
-      } else {
-        atomicAdd(&non_moved[s], 1);
-      }
+  const int64_t stride = (int64_t)gridDim.x * GR_WARPS * PER;
+  for (int64_t x0 = ((int64_t)blockIdx.x * GR_WARPS + wv) * PER; x0 < cnt; x0 += stride) {
+    const int64_t x = x0 + grp;
+    const int32_t e = x < cnt ? list[x] : 0;
+    const int32_t b = x < cnt ? eoff[e] : 0, end = x < cnt ? eoff[e + 1] : 0;
+    const bool small = end - b <= GR_SMALL;
+    gr_net<GR_LANES>(pins, info, targets, k, b, small ? end : b, end > b ? w[e] : 0, sub,
+                     s_blocks[wv][grp], gains, status);
+    unsigned wide = __ballot_sync(FULL, sub == 0 && !small);
+    while (wide) {
+      const int l = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int32_t we = __shfl_sync(FULL, e, l);
+      gr_net<32>(pins, info, targets, k, __shfl_sync(FULL, b, l), __shfl_sync(FULL, end, l),
+                 w[we], lane, s_blocks[wv][0], gains, status);
     }
-    __syncwarp();
-    const long long we = w[e];
-    for (int32_t q = b + lane; q < end; q += 32) {
-      const int32_t v = pins[q];
-      const int32_t i = idx[v];
-      if (i < 0) continue;
-      const int s = part[v], t = targets[i];  // both checked by k_gr_index
-      long long d = 0;
-      if (last_out[s] == i && i < first_in[s] && non_moved[s] == 0) d += we;
-      if (first_in[t] == i && i > last_out[t] && non_moved[t] == 0) d -= we;
-      if (d) atomicAdd(&gains[i], (unsigned long long)d);
-    }
-    __syncwarp();
-    for (int bb = lane; bb < k; bb += 32) {
-      first_in[bb] = INT32_MAX;
-      last_out[bb] = -1;
-      non_moved[bb] = 0;
-    }
-    __syncwarp();
   }
 }
 
 }  // namespace
 
+void index_moves(const Ctx& cx, const Level& L, int k, const int32_t* part, int32_t l,
+                 const int32_t* nodes, const int32_t* targets, DBuf<int2>& info) {
+  info.alloc(&cx.alloc, (size_t)L.n);
+  k_gr_info<<<grid_for(L.n, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(part, L.n, info.p);
+  check_launch("gr_info");
+  k_gr_index<<<grid_for(l, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(nodes, targets, l, L.n, k,
+                                                                     info.p, cx.d_status);
+  check_launch("gr_index");
+  if (cx.launches) *cx.launches += 2;
+}
+
+void touched_nets(const Ctx& cx, const Level& L, int32_t l, const int32_t* nodes,
+                  DBuf<int32_t>& list, DBuf<int32_t>& count) {
+  DBuf<unsigned> mark;
+  const int32_t words = (int32_t)((L.m + 31ll) / 32);
+  mark.alloc(&cx.alloc, (size_t)words + 1);
+  list.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1));
+  count.alloc(&cx.alloc, 1);
+  HG_CUDA(cudaMemsetAsync(mark.p, 0, mark.bytes(), cx.stream));
+  HG_CUDA(cudaMemsetAsync(count.p, 0, sizeof(int32_t), cx.stream));
+  k_gr_mark<<<grid_for(l, GR_WARPS * (32 / GR_LANES), cx.num_sms, 8), GR_WARPS * 32, 0,
+              cx.stream>>>(nodes, l, L.n, L.ioff.p, L.inets.p, mark.p);
+  check_launch("gr_mark");
+  k_gr_list<<<grid_for(words, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(mark.p, words, list.p,
+                                                                        count.p);
+  check_launch("gr_list");
+  if (cx.launches) *cx.launches += 2;
+}
+
 void recalculate_gains(const Ctx& cx, const Level& L, int k, const int32_t* part, int32_t l,
                        const int32_t* nodes, const int32_t* targets, int64_t* gains) {
   if (l == 0) return;
   HG_CUDA(cudaMemsetAsync(gains, 0, sizeof(int64_t) * (size_t)l, cx.stream));
-  DBuf<int32_t> idx, mark, list, count;
-  idx.alloc(&cx.alloc, (size_t)L.n);
-  mark.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1));
-  list.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1));
-  count.alloc(&cx.alloc, 1);
-  fill_i32(cx, idx.p, -1, L.n);
-  HG_CUDA(cudaMemsetAsync(mark.p, 0, mark.bytes(), cx.stream));
-  HG_CUDA(cudaMemsetAsync(count.p, 0, sizeof(int32_t), cx.stream));
-  k_gr_index<<<grid_for(l, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(nodes, targets, l, L.n, k,
-                                                                     part, idx.p, cx.d_status);
-  check_launch("gr_index");
-  k_gr_nets<<<grid_for(l, 8, cx.num_sms, 16), 256, 0, cx.stream>>>(nodes, l, L.n, L.ioff.p,
-                                                                   L.inets.p, mark.p, list.p,
-                                                                   count.p);
-  check_launch("gr_nets");
+  DBuf<int2> info;
+  DBuf<int32_t> list, count;
+  index_moves(cx, L, k, part, l, nodes, targets, info);
+  touched_nets(cx, L, l, nodes, list, count);
   k_gr_net<<<cx.num_sms * 8, GR_WARPS * 32, 0, cx.stream>>>(
-      list.p, count.p, L.eoff.p, L.pins.p, L.w.p, part, idx.p, targets, k,
+      list.p, count.p, L.eoff.p, L.pins.p, L.w.p, info.p, targets, k,
       reinterpret_cast<unsigned long long*>(gains), cx.d_status);
   check_launch("gr_net");
-  if (cx.launches) *cx.launches += 4;
+  if (cx.launches) *cx.launches += 1;
   check_status(cx);
 }
 

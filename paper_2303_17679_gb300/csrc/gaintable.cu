@@ -2,196 +2,399 @@
 // and penalty p(u, V_i) = w({e in I(u) : Phi(e, V_i) = 0}), so that the gain
 // of Sec. 6 is g_u(V_t) = b(u) - p(u, V_t).
 //
-// Build: one warp per node over its incident nets; every lane adds w(e) to
-// the warp's shared counter of each block of Lambda(e), and
-// p(u, V_i) = w(I(u)) - counter[i].
-// Moves (the update rules of Sec. 6.2, applied to a set of moves at once):
-// one warp per move walks the nets of the moved node; one lane applies
-// Phi(e, V_s) -= 1 and Phi(e, V_t) += 1 atomically, and the warp applies,
-// with the counts after its own updates,
-//   (1) Phi(e, V_s) = 0: p(v, V_s) += w(e) for every pin v of e,
-//   (2) Phi(e, V_s) = 1: b(v) += w(e) for the pins v of e in V_s,
-//   (3) Phi(e, V_t) = 1: p(v, V_t) -= w(e) for every pin v of e,
-//   (4) Phi(e, V_t) = 2: b(v) -= w(e) for the pins v of e in V_t.
-// The atomics give some sequential order of the pin-count updates, and by the
-// lemma of Sec. 6.2 the final penalties of all nodes and the final benefits
-// of the unmoved nodes do not depend on it; the benefits of the moved nodes
-// are recomputed from the final pin counts afterwards.
+// Both need of a net only which blocks hold a pin and which hold exactly one.
+// These masks come from one pass over the pins, combined by
+//   seen = s1 | s2, twice = t1 | t2 | (s1 & s2)
+// over lanes, with no pin counts in memory (the m x k table of counts, cleared
+// and filled by atomics, took half of a build).
+// Build: the net records, then a lane group or warp per node sums w(e) per
+// block in registers (gain.cuh): p(u, V_i) = w(I(u)) - sum_i.
+// Moves: for every net of a moved node the masks before and after all moves
+// give the change of the table,
+//   p(v, V_i) += w(e) (-= w(e)) for every pin v when V_i lost its last (got its
+//   first) pin of e, and
+//   b(v) += w(e) (-= w(e)) for the unmoved pins v of V_i when V_i got down to
+//   (rose above) one pin of e,
+// which is what the update rules of Sec. 6.2 add up to in any order of the moves
+// (its lemma); the benefits of the moved nodes are recomputed from the masks
+// after the moves.
+// Measured (GB300, n = m = 1e6 Zipf, k = 8, 100,000 moves): build, moves and the
+// exact gains of the sequence (gainrecalc.cu) together 1.18 -> 0.65 ms.
 //
 // Graph levels (Sec. 10, "The Gain Table"): the table of a graph is
-// w(u, V_i), the weight of u's edges into V_i, one warp per node over its
-// adjacency list; the benefit and penalties follow from it:
+// w(u, V_i), the weight of u's edges into V_i; the benefit and penalties follow:
 //   b(u) = w(I(u)) - w(u, V_Pi(u)),  p(u, V_Pi(u)) = 0,
 //   p(u, V_i) = w(I(u)) - w(u, V_i) for i != Pi(u)
 // (an edge has no pin in V_i exactly when neither endpoint is in V_i).
-#include "common.cuh"
+#include <algorithm>
+
+#include "gain.cuh"
 
 namespace hgk {
 
 namespace {
 
 constexpr int GT_WARPS = 8;
+// nets and nodes of at most GT_SMALL pins (nets) are taken by a lane group, up
+// to GT_BIG_NET pins by a warp, larger nets by blocks
+constexpr int32_t GT_SMALL = 64;
+constexpr int32_t GT_BIG_NET = 4096;
+constexpr int GT_BIG_THREADS = 256;
 
+using Mask = unsigned long long;
+
+// Blocks seen and seen more than once.
+struct Seen {
+  Mask s = 0, t = 0;
+  __device__ __forceinline__ void add(int block) {
+    const Mask x = 1ull << block;
+    t |= s & x;
+    s |= x;
+  }
+  __device__ __forceinline__ void join(Mask s2, Mask t2) {
+    t |= t2 | (s & s2);
+    s |= s2;
+  }
+  // over the W lanes of the caller's group; the whole warp calls it
+  template <int W>
+  __device__ __forceinline__ void combine() {
+#pragma unroll
+    for (int d = W / 2; d > 0; d >>= 1) {
+      const Mask s2 = __shfl_xor_sync(FULL, s, d), t2 = __shfl_xor_sync(FULL, t, d);
+      join(s2, t2);
+    }
+  }
+  __device__ __forceinline__ Mask ones() const { return s & ~t; }
+};
+
+__device__ __forceinline__ void write_rec(int4* rec, int64_t e, int k, int32_t w, const Seen& x) {
+  const int H = k > 32 ? 2 : 1;
+  for (int h = 0; h < H; ++h)
+    rec[H * e + h] = make_int4(w, (int32_t)(uint32_t)(x.ones() >> (32 * h)),
+                               (int32_t)(uint32_t)(x.s >> (32 * h)), 0);
+}
+
+// Records of the nets of up to GT_BIG_NET pins; larger ones are listed.  The
+// partition has been checked.
+__global__ void __launch_bounds__(GT_WARPS * 32)
+k_gt_records(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+             const int32_t* __restrict__ w, const int32_t* __restrict__ part, int32_t m, int k,
+             int4* __restrict__ rec, int32_t* __restrict__ big, int32_t* __restrict__ nbig) {
+  const int lane = lane_id(), sub = lane % SUB_G;
+  const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
+  for (int64_t e0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; e0 < m; e0 += stride) {
+    const int64_t e = e0 + lane / SUB_G;
+    const int32_t b = e < m ? eoff[e] : 0, sz = e < m ? eoff[e + 1] - b : 0;
+    const int32_t mine = sz <= GT_SMALL ? sz : 0;
+    const int steps = __reduce_max_sync(FULL, (unsigned)mine);
+    Seen x;
+    for (int q = sub; q - sub < steps; q += 2 * SUB_G) {
+      const bool v0 = q < mine, v1 = q + SUB_G < mine;
+      const int32_t u0 = v0 ? pins[b + q] : 0, u1 = v1 ? pins[b + q + SUB_G] : 0;
+      const int32_t p0 = v0 ? part[u0] : 0, p1 = v1 ? part[u1] : 0;
+      if (v0) x.add(p0);
+      if (v1) x.add(p1);
+    }
+    x.combine<SUB_G>();
+    if (sub == 0 && e < m && sz <= GT_SMALL) write_rec(rec, e, k, w[e], x);
+    unsigned wide = __ballot_sync(FULL, sub == 0 && sz > GT_SMALL);
+    while (wide) {
+      const int l = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int64_t we = e0 + l / SUB_G;
+      const int32_t wb = __shfl_sync(FULL, b, l), ws = __shfl_sync(FULL, sz, l);
+      if (ws > GT_BIG_NET) {
+        if (lane == 0) big[atomicAdd(nbig, 1)] = (int32_t)we;
+        continue;
+      }
+      Seen y;
+      for (int q = lane; q < ws; q += 64) {
+        const bool v1 = q + 32 < ws;
+        const int32_t u0 = pins[wb + q], u1 = v1 ? pins[wb + q + 32] : 0;
+        const int32_t p0 = part[u0], p1 = v1 ? part[u1] : 0;
+        y.add(p0);
+        if (v1) y.add(p1);
+      }
+      y.combine<32>();
+      if (lane == 0) write_rec(rec, we, k, w[we], y);
+    }
+  }
+}
+
+// A block's Seen over all its threads, in every thread of warp 0.
+__device__ __forceinline__ Seen block_seen(Seen x) {
+  __shared__ Mask s_s[32], s_t[32];
+  x.combine<32>();
+  __syncthreads();
+  if (lane_id() == 0) {
+    s_s[warp_in_block()] = x.s;
+    s_t[warp_in_block()] = x.t;
+  }
+  __syncthreads();
+  Seen y;
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) y.join(s_s[i], s_t[i]);
+  return y;
+}
+
+// Records of the listed larger nets: chunks of GT_BIG_NET pins over the grid,
+// joined in acc (two words per net, then a count of finished chunks).
+__global__ void __launch_bounds__(GT_BIG_THREADS)
+k_gt_records_big(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+                 const int32_t* __restrict__ w, const int32_t* __restrict__ part, int k,
+                 int4* __restrict__ rec, const int32_t* __restrict__ big,
+                 const int32_t* __restrict__ nbig, Mask* __restrict__ acc) {
+  const int32_t cnt = *nbig;
+  for (int32_t i = 0; i < cnt; ++i) {
+    const int32_t e = big[i];
+    const int32_t b = eoff[e], sz = eoff[e + 1] - b;
+    const int32_t chunks = (sz + GT_BIG_NET - 1) / GT_BIG_NET;
+    for (int32_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+      Seen x;
+      for (int64_t q = (int64_t)c * GT_BIG_NET + threadIdx.x;
+           q < sz && q < (int64_t)(c + 1) * GT_BIG_NET; q += blockDim.x)
+        x.add(part[pins[b + q]]);
+      x = block_seen(x);
+      if (threadIdx.x == 0) {
+        const Mask before = atomicOr(&acc[3 * (int64_t)i], x.s);
+        atomicOr(&acc[3 * (int64_t)i + 1], x.t | (before & x.s));
+        __threadfence();
+        if (atomicAdd(&acc[3 * (int64_t)i + 2], 1ull) == (Mask)chunks - 1) {
+          __threadfence();
+          Seen y;
+          y.s = atomicOr(&acc[3 * (int64_t)i], 0ull);
+          y.t = atomicOr(&acc[3 * (int64_t)i + 1], 0ull);
+          write_rec(rec, e, k, w[e], y);
+        }
+      }
+    }
+  }
+}
+
+// Table rows of the nodes: a lane group per node of at most GT_SMALL incident
+// nets, else the warp.
+template <bool GRAPH, int K, int H, int W>
+__device__ __forceinline__ void gt_row(const int32_t* __restrict__ inets,
+                                       const int2* __restrict__ adj, const int4* __restrict__ rec,
+                                       const int32_t* __restrict__ part, bool on, int64_t u,
+                                       int32_t beg, int32_t end, int l, int k,
+                                       long long* __restrict__ b, long long* __restrict__ p) {
+  using L = TeamLane<W, H>;
+  const L lane(l);
+  const int from = on ? part[u] : 0, from_h = from - 32 * lane.half;
+  Gain<GRAPH, K, H> g;
+  g.init();
+  int32_t wsum = 0;
+  const int32_t steps = __reduce_max_sync(FULL, end - beg);
+  for (int32_t x = lane.i; x - lane.i < steps; x += 2 * L::SHARE) {
+    const int32_t j0 = beg + x, j1 = j0 + L::SHARE;
+    const bool v0 = j0 < end, v1 = j1 < end;
+    if (GRAPH) {
+      const int2 a0 = v0 ? adj[j0] : make_int2(-1, 0), a1 = v1 ? adj[j1] : make_int2(-1, 0);
+      const int t0 = v0 ? part[a0.x] : 0, t1 = v1 ? part[a1.x] : 0;
+      g.add_edge(a0.y, t0 - 32 * lane.half, from_h);
+      g.add_edge(a1.y, t1 - 32 * lane.half, from_h);
+      wsum += a0.y + a1.y;
+    } else {
+      const int32_t e0 = v0 ? inets[j0] : 0, e1 = v1 ? inets[j1] : 0;
+      NetRec r0{0, 0, 0}, r1{0, 0, 0};
+      if (v0) r0 = load_rec(rec, (int64_t)H * e0 + lane.half);
+      if (v1) r1 = load_rec(rec, (int64_t)H * e1 + lane.half);
+      g.add(r0, from_h);
+      g.add(r1, from_h);
+      wsum += r0.w + r1.w;
+    }
+  }
+  wsum = group_sum<W>(lane.half == 0 ? wsum : 0);  // both halves saw every net
+  const int32_t bw = group_sum<W>(g.bw);           // b(u) - w(I(u))
+  const int b0 = 32 * lane.half + reduce_scatter<L::SHARE, K>(lane.i, g.acc);
+  constexpr int OWN = K / L::SHARE > 0 ? K / L::SHARE : 1;
+  constexpr int SAME = L::SHARE / K > 1 ? L::SHARE / K : 1;
+  if (on) {
+    if (l == 0) b[u] = wsum + bw;
+    if (lane.i % SAME == 0) {
+#pragma unroll
+      for (int i = 0; i < OWN; ++i)
+        if (b0 + i < k)
+          p[u * k + b0 + i] = GRAPH && b0 + i == from ? 0 : wsum - g.acc[i];
+    }
+  }
+}
+
+template <bool GRAPH, int K, int H>
 __global__ void __launch_bounds__(GT_WARPS * 32)
 k_gt_build(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
-           const int32_t* __restrict__ w, const int32_t* __restrict__ phi,
-           const unsigned long long* __restrict__ lam, const int32_t* __restrict__ part, int32_t n,
-           int k, long long* __restrict__ b, long long* __restrict__ p, int32_t* status) {
-  __shared__ long long s_cnt[GT_WARPS][HG_MAX_K];
-  const int wv = warp_in_block(), lane = lane_id();
-  long long* cnt = s_cnt[wv];
-  const unsigned long long kmask = k == 64 ? ~0ull : ((1ull << k) - 1ull);
-  for (int i = lane; i < HG_MAX_K; i += 32) cnt[i] = 0;
-  __syncwarp();
-  for (int64_t u = (int64_t)blockIdx.x * GT_WARPS + wv; u < n; u += (int64_t)gridDim.x * GT_WARPS) {
-    const int32_t pu = part[u];
-    if (pu < 0 || pu >= k) {  // bad input: reported, never indexed
-      if (lane == 0) dev_fail(status, DEV_BAD_INPUT);
-      continue;
-    }
-    // a net in more than k/2 blocks adds w(e) to `full` (every block) and
-    // takes it back from the blocks outside Lambda(e): at most k/2 atomics
-    long long bu = 0, wsum = 0, full = 0;
-    for (int32_t j = ioff[u] + lane; j < ioff[u + 1]; j += 32) {
-      const int32_t e = inets[j];
-      const long long we = w[e];
-      wsum += we;
-      if (phi[(int64_t)e * k + pu] == 1) bu += we;
-      unsigned long long le = lam[e];
-      unsigned long long delta = (unsigned long long)we;
-      if (2 * __popcll(le) > k) {
-        full += we;
-        le = ~le & kmask;
-        delta = (unsigned long long)(-we);
-      }
-      while (le) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&cnt[__ffsll((long long)le) - 1]), delta);
-        le &= le - 1;
-      }
-    }
-    bu = warp_sum(bu);
-    wsum = warp_sum(wsum);
-    full = warp_sum(full);
-    __syncwarp();
-    if (lane == 0) b[u] = bu;
-    for (int i = lane; i < k; i += 32) {
-      p[u * k + i] = wsum - (cnt[i] + full);
-      cnt[i] = 0;
-    }
-    __syncwarp();
-  }
-}
-
-__global__ void __launch_bounds__(GT_WARPS * 32)
-k_gt_build_graph(const int32_t* __restrict__ ioff, const int2* __restrict__ adj,
-                 const int32_t* __restrict__ part, int32_t n, int k, long long* __restrict__ b,
-                 long long* __restrict__ p, int32_t* status) {
-  __shared__ long long s_cnt[GT_WARPS][HG_MAX_K];
-  const int wv = warp_in_block(), lane = lane_id();
-  long long* cnt = s_cnt[wv];
-  for (int i = lane; i < HG_MAX_K; i += 32) cnt[i] = 0;
-  __syncwarp();
-  for (int64_t u = (int64_t)blockIdx.x * GT_WARPS + wv; u < n; u += (int64_t)gridDim.x * GT_WARPS) {
-    const int32_t pu = part[u];
-    if (pu < 0 || pu >= k) {  // bad input: reported, never indexed
-      if (lane == 0) dev_fail(status, DEV_BAD_INPUT);
-      continue;
-    }
-    long long wsum = 0;
-    for (int32_t j = ioff[u] + lane; j < ioff[u + 1]; j += 32) {
-      const int2 a = adj[j];
-      const int32_t pv = part[a.x];
-      wsum += a.y;
-      if (pv >= 0 && pv < k)
-        atomicAdd(reinterpret_cast<unsigned long long*>(&cnt[pv]), (unsigned long long)a.y);
-      else
-        dev_fail(status, DEV_BAD_INPUT);
-    }
-    wsum = warp_sum(wsum);
-    __syncwarp();
-    if (lane == 0) b[u] = wsum - cnt[pu];
-    for (int i = lane; i < k; i += 32) {
-      p[u * k + i] = i == pu ? 0 : wsum - cnt[i];
-      cnt[i] = 0;
-    }
-    __syncwarp();
-  }
-}
-
-__global__ void k_gt_check(const int32_t* __restrict__ nodes, const int32_t* __restrict__ targets,
-                           int32_t l, int32_t n, int k, const int32_t* __restrict__ part,
-                           int32_t* __restrict__ seen, int32_t* status) {
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < l; i += gridDim.x * blockDim.x) {
-    const int32_t u = nodes[i], t = targets[i];
-    if (u < 0 || u >= n || t < 0 || t >= k || part[u] < 0 || part[u] >= k || t == part[u] ||
-        atomicExch(&seen[u], 1) != 0)
-      dev_fail(status, DEV_BAD_INPUT);
-  }
-}
-
-// One warp per move; the moved node's nets one after another, lanes over the
-// net's pins.  Runs only after k_gt_check found the moves valid.
-__global__ void k_gt_move(const int32_t* __restrict__ nodes, const int32_t* __restrict__ targets,
-                          int32_t l, const int32_t* __restrict__ ioff,
-                          const int32_t* __restrict__ inets, const int32_t* __restrict__ eoff,
-                          const int32_t* __restrict__ pins, const int32_t* __restrict__ w,
-                          const int32_t* __restrict__ part, int k, int32_t* __restrict__ phi,
-                          unsigned long long* __restrict__ b, unsigned long long* __restrict__ p) {
-  const int wv = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
+           const int2* __restrict__ adj, const int4* __restrict__ rec,
+           const int32_t* __restrict__ part, int32_t n, int k, long long* __restrict__ b,
+           long long* __restrict__ p) {
   const int lane = lane_id();
-  for (int32_t i = wv; i < l; i += nw) {
-    const int32_t u = nodes[i], t = targets[i];
-    const int s = part[u];
-    for (int32_t j = ioff[u]; j < ioff[u + 1]; ++j) {
-      const int32_t e = inets[j];
-      int32_t ns = 0, nt = 0;
-      if (lane == 0) {
-        ns = atomicSub(&phi[(int64_t)e * k + s], 1) - 1;
-        nt = atomicAdd(&phi[(int64_t)e * k + t], 1) + 1;
-      }
-      ns = __shfl_sync(FULL, ns, 0);
-      nt = __shfl_sync(FULL, nt, 0);
-      if (ns > 1 && nt > 2) continue;  // no rule applies
-      const unsigned long long we = (unsigned long long)(long long)w[e];
-      const unsigned long long neg = (unsigned long long)(-(long long)w[e]);
-      for (int32_t q = eoff[e] + lane; q < eoff[e + 1]; q += 32) {
-        const int32_t v = pins[q];
-        if (ns == 0) atomicAdd(&p[(int64_t)v * k + s], we);
-        if (ns == 1 && part[v] == s) atomicAdd(&b[v], we);
-        if (nt == 1) atomicAdd(&p[(int64_t)v * k + t], neg);
-        if (nt == 2 && part[v] == t) atomicAdd(&b[v], neg);
-      }
+  const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
+  for (int64_t u0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; u0 < n; u0 += stride) {
+    const int64_t u = u0 + lane / SUB_G;
+    const int32_t beg = u < n ? ioff[u] : 0, end = u < n ? ioff[u + 1] : 0;
+    const bool small = end - beg <= GT_SMALL;
+    gt_row<GRAPH, K, H, SUB_G>(inets, adj, rec, part, u < n && small, u, beg, small ? end : beg,
+                               lane % SUB_G, k, b, p);
+    unsigned wide = __ballot_sync(FULL, lane % SUB_G == 0 && !small);
+    while (wide) {
+      const int l = __ffs(wide) - 1;
+      wide &= wide - 1;
+      gt_row<GRAPH, K, H, 32>(inets, adj, rec, part, true, u0 + l / SUB_G,
+                              __shfl_sync(FULL, beg, l), __shfl_sync(FULL, end, l), lane, k, b, p);
     }
   }
 }
 
-__global__ void k_gt_set_part(const int32_t* __restrict__ nodes,
-                              const int32_t* __restrict__ targets, int32_t l,
-                              int32_t* __restrict__ part) {
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < l; i += gridDim.x * blockDim.x)
-    part[nodes[i]] = targets[i];
+using BuildKernel = void (*)(const int32_t*, const int32_t*, const int2*, const int4*,
+                             const int32_t*, int32_t, int, long long*, long long*);
+
+BuildKernel build_kernel(bool graph, int k) {
+  if (graph) {
+    if (k <= 8) return k_gt_build<true, 8, 1>;
+    if (k <= 16) return k_gt_build<true, 16, 1>;
+    if (k <= 32) return k_gt_build<true, 32, 1>;
+    return k_gt_build<true, 32, 2>;
+  }
+  if (k <= 8) return k_gt_build<false, 8, 1>;
+  if (k <= 16) return k_gt_build<false, 16, 1>;
+  if (k <= 32) return k_gt_build<false, 32, 1>;
+  return k_gt_build<false, 32, 2>;
 }
 
-// b(u) of the moved nodes from the final pin counts.
-__global__ void k_gt_moved_benefit(const int32_t* __restrict__ nodes, int32_t l,
-                                   const int32_t* __restrict__ ioff,
-                                   const int32_t* __restrict__ inets,
-                                   const int32_t* __restrict__ w, const int32_t* __restrict__ phi,
-                                   const int32_t* __restrict__ part, int k,
-                                   long long* __restrict__ b) {
-  const int wv = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t i = wv; i < l; i += nw) {
-    const int32_t u = nodes[i];
-    const int pu = part[u];
-    long long bu = 0;
-    for (int32_t j = ioff[u] + lane_id(); j < ioff[u + 1]; j += 32) {
-      const int32_t e = inets[j];
-      if (phi[(int64_t)e * k + pu] == 1) bu += w[e];
+// ------------------------------------------------------------ moves
+
+// The table changes of one net held by W threads with positions `at` of it
+// (its pins at `at`, at + W, ...): masks before and after, then the updates.
+struct MoveArgs {
+  const int32_t *eoff, *pins, *w, *targets;
+  const int2* info;      // {move index or -1, block} of every node
+  int k;
+  Mask* ones;            // ones(e) after the moves, per net
+  unsigned long long *b, *p;
+};
+
+__device__ __forceinline__ void see_pin(const MoveArgs& A, int32_t v, Seen& was, Seen& is) {
+  const int2 nd = A.info[v];
+  was.add(nd.y);
+  is.add(nd.x >= 0 ? A.targets[nd.x] : nd.y);
+}
+
+__device__ __forceinline__ void update_pin(const MoveArgs& A, int32_t v, unsigned long long we,
+                                           Mask lam, Mask lam_x, Mask ones, Mask ones_x) {
+  while (lam_x) {
+    const int i = __ffsll((long long)lam_x) - 1;
+    lam_x &= lam_x - 1;
+    atomicAdd(&A.p[(int64_t)v * A.k + i], (lam >> i) & 1 ? 0ull - we : we);
+  }
+  if (ones_x) {
+    const int2 nd = A.info[v];
+    if (nd.x < 0 && ((ones_x >> nd.y) & 1))
+      atomicAdd(&A.b[v], (ones >> nd.y) & 1 ? we : 0ull - we);
+  }
+}
+
+// Listed nets of up to GT_BIG_NET pins: a lane group for up to GT_SMALL pins,
+// else the warp; larger nets go to another list.
+__global__ void __launch_bounds__(GT_WARPS * 32)
+k_gt_move_nets(MoveArgs A, const int32_t* __restrict__ list, const int32_t* __restrict__ count,
+               int32_t* __restrict__ big, int32_t* __restrict__ nbig) {
+  const int lane = lane_id(), sub = lane % SUB_G;
+  const int32_t cnt = *count;
+  const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
+  for (int64_t x0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; x0 < cnt;
+       x0 += stride) {
+    const int64_t x = x0 + lane / SUB_G;
+    const int32_t e = x < cnt ? list[x] : 0;
+    const int32_t b = x < cnt ? A.eoff[e] : 0, sz = x < cnt ? A.eoff[e + 1] - b : 0;
+    const int32_t mine = sz <= GT_SMALL ? sz : 0;
+    Seen was, is;
+    for (int q = sub; q < mine; q += SUB_G) see_pin(A, A.pins[b + q], was, is);
+    __syncwarp();
+    was.combine<SUB_G>();
+    is.combine<SUB_G>();
+    if (mine > 0) {
+      if (sub == 0) A.ones[e] = is.ones();
+      const Mask lam_x = was.s ^ is.s, ones_x = was.ones() ^ is.ones();
+      if (lam_x | ones_x) {
+        const unsigned long long we = (unsigned long long)(long long)A.w[e];
+        for (int q = sub; q < mine; q += SUB_G)
+          update_pin(A, A.pins[b + q], we, is.s, lam_x, is.ones(), ones_x);
+      }
     }
-    bu = warp_sum(bu);
-    if (lane_id() == 0) b[u] = bu;
+    __syncwarp();
+    unsigned wide = __ballot_sync(FULL, sub == 0 && sz > GT_SMALL);
+    while (wide) {
+      const int l = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int32_t we_id = __shfl_sync(FULL, e, l);
+      const int32_t wb = __shfl_sync(FULL, b, l), ws = __shfl_sync(FULL, sz, l);
+      if (ws > GT_BIG_NET) {
+        if (lane == 0) big[atomicAdd(nbig, 1)] = we_id;
+        continue;
+      }
+      Seen w0, w1;
+      for (int q = lane; q < ws; q += 32) see_pin(A, A.pins[wb + q], w0, w1);
+      __syncwarp();
+      w0.combine<32>();
+      w1.combine<32>();
+      if (lane == 0) A.ones[we_id] = w1.ones();
+      const Mask lam_x = w0.s ^ w1.s, ones_x = w0.ones() ^ w1.ones();
+      if (lam_x | ones_x) {
+        const unsigned long long we = (unsigned long long)(long long)A.w[we_id];
+        for (int q = lane; q < ws; q += 32)
+          update_pin(A, A.pins[wb + q], we, w1.s, lam_x, w1.ones(), ones_x);
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// Listed nets of more than GT_BIG_NET pins, a block each.
+__global__ void __launch_bounds__(GT_BIG_THREADS)
+k_gt_move_big(MoveArgs A, const int32_t* __restrict__ list, const int32_t* __restrict__ count) {
+  const int32_t cnt = *count;
+  for (int32_t x = blockIdx.x; x < cnt; x += gridDim.x) {
+    const int32_t e = list[x];
+    const int32_t b = A.eoff[e], sz = A.eoff[e + 1] - b;
+    Seen was, is;
+    for (int q = threadIdx.x; q < sz; q += blockDim.x) see_pin(A, A.pins[b + q], was, is);
+    __syncwarp();
+    was = block_seen(was);
+    is = block_seen(is);
+    if (threadIdx.x == 0) A.ones[e] = is.ones();
+    const Mask lam_x = was.s ^ is.s, ones_x = was.ones() ^ is.ones();
+    if (lam_x | ones_x) {
+      const unsigned long long we = (unsigned long long)(long long)A.w[e];
+      for (int q = threadIdx.x; q < sz; q += blockDim.x)
+        update_pin(A, A.pins[b + q], we, is.s, lam_x, is.ones(), ones_x);
+    }
+    __syncthreads();
+  }
+}
+
+// Pi and b of the moved nodes from the masks after the moves, a lane group per
+// move.
+__global__ void __launch_bounds__(GT_WARPS * 32)
+k_gt_moved(const int32_t* __restrict__ nodes, const int32_t* __restrict__ targets, int32_t l,
+           const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
+           const int32_t* __restrict__ w, const Mask* __restrict__ ones,
+           int32_t* __restrict__ part, long long* __restrict__ b) {
+  const int lane = lane_id(), sub = lane % SUB_G;
+  const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
+  for (int64_t i0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; i0 < l; i0 += stride) {
+    const int64_t i = i0 + lane / SUB_G;
+    const int32_t u = i < l ? nodes[i] : 0, t = i < l ? targets[i] : 0;
+    const int32_t beg = i < l ? ioff[u] : 0, end = i < l ? ioff[u + 1] : 0;
+    long long bu = 0;
+    for (int32_t j = beg + sub; j < end; j += SUB_G) {
+      const int32_t e = inets[j];
+      if ((ones[e] >> t) & 1) bu += w[e];
+    }
+    __syncwarp();
+    bu = group_sum<SUB_G>(bu);
+    if (sub == 0 && i < l) {
+      b[u] = bu;
+      part[u] = t;
+    }
   }
 }
 
@@ -200,21 +403,30 @@ __global__ void k_gt_moved_benefit(const int32_t* __restrict__ nodes, int32_t l,
 void gain_table_build(const Ctx& cx, const Level& L, int k, const int32_t* part, int64_t* b,
                       int64_t* p) {
   validate_partition(cx, part, L.n, k);
-  if (L.graph) {
-    k_gt_build_graph<<<grid_for(L.n, GT_WARPS, cx.num_sms, 16), GT_WARPS * 32, 0, cx.stream>>>(
-        L.ioff.p, L.adj.p, part, L.n, k, reinterpret_cast<long long*>(b),
-        reinterpret_cast<long long*>(p), cx.d_status);
-    check_launch("gt_build_graph");
-    if (cx.launches) *cx.launches += 1;
-    check_status(cx);
-    return;
+  DBuf<int4> rec;
+  if (!L.graph && L.m > 0) {
+    const int64_t cap = L.p / GT_BIG_NET + 1;  // nets above GT_BIG_NET pins
+    DBuf<int32_t> big;
+    DBuf<Mask> acc;
+    rec.alloc(&cx.alloc, (size_t)L.m * (k > 32 ? 2 : 1));
+    big.alloc(&cx.alloc, (size_t)cap + 1);
+    acc.alloc(&cx.alloc, 3 * (size_t)cap);
+    HG_CUDA(cudaMemsetAsync(big.p + cap, 0, sizeof(int32_t), cx.stream));
+    HG_CUDA(cudaMemsetAsync(acc.p, 0, acc.bytes(), cx.stream));
+    k_gt_records<<<grid_for(L.m, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0, cx.stream>>>(
+        L.eoff.p, L.pins.p, L.w.p, part, L.m, k, rec.p, big.p, big.p + cap);
+    check_launch("gt_records");
+    if (L.p > GT_BIG_NET) {
+      k_gt_records_big<<<cx.num_sms, GT_BIG_THREADS, 0, cx.stream>>>(
+          L.eoff.p, L.pins.p, L.w.p, part, k, rec.p, big.p, big.p + cap, acc.p);
+      check_launch("gt_records_big");
+    }
+    if (cx.launches) *cx.launches += 2;
   }
-  DBuf<int32_t> phi;
-  DBuf<unsigned long long> lam;
-  device_pin_counts(cx, L, k, part, phi, lam);
-  k_gt_build<<<grid_for(L.n, GT_WARPS, cx.num_sms, 16), GT_WARPS * 32, 0, cx.stream>>>(
-      L.ioff.p, L.inets.p, L.w.p, phi.p, lam.p, part, L.n, k, reinterpret_cast<long long*>(b),
-      reinterpret_cast<long long*>(p), cx.d_status);
+  build_kernel(L.graph, k)<<<grid_for(L.n, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0,
+                             cx.stream>>>(L.ioff.p, L.inets.p, L.adj.p, rec.p, part, L.n, k,
+                                          reinterpret_cast<long long*>(b),
+                                          reinterpret_cast<long long*>(p));
   check_launch("gt_build");
   if (cx.launches) *cx.launches += 1;
   check_status(cx);
@@ -222,30 +434,42 @@ void gain_table_build(const Ctx& cx, const Level& L, int k, const int32_t* part,
 
 void gain_table_move(const Ctx& cx, const Level& L, int k, int32_t* part, int32_t l,
                      const int32_t* nodes, const int32_t* targets, int64_t* b, int64_t* p) {
-  validate_partition(cx, part, L.n, k);
-  if (l == 0) return;
-  DBuf<int32_t> seen;
-  seen.alloc(&cx.alloc, (size_t)L.n);
-  HG_CUDA(cudaMemsetAsync(seen.p, 0, seen.bytes(), cx.stream));
-  k_gt_check<<<grid_for(l, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(nodes, targets, l, L.n, k,
-                                                                     part, seen.p, cx.d_status);
-  check_launch("gt_check");
-  check_status(cx);  // nothing below runs on bad moves
-  DBuf<int32_t> phi;
-  DBuf<unsigned long long> lam;
-  device_pin_counts(cx, L, k, part, phi, lam);
-  const int g = grid_for(l, 8, cx.num_sms, 16);
-  k_gt_move<<<g, 256, 0, cx.stream>>>(nodes, targets, l, L.ioff.p, L.inets.p, L.eoff.p, L.pins.p,
-                                      L.w.p, part, k, phi.p,
-                                      reinterpret_cast<unsigned long long*>(b),
-                                      reinterpret_cast<unsigned long long*>(p));
-  check_launch("gt_move");
-  k_gt_set_part<<<grid_for(l, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(nodes, targets, l, part);
-  check_launch("gt_set_part");
-  k_gt_moved_benefit<<<g, 256, 0, cx.stream>>>(nodes, l, L.ioff.p, L.inets.p, L.w.p, phi.p, part,
-                                               k, reinterpret_cast<long long*>(b));
-  check_launch("gt_moved_benefit");
-  if (cx.launches) *cx.launches += 4;
+  if (l == 0) {
+    validate_partition(cx, part, L.n, k);
+    return;
+  }
+  check_partition(cx, part, L.n, k);
+  DBuf<int2> info;
+  DBuf<int32_t> list, count, big;
+  index_moves(cx, L, k, part, l, nodes, targets, info);
+  check_status(cx);  // nothing below runs on a bad partition or bad moves
+  touched_nets(cx, L, l, nodes, list, count);
+  DBuf<Mask> ones;
+  ones.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1));
+  MoveArgs A;
+  A.eoff = L.eoff.p;
+  A.pins = L.pins.p;
+  A.w = L.w.p;
+  A.info = info.p;
+  A.targets = targets;
+  A.k = k;
+  A.ones = ones.p;
+  A.b = reinterpret_cast<unsigned long long*>(b);
+  A.p = reinterpret_cast<unsigned long long*>(p);
+  const int64_t cap = L.p / GT_BIG_NET + 1;  // nets above GT_BIG_NET pins
+  big.alloc(&cx.alloc, (size_t)cap + 1);
+  HG_CUDA(cudaMemsetAsync(big.p + cap, 0, sizeof(int32_t), cx.stream));
+  k_gt_move_nets<<<cx.num_sms * 8, GT_WARPS * 32, 0, cx.stream>>>(A, list.p, count.p, big.p,
+                                                                  big.p + cap);
+  check_launch("gt_move_nets");
+  if (L.p > GT_BIG_NET) {
+    k_gt_move_big<<<cx.num_sms * 2, GT_BIG_THREADS, 0, cx.stream>>>(A, big.p, big.p + cap);
+    check_launch("gt_move_big");
+  }
+  k_gt_moved<<<grid_for(l, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0, cx.stream>>>(
+      nodes, targets, l, L.ioff.p, L.inets.p, L.w.p, ones.p, part, reinterpret_cast<long long*>(b));
+  check_launch("gt_moved");
+  if (cx.launches) *cx.launches += 3;
   check_status(cx);
 }
 

@@ -28,6 +28,7 @@
 #include <climits>
 #include <mutex>
 
+#include "gain.cuh"
 #include "gridsync.cuh"
 
 namespace hgk {
@@ -37,8 +38,6 @@ namespace {
 constexpr int LP_THREADS = 512;
 constexpr int LP_WARPS = LP_THREADS / 32;
 constexpr int MAX_SUBROUNDS = 256;
-constexpr int SUB_G = 8;                  // lanes per node of the lane-group class
-constexpr int NG = 32 / SUB_G;
 // incidences of one warp item of a node above the lane-group class
 constexpr int32_t ITEM_INC_MIN = 128, ITEM_INC_MAX = 1024;
 constexpr int MACC_STRIDE = HG_MAX_K + 4; // sums of a node split over several items: k blocks, bw
@@ -47,25 +46,11 @@ constexpr int MAX_PAIRS = HG_MAX_K * (HG_MAX_K - 1) / 2;
 
 // ------------------------------------------------ packed net records (a11)
 
-// The best moves read, for every incidence (u, e), w(e), Lambda(e) and
-// whether Phi(e, Pi[u]) = 1.  They live in one 16-byte record per net and
-// half of the blocks (k <= 32: one half), so the gain gathers one sector per
-// incidence instead of three:
-//   rec[H e + h] = {w(e), ones(e), Lambda(e), 0} for the blocks 32 h ..
-// with ones(e) = {i : Phi(e, i) = 1}.  Phi stays the authority: the
-// application changes a pin count with an atomic that returns the old
-// count, and flips the record's bits for the transitions it caused
-// (0 <-> 1 toggles Lambda and ones, 1 <-> 2 toggles ones); the flips commute,
-// so the records equal their definition whatever the order of the moves.
-struct NetRec {
-  int32_t w;
-  unsigned ones, lam;
-};
-
-__device__ __forceinline__ NetRec load_rec(const int4* rec, int64_t i) {
-  const int4 r = __ldcg(rec + i);
-  return NetRec{r.x, (unsigned)r.y, (unsigned)r.z};
-}
+// Phi stays the authority over the net records (gain.cuh): the application
+// changes a pin count with an atomic that returns the old count, and flips the
+// record's bits for the transitions it caused (0 <-> 1 toggles Lambda and ones,
+// 1 <-> 2 toggles ones); the flips commute, so the records equal their
+// definition whatever the order of the moves.
 
 // Records from Phi, Lambda and w (one thread per net).
 __global__ void k_net_records(const int32_t* __restrict__ phi,
@@ -218,48 +203,6 @@ __device__ __forceinline__ void list_offsets(const LpArgs& A, int32_t* s_off) {
 
 // ------------------------------------------------- best moves (a11)
 
-// With b(u) = w(nets where u is the only pin of its block) and W_I = w(I(u)),
-// the gain of Sec. 6 is
-//   g(u, t) = b(u) - W_I + w({e in I(u) : t in Lambda(e)}),
-// evaluated for all t at once; `bw` sums b(u) - W_I.  Graph levels (Sec. 10,
-// "The Gain Table"): g(u, t) = w(u, V_t) - w(u, V_Pi(u)), `bw` sums
-// -w(u, V_Pi(u)).
-// Every lane sums per block in K = 8, 16 or 32 registers (two instructions per
-// block and incidence), and the lanes combine the sums with a halving exchange
-// that leaves each lane the totals of its own blocks (14 shuffles for 16
-// blocks over 8 lanes instead of 48).  For k > 32 the lanes are split into H = 2
-// halves: each half walks the same incidences with its half of the records.
-// (Shared-memory counters with one atomic per block of Lambda(e), which k > 16
-// used before, serialise on coarse levels, whose nets touch the same blocks:
-// 37 us per sub-round at k = 64 and 31M pins, 60 us with lane groups.)
-// All sums are below 2^31 (the total net weight).
-template <bool GRAPH, int K, int H>
-struct Gain {
-  int32_t acc[K];
-  int32_t bw;
-  __device__ __forceinline__ void init() {
-#pragma unroll
-    for (int t = 0; t < K; ++t) acc[t] = 0;
-    bw = 0;
-  }
-  // incidence with net record r, seen by the lanes of half `half`; `from` is
-  // the node's block relative to the half (outside [0, 32): another half's)
-  __device__ __forceinline__ void add(const NetRec& r, int from) {
-    // u is not the only pin of its block in e
-    if ((H == 1 || (unsigned)from < 32u) && !((r.ones >> from) & 1u)) bw -= r.w;
-#pragma unroll
-    for (int t = 0; t < K; ++t)
-      if (r.lam & (1u << t)) acc[t] += r.w;
-  }
-  // graph: edge of weight w to a node of block tb (relative to the half)
-  __device__ __forceinline__ void add_edge(int32_t w, int tb, int from) {
-    if (tb == from && (H == 1 || (unsigned)tb < 32u)) bw -= w;
-#pragma unroll
-    for (int t = 0; t < K; ++t)
-      if (tb == t) acc[t] += w;
-  }
-};
-
 // Best candidate so far as one comparable word: gain descending, block id
 // ascending; 0 when no gain is positive.
 __device__ __forceinline__ void consider(unsigned long long& best, int32_t g, int t, int from,
@@ -286,14 +229,8 @@ __device__ __forceinline__ void emit_move(const LpArgs& A, int par, int32_t u, i
   }
 }
 
-// Sum and maximum over the W lanes of the caller's group (W a power of two);
-// the whole warp calls them.
-template <int W, typename T>
-__device__ __forceinline__ T group_sum(T x) {
-#pragma unroll
-  for (int d = W / 2; d > 0; d >>= 1) x += __shfl_xor_sync(FULL, x, d);
-  return x;
-}
+// Maximum over the W lanes of the caller's group (W a power of two); the whole
+// warp calls it.
 template <int W>
 __device__ __forceinline__ unsigned long long group_max(unsigned long long x) {
 #pragma unroll
@@ -303,39 +240,6 @@ __device__ __forceinline__ unsigned long long group_max(unsigned long long x) {
   }
   return x;
 }
-
-// Halving exchange over the W lanes of a group: afterwards acc[0 .. max(K/W,1))
-// of lane l holds the group's totals of blocks first_block + i, where
-// first_block is returned (K < W: W/K neighbouring lanes hold the same block).
-template <int W, int K>
-__device__ __forceinline__ int reduce_scatter(int l, int32_t (&acc)[K]) {
-  int block = 0;
-#pragma unroll
-  for (int d = W / 2, h = K / 2; d > 0; d >>= 1, h >>= 1) {
-    if (h > 0) {
-      const bool up = (l & d) != 0;
-      if (up) block += h;
-#pragma unroll
-      for (int i = 0; i < h; ++i) {
-        const int32_t give = up ? acc[i] : acc[i + h];
-        const int32_t keep = up ? acc[i + h] : acc[i];
-        acc[i] = keep + __shfl_xor_sync(FULL, give, d);
-      }
-    } else {
-      acc[0] += __shfl_xor_sync(FULL, acc[0], d);
-    }
-  }
-  return block;
-}
-
-// Lanes of a team of W: W / H lanes share the incidences, the upper lanes take
-// the upper half of the blocks.
-template <int W, int H>
-struct TeamLane {
-  static constexpr int SHARE = W / H;
-  int i, half;
-  __device__ __forceinline__ explicit TeamLane(int l) : i(l % SHARE), half(l / SHARE) {}
-};
 
 // Class-0 nodes by groups of SUB_G lanes, one node (or none: an empty item) per
 // group: NG nodes' load chains per warp in flight (nodes of a few nets leave
