@@ -376,6 +376,123 @@ __global__ void k_compact(const int32_t* __restrict__ keep, const int32_t* __res
   }
 }
 
+// ------------------------------------------------------------ graph levels
+
+// A net of two pins is its pair of coarse nodes: the pair itself, {smaller,
+// larger} in 64 bits, is the hash-table key, so equal keys are identical nets
+// and the weights are summed at the key.  Three passes over the edges (insert,
+// flag, write) instead of the general path's lists, fingerprints, pin-by-pin
+// comparison and second scan; each is bound by its random table sectors.
+// Measured (GB300, 1e6 nodes, 4e6 edges, k = 8, all nine levels): coarsening 20.4
+// -> 13.3 ms.
+__global__ void k_edge_insert(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+                              const int32_t* __restrict__ map, const int32_t* __restrict__ w,
+                              int32_t m, unsigned long long* __restrict__ tkey,
+                              int2* __restrict__ tval, uint64_t mask,
+                              int32_t* __restrict__ slot_of, int32_t* status) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t b = eoff[e];
+    const int32_t x = map[pins[b]], y = map[pins[b + 1]];
+    int32_t slot = -1;
+    if (x != y) {
+      const unsigned long long f =
+          ((unsigned long long)(uint32_t)min(x, y) << 32) | (uint32_t)max(x, y);
+      uint64_t h = mix64(f) & mask;
+      for (uint64_t probe = 0; probe <= mask; ++probe) {
+        const unsigned long long k = tkey[h];
+        if (k == f) { slot = (int32_t)h; break; }
+        if (k == EMPTY_FP) {
+          const unsigned long long old = atomicCAS(&tkey[h], EMPTY_FP, f);
+          if (old == EMPTY_FP || old == f) { slot = (int32_t)h; break; }
+        }
+        h = (h + 1) & mask;
+      }
+      if (slot < 0) {
+        dev_fail(status, DEV_HASH_FULL);
+      } else {
+        atomicMin(&tval[slot].x, (int32_t)e);  // the representative: smallest id
+        atomicAdd(&tval[slot].y, w[e]);
+      }
+    }
+    slot_of[e] = slot;
+  }
+}
+
+__global__ void k_edge_flag(const int32_t* __restrict__ slot_of, const int2* __restrict__ tval,
+                            int32_t m, int32_t* __restrict__ keep) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t sl = slot_of[e];
+    keep[e] = sl >= 0 && tval[sl].x == (int32_t)e ? 1 : 0;
+  }
+}
+
+// Kept edges by the rank of their representative: offsets, pins ascending,
+// weights.
+__global__ void k_edge_write(const int32_t* __restrict__ slot_of,
+                             const unsigned long long* __restrict__ tkey,
+                             const int2* __restrict__ tval, const int32_t* __restrict__ newid,
+                             int32_t m, int32_t m2, int32_t* __restrict__ eoff2,
+                             int2* __restrict__ pins2, int32_t* __restrict__ w2) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t sl = slot_of[e];
+    if (sl < 0) continue;
+    const int2 v = tval[sl];
+    if (v.x != (int32_t)e) continue;
+    const int32_t id = newid[e];
+    const unsigned long long f = tkey[sl];
+    pins2[id] = make_int2((int32_t)(f >> 32), (int32_t)(uint32_t)f);
+    w2[id] = v.y;
+    eoff2[id] = 2 * id;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) eoff2[m2] = 2 * m2;
+}
+
+__global__ void k_edge_table(unsigned long long* __restrict__ tkey, int2* __restrict__ tval,
+                             uint64_t cap) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cap;
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    tkey[i] = EMPTY_FP;
+    tval[i] = make_int2(INT_MAX, 0);
+  }
+}
+
+void contract_edges(const Ctx& cx, const Level& L, Level& out) {
+  const int32_t m = L.m;
+  uint64_t cap = 2;
+  while (cap < 2 * (uint64_t)m) cap <<= 1;
+  DBuf<unsigned long long> tkey;
+  DBuf<int2> tval;
+  DBuf<int32_t> slot_of, keep, total;
+  tkey.alloc(&cx.alloc, (size_t)cap);
+  tval.alloc(&cx.alloc, (size_t)cap);
+  slot_of.alloc(&cx.alloc, (size_t)m);
+  keep.alloc(&cx.alloc, (size_t)m);
+  total.alloc(&cx.alloc, 1);
+  const int g = grid_for(m, 256, cx.num_sms, 8);
+  k_edge_table<<<grid_for((int64_t)cap, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(tkey.p, tval.p,
+                                                                                cap);
+  check_launch("edge_table");
+  k_edge_insert<<<g, 256, 0, cx.stream>>>(L.eoff.p, L.pins.p, L.map.p, L.w.p, m, tkey.p, tval.p,
+                                          cap - 1, slot_of.p, cx.d_status);
+  check_launch("edge_insert");
+  k_edge_flag<<<g, 256, 0, cx.stream>>>(slot_of.p, tval.p, m, keep.p);
+  check_launch("edge_flag");
+  scan_exclusive_i32(cx, keep.p, keep.p, m, total.p);  // keep flag -> new id
+  const int32_t m2 = read_i32(cx, total.p);
+  out.m = m2;
+  out.p = 2 * (int64_t)m2;
+  out.eoff.alloc(&cx.alloc, (size_t)m2 + 1);
+  out.pins.alloc(&cx.alloc, (size_t)std::max<int64_t>(out.p, 1));
+  out.w.alloc(&cx.alloc, (size_t)std::max<int32_t>(m2, 1));
+  k_edge_write<<<g, 256, 0, cx.stream>>>(slot_of.p, tkey.p, tval.p, keep.p, m, m2, out.eoff.p,
+                                         reinterpret_cast<int2*>(out.pins.p), out.w.p);
+  check_launch("edge_write");
+  if (cx.launches) *cx.launches += 4;
+}
+
 // Community of every coarse node: the community of its members (a cluster
 // never spans two communities).
 __global__ void k_coarse_comm(const int32_t* __restrict__ map, const int32_t* __restrict__ comm,
@@ -423,6 +540,17 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
     out.eoff.alloc(&cx.alloc, 1);
     HG_CUDA(cudaMemsetAsync(out.eoff.p, 0, sizeof(int32_t), cx.stream));
     build_incidence(cx, out);
+    coarse_communities(cx, L, out);
+    L.coarsened = true;
+    return;
+  }
+
+  // a6 - a8 of a graph level (a graph's coarse nets have two pins again: one-pin
+  // nets are dropped)
+  if (L.graph) {
+    contract_edges(cx, L, out);
+    build_incidence(cx, out);
+    if (out.m > 0) build_graph_adjacency(cx, out);
     coarse_communities(cx, L, out);
     L.coarsened = true;
     return;
@@ -532,8 +660,6 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
                           cudaMemcpyDeviceToDevice, cx.stream));
   if (cx.launches) *cx.launches += 2;
   build_incidence(cx, out);
-  // a graph's coarse nets have two pins again (one-pin nets are dropped)
-  if (L.graph && out.m > 0) build_graph_adjacency(cx, out);
   coarse_communities(cx, L, out);
   L.coarsened = true;
 }
