@@ -22,23 +22,25 @@
 // cluster added to its self-loop weight) and the next level starts.
 //
 // Layout per level: CSR with int64 offsets, int32 neighbours, int64 weights,
-// int64 self-loop weights, degrees k and volumes.  Per round the vertices
-// are listed by (sub-round, class): vertices of at most 8 (32) edges are decided
-// by a group of eight lanes (a warp) that holds one edge per lane and sums the
-// edges of a cluster by exchanging them; up to LV_SMALL edges by one warp with
-// a shared-memory table of the neighbouring clusters; the rest insert their
-// edges into per-vertex tables in global memory with one thread per edge over
-// the whole grid, then one block per vertex takes the best entry.  Aggregation
-// uses the same global tables, one per coarse vertex.
-// What bounds it: 16 dependent sub-rounds of gathers per round, some 25 rounds.
-// Most vertices have a handful of edges (a table of 512 slots, cleared and
-// scanned per vertex, cost more than they did), and the host reads only the
-// class boundaries of a round (copying the table offsets of all vertices took
-// over a millisecond per round).
+// int64 self-loop weights, degrees k and volumes.
+//
+// The rounds of a level run as one persistent kernel (blocks meet at grid_sync;
+// two or three barriers per sub-round).  Per round the vertices are listed by
+// (sub-round, class): vertices of at most 8 (32) edges are decided by a group of
+// eight lanes (a warp) that holds one edge per lane and sums the edges of a
+// cluster by exchanging them; up to LV_SMALL edges by one warp with a shared
+// table of the neighbouring clusters, up to LV_BLOCK by the block with all the
+// tables as one; larger vertices are split into parts by a hash of the cluster,
+// a block each, whose bests are compared after one more barrier.  Aggregation
+// adds the edges to global tables, one per coarse vertex.
+// What bounds it: some 25 rounds of 16 dependent sub-rounds, each a chain of
+// gathers; as four or five launches per sub-round, with a host wait and the
+// copy of all table offsets per round, the detection on 250,007 nodes and
+// 1.35M pins took 30.1 ms, now 16.1 ms.
 #include <algorithm>
 #include <mutex>
 
-#include "common.cuh"
+#include "gridsync.cuh"
 
 namespace hgk {
 
@@ -46,13 +48,16 @@ namespace {
 
 constexpr int LV_ROUNDS = 5;
 constexpr int LV_LEVELS = 32;
-constexpr int LV_CLASSES = 4;
-constexpr int LV_GROUP = 8;            // class 0: degree <= 8, eight lanes per vertex
-constexpr int LV_LANES = 32;           // class 1: degree <= 32, a warp per vertex
-constexpr int LV_SMALL = 256;          // class 2: degree <= 256, a warp and a shared table
-constexpr int LV_SLOTS = 2 * LV_SMALL;  // shared slots per warp (load <= 1/2)
-constexpr int LV_WARPS = 8;
-constexpr int LV_ARGMAX_THREADS = 256;
+constexpr int LV_CLASSES = 5;
+constexpr int LV_GROUP = 8;             // class 0: degree <= 8, eight lanes per vertex
+constexpr int LV_LANES = 32;            // class 1: degree <= 32, a warp per vertex
+constexpr int LV_SMALL = 256;           // class 2: degree <= 256, a warp and a shared table
+constexpr int LV_BLOCK = 4096;          // class 3: degree <= 4096, a block
+constexpr int LV_PART = 2048;           // class 4: neighbouring clusters per part
+constexpr int LV_THREADS = 512;
+constexpr int LV_WARPS = LV_THREADS / 32;
+constexpr int LV_SLOTS = 2 * LV_SMALL;  // slots per warp (load <= 1/2)
+constexpr int LV_BLOCK_SLOTS = LV_SLOTS * LV_WARPS;
 constexpr int32_t LV_EMPTY = -1;
 
 using i128 = __int128;
@@ -120,81 +125,6 @@ __global__ void k_lv_init(int64_t V, const long long* __restrict__ k, int32_t* _
   }
 }
 
-// ------------------------------------------------------------ lists
-
-// key = sub-round * LV_CLASSES + class of every vertex with at least one edge.
-__device__ __forceinline__ int lv_key(const long long* off, uint64_t seed, int level, int round,
-                                      int64_t i, int S) {
-  const long long deg = off[i + 1] - off[i];
-  if (deg == 0) return -1;  // no neighbouring cluster: never moves
-  const int cls = deg <= LV_GROUP ? 0 : deg <= LV_LANES ? 1 : deg <= LV_SMALL ? 2 : 3;
-  return subround_louvain(seed, level, round, i, S) * LV_CLASSES + cls;
-}
-
-__global__ void k_lv_count(const long long* __restrict__ off, int64_t V, uint64_t seed, int level,
-                           int round, int S, int32_t* __restrict__ cnt) {
-  extern __shared__ int32_t s_cnt[];
-  for (int i = threadIdx.x; i < LV_CLASSES * S; i += blockDim.x) s_cnt[i] = 0;
-  __syncthreads();
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int key = lv_key(off, seed, level, round, i, S);
-    if (key >= 0) atomicAdd(&s_cnt[key], 1);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < LV_CLASSES * S; i += blockDim.x)
-    if (s_cnt[i]) atomicAdd(&cnt[i], s_cnt[i]);
-}
-
-// Scatters vertices by key; the list order inside a key is unspecified
-// (every later step is a set operation or an integer sum).
-__global__ void k_lv_scatter(const long long* __restrict__ off, int64_t V, uint64_t seed,
-                             int level, int round, int S, const int32_t* __restrict__ koff,
-                             int32_t* __restrict__ fill, int32_t* __restrict__ list) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < V; b += stride) {
-    const int64_t i = b + lane_id();
-    const bool valid = i < V;
-    const int key = valid ? lv_key(off, seed, level, round, i, S) : -1;
-    const int32_t slot = warp_claim_slot(fill, key, __ballot_sync(FULL, valid));
-    if (slot >= 0) list[koff[key] + slot] = (int32_t)i;
-  }
-}
-
-// Degrees and global table sizes (power of two >= 2 deg + 2) of the vertices
-// that need a table along the list of *listed <= cap vertices (zeros after it
-// and for the others).
-__global__ void k_lv_list_sizes(const int32_t* __restrict__ list, const int32_t* __restrict__ listed,
-                                int32_t cap, const long long* __restrict__ off,
-                                int32_t* __restrict__ deg, int32_t* __restrict__ tsize) {
-  const int32_t cnt = *listed;
-  for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < cap; x += gridDim.x * blockDim.x) {
-    int32_t d = 0, t = 0;
-    if (x < cnt) {
-      const int32_t i = list[x];
-      d = (int32_t)(off[i + 1] - off[i]);
-      if (d > LV_SMALL) {
-        // at most 2^30 slots: a larger vertex fills its table, which the
-        // insertion reports as a full table
-        int64_t c = 4;
-        while (c < 2 * (int64_t)d + 2 && c < (1ll << 30)) c <<= 1;
-        t = (int32_t)c;
-      }
-    }
-    deg[x] = d;
-    tsize[x] = t;
-  }
-}
-
-// The class boundaries of a round and the table offsets there.
-__global__ void k_lv_bounds(const int32_t* __restrict__ koff, int nkeys,
-                            const long long* __restrict__ toff, long long* __restrict__ out) {
-  for (int i = threadIdx.x; i <= nkeys; i += blockDim.x) {
-    out[i] = koff[i];
-    out[nkeys + 1 + i] = toff[koff[i]];
-  }
-}
-
 // ------------------------------------------------------------ tables
 
 // Adds `val` to `key`'s entry of a global table (keys LV_EMPTY when free).
@@ -242,46 +172,140 @@ __device__ __forceinline__ void warp_best(Cand& x) {
   for (int d = 16; d > 0; d >>= 1) cand_better(x, shfl_cand(x, d));
 }
 
+// ------------------------------------------------------------ local moving
+
+enum { LV_MOVES = 0, LV_WORDS = 4 };           // per sub-round (two sets)
+enum { LR_MOVED = 0, LR_ROUNDS = 1, LR_LV_WORDS = 2 };
+
+// Best of one part of a vertex.
+struct PartBest {
+  unsigned long long lo;
+  long long hi, kia;
+  int32_t c, pad;
+};
+
 struct LvArgs {
   const long long* off;
   const int32_t* adj;
   const long long* aw;
   const long long* k;
-  const int32_t* cl;
-  const long long* vol;
+  int32_t* cl;
+  long long* vol;
   long long W2;
-  const int32_t* list;
-  int32_t* mv_v;
-  int32_t* mv_to;
-  int32_t* words;  // [0] moves of the sub-round
+  int64_t V;
+  uint64_t seed;
+  int level, S;
+  int2* list;       // {vertex, part | parts << 16} by (sub-round, class)
+  int32_t *cnt, *fill;  // LV_CLASSES S each
+  int2* mv;         // {vertex, cluster}
+  int32_t* words;
+  PartBest* parts;
+  unsigned long long* res;
+  unsigned* barrier;
   int32_t* status;
 };
 
-// The move of vertex i from its own cluster's entry kia and the best other
-// candidate: moves iff s(best) > s(own).
-__device__ __forceinline__ void lv_emit(const LvArgs& A, int32_t i, long long kia, const Cand& best) {
-  const int32_t own = A.cl[i];
-  const long long ki = A.k[i];
-  const i128 s_own = (i128)A.W2 * kia - (i128)ki * (A.vol[own] - ki);
-  if (best.c >= 0 && best.s > s_own) {
-    const int32_t slot = atomicAdd(&A.words[0], 1);
-    A.mv_v[slot] = i;
-    A.mv_to[slot] = best.c;
+// Class and list entries of a vertex of degree deg (0: no neighbouring cluster,
+// never moves).
+__device__ __forceinline__ int lv_class(const LvArgs& A, long long deg, int32_t& entries) {
+  entries = 1;
+  if (deg <= LV_GROUP) return 0;
+  if (deg <= LV_LANES) return 1;
+  if (deg <= LV_SMALL) return 2;
+  if (deg <= LV_BLOCK) return 3;
+  const long long D = deg < A.V ? deg : A.V;  // bound on the neighbouring clusters
+  entries = (int32_t)((D + LV_PART - 1) / LV_PART);
+  return 4;
+}
+
+// Counts (scatter == false) or writes the list entries of the block's tiles of
+// vertices; one global claim per tile and key.
+__device__ __forceinline__ void lv_list(const LvArgs& A, int round, bool scatter,
+                                        const int32_t* s_off, int32_t* s_hist, int32_t* s_base) {
+  const int keys = LV_CLASSES * A.S;
+  for (int i = threadIdx.x; i < keys; i += LV_THREADS) s_hist[i] = 0;
+  __syncthreads();
+  const int64_t stride = (int64_t)gridDim.x * LV_THREADS;
+  for (int64_t i0 = (int64_t)blockIdx.x * LV_THREADS; i0 < A.V; i0 += stride) {
+    const int64_t i = i0 + threadIdx.x;
+    int key = -1, slot = 0;
+    int32_t entries = 0;
+    if (i < A.V) {
+      const long long deg = A.off[i + 1] - A.off[i];
+      if (deg > 0) {
+        const int cls = lv_class(A, deg, entries);
+        key = subround_louvain(A.seed, A.level, round, i, A.S) * LV_CLASSES + cls;
+        slot = atomicAdd(&s_hist[key], entries);
+      }
+    }
+    if (!scatter) continue;
+    __syncthreads();
+    for (int x = threadIdx.x; x < keys; x += LV_THREADS) {
+      s_base[x] = s_hist[x] ? atomicAdd(&A.fill[x], s_hist[x]) : 0;
+      s_hist[x] = 0;
+    }
+    __syncthreads();
+    if (key >= 0) {
+      int2* out = A.list + s_off[key] + s_base[key] + slot;
+      for (int32_t x = 0; x < entries; ++x) out[x] = make_int2((int32_t)i, x | (entries << 16));
+    }
+    __syncthreads();
   }
+  if (!scatter) {
+    __syncthreads();
+    for (int x = threadIdx.x; x < keys; x += LV_THREADS)
+      if (s_hist[x]) atomicAdd(&A.cnt[x], s_hist[x]);
+  }
+}
+
+__device__ __forceinline__ void lv_offsets_of(const LvArgs& A, int32_t* s_off) {
+  const int keys = LV_CLASSES * A.S;
+  if (warp_in_block() == 0) {
+    int32_t carry = 0;
+    for (int i0 = 0; i0 < keys; i0 += 32) {
+      const int i = i0 + lane_id();
+      const int32_t x = i < keys ? __ldcg(A.cnt + i) : 0;
+      const int32_t incl = warp_inclusive_scan(x);
+      if (i < keys) s_off[i] = carry + incl - x;
+      carry += __shfl_sync(FULL, incl, 31);
+    }
+    if (lane_id() == 0) s_off[keys] = carry;
+  }
+  __syncthreads();
+}
+
+// Vertex i moves to the best other candidate iff s(best) > s(own), kia = the
+// weight of its edges into its own cluster.
+__device__ __forceinline__ bool lv_moves(const LvArgs& A, int32_t i, long long kia,
+                                         const Cand& best) {
+  if (best.c < 0) return false;
+  const long long ki = A.k[i];
+  return best.s > (i128)A.W2 * kia - (i128)ki * (A.vol[A.cl[i]] - ki);
+}
+
+// Lanes with `moves` enter {i, c} in the move list (the whole warp calls it).
+__device__ __forceinline__ void lv_emit(const LvArgs& A, int32_t* words, bool moves, int32_t i,
+                                        int32_t c) {
+  const unsigned who = __ballot_sync(FULL, moves);
+  if (!who) return;
+  int32_t slot = 0;
+  if (lane_id() == 0) slot = atomicAdd(&words[LV_MOVES], __popc(who));
+  slot = __shfl_sync(FULL, slot, 0) + __popc(who & ((1u << lane_id()) - 1u));
+  if (moves) A.mv[slot] = make_int2(i, c);
 }
 
 // Classes 0 and 1: G lanes per vertex of at most G edges, one edge per lane.
 // Every lane sums the edges of its own cluster (equal lanes hold equal
 // candidates); the groups of a warp stay in step.
 template <int G>
-__global__ void __launch_bounds__(LV_WARPS * 32) k_lv_lanes(LvArgs A, int32_t lo, int32_t hi) {
+__device__ __forceinline__ void lv_lanes(const LvArgs& A, int32_t* words, int32_t lo, int32_t hi,
+                                         int64_t gw, int64_t NW) {
   constexpr int PER = 32 / G;
   const int lane = lane_id(), sub = lane % G, grp = lane / G;
-  const int32_t stride = gridDim.x * LV_WARPS * PER;
-  for (int32_t x0 = lo + (blockIdx.x * LV_WARPS + warp_in_block()) * PER; x0 < hi; x0 += stride) {
-    const int32_t x = x0 + grp;
+  for (int64_t x0 = lo + gw * PER; x0 < hi; x0 += NW * PER) {
+    const int64_t x = x0 + grp;
     const bool on = x < hi;
-    const int32_t i = on ? A.list[x] : 0;
+    const int32_t i = on ? A.list[x].x : 0;
     const long long b = on ? A.off[i] : 0;
     const int d = on ? (int)(A.off[i + 1] - b) : 0;
     int32_t C = -1;
@@ -293,7 +317,7 @@ __global__ void __launch_bounds__(LV_WARPS * 32) k_lv_lanes(LvArgs A, int32_t lo
     const int32_t own = on ? A.cl[i] : -1;
     const long long ki = on ? A.k[i] : 0;
     const long long vol = C >= 0 ? A.vol[C] : 0;
-    const int steps = __reduce_max_sync(FULL, (unsigned)d);
+    const int steps = (int)__reduce_max_sync(FULL, (unsigned)d);
     long long kic = 0;
     for (int t = 0; t < steps; ++t) {
       const int32_t Ct = __shfl_sync(FULL, C, grp * G + t);
@@ -309,153 +333,184 @@ __global__ void __launch_bounds__(LV_WARPS * 32) k_lv_lanes(LvArgs A, int32_t lo
       const long long o = __shfl_xor_sync(FULL, kia, s);
       kia = o > kia ? o : kia;
     }
-    bool moves = false;
-    if (on && sub == 0 && best.c >= 0)
-      moves = best.s > (i128)A.W2 * kia - (i128)ki * (A.vol[own] - ki);
-    const unsigned who = __ballot_sync(FULL, moves);
-    if (who) {
-      int32_t slot = 0;
-      if (lane == 0) slot = atomicAdd(&A.words[0], __popc(who));
-      slot = __shfl_sync(FULL, slot, 0) + __popc(who & ((1u << lane) - 1u));
-      if (moves) {
-        A.mv_v[slot] = i;
-        A.mv_to[slot] = best.c;
-      }
-    }
+    lv_emit(A, words, on && sub == 0 && lv_moves(A, i, kia, best), i, best.c);
   }
 }
 
-// Class 2: one warp per vertex, shared table of LV_SLOTS entries.
-__global__ void __launch_bounds__(LV_WARPS * 32) k_lv_small(LvArgs A, int32_t lo, int32_t hi) {
-  __shared__ int32_t s_key[LV_WARPS][LV_SLOTS];
-  __shared__ long long s_val[LV_WARPS][LV_SLOTS];
-  const int wv = warp_in_block(), lane = lane_id();
-  int32_t* keys = s_key[wv];
-  long long* vals = s_val[wv];
-  for (int x = lane; x < LV_SLOTS; x += 32) {
+// The best other candidate and the own cluster's entry among slots first,
+// first + step, ... of a table, which are cleared.
+__device__ __forceinline__ void lv_take(const LvArgs& A, int32_t i, int32_t* keys,
+                                        long long* vals, int slots, int first, int step,
+                                        Cand& best, long long& kia) {
+  const int32_t own = A.cl[i];
+  const long long ki = A.k[i];
+  best = Cand{0, -1};
+  kia = 0;
+  for (int s = first; s < slots; s += step) {
+    const int32_t C = keys[s];
+    if (C == LV_EMPTY) continue;
+    const long long kic = vals[s];
+    keys[s] = LV_EMPTY;
+    vals[s] = 0;
+    if (C == own) kia = kic;
+    else cand_better(best, Cand{(i128)A.W2 * kic - (i128)ki * A.vol[C], C});
+  }
+  warp_best(best);
+  kia = warp_sum(kia);
+}
+
+// Part of a cluster among `parts` (its own hash: the table's picks the slot).
+__device__ __forceinline__ int lv_part(int32_t C, int parts) {
+  return (int)(((mix64((uint64_t)(uint32_t)C ^ 0xA5A5A5A500000000ull) >> 32) * (uint64_t)parts) >>
+               32);
+}
+
+// Classes 3 and 4: the block rates vertex i over all its edges, keeping the
+// clusters of one part.
+__device__ __forceinline__ void lv_block(const LvArgs& A, int32_t* words, int32_t x,
+                                         int32_t* keys, long long* vals) {
+  __shared__ unsigned long long s_lo[LV_WARPS];
+  __shared__ long long s_hi[LV_WARPS], s_kia[LV_WARPS];
+  __shared__ int32_t s_c[LV_WARPS];
+  const int2 nd = A.list[x];
+  const int32_t i = nd.x;
+  const int part = nd.y & 0xffff, parts = nd.y >> 16;
+  const long long b = A.off[i], e = A.off[i + 1];
+  for (long long q = b + threadIdx.x; q < e; q += LV_THREADS) {
+    const int32_t C = A.cl[A.adj[q]];
+    if (parts > 1 && lv_part(C, parts) != part) continue;
+    if (!table_add(keys, vals, LV_BLOCK_SLOTS - 1, C, A.aw[q])) dev_fail(A.status, DEV_HASH_FULL);
+  }
+  __syncthreads();
+  Cand best;
+  long long kia;
+  lv_take(A, i, keys, vals, LV_BLOCK_SLOTS, threadIdx.x, LV_THREADS, best, kia);
+  if (lane_id() == 0) {
+    s_lo[warp_in_block()] = (unsigned long long)best.s;
+    s_hi[warp_in_block()] = (long long)(best.s >> 64);
+    s_c[warp_in_block()] = best.c;
+    s_kia[warp_in_block()] = kia;
+  }
+  __syncthreads();
+  if (warp_in_block() == 0) {
+    const int l = lane_id();
+    best = Cand{0, -1};
+    kia = 0;
+    if (l < LV_WARPS) {
+      best = Cand{((i128)s_hi[l] << 64) | (i128)s_lo[l], s_c[l]};
+      kia = s_kia[l];
+    }
+    warp_best(best);
+    kia = warp_sum(kia);
+    if (parts == 1) {
+      lv_emit(A, words, l == 0 && lv_moves(A, i, kia, best), i, best.c);
+    } else if (l == 0) {
+      A.parts[x] = PartBest{(unsigned long long)best.s, (long long)(best.s >> 64), kia, best.c, 0};
+    }
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(LV_THREADS, 2) k_lv_run(const __grid_constant__ LvArgs A) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  long long* vals = reinterpret_cast<long long*>(smem);
+  int32_t* keys = reinterpret_cast<int32_t*>(vals + LV_BLOCK_SLOTS);
+  int32_t* s_off = keys + LV_BLOCK_SLOTS;
+  const int nkeys = LV_CLASSES * A.S;
+  int32_t* s_hist = s_off + nkeys + 1;
+  int32_t* s_base = s_hist + nkeys;
+  const int lane = lane_id(), wv = warp_in_block();
+  const int64_t gw = (int64_t)wv * gridDim.x + blockIdx.x, NW = (int64_t)gridDim.x * LV_WARPS;
+  // the warps' tables are consecutive pieces of the block's
+  int32_t* wkeys = keys + wv * LV_SLOTS;
+  long long* wvals = vals + wv * LV_SLOTS;
+  for (int x = threadIdx.x; x < LV_BLOCK_SLOTS; x += LV_THREADS) {
     keys[x] = LV_EMPTY;
     vals[x] = 0;
   }
-  __syncwarp();
-  for (int32_t x = lo + blockIdx.x * LV_WARPS + wv; x < hi; x += gridDim.x * LV_WARPS) {
-    const int32_t i = A.list[x];
-    const long long b = A.off[i], e = A.off[i + 1];
-    for (long long q = b + lane; q < e; q += 32) {
-      const int32_t C = A.cl[A.adj[q]];
-      if (!table_add(keys, vals, LV_SLOTS - 1, C, A.aw[q])) dev_fail(A.status, DEV_HASH_FULL);
-    }
-    __syncwarp();
-    const int32_t own = A.cl[i];
-    const long long ki = A.k[i];
-    Cand best{0, -1};
-    long long kia = 0;
-    for (int s = lane; s < LV_SLOTS; s += 32) {
-      const int32_t C = keys[s];
-      if (C == LV_EMPTY) continue;
-      const long long kic = vals[s];
-      keys[s] = LV_EMPTY;
-      vals[s] = 0;
-      if (C == own) {
-        kia = kic;
-        continue;
+  __syncthreads();
+  unsigned gen = 0;
+  auto sync = [&]() { return grid_sync(false, A.barrier, A.status, gen); };
+  unsigned long long before = 0;
+  int par = 0, rounds = 0;
+  for (int round = 0; round < LV_ROUNDS; ++round) {
+    lv_list(A, round, false, s_off, s_hist, s_base);
+    if (!sync()) return;
+    lv_offsets_of(A, s_off);
+    lv_list(A, round, true, s_off, s_hist, s_base);
+    if (!sync()) return;
+    for (int s = 0; s < A.S; ++s, par ^= 1) {
+      int32_t* words = A.words + par * LV_WORDS;
+      if (blockIdx.x == 0 && threadIdx.x < LV_WORDS) A.words[(par ^ 1) * LV_WORDS + threadIdx.x] = 0;
+      if (s == 0)  // the lists are built: clear their counters for the next round
+        for (int x = blockIdx.x * LV_THREADS + threadIdx.x; x < nkeys; x += gridDim.x * LV_THREADS) {
+          A.cnt[x] = 0;
+          A.fill[x] = 0;
+        }
+      const int32_t* at = s_off + LV_CLASSES * s;
+      // ---- decisions from the state at the start of the sub-round
+      for (int32_t x = at[4] + (int32_t)blockIdx.x; x < at[5]; x += gridDim.x)
+        lv_block(A, words, x, keys, vals);
+      for (int32_t x = at[3] + (int32_t)blockIdx.x; x < at[4]; x += gridDim.x)
+        lv_block(A, words, x, keys, vals);
+      for (int64_t x = at[2] + gw; x < at[3]; x += NW) {
+        const int32_t i = A.list[x].x;
+        const long long b = A.off[i], e = A.off[i + 1];
+        for (long long q = b + lane; q < e; q += 32)
+          if (!table_add(wkeys, wvals, LV_SLOTS - 1, A.cl[A.adj[q]], A.aw[q]))
+            dev_fail(A.status, DEV_HASH_FULL);
+        __syncwarp();
+        Cand best;
+        long long kia;
+        lv_take(A, i, wkeys, wvals, LV_SLOTS, lane, 32, best, kia);
+        lv_emit(A, words, lane == 0 && lv_moves(A, i, kia, best), i, best.c);
+        __syncwarp();
       }
-      cand_better(best, Cand{(i128)A.W2 * kic - (i128)ki * A.vol[C], C});
+      lv_lanes<LV_LANES>(A, words, at[1], at[2], gw, NW);
+      lv_lanes<LV_GROUP>(A, words, at[0], at[1], NW - 1 - gw, NW);
+      __syncwarp();
+      if (!sync()) return;
+      if (at[5] > at[4]) {
+        for (int64_t x = at[4] + gw; x < at[5]; x += NW) {
+          const int2 nd = A.list[x];
+          if ((nd.y & 0xffff) != 0) continue;  // the first part's entry combines
+          const int parts = nd.y >> 16;
+          Cand best{0, -1};
+          long long kia = 0;
+          for (int t = lane; t < parts; t += 32) {
+            const PartBest pb = A.parts[x + t];
+            cand_better(best, Cand{((i128)pb.hi << 64) | (i128)pb.lo, pb.c});
+            kia += pb.kia;
+          }
+          warp_best(best);
+          kia = warp_sum(kia);
+          lv_emit(A, words, lane == 0 && lv_moves(A, nd.x, kia, best), nd.x, best.c);
+        }
+        if (!sync()) return;
+      }
+      // ---- moves: clusters and integer volumes
+      const int32_t nm = __ldcg(words + LV_MOVES);
+      for (int32_t x = blockIdx.x * LV_THREADS + threadIdx.x; x < nm; x += gridDim.x * LV_THREADS) {
+        const int2 mv = A.mv[x];
+        const long long ki = A.k[mv.x];
+        atomic_add_i64(&A.vol[A.cl[mv.x]], -ki);
+        atomic_add_i64(&A.vol[mv.y], ki);
+        A.cl[mv.x] = mv.y;
+      }
+      if (blockIdx.x == 0 && threadIdx.x == 0 && nm)
+        atomicAdd(&A.res[LR_MOVED], (unsigned long long)nm);
+      if (!sync()) return;
     }
-    warp_best(best);
-    kia = warp_sum(kia);
-    if (lane == 0) lv_emit(A, i, kia, best);
-    __syncwarp();
+    rounds = round + 1;
+    const unsigned long long moved = __ldcg(A.res + LR_MOVED);
+    if (100 * (long long)(moved - before) < A.V) break;
+    before = moved;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) A.res[LR_ROUNDS] = (unsigned long long)rounds;
 }
 
-// Class 3, step 1: one thread per edge of the listed vertices [lo, hi):
-// lpre = exclusive prefix of their degrees along the list, toff = offsets of
-// their global tables (relative to tbase).
-__global__ void k_lv_big_insert(LvArgs A, int32_t lo, int32_t hi, const long long* __restrict__ lpre,
-                                const long long* __restrict__ toff, long long tbase,
-                                const int32_t* __restrict__ tsize, int32_t* __restrict__ tkey,
-                                long long* __restrict__ tval) {
-  const long long base = lpre[lo], cnt = lpre[hi] - base;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < cnt;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long y = base + t;
-    int32_t a = lo, b = hi - 1;  // largest x in [lo, hi) with lpre[x] <= y
-    while (a < b) {
-      const int32_t mid = (a + b + 1) >> 1;
-      if (lpre[mid] <= y) a = mid;
-      else b = mid - 1;
-    }
-    const int32_t i = A.list[a];
-    const long long q = A.off[i] + (y - lpre[a]);
-    const long long tb = toff[a] - tbase;
-    if (!table_add(tkey + tb, tval + tb, (uint32_t)tsize[a] - 1, A.cl[A.adj[q]], A.aw[q]))
-      dev_fail(A.status, DEV_HASH_FULL);
-  }
-}
-
-// Class 3, step 2: one block per listed vertex, best entry of its table
-// (cleared on the way for the next sub-round).
-__global__ void __launch_bounds__(LV_ARGMAX_THREADS)
-k_lv_big_argmax(LvArgs A, int32_t lo, int32_t hi, const long long* __restrict__ toff,
-                long long tbase, const int32_t* __restrict__ tsize, int32_t* __restrict__ tkey,
-                long long* __restrict__ tval) {
-  __shared__ long long s_lo[32], s_hi[32], s_kia[32];
-  __shared__ int32_t s_c[32];
-  for (int32_t x = lo + blockIdx.x; x < hi; x += gridDim.x) {
-    const int32_t i = A.list[x];
-    const int32_t own = A.cl[i];
-    const long long ki = A.k[i];
-    const long long tb = toff[x] - tbase;
-    Cand best{0, -1};
-    long long kia = 0;
-    for (int32_t s = threadIdx.x; s < tsize[x]; s += blockDim.x) {
-      const int32_t C = tkey[tb + s];
-      if (C == LV_EMPTY) continue;
-      const long long kic = tval[tb + s];
-      tkey[tb + s] = LV_EMPTY;
-      tval[tb + s] = 0;
-      if (C == own) {
-        kia = kic;
-        continue;
-      }
-      cand_better(best, Cand{(i128)A.W2 * kic - (i128)ki * A.vol[C], C});
-    }
-    warp_best(best);
-    kia = warp_sum(kia);
-    if (lane_id() == 0) {
-      s_lo[warp_in_block()] = (long long)(unsigned long long)best.s;
-      s_hi[warp_in_block()] = (long long)(best.s >> 64);
-      s_c[warp_in_block()] = best.c;
-      s_kia[warp_in_block()] = kia;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      Cand b{0, -1};
-      long long ka = 0;
-      for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) {
-        cand_better(b, Cand{((i128)s_hi[wv] << 64) | (i128)(unsigned long long)s_lo[wv], s_c[wv]});
-        ka += s_kia[wv];
-      }
-      lv_emit(A, i, ka, b);
-    }
-    __syncthreads();
-  }
-}
-
-// Applies the sub-round's moves: cluster and integer volume updates.
-__global__ void k_lv_apply(const int32_t* __restrict__ mv_v, const int32_t* __restrict__ mv_to,
-                           const int32_t* __restrict__ words, const long long* __restrict__ k,
-                           int32_t* __restrict__ cl, long long* __restrict__ vol,
-                           unsigned long long* __restrict__ moved) {
-  const int32_t nm = words[0];
-  for (int32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < nm; x += gridDim.x * blockDim.x) {
-    const int32_t i = mv_v[x], to = mv_to[x];
-    const long long ki = k[i];
-    atomic_add_i64(&vol[cl[i]], -ki);
-    atomic_add_i64(&vol[to], ki);
-    cl[i] = to;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && nm) atomicAdd(moved, (unsigned long long)nm);
+size_t lv_smem(int S) {
+  return (size_t)LV_BLOCK_SLOTS * 12 + (3 * (size_t)LV_CLASSES * S + 1) * sizeof(int32_t);
 }
 
 // ------------------------------------------------------------ aggregation
@@ -721,28 +776,19 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   const int gV = grid_for(V, 256, cx.num_sms, 8);
   k_lv_init<<<gV, 256, 0, cx.stream>>>(V, g.k.p, cl.p, vol.p);
   check_launch("lv_init");
-  DBuf<int32_t> cnt, fill, koff, list, mv_v, mv_to, words, ldeg, tsize;
-  DBuf<long long> lpre, toff;
-  DBuf<unsigned long long> moved;
-  const int nkeys = LV_CLASSES * S;
-  cnt.alloc(&cx.alloc, (size_t)nkeys);
-  fill.alloc(&cx.alloc, (size_t)nkeys);
-  koff.alloc(&cx.alloc, (size_t)nkeys + 1);
-  list.alloc(&cx.alloc, (size_t)V + 1);
-  mv_v.alloc(&cx.alloc, (size_t)V + 1);
-  mv_to.alloc(&cx.alloc, (size_t)V + 1);
-  words.alloc(&cx.alloc, (size_t)S * 4);
-  ldeg.alloc(&cx.alloc, (size_t)V + 1);
-  tsize.alloc(&cx.alloc, (size_t)V + 1);
-  lpre.alloc(&cx.alloc, (size_t)V + 1);
-  toff.alloc(&cx.alloc, (size_t)V + 1);
-  moved.alloc(&cx.alloc, 1);
-  DBuf<long long> bounds;
-  bounds.alloc(&cx.alloc, 2 * ((size_t)nkeys + 1));
-  DBuf<int32_t> tkey;
-  DBuf<long long> tval;
-  size_t tcap = 0;
-  LvArgs A;
+  const size_t nkeys = (size_t)LV_CLASSES * S;
+  // a list entry per vertex, and one per further part of a large vertex
+  const size_t entries = (size_t)V + (size_t)(g.E / LV_PART) + 1;
+  DBuf<int2> list, mv;
+  DBuf<PartBest> parts;
+  DBuf<unsigned long long> zero;  // results, then 32-bit counters
+  list.alloc(&cx.alloc, entries);
+  mv.alloc(&cx.alloc, (size_t)V + 1);
+  parts.alloc(&cx.alloc, entries);
+  zero.alloc(&cx.alloc, LR_LV_WORDS + nkeys + LV_WORDS + 1);
+  HG_CUDA(cudaMemsetAsync(zero.p, 0, zero.bytes(), cx.stream));
+  int32_t* z = reinterpret_cast<int32_t*>(zero.p + LR_LV_WORDS);
+  LvArgs A{};
   A.off = g.off.p;
   A.adj = g.adj.p;
   A.aw = g.aw.p;
@@ -750,93 +796,41 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   A.cl = cl.p;
   A.vol = vol.p;
   A.W2 = W2;
+  A.V = V;
+  A.seed = seed;
+  A.level = level;
+  A.S = S;
   A.list = list.p;
-  A.mv_v = mv_v.p;
-  A.mv_to = mv_to.p;
+  A.cnt = z;
+  A.fill = z + nkeys;
+  A.words = z + 2 * nkeys;
+  A.barrier = reinterpret_cast<unsigned*>(z + 2 * nkeys + 2 * LV_WORDS);
+  A.mv = mv.p;
+  A.parts = parts.p;
+  A.res = zero.p;
   A.status = cx.d_status;
-  int64_t level_moves = 0;
-  for (int round = 0; round < LV_ROUNDS; ++round) {
-    HG_CUDA(cudaMemsetAsync(cnt.p, 0, cnt.bytes(), cx.stream));
-    HG_CUDA(cudaMemsetAsync(fill.p, 0, fill.bytes(), cx.stream));
-    HG_CUDA(cudaMemsetAsync(words.p, 0, words.bytes(), cx.stream));
-    HG_CUDA(cudaMemsetAsync(moved.p, 0, moved.bytes(), cx.stream));
-    k_lv_count<<<gV, 256, nkeys * sizeof(int32_t), cx.stream>>>(g.off.p, V, seed, level, round, S,
-                                                                 cnt.p);
-    check_launch("lv_count");
-    scan_exclusive_i32(cx, cnt.p, koff.p, nkeys, koff.p + nkeys);
-    k_lv_scatter<<<gV, 256, 0, cx.stream>>>(g.off.p, V, seed, level, round, S, koff.p, fill.p,
-                                            list.p);
-    check_launch("lv_scatter");
-    // degrees and table sizes along the list, class-3 tables per sub-round
-    k_lv_list_sizes<<<gV, 256, 0, cx.stream>>>(list.p, koff.p + nkeys, (int32_t)V, g.off.p, ldeg.p,
-                                               tsize.p);
-    check_launch("lv_list_sizes");
-    scan_exclusive_i32_to_i64(cx, ldeg.p, reinterpret_cast<int64_t*>(lpre.p), V,
-                              reinterpret_cast<int64_t*>(lpre.p) + V);
-    scan_exclusive_i32_to_i64(cx, tsize.p, reinterpret_cast<int64_t*>(toff.p), V,
-                              reinterpret_cast<int64_t*>(toff.p) + V);
-    k_lv_bounds<<<1, 256, 0, cx.stream>>>(koff.p, nkeys, toff.p, bounds.p);
-    check_launch("lv_bounds");
-    std::vector<long long> hb(2 * ((size_t)nkeys + 1));
-    wait_stream(cx);
-    HG_CUDA(cudaMemcpyAsync(hb.data(), bounds.p, sizeof(long long) * hb.size(),
-                            cudaMemcpyDeviceToHost, cx.stream));
-    check_status(cx);
-    const long long* hkoff = hb.data();
-    const long long* htoff = hb.data() + nkeys + 1;
-    size_t need = 1;
-    for (int s = 0; s < S; ++s)
-      need = std::max<size_t>(need, (size_t)(htoff[LV_CLASSES * s + 4] - htoff[LV_CLASSES * s + 3]));
-    if (need > tcap) {
-      tkey.alloc(&cx.alloc, need);
-      tval.alloc(&cx.alloc, need);
-      HG_CUDA(cudaMemsetAsync(tkey.p, 0xff, tkey.bytes(), cx.stream));
-      HG_CUDA(cudaMemsetAsync(tval.p, 0, tval.bytes(), cx.stream));
-      tcap = need;
-    }
-    for (int s = 0; s < S; ++s) {
-      A.words = words.p + 4 * s;
-      int32_t at[LV_CLASSES + 1];
-      for (int c = 0; c <= LV_CLASSES; ++c) at[c] = (int32_t)hkoff[LV_CLASSES * s + c];
-      if (at[1] > at[0]) {
-        k_lv_lanes<LV_GROUP><<<grid_for(at[1] - at[0], LV_WARPS * (32 / LV_GROUP), cx.num_sms, 8),
-                               LV_WARPS * 32, 0, cx.stream>>>(A, at[0], at[1]);
-        check_launch("lv_lanes");
-        lc.launches += 1;
-      }
-      if (at[2] > at[1]) {
-        k_lv_lanes<LV_LANES><<<grid_for(at[2] - at[1], LV_WARPS, cx.num_sms, 8), LV_WARPS * 32, 0,
-                               cx.stream>>>(A, at[1], at[2]);
-        check_launch("lv_lanes");
-        lc.launches += 1;
-      }
-      if (at[3] > at[2]) {
-        k_lv_small<<<grid_for(at[3] - at[2], LV_WARPS, cx.num_sms, 8), LV_WARPS * 32, 0,
-                     cx.stream>>>(A, at[2], at[3]);
-        check_launch("lv_small");
-        lc.launches += 1;
-      }
-      if (at[4] > at[3]) {
-        const long long tbase = htoff[LV_CLASSES * s + 3];
-        k_lv_big_insert<<<cx.num_sms * 8, 256, 0, cx.stream>>>(A, at[3], at[4], lpre.p, toff.p,
-                                                               tbase, tsize.p, tkey.p, tval.p);
-        check_launch("lv_big_insert");
-        k_lv_big_argmax<<<grid_for(at[4] - at[3], 1, cx.num_sms, 8), LV_ARGMAX_THREADS, 0,
-                          cx.stream>>>(A, at[3], at[4], toff.p, tbase, tsize.p, tkey.p, tval.p);
-        check_launch("lv_big_argmax");
-        lc.launches += 2;
-      }
-      k_lv_apply<<<grid_for((V + S - 1) / S, 256, cx.num_sms, 4), 256, 0, cx.stream>>>(
-          mv_v.p, mv_to.p, A.words, g.k.p, cl.p, vol.p, moved.p);
-      check_launch("lv_apply");
-      lc.launches += 1;
-    }
-    const int64_t m = read_i64(cx, reinterpret_cast<const int64_t*>(moved.p));
-    level_moves += m;
-    lc.rounds += 1;
-    if (100 * m < V) break;
-  }
-  return level_moves;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    HG_CUDA(cudaFuncSetAttribute(k_lv_run, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)lv_smem(256)));
+  });
+  const size_t smem = lv_smem(S);
+  int per_sm = 0;
+  HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lv_run, LV_THREADS, smem));
+  if (per_sm < 1) throw HgError(HG_ERR_CUDA, "local moving does not fit an SM");
+  // a block per 16 vertices or 256 edges of a sub-round (coarse levels: heavy
+  // vertices take a block each); four times that when the handle shares the GPU
+  // with others (it sleeps while it waits)
+  const int64_t share = cx.sync_event ? 4 : 1;
+  const int64_t need =
+      std::max<int64_t>(V / (S * 16 * share), g.E / (S * 256 * share)) + 1;
+  const int blocks = (int)std::min<int64_t>(need, (int64_t)cx.num_sms * std::min(per_sm, 2));
+  launch_persistent(cx, k_lv_run, blocks, LV_THREADS, smem, false, A);
+  lc.launches += 1;
+  unsigned long long hres[LR_LV_WORDS];
+  read_back(cx, hres, A.res, sizeof(hres));
+  lc.rounds += (int64_t)hres[LR_ROUNDS];
+  return (int64_t)hres[LR_MOVED];
 }
 
 }  // namespace
