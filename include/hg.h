@@ -132,7 +132,7 @@ typedef struct {
   double ms_lp_select;  /* move gathering or bucketing and prefix selection (a12) */
   double ms_lp_apply;   /* move application (a13) */
   double ms_objective;  /* objective (a14) */
-  double ms_initial;    /* host initial partition incl. copies */
+  double ms_initial;    /* initial partition */
   int64_t launches;     /* kernels launched */
   int64_t rating_launches;
   int64_t rating_pin_visits;  /* pins read by the rating kernels */
@@ -206,8 +206,8 @@ int hg_level_info(const hg_t* h, int32_t level, int32_t* out_n, int32_t* out_m, 
 /* Seeded initial partition of a level (the paper's portfolio of Sec. 5 is
  * replaced by one deterministic rule): nodes in order of
  * (mix64(seed ^ 2^63 ^ u), u), each to the lightest block so far, ties to the
- * smaller block id; mix64 = the SplitMix64 output function.  Computed on the
- * host from the level's node weights.  part: device, n_level int32, written. */
+ * smaller block id; mix64 = the SplitMix64 output function.  part: device,
+ * n_level int32, written.  Synchronizes the stream. */
 int hg_initial_partition(hg_t* h, int32_t level, int32_t k, int32_t* part);
 
 /* Projection Pi_l[u] = Pi_{l+1}[map(u)] from level coarse_level (>= 1) to

@@ -1,11 +1,9 @@
 // C ABI of the library (declared in include/hg.h): the handle holding the
-// level hierarchy, argument checking, the multilevel loop of Algorithm 1 and
-// the seeded host-side initial partition.
+// level hierarchy, argument checking and the multilevel loop of Algorithm 1.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <memory>
-#include <numeric>
 #include <thread>
 #include <vector>
 
@@ -361,27 +359,9 @@ int hg_initial_partition(hg_t* h, int32_t level, int32_t k, int32_t* part) {
   if (!valid_level(h, level)) return HG_ERR_STATE;
   return guarded(h, [&]() -> int {
     hgk::EventTimer tm(h->cx, &h->stats.ms_initial);
-    const Level& L = *h->levels[level];
-    std::vector<int32_t> c((size_t)L.n), out((size_t)L.n);
-    HG_CUDA(cudaMemcpyAsync(c.data(), L.c.p, sizeof(int32_t) * (size_t)L.n,
-                            cudaMemcpyDeviceToHost, h->cx.stream));
-    HG_CUDA(cudaStreamSynchronize(h->cx.stream));
-    // order of (mix64(seed ^ 2^63 ^ u), u); each node to the lightest block
-    std::vector<std::pair<uint64_t, int32_t>> order((size_t)L.n);
-    for (int32_t u = 0; u < L.n; ++u)
-      order[u] = {hgk::mix64(h->opt.seed ^ (1ull << 63) ^ (uint64_t)(uint32_t)u), u};
-    std::sort(order.begin(), order.end());
-    std::vector<int64_t> bw((size_t)k, 0);
-    for (const auto& kv : order) {
-      int best = 0;
-      for (int b = 1; b < k; ++b)
-        if (bw[b] < bw[best]) best = b;
-      out[kv.second] = best;
-      bw[best] += c[kv.second];
-    }
-    HG_CUDA(cudaMemcpyAsync(part, out.data(), sizeof(int32_t) * (size_t)L.n,
-                            cudaMemcpyHostToDevice, h->cx.stream));
-    HG_CUDA(cudaStreamSynchronize(h->cx.stream));
+    hgk::initial_partition(h->cx, *h->levels[level], k, h->opt.seed, part);
+    sync_stats(h);
+    hgk::wait_stream(h->cx);
     return HG_OK;
   });
 }

@@ -408,6 +408,9 @@ struct PinState {
 void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, PinState& st,
                      bool counts);
 
+// Seeded initial partition of a level into k blocks (initial.cu).
+void initial_partition(const Ctx& cx, const Level& L, int k, uint64_t seed, int32_t* part);
+
 void project_partition(const Ctx& cx, const Level& fine, const int32_t* coarse_part,
                        int32_t* fine_part);
 
