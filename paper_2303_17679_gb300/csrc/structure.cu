@@ -90,8 +90,10 @@ __global__ void k_validate_nodes(const int32_t* __restrict__ c, int32_t n, int32
 // No node twice in a net.  One warp per net of at most DISTINCT_SMALL pins:
 // nets of at most 32 pins compare lanes with a match; larger ones insert
 // their pins into a per-warp hash set in shared memory (a pin found already
-// present is a repeat).  Larger nets are left to k_distinct_big.  Runs only
-// on offsets and pins already checked, so every read stays in bounds.
+// present is a repeat).  Larger nets are listed for k_distinct_big (a block
+// that looks for them among all nets waits on two offsets per net: 5 of 6 ms at
+// 2e6 nets).  Runs only on offsets and pins already checked, so every read
+// stays in bounds.
 constexpr int DISTINCT_WARPS = 4;
 constexpr int DISTINCT_SMALL = 1024;
 // largest total of the per-block node bitmaps of k_distinct_big_bitmap
@@ -124,7 +126,7 @@ __device__ __forceinline__ void set_erase(int32_t* set, uint32_t mask, int32_t v
 
 __global__ void __launch_bounds__(DISTINCT_WARPS * 32)
 k_distinct_small(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins, int32_t m,
-                 int32_t* status) {
+                 int32_t* __restrict__ big, int32_t* __restrict__ nbig, int32_t* status) {
   __shared__ int32_t s_set[DISTINCT_WARPS][DISTINCT_SET];
   const int wv = warp_in_block(), lane = lane_id();
   int32_t* set = s_set[wv];
@@ -133,7 +135,10 @@ k_distinct_small(const int32_t* __restrict__ eoff, const int32_t* __restrict__ p
   for (int64_t e = (int64_t)blockIdx.x * DISTINCT_WARPS + wv; e < m;
        e += (int64_t)gridDim.x * DISTINCT_WARPS) {
     const int32_t b = eoff[e], sz = eoff[e + 1] - b;
-    if (sz > DISTINCT_SMALL) continue;
+    if (sz > DISTINCT_SMALL) {
+      if (lane == 0) big[atomicAdd(nbig, 1)] = (int32_t)e;
+      continue;
+    }
     bool dup = false;
     if (sz <= 32) {
       const int32_t v = lane < sz ? pins[b + lane] : -1 - lane;
@@ -152,13 +157,14 @@ k_distinct_small(const int32_t* __restrict__ eoff, const int32_t* __restrict__ p
 // slots (a power of two >= twice the largest net) in this block's region of
 // `scratch` (all slots -1 on entry, restored before the block moves on).
 __global__ void k_distinct_big(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
-                               int32_t m, int32_t* __restrict__ scratch, uint32_t cap,
-                               int32_t* status) {
+                               const int32_t* __restrict__ big, const int32_t* __restrict__ nbig,
+                               int32_t* __restrict__ scratch, uint32_t cap, int32_t* status) {
   int32_t* set = scratch + (size_t)blockIdx.x * cap;
   __shared__ int s_dup;
-  for (int64_t e = blockIdx.x; e < m; e += gridDim.x) {
+  const int32_t cnt = *nbig;
+  for (int32_t x = blockIdx.x; x < cnt; x += gridDim.x) {
+    const int32_t e = big[x];
     const int32_t b = eoff[e], sz = eoff[e + 1] - b;
-    if (sz <= DISTINCT_SMALL) continue;
     if (threadIdx.x == 0) s_dup = 0;
     __syncthreads();
     bool dup = false;
@@ -175,14 +181,17 @@ __global__ void k_distinct_big(const int32_t* __restrict__ eoff, const int32_t* 
 // bitmaps of all blocks are small: one atomicOr per pin finds a repeat and one
 // atomicAnd per pin clears the net's bits again, with no probing.
 __global__ void k_distinct_big_bitmap(const int32_t* __restrict__ eoff,
-                                      const int32_t* __restrict__ pins, int32_t m,
+                                      const int32_t* __restrict__ pins,
+                                      const int32_t* __restrict__ big,
+                                      const int32_t* __restrict__ nbig,
                                       uint32_t* __restrict__ scratch, int64_t words,
                                       int32_t* status) {
   uint32_t* set = scratch + (size_t)blockIdx.x * (size_t)words;
   __shared__ int s_dup;
-  for (int64_t e = blockIdx.x; e < m; e += gridDim.x) {
+  const int32_t cnt = *nbig;
+  for (int32_t x = blockIdx.x; x < cnt; x += gridDim.x) {
+    const int32_t e = big[x];
     const int32_t b = eoff[e], sz = eoff[e + 1] - b;
-    if (sz <= DISTINCT_SMALL) continue;
     if (threadIdx.x == 0) s_dup = 0;
     __syncthreads();
     bool dup = false;
@@ -314,8 +323,13 @@ bool distinct_pins(const Ctx& cx, const Level& L) {
   HG_CUDA(cudaMemsetAsync(mx.p, 0, sizeof(int32_t), cx.stream));
   k_max_net_size<<<grid_for(L.m, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(L.eoff.p, L.m, mx.p);
   check_launch("max_net_size");
+  DBuf<int32_t> big;  // nets above DISTINCT_SMALL pins, then their number
+  const size_t nb = (size_t)(L.p / (DISTINCT_SMALL + 1)) + 1;
+  big.alloc(&cx.alloc, nb + 1);
+  int32_t* nbig = big.p + nb;
+  HG_CUDA(cudaMemsetAsync(nbig, 0, sizeof(int32_t), cx.stream));
   k_distinct_small<<<grid_for(L.m, DISTINCT_WARPS, cx.num_sms, 16), DISTINCT_WARPS * 32, 0,
-                     cx.stream>>>(L.eoff.p, L.pins.p, L.m, cx.d_status);
+                     cx.stream>>>(L.eoff.p, L.pins.p, L.m, big.p, nbig, cx.d_status);
   check_launch("distinct_small");
   const int32_t biggest = read_i32(cx, mx.p);
   const int64_t words = ((int64_t)L.n + 31) / 32;
@@ -324,8 +338,8 @@ bool distinct_pins(const Ctx& cx, const Level& L) {
     DBuf<uint32_t> scratch;
     scratch.alloc(&cx.alloc, (size_t)blocks * (size_t)words);
     HG_CUDA(cudaMemsetAsync(scratch.p, 0, scratch.bytes(), cx.stream));
-    k_distinct_big_bitmap<<<blocks, 256, 0, cx.stream>>>(L.eoff.p, L.pins.p, L.m, scratch.p,
-                                                         words, cx.d_status);
+    k_distinct_big_bitmap<<<blocks, 1024, 0, cx.stream>>>(L.eoff.p, L.pins.p, big.p, nbig,
+                                                          scratch.p, words, cx.d_status);
     check_launch("distinct_big_bitmap");
   } else if (biggest > DISTINCT_SMALL) {
     uint32_t cap = 1;
@@ -334,8 +348,8 @@ bool distinct_pins(const Ctx& cx, const Level& L) {
     DBuf<int32_t> scratch;
     scratch.alloc(&cx.alloc, (size_t)blocks * cap);
     HG_CUDA(cudaMemsetAsync(scratch.p, 0xff, scratch.bytes(), cx.stream));
-    k_distinct_big<<<blocks, 256, 0, cx.stream>>>(L.eoff.p, L.pins.p, L.m, scratch.p, cap,
-                                                  cx.d_status);
+    k_distinct_big<<<blocks, 1024, 0, cx.stream>>>(L.eoff.p, L.pins.p, big.p, nbig, scratch.p,
+                                                   cap, cx.d_status);
     check_launch("distinct_big");
   }
   if (read_status(cx, nullptr, nullptr, 0) != DEV_OK) {
