@@ -14,6 +14,7 @@
 //       sums over a keep flag and the kept sizes, then the incidence lists.
 #include <algorithm>
 #include <climits>
+#include <mutex>
 
 #include "common.cuh"
 
@@ -21,10 +22,24 @@ namespace hgk {
 
 namespace {
 
+// Net size classes of the remap: a thread, a warp, a block, a block per net.  A
+// block per net of 33..1024 pins spends its time at the barriers of its sort and
+// two block-wide sums; a warp needs none.  Where the coarse nodes fit a bitmap in
+// shared memory, marking them replaces the O(log^2) steps of the sort and the
+// cleared bitmap in global memory.  Measured (GB300, with compaction and the
+// comparison of identical nets by eight lanes per net): coarsening of a 4e6-node
+// large-net input, k = 64: 104.9 -> 95.8 ms; of 1e6 Zipf nodes, k = 8: 56 -> 52.5 ms.
 constexpr int SMALL_NET = 32;
+constexpr int WARP_NET = 1024;
 constexpr int MID_NET = 4096;
+constexpr int NCLS = 4;
+constexpr int WARP_NETS = 8;        // warps per block of the warp class
 constexpr int MID_THREADS = 256;
 constexpr int BIG_THREADS = 512;
+// Coarse nodes up to which a net's pins are marked in a shared bitmap instead
+// of being sorted: a warp's bitmap of 2 KB, a block's of 64 KB.
+constexpr int32_t WARP_BITMAP_N = 16384;
+constexpr int32_t BLOCK_BITMAP_N = 1 << 19;
 constexpr unsigned long long EMPTY_FP = ~0ull;
 
 __global__ void k_rep_flags(const int32_t* __restrict__ rep, int32_t n, int32_t* __restrict__ flag) {
@@ -53,7 +68,7 @@ __global__ void k_classify_nets(const int32_t* __restrict__ eoff, int32_t m,
     int cls = -1;
     if (valid) {
       const int32_t sz = eoff[e + 1] - eoff[e];
-      cls = sz <= SMALL_NET ? 0 : (sz <= MID_NET ? 1 : 2);
+      cls = sz <= SMALL_NET ? 0 : sz <= WARP_NET ? 1 : sz <= MID_NET ? 2 : 3;
     }
     const int32_t slot = warp_claim_slot(counts, cls, __ballot_sync(FULL, valid));
     if (valid) lists[(int64_t)cls * m + slot] = (int32_t)e;
@@ -102,7 +117,221 @@ __global__ void k_remap_small(const int32_t* __restrict__ list, int32_t count,
   }
 }
 
-// Nets of 33..4096 pins: one block per net, bitonic sort with the keys in
+// Nets of 33..1024 pins on levels of few coarse nodes: one warp per net marks
+// the coarse nodes in a bitmap in shared memory and writes the set bits in
+// ascending order (each lane a run of words).
+__global__ void __launch_bounds__(WARP_NETS * 32)
+k_remap_warp_bitmap(const int32_t* __restrict__ list, int32_t count,
+                    const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+                    const int32_t* __restrict__ map, int32_t words, int fp_bits,
+                    int32_t* __restrict__ tpins, int32_t* __restrict__ tsize,
+                    unsigned long long* __restrict__ fp) {
+  // one pad word per 32, so that the lanes' runs start in different banks
+  constexpr int CAP = WARP_BITMAP_N / 32;
+  __shared__ unsigned s_bits[WARP_NETS][CAP + CAP / 32 + 1];
+  unsigned* bits = s_bits[warp_in_block()];
+  const int lane = lane_id();
+  const int per = (words + 31) / 32;  // words per lane
+  auto at = [](int w) { return w + (w >> 5); };
+  for (int w = lane; w < words; w += 32) bits[at(w)] = 0u;
+  __syncwarp();
+  for (int32_t i = blockIdx.x * WARP_NETS + warp_in_block(); i < count;
+       i += gridDim.x * WARP_NETS) {
+    const int32_t e = list[i];
+    const int32_t b = eoff[e], sz = eoff[e + 1] - b;
+    for (int q = lane; q < sz; q += 64) {
+      const bool two = q + 32 < sz;
+      const int32_t p0 = pins[b + q], p1 = two ? pins[b + q + 32] : p0;
+      const int32_t v0 = map[p0], v1 = map[p1];
+      atomicOr(&bits[at(v0 >> 5)], 1u << (v0 & 31));
+      if (two) atomicOr(&bits[at(v1 >> 5)], 1u << (v1 & 31));
+    }
+    __syncwarp();
+    int c = 0;
+    for (int x = 0; x < per; ++x) {
+      const int w = lane * per + x;
+      if (w < words) c += __popc(bits[at(w)]);
+    }
+    const int incl = warp_inclusive_scan(c);
+    int32_t pos = b + incl - c;
+    unsigned long long sum = 0;
+    for (int x = 0; x < per; ++x) {
+      const int w = lane * per + x;
+      if (w >= words) break;
+      unsigned rest = bits[at(w)];
+      bits[at(w)] = 0u;
+      while (rest) {
+        const int32_t v = (w << 5) + __ffs(rest) - 1;
+        rest &= rest - 1;
+        tpins[pos++] = v;
+        sum += mix64((unsigned long long)(uint32_t)v);
+      }
+    }
+    sum = warp_sum(sum);
+    if (lane == 31) {
+      tsize[e] = incl;
+      fp[e] = fingerprint_finish(sum, incl, fp_bits);
+    }
+    __syncwarp();
+  }
+}
+
+// One net of at most 32 R pins by the warp: a bitonic sort with R keys per lane
+// in registers (in-thread swaps below R, lane shuffles above), then the first
+// key of every run is kept.
+template <int R>
+__device__ __forceinline__ void remap_sort(int32_t e, int32_t b, int32_t sz,
+                                           const int32_t* __restrict__ pins,
+                                           const int32_t* __restrict__ map, int fp_bits,
+                                           int32_t* __restrict__ tpins,
+                                           int32_t* __restrict__ tsize,
+                                           unsigned long long* __restrict__ fp) {
+  const int lane = lane_id();
+  int32_t v[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int32_t i = r * 32 + lane;  // any arrangement sorts
+    v[r] = i < sz ? map[pins[b + i]] : INT_MAX;
+  }
+#pragma unroll 1
+  for (int kk = 2; kk <= 32 * R; kk <<= 1) {
+#pragma unroll 1
+    for (int j = kk >> 1; j >= R; j >>= 1) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = lane * R + r;
+        const int32_t y = __shfl_xor_sync(FULL, v[r], j / R);
+        const bool keep_min = ((i & kk) == 0) == ((i & j) == 0);
+        v[r] = keep_min ? min(v[r], y) : max(v[r], y);
+      }
+    }
+#pragma unroll
+    for (int j = R / 2; j > 0; j >>= 1) {
+      if (j >= kk) continue;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if ((r ^ j) > r) {
+          const bool up = ((lane * R + r) & kk) == 0;
+          const int32_t lo = min(v[r], v[r ^ j]), hi = max(v[r], v[r ^ j]);
+          v[r] = up ? lo : hi;
+          v[r ^ j] = up ? hi : lo;
+        }
+      }
+    }
+  }
+  // lane l holds keys l R .. l R + R - 1 of the sorted net
+  const int32_t before = __shfl_up_sync(FULL, v[R - 1], 1);
+  int c = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int32_t prev = r == 0 ? (lane == 0 ? -1 : before) : v[r - 1];
+    c += v[r] != INT_MAX && v[r] != prev;
+  }
+  const int incl = warp_inclusive_scan(c);
+  int32_t pos = b + incl - c;
+  unsigned long long sum = 0;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int32_t prev = r == 0 ? (lane == 0 ? -1 : before) : v[r - 1];
+    if (v[r] != INT_MAX && v[r] != prev) {
+      tpins[pos++] = v[r];
+      sum += mix64((unsigned long long)(uint32_t)v[r]);
+    }
+  }
+  sum = warp_sum(sum);
+  if (lane == 31) {
+    tsize[e] = incl;
+    fp[e] = fingerprint_finish(sum, incl, fp_bits);
+  }
+}
+
+// Nets of 33..1024 pins on the other levels, one warp per net.
+__global__ void __launch_bounds__(WARP_NETS * 32)
+k_remap_warp_sort(const int32_t* __restrict__ list, int32_t count,
+                  const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+                  const int32_t* __restrict__ map, int fp_bits, int32_t* __restrict__ tpins,
+                  int32_t* __restrict__ tsize, unsigned long long* __restrict__ fp) {
+  for (int32_t i = blockIdx.x * WARP_NETS + warp_in_block(); i < count;
+       i += gridDim.x * WARP_NETS) {
+    const int32_t e = list[i];
+    const int32_t b = eoff[e], sz = eoff[e + 1] - b;
+    if (sz <= 128) remap_sort<4>(e, b, sz, pins, map, fp_bits, tpins, tsize, fp);
+    else if (sz <= 512) remap_sort<16>(e, b, sz, pins, map, fp_bits, tpins, tsize, fp);
+    else remap_sort<32>(e, b, sz, pins, map, fp_bits, tpins, tsize, fp);
+  }
+}
+
+// Nets of more than 1024 pins on levels whose coarse nodes fit a bitmap in
+// shared memory: one block per net, every thread a run of words, one block-wide
+// scan per net.
+__global__ void __launch_bounds__(BIG_THREADS)
+k_remap_block_bitmap(const int32_t* __restrict__ list, int32_t count,
+                     const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+                     const int32_t* __restrict__ map, int32_t words, int fp_bits,
+                     int32_t* __restrict__ tpins, int32_t* __restrict__ tsize,
+                     unsigned long long* __restrict__ fp) {
+  extern __shared__ unsigned bits[];  // one pad word per 32
+  __shared__ int32_t s_wsum[BIG_THREADS / 32];
+  __shared__ unsigned long long s_red[32];
+  const int per = (words + BIG_THREADS - 1) / BIG_THREADS;
+  auto at = [](int w) { return w + (w >> 5); };
+  for (int w = threadIdx.x; w < words; w += BIG_THREADS) bits[at(w)] = 0u;
+  __syncthreads();
+  for (int32_t i = blockIdx.x; i < count; i += gridDim.x) {
+    const int32_t e = list[i];
+    const int32_t b = eoff[e], sz = eoff[e + 1] - b;
+    for (int32_t q0 = threadIdx.x; q0 < sz; q0 += 4 * BIG_THREADS) {
+      int32_t v[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int64_t q = (int64_t)q0 + x * BIG_THREADS;
+        v[x] = q < sz ? pins[b + q] : -1;
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        if (v[x] >= 0) v[x] = map[v[x]];
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        if (v[x] >= 0) atomicOr(&bits[at(v[x] >> 5)], 1u << (v[x] & 31));
+    }
+    __syncthreads();
+    int c = 0;
+    for (int x = 0; x < per; ++x) {
+      const int w = threadIdx.x * per + x;
+      if (w < words) c += __popc(bits[at(w)]);
+    }
+    const int incl = warp_inclusive_scan(c);
+    if (lane_id() == 31) s_wsum[warp_in_block()] = incl;
+    __syncthreads();
+    int32_t before = 0, total = 0;
+#pragma unroll
+    for (int x = 0; x < BIG_THREADS / 32; ++x) {
+      if (x < warp_in_block()) before += s_wsum[x];
+      total += s_wsum[x];
+    }
+    int32_t pos = b + before + incl - c;
+    unsigned long long sum = 0;
+    for (int x = 0; x < per; ++x) {
+      const int w = threadIdx.x * per + x;
+      if (w >= words) break;
+      unsigned rest = bits[at(w)];
+      bits[at(w)] = 0u;
+      while (rest) {
+        const int32_t v = (w << 5) + __ffs(rest) - 1;
+        rest &= rest - 1;
+        tpins[pos++] = v;
+        sum += mix64((unsigned long long)(uint32_t)v);
+      }
+    }
+    sum = block_sum(sum, s_red);  // ends with the bitmap clear and a barrier passed
+    if (threadIdx.x == 0) {
+      tsize[e] = total;
+      fp[e] = fingerprint_finish(sum, total, fp_bits);
+    }
+  }
+}
+
+// Nets of 1025..4096 pins on the other levels: one block per net, bitonic sort with the keys in
 // registers (shared memory only for the exchanges between warps).
 __global__ void __launch_bounds__(MID_THREADS, 1024 / MID_THREADS)
 k_remap_mid(const int32_t* __restrict__ list, int32_t count, const int32_t* __restrict__ eoff,
@@ -311,33 +540,50 @@ __global__ void k_ident_insert(const int32_t* __restrict__ list, const int32_t* 
   }
 }
 
-// One warp per candidate net: compare with its group's smallest id.
+// Eight lanes per candidate net: compare with its group's smallest id (nets of
+// many pins by the whole warp).
+constexpr int CMP_LANES = 8;
+constexpr int32_t CMP_SMALL = 128;
+
 __global__ void k_ident_compare(const int32_t* __restrict__ list, const int32_t* __restrict__ count,
                                 const int32_t* __restrict__ eoff, const int32_t* __restrict__ tpins,
                                 const int32_t* __restrict__ tsize,
                                 const int32_t* __restrict__ slot_of_net,
                                 const int32_t* __restrict__ tmin, int32_t* __restrict__ repnet,
                                 int32_t* __restrict__ failed, int32_t* __restrict__ nfailed) {
+  constexpr int PER = 32 / CMP_LANES;
   const int32_t cnt = *count;
-  const int wv = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t i = wv; i < cnt; i += nwarps) {
-    const int32_t e = list[i];
-    const int32_t r = tmin[slot_of_net[e]];
+  const int lane = lane_id(), sub = lane % CMP_LANES, grp = lane / CMP_LANES;
+  const unsigned mine = ((1u << CMP_LANES) - 1u) << (grp * CMP_LANES);
+  const int64_t stride = (((int64_t)gridDim.x * blockDim.x) >> 5) * PER;
+  for (int64_t i0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * PER; i0 < cnt;
+       i0 += stride) {
+    const int64_t i = i0 + grp;
+    const bool on = i < cnt;
+    const int32_t e = on ? list[i] : 0;
+    const int32_t r = on ? tmin[slot_of_net[e]] : 0;
+    const int32_t sz = on ? tsize[e] : 0;
     bool same = true;
-    if (r != e) {
-      const int32_t sz = tsize[e];
-      if (tsize[r] != sz) {
-        same = false;
-      } else {
-        const int32_t* a = tpins + eoff[e];
-        const int32_t* bb = tpins + eoff[r];
-        for (int32_t q = lane_id(); q < sz; q += 32)
-          if (a[q] != bb[q]) same = false;
-        same = __all_sync(FULL, same);
-      }
+    const bool check = on && r != e;
+    if (check) same = tsize[r] == sz;
+    const int32_t ea = on ? eoff[e] : 0, eb = on ? eoff[r] : 0;
+    const bool walk = check && same;
+    for (int32_t q = sub; walk && sz <= CMP_SMALL && q < sz; q += CMP_LANES)
+      if (tpins[ea + q] != tpins[eb + q]) same = false;
+    __syncwarp();
+    unsigned wide = __ballot_sync(FULL, walk && sz > CMP_SMALL && sub == 0);
+    while (wide) {
+      const int l = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int32_t wa = __shfl_sync(FULL, ea, l), wb = __shfl_sync(FULL, eb, l);
+      const int32_t ws = __shfl_sync(FULL, sz, l);
+      bool eq = true;
+      for (int32_t q = lane; q < ws; q += 32) eq &= tpins[wa + q] == tpins[wb + q];
+      eq = __all_sync(FULL, eq);
+      if (lane / CMP_LANES == l / CMP_LANES) same = eq;
     }
-    if (lane_id() == 0) {
+    same = (__ballot_sync(FULL, same) & mine) == mine;
+    if (sub == 0 && on) {
       if (same) repnet[e] = r;
       else failed[atomicAdd(nfailed, 1)] = e;
     }
@@ -357,21 +603,45 @@ __global__ void k_net_weights(const int32_t* __restrict__ tsize, const int32_t* 
   }
 }
 
-// One warp per kept net: write its coarse offset, weight and pins.
+// Eight lanes per kept net write its coarse offset, weight and pins (nets of
+// many pins by the whole warp, four pins per lane in flight).
+constexpr int CP_LANES = 8;
+constexpr int32_t CP_SMALL = 64;
+
 __global__ void k_compact(const int32_t* __restrict__ keep, const int32_t* __restrict__ newid,
                           const int32_t* __restrict__ poff, const int32_t* __restrict__ eoff,
                           const int32_t* __restrict__ tpins, const int32_t* __restrict__ tsize,
                           const int32_t* __restrict__ wsum, int32_t m, int32_t* __restrict__ eoff2,
                           int32_t* __restrict__ pins2, int32_t* __restrict__ w2) {
-  const int wv = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int32_t e = wv; e < m; e += nwarps) {
-    if (!keep[e]) continue;
-    const int32_t id = newid[e], dst = poff[e], src = eoff[e], sz = tsize[e];
-    for (int32_t q = lane_id(); q < sz; q += 32) pins2[dst + q] = tpins[src + q];
-    if (lane_id() == 0) {
+  constexpr int PER = 32 / CP_LANES;
+  const int lane = lane_id(), sub = lane % CP_LANES;
+  const int64_t stride = (((int64_t)gridDim.x * blockDim.x) >> 5) * PER;
+  for (int64_t e0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * PER; e0 < m;
+       e0 += stride) {
+    const int64_t e = e0 + lane / CP_LANES;
+    const bool on = e < m && keep[e];
+    const int32_t dst = on ? poff[e] : 0, src = on ? eoff[e] : 0, sz = on ? tsize[e] : 0;
+    if (on && sub == 0) {
+      const int32_t id = newid[e];
       eoff2[id] = dst;
       w2[id] = wsum[e];
+    }
+    for (int32_t q = sub; sz <= CP_SMALL && q < sz; q += CP_LANES) pins2[dst + q] = tpins[src + q];
+    __syncwarp();
+    unsigned wide = __ballot_sync(FULL, sub == 0 && sz > CP_SMALL);
+    while (wide) {
+      const int l = __ffs(wide) - 1;
+      wide &= wide - 1;
+      const int32_t wd = __shfl_sync(FULL, dst, l), ws = __shfl_sync(FULL, src, l);
+      const int32_t wz = __shfl_sync(FULL, sz, l);
+      for (int32_t q0 = lane; q0 < wz; q0 += 128) {
+        int32_t v[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) v[x] = q0 + 32 * x < wz ? tpins[ws + q0 + 32 * x] : 0;
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+          if (q0 + 32 * x < wz) pins2[wd + q0 + 32 * x] = v[x];
+      }
     }
   }
 }
@@ -560,35 +830,65 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
   const int gm = grid_for(m, 256, cx.num_sms, 4);
   DBuf<int32_t> lists, counts, tpins, tsize;
   DBuf<unsigned long long> fp;
-  lists.alloc(&cx.alloc, (size_t)m * 3);
-  counts.alloc(&cx.alloc, 4);
+  lists.alloc(&cx.alloc, (size_t)m * NCLS);
+  counts.alloc(&cx.alloc, NCLS);
   tpins.alloc(&cx.alloc, (size_t)std::max<int64_t>(L.p, 1));
   tsize.alloc(&cx.alloc, (size_t)m);
   fp.alloc(&cx.alloc, (size_t)m);
   HG_CUDA(cudaMemsetAsync(counts.p, 0, counts.bytes(), cx.stream));
   k_classify_nets<<<gm, 256, 0, cx.stream>>>(L.eoff.p, m, lists.p, counts.p);
   check_launch("classify_nets");
-  int32_t hc[4];
+  int32_t hc[NCLS];
   read_back(cx, hc, counts.p, sizeof(hc));
   if (hc[0])
     k_remap_small<<<grid_for(hc[0], 128, cx.num_sms, 16), 128, 0, cx.stream>>>(
         lists.p, hc[0], L.eoff.p, L.pins.p, L.map.p, fingerprint_bits, tpins.p, tsize.p, fp.p);
-  if (hc[1])
-    k_remap_mid<<<grid_for(hc[1], 1, cx.num_sms, 8), MID_THREADS, 0, cx.stream>>>(
-        lists.p + m, hc[1], L.eoff.p, L.pins.p, L.map.p, fingerprint_bits, tpins.p, tsize.p, fp.p);
+  const int32_t words = (n2 + 31) / 32;
+  if (hc[1]) {
+    const int gw = grid_for(hc[1], WARP_NETS, cx.num_sms, 8);
+    if (n2 <= WARP_BITMAP_N)
+      k_remap_warp_bitmap<<<gw, WARP_NETS * 32, 0, cx.stream>>>(
+          lists.p + m, hc[1], L.eoff.p, L.pins.p, L.map.p, words, fingerprint_bits, tpins.p,
+          tsize.p, fp.p);
+    else
+      k_remap_warp_sort<<<gw, WARP_NETS * 32, 0, cx.stream>>>(lists.p + m, hc[1], L.eoff.p,
+                                                              L.pins.p, L.map.p, fingerprint_bits,
+                                                              tpins.p, tsize.p, fp.p);
+  }
   DBuf<unsigned> bitmaps;
-  if (hc[2]) {
-    const int32_t words = (n2 + 31) / 32;
-    const int blocks = (int)std::max<int64_t>(
-        1, std::min<int64_t>({(int64_t)hc[2], (int64_t)cx.num_sms * 2,
-                              (int64_t)((256ll << 20) / ((int64_t)words * 4 + 1))}));
-    bitmaps.alloc(&cx.alloc, (size_t)blocks * words);
-    k_remap_big<<<blocks, BIG_THREADS, 0, cx.stream>>>(lists.p + 2 * (size_t)m, hc[2], L.eoff.p,
-                                                       L.pins.p, L.map.p, words, bitmaps.p,
-                                                       fingerprint_bits, tpins.p, tsize.p, fp.p);
+  const int32_t* mid = lists.p + 2 * (size_t)m;
+  const int32_t* big = lists.p + 3 * (size_t)m;
+  if (n2 <= BLOCK_BITMAP_N) {
+    const size_t bytes = ((size_t)words + words / 32 + 1) * sizeof(unsigned);
+    const int per_sm = std::max(1, std::min(4, (int)(200 * 1024 / bytes)));
+    static std::once_flag once;
+    std::call_once(once, [] {
+      HG_CUDA(cudaFuncSetAttribute(k_remap_block_bitmap,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (BLOCK_BITMAP_N / 32 + BLOCK_BITMAP_N / 1024 + 1) * 4));
+    });
+    for (int c = 2; c < NCLS; ++c)
+      if (hc[c])
+        k_remap_block_bitmap<<<grid_for(hc[c], 1, cx.num_sms, per_sm), BIG_THREADS, bytes,
+                               cx.stream>>>(c == 2 ? mid : big, hc[c], L.eoff.p, L.pins.p,
+                                            L.map.p, words, fingerprint_bits, tpins.p, tsize.p,
+                                            fp.p);
+  } else {
+    if (hc[2])
+      k_remap_mid<<<grid_for(hc[2], 1, cx.num_sms, 8), MID_THREADS, 0, cx.stream>>>(
+          mid, hc[2], L.eoff.p, L.pins.p, L.map.p, fingerprint_bits, tpins.p, tsize.p, fp.p);
+    if (hc[3]) {
+      const int blocks = (int)std::max<int64_t>(
+          1, std::min<int64_t>({(int64_t)hc[3], (int64_t)cx.num_sms * 2,
+                                (int64_t)((256ll << 20) / ((int64_t)words * 4 + 1))}));
+      bitmaps.alloc(&cx.alloc, (size_t)blocks * words);
+      k_remap_big<<<blocks, BIG_THREADS, 0, cx.stream>>>(big, hc[3], L.eoff.p, L.pins.p, L.map.p,
+                                                         words, bitmaps.p, fingerprint_bits,
+                                                         tpins.p, tsize.p, fp.p);
+    }
   }
   check_launch("remap");
-  if (cx.launches) *cx.launches += 1 + (hc[0] > 0) + (hc[1] > 0) + (hc[2] > 0);
+  if (cx.launches) *cx.launches += 1 + (hc[0] > 0) + (hc[1] > 0) + (hc[2] > 0) + (hc[3] > 0);
   bitmaps.release();
 
   // a7: identical nets
@@ -608,7 +908,7 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
   k_candidates<<<gm, 256, 0, cx.stream>>>(tsize.p, m, cand.p, ncand.p);
   check_launch("candidates");
   const int g_ins = grid_for(m, 256, cx.num_sms, 8);
-  const int g_cmp = grid_for(m, 8, cx.num_sms, 16);
+  const int g_cmp = grid_for(m, 8 * (32 / CMP_LANES), cx.num_sms, 8);
   for (int round = 0;; ++round) {
     HG_CUDA(cudaMemsetAsync(tkey.p, 0xff, tkey.bytes(), cx.stream));
     HG_CUDA(cudaMemsetAsync(tmin.p, 0x7f, tmin.bytes(), cx.stream));
@@ -652,7 +952,7 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
   out.eoff.alloc(&cx.alloc, (size_t)out.m + 1);
   out.pins.alloc(&cx.alloc, (size_t)std::max<int64_t>(out.p, 1));
   out.w.alloc(&cx.alloc, (size_t)std::max<int32_t>(out.m, 1));
-  k_compact<<<grid_for(m, 8, cx.num_sms, 16), 256, 0, cx.stream>>>(
+  k_compact<<<grid_for(m, 8 * (32 / CP_LANES), cx.num_sms, 8), 256, 0, cx.stream>>>(
       kflag.p, newid.p, ksize.p, L.eoff.p, tpins.p, tsize.p, wsum.p, m, out.eoff.p, out.pins.p,
       out.w.p);
   check_launch("compact");
