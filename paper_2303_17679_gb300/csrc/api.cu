@@ -265,8 +265,8 @@ int hg_create(int32_t n, int32_t m, const int32_t* net_offsets, const int32_t* p
     h->W0 = W;
     {
       hgk::EventTimer tm(h->cx, &h->stats.ms_transpose);
+      L->graph = o.graph_path == 0 && hgk::level_is_graph(h->cx, *L);
       hgk::build_incidence(h->cx, *L);
-      if (o.graph_path == 0 && hgk::level_is_graph(h->cx, *L)) hgk::build_graph_adjacency(h->cx, *L);
     }
     hgk::check_status(h->cx);
     h->levels.push_back(std::move(L));

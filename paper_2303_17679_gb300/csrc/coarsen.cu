@@ -103,13 +103,17 @@ __device__ __forceinline__ int rate_class(int64_t W, int32_t records, int32_t n,
 // floor(w(e) * 2^20 / (|e| - 1)) for the rated nets (2 <= |e| <= T), else 0;
 // at least 1 for a rated net since |e| - 1 < 2^20.
 __global__ void k_net_terms(const int32_t* __restrict__ eoff, const int32_t* __restrict__ w,
-                            int32_t m, int T, unsigned long long* __restrict__ rterm) {
+                            int32_t m, int T, IncMeta* __restrict__ nmeta) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t sz = eoff[e + 1] - eoff[e];
-    rterm[e] = (sz >= 2 && sz <= T)
-                   ? (((unsigned long long)w[e]) << 20) / (unsigned long long)(sz - 1)
-                   : 0ull;
+    IncMeta x;
+    x.start = eoff[e];
+    x.eff = eoff[e + 1] - x.start;
+    x.r = (x.eff >= 2 && x.eff <= T)
+              ? (((unsigned long long)w[e]) << 20) / (unsigned long long)(x.eff - 1)
+              : 0ull;
+    if (x.r == 0) x.eff = 0;
+    nmeta[e] = x;
   }
 }
 
@@ -175,6 +179,11 @@ __device__ __forceinline__ bool level_grouped(const unsigned long long* heavy, i
   return comm || GROUP_HEAVY_DEN * *heavy >= GROUP_HEAVY_NUM * (unsigned long long)p;
 }
 
+// The lowest weight bucket goes to the net record's upper bits (terms stay
+// below 2^51): a node whose bound lies below it has no candidate in the net.
+constexpr int TERM_BITS = 56;
+constexpr unsigned long long TERM_MASK = (1ull << TERM_BITS) - 1;
+
 // Sorts the sz <= 32 R pins of one net by group key with the warp: a bitonic
 // network over {key, index in the net} words held R per lane (in-thread swaps
 // below R, lane shuffles above).  The order of equal keys does not matter.
@@ -183,8 +192,8 @@ __device__ __forceinline__ void group_sort(int32_t b, int32_t sz, const int32_t*
                                            const int32_t* __restrict__ c,
                                            const int32_t* __restrict__ comm,
                                            int32_t* __restrict__ gpins,
-                                           int32_t* __restrict__ qnew,
-                                           uint32_t* __restrict__ gkey) {
+                                           uint32_t* __restrict__ gkey,
+                                           IncMeta* __restrict__ nmeta) {
   const int lane = lane_id();
   uint32_t v[R];
 #pragma unroll
@@ -222,43 +231,42 @@ __device__ __forceinline__ void group_sort(int32_t b, int32_t sz, const int32_t*
       }
     }
   }
+  uint32_t low = GROUP_W_MASK;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int32_t i = lane * R + r;
     if (i < sz) {
+      low = min(low, (v[r] >> GROUP_IDX_BITS) & GROUP_W_MASK);
       const int32_t from = b + (int32_t)(v[r] & (GROUP_NET - 1));
       gpins[b + i] = pins[from];
       gkey[b + i] = v[r] >> GROUP_IDX_BITS;
-      qnew[from] = b + i;
     }
   }
+  low = __reduce_min_sync(FULL, low);
+  if (lane == 0) nmeta->r |= (unsigned long long)low << TERM_BITS;
 }
 
-// One warp per net: gpins = the grouped pin order, qnew[q] = new position of
-// pin position q, gkey = group key per new position.  Unrated nets and nets
-// of more than GROUP_NET pins keep their order.
+// One warp per net: gpins = the grouped pin order, gkey = group key per
+// position.  Unrated nets and nets of more than GROUP_NET pins keep their order.
 __global__ void __launch_bounds__(GROUP_WARPS * 32)
 k_group_nets(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins, int32_t m, int T,
              const int32_t* __restrict__ c, const int32_t* __restrict__ comm, int64_t p,
              const unsigned long long* __restrict__ heavy, int32_t* __restrict__ gpins,
-             int32_t* __restrict__ qnew, uint32_t* __restrict__ gkey) {
+             uint32_t* __restrict__ gkey, IncMeta* __restrict__ nmeta) {
   if (!level_grouped(heavy, p, comm != nullptr)) return;
   for (int64_t e = (int64_t)blockIdx.x * GROUP_WARPS + warp_in_block(); e < m;
        e += (int64_t)gridDim.x * GROUP_WARPS) {
     const int32_t b = eoff[e], sz = eoff[e + 1] - b;
     if (sz < 2 || sz > T || sz > GROUP_NET) {
-      for (int32_t q = b + lane_id(); q < b + sz; q += 32) {
-        gpins[q] = pins[q];
-        qnew[q] = q;
-      }
+      for (int32_t q = b + lane_id(); q < b + sz; q += 32) gpins[q] = pins[q];
     } else if (sz <= 32) {
-      group_sort<1>(b, sz, pins, c, comm, gpins, qnew, gkey);
+      group_sort<1>(b, sz, pins, c, comm, gpins, gkey, nmeta + e);
     } else if (sz <= 128) {
-      group_sort<4>(b, sz, pins, c, comm, gpins, qnew, gkey);
+      group_sort<4>(b, sz, pins, c, comm, gpins, gkey, nmeta + e);
     } else if (sz <= 512) {
-      group_sort<16>(b, sz, pins, c, comm, gpins, qnew, gkey);
+      group_sort<16>(b, sz, pins, c, comm, gpins, gkey, nmeta + e);
     } else {
-      group_sort<32>(b, sz, pins, c, comm, gpins, qnew, gkey);
+      group_sort<32>(b, sz, pins, c, comm, gpins, gkey, nmeta + e);
     }
   }
 }
@@ -274,42 +282,6 @@ __device__ __forceinline__ int32_t group_lower(const uint32_t* __restrict__ gkey
   return lo;
 }
 
-// IncMeta of every incidence of a hypergraph level; on grouped levels the
-// range of u's possible candidates in the net.
-__global__ void k_inc_meta(const int32_t* __restrict__ inets, const int32_t* __restrict__ ipin,
-                           const int32_t* __restrict__ eoff,
-                           const unsigned long long* __restrict__ rterm, int64_t p,
-                           const int32_t* __restrict__ c, int32_t c_max, bool comm,
-                           const unsigned long long* __restrict__ heavy,
-                           const int32_t* __restrict__ gpins, const int32_t* __restrict__ qnew,
-                           const uint32_t* __restrict__ gkey, IncMeta* __restrict__ imeta) {
-  const bool grouped = level_grouped(heavy, p, comm);
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t e = inets[j];
-    const unsigned long long r = rterm[e];
-    IncMeta x;
-    x.start = eoff[e];
-    x.eff = r != 0 ? eoff[e + 1] - x.start : 0;
-    x.r = r;
-    if (grouped) {
-      if (x.eff != 0 && x.eff <= GROUP_NET) {
-        const int32_t qn = qnew[ipin[j]];
-        const int32_t end = x.start + x.eff, left = c_max - c[gpins[qn]];
-        x.eff = 0;
-        if (left > 0) {
-          const uint32_t key = gkey[qn], base = key & ~GROUP_W_MASK, top = weight_bucket(left);
-          if (comm) x.start = group_lower(gkey, x.start, qn, base);
-          x.eff = group_lower(gkey, x.start, end, base + top + 1) - x.start;
-          // a range holding u alone has no candidate
-          if (x.eff == 1 && (key & GROUP_W_MASK) <= top) x.eff = 0;
-        }
-      }
-    }
-    imeta[j] = x;
-  }
-}
-
 // {u, ioff[u], rend[u], c(u)} of every listed node.
 __global__ void k_list_nodes(const int32_t* __restrict__ list, int32_t cnt,
                              const int32_t* __restrict__ ioff, const int32_t* __restrict__ rend,
@@ -320,60 +292,242 @@ __global__ void k_list_nodes(const int32_t* __restrict__ list, int32_t cnt,
   }
 }
 
-// One warp per node, lanes over its incident nets.  Hypergraph levels: over
-// their records, and the records that hold a visit are moved to the front of
-// the node's range (rend[u] = their end), so the walks never load the records
-// of unrated nets or of nets without a candidate (on large-net inputs most
-// incidences are of unrated nets; on grouped coarse levels a node of thousands
-// of nets may have a handful left).  Visits bound the records a walk loads.
-__global__ void k_node_work(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
-                            IncMeta* __restrict__ imeta,
-                            const unsigned long long* __restrict__ rterm, int32_t n, bool graph,
-                            int32_t* __restrict__ wof, int32_t* __restrict__ rend,
-                            unsigned long long* __restrict__ max_r) {
-  unsigned long long lr = 0, lw = 0;
+// The weight and records of every node.  A record is the net's {start, pins,
+// term} (one 16-byte gather), on grouped levels cut to the range of u's possible
+// candidates; the records that hold a visit are written to the front of the
+// node's range (rend[u] = their end), so the walks never load the records of
+// unrated nets or of nets without a candidate (on large-net inputs most
+// incidences are of unrated nets; on grouped coarse levels a node of thousands of
+// nets may have a handful left).  Visits bound the records a walk loads.
+//
+// Bound by the gathers of the net records and, on grouped levels, by the
+// dependent steps of the range searches: eight lanes take a node, a warp one of
+// more than WORK_SMALL nets, a block one of more than WORK_WIDE, and warps queue
+// the records that need a search until every lane has one (an incidence in ten or
+// fewer does on coarse levels).
+constexpr int WORK_LANES = 8;
+constexpr int32_t WORK_SMALL = 64, WORK_WIDE = 512;
+constexpr int WORK_WARPS = 8;
+
+struct NodeRange {     // of a node on a grouped level
+  uint32_t base, top;  // community part of its group key, highest weight bucket
+  uint32_t own;        // its own weight bucket
+  int32_t left;        // weight left beside it
+};
+
+struct WorkArgs {
+  const int32_t *ioff, *inets;
+  const IncMeta* nmeta;
+  int32_t n;
+  int64_t p;
+  bool graph;
+  const int32_t *c, *comm;
+  int32_t c_max;
+  const uint32_t* gkey;
+  IncMeta* imeta;
+  int32_t *wof, *rend;
+  unsigned long long* max_r;  // largest rating, incidences of heavy nodes, total W
+  int32_t *big, *nbig;        // nodes of more than WORK_WIDE nets
+};
+
+__device__ __forceinline__ NodeRange node_range(const WorkArgs& A, int64_t u) {
+  const int32_t cu = A.c[u];
+  NodeRange r;
+  r.left = A.c_max - cu;
+  r.top = r.left > 0 ? weight_bucket(r.left) : 0u;
+  r.own = weight_bucket(cu);
+  r.base = group_key(A.comm ? A.comm[u] : 0, cu) & ~GROUP_W_MASK;
+  return r;
+}
+
+// The record of net e, empty if the lowest bucket already says so.
+__device__ __forceinline__ IncMeta net_record(const WorkArgs& A, bool grouped, int32_t e,
+                                              const NodeRange& r) {
+  IncMeta x = A.nmeta[e];
+  if (grouped) {
+    const uint32_t low = (uint32_t)(x.r >> TERM_BITS);
+    x.r &= TERM_MASK;
+    if (x.eff <= GROUP_NET && (r.left <= 0 || low > r.top)) x.eff = 0;
+  }
+  return x;
+}
+
+// The range of the node's possible candidates (grouped levels).
+__device__ __forceinline__ void cut_record(const WorkArgs& A, IncMeta& x, const NodeRange& r) {
+  if (x.eff == 0 || x.eff > GROUP_NET) return;
+  const int32_t end = x.start + x.eff;
+  if (A.comm) x.start = group_lower(A.gkey, x.start, end, r.base);
+  x.eff = group_lower(A.gkey, x.start, end, r.base + r.top + 1) - x.start;
+  // a range holding u alone has no candidate
+  if (x.eff == 1 && r.own <= r.top) x.eff = 0;
+}
+
+// The records [beg, end) of one node by `warps` warps, this one number wv;
+// *to (shared) counts the records written.
+__device__ __forceinline__ void walk_node(const WorkArgs& A, bool grouped, int32_t beg,
+                                          int32_t end, const NodeRange& r, int wv, int warps,
+                                          IncMeta* queue, int32_t* to, long long& W,
+                                          unsigned long long& R) {
   const int lane = lane_id();
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += nw) {
-    long long W = 0;
-    unsigned long long R = 0;
-    const int32_t beg = ioff[u], end = ioff[u + 1];
-    int32_t out = beg;
-    if (graph) {
-      for (int32_t j = beg + lane; j < end; j += 32) {
-        const unsigned long long r = rterm[inets[j]];
-        W += r != 0;  // a graph visits the other endpoint only
-        R += r;
-      }
-      out = end;
-    } else {
-      for (int32_t j0 = beg; j0 < end; j0 += 32) {
-        const int32_t j = j0 + lane;
-        IncMeta x{0, 0, 0};
-        if (j < end) x = imeta[j];
-        const unsigned live = __ballot_sync(FULL, x.eff != 0);
-        if (x.eff != 0) {
-          W += x.eff;
-          R += x.r;
-          // never past the records this warp has read
-          const int32_t to = out + __popc(live & ((1u << lane) - 1u));
-          if (to != j) imeta[to] = x;
-        }
-        out += __popc(live);
-      }
+  const unsigned below = (1u << lane) - 1u;
+  int held = 0;
+  auto emit = [&](const IncMeta& x) {
+    const unsigned live = __ballot_sync(FULL, x.eff != 0);
+    if (!live) return;
+    int32_t at = 0;
+    if (lane == 0) at = atomicAdd(to, __popc(live));
+    at = beg + __shfl_sync(FULL, at, 0) + __popc(live & below);
+    if (x.eff != 0) {
+      W += A.graph ? 1 : x.eff;  // a graph visits the other endpoint only
+      R += x.r;
+      if (!A.graph) A.imeta[at] = x;
     }
-    W = warp_sum(W);
-    R = warp_sum(R);
-    lr = R > lr ? R : lr;
-    lw += (unsigned long long)W;
-    if (lane == 0) {
-      wof[u] = W > 0x7fffffff ? 0x7fffffff : (int32_t)W;
-      rend[u] = out;
+  };
+  auto drain = [&](int count) {
+    IncMeta x{0, 0, 0};
+    held -= count;
+    if (lane < count) x = queue[held + lane];
+    __syncwarp();
+    cut_record(A, x, r);
+    emit(x);
+  };
+  for (int32_t j0 = beg + wv * 64; j0 < end; j0 += warps * 64) {
+    const int32_t ja = j0 + lane, jb = ja + 32;
+    IncMeta x[2] = {{0, 0, 0}, {0, 0, 0}};
+    const int32_t ea = ja < end ? A.inets[ja] : -1, eb = jb < end ? A.inets[jb] : -1;
+    if (ea >= 0) x[0] = net_record(A, grouped, ea, r);
+    if (eb >= 0) x[1] = net_record(A, grouped, eb, r);
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      if (!grouped) {
+        emit(x[y]);
+        continue;
+      }
+      const unsigned live = __ballot_sync(FULL, x[y].eff != 0);
+      if (x[y].eff != 0) queue[held + __popc(live & below)] = x[y];
+      __syncwarp();
+      held += __popc(live);
+      if (held >= 32) drain(32);
     }
   }
-  if (lane == 0 && lr) atomicMax(max_r, lr);
-  const unsigned long long wv[1] = {lane == 0 ? lw : 0ull};
-  block_add_counters(max_r + 2, wv);
+  if (held > 0) drain(held);
+}
+
+__global__ void __launch_bounds__(WORK_WARPS * 32) k_node_work(WorkArgs A) {
+  constexpr int PER = 32 / WORK_LANES;
+  __shared__ IncMeta s_queue[WORK_WARPS][64];
+  __shared__ int32_t s_to[WORK_WARPS];
+  unsigned long long lr = 0, lw = 0;
+  const bool grouped = !A.graph && level_grouped(A.max_r + 1, A.p, A.comm != nullptr);
+  const int lane = lane_id(), sub = lane % WORK_LANES, first = lane - sub;
+  const int wv = warp_in_block();
+  const int64_t stride = (((int64_t)gridDim.x * blockDim.x) >> 5) * PER;
+  for (int64_t u0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * PER; u0 < A.n;
+       u0 += stride) {
+    const int64_t u = u0 + lane / WORK_LANES;
+    const bool on = u < A.n;
+    const int32_t beg = on ? A.ioff[u] : 0, end = on ? A.ioff[u + 1] : 0;
+    NodeRange r{0u, 0u, 0u, 0};
+    if (grouped && on) r = node_range(A, u);
+    long long W = 0;
+    unsigned long long R = 0;
+    int32_t out = beg;
+    const bool wide = end - beg > WORK_SMALL, big = end - beg > WORK_WIDE;
+    const int32_t stop = wide ? beg : end;
+    for (int32_t j0 = beg; __any_sync(FULL, j0 < stop); j0 += WORK_LANES) {
+      const int32_t j = j0 + sub;
+      IncMeta x{0, 0, 0};
+      if (j < stop) {
+        x = net_record(A, grouped, A.inets[j], r);
+        if (grouped) cut_record(A, x, r);
+      }
+      const unsigned live =
+          (__ballot_sync(FULL, x.eff != 0) >> first) & ((1u << WORK_LANES) - 1u);
+      if (x.eff != 0) {
+        W += A.graph ? 1 : x.eff;
+        R += x.r;
+        if (!A.graph) A.imeta[out + __popc(live & ((1u << sub) - 1u))] = x;
+      }
+      out += __popc(live);
+    }
+    for (unsigned rest = __ballot_sync(FULL, sub == 0 && wide && !big); rest; rest &= rest - 1) {
+      const int l = __ffs(rest) - 1;
+      const int32_t wb = __shfl_sync(FULL, beg, l), we = __shfl_sync(FULL, end, l);
+      NodeRange wr;
+      wr.base = __shfl_sync(FULL, r.base, l);
+      wr.top = __shfl_sync(FULL, r.top, l);
+      wr.own = __shfl_sync(FULL, r.own, l);
+      wr.left = __shfl_sync(FULL, r.left, l);
+      long long WW = 0;
+      unsigned long long RR = 0;
+      if (lane == 0) s_to[wv] = 0;
+      __syncwarp();
+      walk_node(A, grouped, wb, we, wr, 0, 1, s_queue[wv], &s_to[wv], WW, RR);
+      __syncwarp();
+      if (first == l) out = wb + s_to[wv];
+      __syncwarp();
+      // one lane of the node's group takes the warp's sums
+      WW = warp_sum(WW);
+      RR = warp_sum(RR);
+      if (lane == l) {
+        W += WW;
+        R += RR;
+      }
+    }
+#pragma unroll
+    for (int d = WORK_LANES / 2; d > 0; d >>= 1) {
+      W += __shfl_xor_sync(FULL, W, d);
+      R += __shfl_xor_sync(FULL, R, d);
+    }
+    if (sub == 0 && on) {
+      if (big) {
+        A.big[atomicAdd(A.nbig, 1)] = (int32_t)u;
+      } else {
+        lr = R > lr ? R : lr;
+        lw += (unsigned long long)W;
+        A.wof[u] = W > 0x7fffffff ? 0x7fffffff : (int32_t)W;
+        A.rend[u] = A.graph ? end : out;
+      }
+    }
+  }
+  lr = warp_max(lr);
+  if (lane == 0 && lr) atomicMax(A.max_r, lr);
+  const unsigned long long wsum[1] = {lw};
+  block_add_counters(A.max_r + 2, wsum);
+}
+
+__global__ void __launch_bounds__(WORK_WARPS * 32) k_node_work_big(WorkArgs A) {
+  __shared__ IncMeta s_queue[WORK_WARPS][64];
+  __shared__ int32_t s_to;
+  __shared__ unsigned long long s_red[32];
+  const bool grouped = !A.graph && level_grouped(A.max_r + 1, A.p, A.comm != nullptr);
+  const int32_t count = *A.nbig;
+  unsigned long long lr = 0, lw = 0;
+  for (int32_t i = blockIdx.x; i < count; i += gridDim.x) {
+    const int32_t u = A.big[i];
+    const int32_t beg = A.ioff[u], end = A.ioff[u + 1];
+    NodeRange r{0u, 0u, 0u, 0};
+    if (grouped) r = node_range(A, u);
+    if (threadIdx.x == 0) s_to = 0;
+    __syncthreads();
+    long long W = 0;
+    unsigned long long R = 0;
+    walk_node(A, grouped, beg, end, r, warp_in_block(), WORK_WARPS, s_queue[warp_in_block()],
+              &s_to, W, R);
+    const unsigned long long WS = block_sum((unsigned long long)W, s_red);
+    __syncthreads();
+    R = block_sum(R, s_red);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      lr = R > lr ? R : lr;
+      lw += WS;
+      A.wof[u] = WS > 0x7fffffffull ? 0x7fffffff : (int32_t)WS;
+      A.rend[u] = A.graph ? end : beg + s_to;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0 && lr) atomicMax(A.max_r, lr);
+  if (threadIdx.x == 0 && lw) atomicAdd(A.max_r + 2, lw);
 }
 
 // key = class * S + sub-round of every node with W(u) > 0, and the counts.
@@ -592,39 +746,45 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   k_init_cluster<<<g_nodes, 256, 0, cx.stream>>>(L.c.p, n, P.seed, P.level, S, L.rep.p, cst.p,
                                                  slot_of.p);
   check_launch("init_cluster");
-  DBuf<unsigned long long> rterm;
-  rterm.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1));
+  DBuf<IncMeta> nmeta;
+  nmeta.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1));
   if (L.m > 0) {
     k_net_terms<<<grid_for(L.m, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(L.eoff.p, L.w.p, L.m,
-                                                                          P.T, rterm.p);
+                                                                          P.T, nmeta.p);
     check_launch("net_terms");
   }
   // hypergraph levels: the grouped pin order (where it pays, decided on the
-  // device) and the net record of every incidence
+  // device) and the net records of every node
   DBuf<IncMeta> imeta;
   DBuf<int32_t> gpins, rend;
+  DBuf<uint32_t> gkey;
   rend.alloc(&cx.alloc, ncap);
   if (records) {
-    DBuf<int32_t> qnew;
-    DBuf<uint32_t> gkey;
     gpins.alloc(&cx.alloc, (size_t)L.p);
-    qnew.alloc(&cx.alloc, (size_t)L.p);
     gkey.alloc(&cx.alloc, (size_t)L.p);
     imeta.alloc(&cx.alloc, (size_t)L.p);
     k_heavy_pins<<<g_nodes, 256, 0, cx.stream>>>(L.c.p, L.ioff.p, n, P.c_max, max_r.p + 1);
     check_launch("heavy_pins");
     k_group_nets<<<grid_for(L.m, GROUP_WARPS, cx.num_sms, 16), GROUP_WARPS * 32, 0, cx.stream>>>(
-        L.eoff.p, L.pins.p, L.m, P.T, L.c.p, L.comm.p, L.p, max_r.p + 1, gpins.p, qnew.p, gkey.p);
+        L.eoff.p, L.pins.p, L.m, P.T, L.c.p, L.comm.p, L.p, max_r.p + 1, gpins.p, gkey.p,
+        nmeta.p);
     check_launch("group_nets");
-    k_inc_meta<<<grid_for(L.p, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
-        L.inets.p, L.ipin.p, L.eoff.p, rterm.p, L.p, L.c.p, P.c_max, L.comm.p != nullptr,
-        max_r.p + 1, gpins.p, qnew.p, gkey.p, imeta.p);
-    check_launch("inc_meta");
-    if (cx.launches) *cx.launches += 3;
+    if (cx.launches) *cx.launches += 2;
   }
-  k_node_work<<<grid_for(n, 8, cx.num_sms, 16), 256, 0, cx.stream>>>(
-      L.ioff.p, L.inets.p, imeta.p, rterm.p, n, L.graph, wof.p, rend.p, max_r.p);
+  DBuf<int32_t> big;  // nodes of more than WORK_WIDE nets, then their number
+  const size_t nb = (size_t)(L.p / (WORK_WIDE + 1)) + 1;
+  big.alloc(&cx.alloc, nb + 1);
+  HG_CUDA(cudaMemsetAsync(big.p + nb, 0, sizeof(int32_t), cx.stream));
+  const WorkArgs wa{L.ioff.p, L.inets.p, nmeta.p, n,      L.p,    L.graph, L.c.p, L.comm.p,
+                    P.c_max,  gkey.p,    imeta.p, wof.p,  rend.p, max_r.p, big.p, big.p + nb};
+  k_node_work<<<grid_for(n, WORK_WARPS * (32 / WORK_LANES), cx.num_sms, 8), WORK_WARPS * 32, 0,
+                cx.stream>>>(wa);
   check_launch("node_work");
+  if (L.p > WORK_WIDE) {
+    k_node_work_big<<<grid_for((int64_t)nb, 1, cx.num_sms, 8), WORK_WARPS * 32, 0, cx.stream>>>(wa);
+    check_launch("node_work_big");
+    if (cx.launches) *cx.launches += 1;
+  }
   unsigned long long hmax[3];
   read_back(cx, hmax, max_r.p, sizeof(hmax));
   const unsigned long long hmax_r = hmax[0];
@@ -633,6 +793,8 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
       records && (L.comm.p || GROUP_HEAVY_DEN * hmax[1] >= GROUP_HEAVY_NUM * (unsigned long long)L.p);
   const int32_t* rpins = grouped ? gpins.p : L.pins.p;
   if (!grouped) gpins.release();
+  gkey.release();
+  nmeta.release();
   if (records) {
     tiles.alloc(&cx.alloc, (size_t)num_pin_tiles(L.p) + 1);
     build_tile_index(cx, L.eoff.p, L.m, L.p, tiles.p);

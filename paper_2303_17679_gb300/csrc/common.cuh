@@ -277,7 +277,6 @@ struct Level {
   DBuf<int32_t> c;      // n    node weights
   DBuf<int32_t> ioff;   // n+1  node -> first incident net
   DBuf<int32_t> inets;  // p    incident nets (order unspecified)
-  DBuf<int32_t> ipin;   // p    for every incidence, the index of its pin in `pins`
   DBuf<int32_t> map;    // n    node -> node of the next level (after coarsening)
   DBuf<int32_t> rep;    // n    representative in the clustering that made the next level
   bool coarsened = false;
@@ -322,11 +321,10 @@ void iota_i32(const Ctx& cx, int32_t* p, int64_t n);
 // ---------------------------------------------------- structure (structure.cu)
 
 // Builds ioff/inets of a level from eoff/pins (a1).
+// I(v) of every node; with L.graph set also the adjacency array.
 void build_incidence(const Ctx& cx, Level& L);
 // True when the level has nets and every net has exactly two pins.
 bool level_is_graph(const Ctx& cx, const Level& L);
-// Sets L.graph and builds L.adj (after build_incidence).
-void build_graph_adjacency(const Ctx& cx, Level& L);
 // The pins alone (in range, no node twice in a net) of a level whose offsets
 // are valid: mid-sized host inputs, whose offsets and weights the host checks.
 bool validate_pins_device(const Ctx& cx, const Level& L);

@@ -41,6 +41,7 @@
 #include <mutex>
 
 #include "gridsync.cuh"
+#include "pintile.cuh"
 
 namespace hgk {
 
@@ -73,21 +74,38 @@ __device__ __forceinline__ int subround_louvain(uint64_t seed, int level, int ro
 
 // Bipartite CSR from the hypergraph: node v's edges are its incidences
 // (positions ioff[v]..), net e's edges its pins (positions p + eoff[e]..).
-// One thread per incidence j = (v, e), q = ipin[j] the pin position.
-__global__ void k_lv_bipartite(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
-                               const int32_t* __restrict__ w, const int32_t* __restrict__ inets,
-                               const int32_t* __restrict__ ipin, int32_t n, int64_t p,
-                               int32_t* __restrict__ adj, long long* __restrict__ aw) {
+__device__ __forceinline__ long long lv_net_weight(const int32_t* __restrict__ eoff,
+                                                   const int32_t* __restrict__ w, int32_t e) {
+  const int32_t size = eoff[e + 1] - eoff[e];
+  return (long long)(((unsigned long long)w[e] << 20) / (unsigned long long)size);
+}
+
+// One thread per incidence j = (v, e).
+__global__ void k_lv_node_edges(const int32_t* __restrict__ eoff, const int32_t* __restrict__ w,
+                                const int32_t* __restrict__ inets, int32_t n, int64_t p,
+                                int32_t* __restrict__ adj, long long* __restrict__ aw) {
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p;
        j += (int64_t)gridDim.x * blockDim.x) {
     const int32_t e = inets[j];
-    const int32_t q = ipin[j];
-    const int32_t size = eoff[e + 1] - eoff[e];
-    const long long we = (long long)(((unsigned long long)w[e] << 20) / (unsigned long long)size);
     adj[j] = n + e;
-    aw[j] = we;
-    adj[p + q] = pins[q];
-    aw[p + q] = we;
+    aw[j] = lv_net_weight(eoff, w, e);
+  }
+}
+
+// One thread per pin; adj and aw start at the nets' edges.
+__global__ void __launch_bounds__(PIN_TILE_THREADS)
+k_lv_net_edges(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+               const int32_t* __restrict__ w, const int32_t* __restrict__ tile_net, int32_t m,
+               int64_t p, int32_t* __restrict__ adj, long long* __restrict__ aw) {
+  __shared__ int32_t s_off[PIN_TILE + 3];
+  const int64_t ntiles = num_pin_tiles(p);
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const PinTileView v = stage_pin_tile(eoff, tile_net, m, p, t, s_off);
+    for (int64_t q = v.q0 + threadIdx.x; q < v.q1; q += blockDim.x) {
+      adj[q] = pins[q];
+      aw[q] = lv_net_weight(eoff, w, v.e_lo + net_in_tile(s_off, v.count, q));
+    }
+    __syncthreads();
   }
 }
 
@@ -853,9 +871,18 @@ int32_t detect_communities(const Ctx& cx, const Level& L, int S, uint64_t seed,
   k_lv_offsets<<<grid_for(g.V + 1, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
       L.ioff.p, L.eoff.p, n, m, p, g.off.p);
   check_launch("lv_offsets");
-  k_lv_bipartite<<<grid_for(p, 256, cx.num_sms, 16), 256, 0, cx.stream>>>(
-      L.eoff.p, L.pins.p, L.w.p, L.inets.p, L.ipin.p, n, p, g.adj.p, g.aw.p);
-  check_launch("lv_bipartite");
+  {
+    DBuf<int32_t> tiles;
+    tiles.alloc(&cx.alloc, (size_t)num_pin_tiles(p) + 1);
+    build_tile_index(cx, L.eoff.p, L.m, p, tiles.p);
+    k_lv_node_edges<<<grid_for(p, 256, cx.num_sms, 16), 256, 0, cx.stream>>>(
+        L.eoff.p, L.w.p, L.inets.p, n, p, g.adj.p, g.aw.p);
+    check_launch("lv_node_edges");
+    k_lv_net_edges<<<grid_for(num_pin_tiles(p), 1, cx.num_sms, 8), PIN_TILE_THREADS, 0,
+                     cx.stream>>>(L.eoff.p, L.pins.p, L.w.p, tiles.p, L.m, p, g.adj.p + p,
+                                  g.aw.p + p);
+    check_launch("lv_net_edges");
+  }
   long long W2 = 0;
   lv_degrees(cx, g, &W2);
   for (int level = 0; level < LV_LEVELS; ++level) {

@@ -819,8 +819,8 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
   // nets are dropped)
   if (L.graph) {
     contract_edges(cx, L, out);
+    out.graph = out.m > 0;
     build_incidence(cx, out);
-    if (out.m > 0) build_graph_adjacency(cx, out);
     coarse_communities(cx, L, out);
     L.coarsened = true;
     return;

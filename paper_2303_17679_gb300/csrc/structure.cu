@@ -28,25 +28,37 @@ __global__ void k_degrees(const int32_t* __restrict__ pins, int64_t p, int32_t* 
     atomicAdd(&deg[pins[q]], 1);
 }
 
-// Scatter every pin (e, v) into I(v) at a slot taken from v's cursor; the
-// slot also records the pin's index q in `pins`.
+// Scatter every pin (e, v) into I(v) at a slot taken from v's cursor.
 __global__ void __launch_bounds__(PIN_TILE_THREADS)
 k_scatter_incidence(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
                     const int32_t* __restrict__ tile_net, int32_t m, int64_t p,
-                    int32_t* __restrict__ cursor, int32_t* __restrict__ inets,
-                    int32_t* __restrict__ ipin) {
+                    int32_t* __restrict__ cursor, int32_t* __restrict__ inets) {
   __shared__ int32_t s_off[PIN_TILE + 3];
   const int64_t ntiles = num_pin_tiles(p);
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     PinTileView v = stage_pin_tile(eoff, tile_net, m, p, t, s_off);
     for (int64_t q = v.q0 + threadIdx.x; q < v.q1; q += blockDim.x) {
       const int32_t e = v.e_lo + net_in_tile(s_off, v.count, q);
-      const int32_t u = pins[q];
-      const int32_t slot = atomicAdd(&cursor[u], 1);
-      inets[slot] = e;
-      ipin[slot] = (int32_t)q;
+      inets[atomicAdd(&cursor[pins[q]], 1)] = e;
     }
     __syncthreads();
+  }
+}
+
+// The same for a graph level (net e's pins at 2 e), with the adjacency array:
+// adj[j] = {the other endpoint, w(e)} of incidence j = (u, e).
+__global__ void k_scatter_edges(const int2* __restrict__ pins, const int32_t* __restrict__ w,
+                                int32_t m, int32_t* __restrict__ cursor,
+                                int32_t* __restrict__ inets, int2* __restrict__ adj) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int2 v = pins[e];
+    const int32_t we = w[e];
+    const int32_t a = atomicAdd(&cursor[v.x], 1), b = atomicAdd(&cursor[v.y], 1);
+    inets[a] = (int32_t)e;
+    adj[a] = make_int2(v.y, we);
+    inets[b] = (int32_t)e;
+    adj[b] = make_int2(v.x, we);
   }
 }
 
@@ -237,20 +249,6 @@ __global__ void k_net_size_range(const int32_t* __restrict__ eoff, int32_t m,
   }
 }
 
-// adj[j] = {the other pin of net inets[j], w(inets[j])} for every incidence
-// of a graph level (ipin[j] is the incidence's own pin position).
-__global__ void k_adjacency(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
-                            const int32_t* __restrict__ w, const int32_t* __restrict__ inets,
-                            const int32_t* __restrict__ ipin, int64_t p, int2* __restrict__ adj) {
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < p;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t e = inets[j];
-    const int32_t b = eoff[e];
-    const int32_t other = ipin[j] == b ? b + 1 : b;
-    adj[j] = make_int2(pins[other], w[e]);
-  }
-}
-
 }  // namespace
 
 bool level_is_graph(const Ctx& cx, const Level& L) {
@@ -268,17 +266,6 @@ bool level_is_graph(const Ctx& cx, const Level& L) {
   return h[0] == 2 && h[1] == 2;
 }
 
-void build_graph_adjacency(const Ctx& cx, Level& L) {
-  L.graph = true;
-  L.adj.alloc(&cx.alloc, (size_t)(L.p > 0 ? L.p : 1));
-  if (L.p > 0) {
-    k_adjacency<<<grid_for(L.p, 256, cx.num_sms, 16), 256, 0, cx.stream>>>(
-        L.eoff.p, L.pins.p, L.w.p, L.inets.p, L.ipin.p, L.p, L.adj.p);
-    check_launch("adjacency");
-    if (cx.launches) *cx.launches += 1;
-  }
-}
-
 void build_tile_index(const Ctx& cx, const int32_t* eoff, int32_t m, int64_t p, int32_t* tile_net) {
   const int64_t ntiles = num_pin_tiles(p);
   k_tile_index<<<grid_for(m > 0 ? m : 1, 256, cx.num_sms, 16), 256, 0, cx.stream>>>(eoff, m, ntiles,
@@ -290,7 +277,7 @@ void build_tile_index(const Ctx& cx, const int32_t* eoff, int32_t m, int64_t p, 
 void build_incidence(const Ctx& cx, Level& L) {
   L.ioff.alloc(&cx.alloc, (size_t)L.n + 1);
   L.inets.alloc(&cx.alloc, (size_t)(L.p > 0 ? L.p : 1));
-  L.ipin.alloc(&cx.alloc, (size_t)(L.p > 0 ? L.p : 1));
+  if (L.graph) L.adj.alloc(&cx.alloc, (size_t)(L.p > 0 ? L.p : 1));
   HG_CUDA(cudaMemsetAsync(L.ioff.p, 0, sizeof(int32_t) * ((size_t)L.n + 1), cx.stream));
   if (L.p > 0) {
     k_degrees<<<grid_for(L.p, 256, cx.num_sms, 16), 256, 0, cx.stream>>>(L.pins.p, L.p, L.ioff.p);
@@ -302,11 +289,16 @@ void build_incidence(const Ctx& cx, Level& L) {
     cursor.alloc(&cx.alloc, (size_t)L.n);
     HG_CUDA(cudaMemcpyAsync(cursor.p, L.ioff.p, sizeof(int32_t) * (size_t)L.n,
                             cudaMemcpyDeviceToDevice, cx.stream));
-    tiles.alloc(&cx.alloc, (size_t)num_pin_tiles(L.p) + 1);
-    build_tile_index(cx, L.eoff.p, L.m, L.p, tiles.p);
-    k_scatter_incidence<<<grid_for(num_pin_tiles(L.p), 1, cx.num_sms, 8), PIN_TILE_THREADS, 0,
-                          cx.stream>>>(L.eoff.p, L.pins.p, tiles.p, L.m, L.p, cursor.p,
-                                       L.inets.p, L.ipin.p);
+    if (L.graph) {
+      k_scatter_edges<<<grid_for(L.m, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
+          reinterpret_cast<const int2*>(L.pins.p), L.w.p, L.m, cursor.p, L.inets.p, L.adj.p);
+    } else {
+      tiles.alloc(&cx.alloc, (size_t)num_pin_tiles(L.p) + 1);
+      build_tile_index(cx, L.eoff.p, L.m, L.p, tiles.p);
+      k_scatter_incidence<<<grid_for(num_pin_tiles(L.p), 1, cx.num_sms, 8), PIN_TILE_THREADS, 0,
+                            cx.stream>>>(L.eoff.p, L.pins.p, tiles.p, L.m, L.p, cursor.p,
+                                         L.inets.p);
+    }
     check_launch("scatter_incidence");
     if (cx.launches) *cx.launches += 2;
   }
