@@ -25,6 +25,23 @@ __device__ __forceinline__ NetRec load_rec(const int4* rec, int64_t i) {
   return NetRec{r.x, (unsigned)r.y, (unsigned)r.z};
 }
 
+// Both halves of a record (k > 32).
+struct WideRec {
+  int32_t w;
+  unsigned long long ones, lam;
+};
+
+// One 32-byte load: a gather is bound by its requests, a line each.
+__device__ __forceinline__ WideRec load_wide(const int4* rec, int32_t e) {
+  unsigned w, o0, l0, x0, x1, o1, l1, x2;
+  asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(w), "=r"(o0), "=r"(l0), "=r"(x0), "=r"(x1), "=r"(o1), "=r"(l1), "=r"(x2)
+               : "l"(rec + 2 * (int64_t)e)
+               : "memory");
+  return WideRec{(int32_t)w, (unsigned long long)o0 | (unsigned long long)o1 << 32,
+                 (unsigned long long)l0 | (unsigned long long)l1 << 32};
+}
+
 // Sum over the W lanes of the caller's group (W a power of two); the whole warp
 // calls it.
 template <int W, typename T>
@@ -95,6 +112,9 @@ struct Gain {
   __device__ __forceinline__ void add(const NetRec& r, int from) {
     // u is not the only pin of its block in e
     if ((H == 1 || (unsigned)from < 32u) && !((r.ones >> from) & 1u)) bw -= r.w;
+    add_targets(r);
+  }
+  __device__ __forceinline__ void add_targets(const NetRec& r) {
 #pragma unroll
     for (int t = 0; t < K; ++t)
       if (r.lam & (1u << t)) acc[t] += r.w;

@@ -19,7 +19,7 @@
 // the whole chip (cooperative launch), and no host interaction at all.
 // Measured (GB300, whole call, before -> after): n = 10,000, k = 2 1.47 ->
 // 0.76 ms; n = 500,009 Zipf, k = 16 2.83 -> 1.96 ms; all levels of the 1e6 Zipf
-// V-cycle, k = 8 24.4 -> 19.1 ms; of the 4e6 large-net V-cycle, k = 64 87 -> 66 ms.
+// V-cycle, k = 8 24.4 -> 19.1 ms; of the 4e6 large-net V-cycle, k = 64 87 -> 44 ms.
 //
 // State that changes during the kernel (Pi, Phi, records, lists, counters) is
 // read with ld.cg or atomics, never through L1; the structure (ioff, inets,
@@ -287,17 +287,60 @@ __device__ __forceinline__ void gain_groups(const LpArgs& A, int par, const int4
   __syncwarp();
 }
 
+// The sums of a class-1 item: the node's best move, or, for one of several items,
+// into the node's accumulators; the item that finishes last takes the maximum
+// and clears them for the next pass.
+template <bool GRAPH, int K, int H>
+__device__ __forceinline__ void finish_item(const LpArgs& A, int par, const int4 it, int from,
+                                            Gain<GRAPH, K, H>& g) {
+  using L = TeamLane<32, H>;
+  const int lane = lane_id();
+  const L tl(lane);
+  const int32_t u = it.x, beg = it.y, end = it.z, slot = it.w;
+  int32_t bw = group_sum<32>(g.bw);
+  const int b0 = 32 * tl.half + reduce_scatter<L::SHARE, K>(tl.i, g.acc);
+  constexpr int OWN = K / L::SHARE > 0 ? K / L::SHARE : 1;
+  unsigned long long best = 0;
+  if (slot < 0) {
+#pragma unroll
+    for (int i = 0; i < OWN; ++i) consider(best, bw + g.acc[i], b0 + i, from, A.k);
+  } else {
+    int32_t* macc = A.macc + (int64_t)slot * MACC_STRIDE;
+    constexpr int SAME = L::SHARE / K > 1 ? L::SHARE / K : 1;  // lanes holding the same block
+    if (tl.i % SAME == 0) {
+#pragma unroll
+      for (int i = 0; i < OWN; ++i)
+        if (g.acc[i]) atomicAdd(&macc[b0 + i], g.acc[i]);
+    }
+    if (lane == 0 && bw) atomicAdd(&macc[HG_MAX_K], bw);
+    __threadfence();
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) {
+      const int32_t deg = __ldg(A.ioff + u + 1) - __ldg(A.ioff + u);
+      last = atomicAdd(&A.mtick[slot], end - beg) + (end - beg) == deg;
+    }
+    if (!__shfl_sync(FULL, last, 0)) return;
+    __threadfence();
+    bw = __ldcg(macc + HG_MAX_K);
+    for (int t = lane; t < A.k; t += 32) consider(best, bw + __ldcg(macc + t), t, from, A.k);
+    __syncwarp();
+    for (int t = lane; t < MACC_STRIDE; t += 32) macc[t] = 0;
+    if (lane == 0) A.mtick[slot] = 0;
+  }
+  best = group_max<32>(best);
+  if (lane == 0) emit_move(A, par, u, from, best);
+}
+
 // A class-1 item by a warp: four consecutive incidences per lane and step (one
-// 16-byte load of their net ids).  The items of a node split over several add
-// their sums to the node's accumulators; the one that finishes last takes the
-// maximum and clears them for the next pass.
+// 16-byte load of their net ids).
 template <bool GRAPH, int K, int H>
 __device__ __forceinline__ void gain_item(const LpArgs& A, int par, const int4 it) {
   using L = TeamLane<32, H>;
   const int lane = lane_id();
   const L tl(lane);
-  const int32_t u = it.x, beg = it.y, end = it.z, slot = it.w;
-  const int from = __ldcg(A.part + u), from_h = from - 32 * tl.half;
+  const int32_t beg = it.y, end = it.z;
+  const int from = __ldcg(A.part + it.x), from_h = from - 32 * tl.half;
   Gain<GRAPH, K, H> g;
   g.init();
   if (GRAPH) {
@@ -336,39 +379,133 @@ __device__ __forceinline__ void gain_item(const LpArgs& A, int par, const int4 i
       for (int x = 0; x < 4; ++x) g.add(r[x], from_h);
     }
   }
-  int32_t bw = group_sum<32>(g.bw);
-  const int b0 = 32 * tl.half + reduce_scatter<L::SHARE, K>(tl.i, g.acc);
-  constexpr int OWN = K / L::SHARE > 0 ? K / L::SHARE : 1;
-  unsigned long long best = 0;
-  if (slot < 0) {
-#pragma unroll
-    for (int i = 0; i < OWN; ++i) consider(best, bw + g.acc[i], b0 + i, from, A.k);
-  } else {
-    int32_t* macc = A.macc + (int64_t)slot * MACC_STRIDE;
-    constexpr int SAME = L::SHARE / K > 1 ? L::SHARE / K : 1;  // lanes holding the same block
-    if (tl.i % SAME == 0) {
-#pragma unroll
-      for (int i = 0; i < OWN; ++i)
-        if (g.acc[i]) atomicAdd(&macc[b0 + i], g.acc[i]);
+  finish_item<GRAPH, K, H>(A, par, it, from, g);
+}
+
+// The same for k > 32 (records in two halves).  Most incidences of the nodes of
+// this class are of nets that have pins in every block: those count the same for
+// every target, so they go into bw, nets inside the node's own block into no
+// target at all, and only the others (one in eight on the coarse levels of a
+// large-net input) are queued and added block by block, 16 at a time, each by a
+// lane of either half.  The gathers of the records bound it, at one request
+// each: one lane reads both halves with one load.  Measured (GB300, sub-round of
+// 16,400 nodes and 1.96M incidences, k = 64): best moves 40 -> 19 us (36 us with
+// a load per half).
+__device__ __forceinline__ void gain_item_wide(const LpArgs& A, int par, const int4 it,
+                                               int4* queue) {
+  const int lane = lane_id();
+  const TeamLane<32, 2> tl(lane);
+  const unsigned below = (1u << lane) - 1u;
+  const int32_t beg = it.y, end = it.z;
+  const int from = __ldcg(A.part + it.x);
+  const unsigned long long own = 1ull << from, full = ~0ull >> (64 - A.k);
+  Gain<false, 32, 2> g;
+  g.init();
+  int held = 0;
+  auto drain = [&](int count) {
+    held -= count;
+    NetRec r{0, 0, 0};
+    if (tl.i < count) {
+      const int4 q = queue[held + tl.i];
+      r.w = q.x;
+      r.lam = (unsigned)(tl.half ? q.z : q.y);
     }
-    if (lane == 0 && bw) atomicAdd(&macc[HG_MAX_K], bw);
-    __threadfence();
+    g.add_targets(r);
     __syncwarp();
-    int last = 0;
-    if (lane == 0) {
-      const int32_t deg = __ldg(A.ioff + u + 1) - __ldg(A.ioff + u);
-      last = atomicAdd(&A.mtick[slot], end - beg) + (end - beg) == deg;
+  };
+  // two records in flight per lane, the net ids of the next two loaded ahead
+  int32_t e[2];
+  auto nets = [&](int32_t c0) {
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const int32_t j = c0 + 32 * x + lane;
+      e[x] = j < end ? __ldg(A.inets + j) : -1;
     }
-    if (!__shfl_sync(FULL, last, 0)) return;
-    __threadfence();
-    bw = __ldcg(macc + HG_MAX_K);
-    for (int t = lane; t < A.k; t += 32) consider(best, bw + __ldcg(macc + t), t, from, A.k);
-    __syncwarp();
-    for (int t = lane; t < MACC_STRIDE; t += 32) macc[t] = 0;
-    if (lane == 0) A.mtick[slot] = 0;
+  };
+  nets(beg);
+  for (int32_t c0 = beg; c0 < end; c0 += 64) {
+    WideRec r[2];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      r[x] = WideRec{0, 0, 0};
+      if (e[x] >= 0) r[x] = load_wide(A.rec, e[x]);
+    }
+    nets(c0 + 64);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const bool all = r[x].lam == full;
+      if (all) g.bw += r[x].w;
+      if (!(r[x].ones & own)) g.bw -= r[x].w;
+      const bool mid = !all && (r[x].lam & ~own) != 0;
+      const unsigned live = __ballot_sync(FULL, mid);
+      if (mid)
+        queue[held + __popc(live & below)] = make_int4(
+            r[x].w, (int32_t)(uint32_t)r[x].lam, (int32_t)(uint32_t)(r[x].lam >> 32), 0);
+      __syncwarp();
+      held += __popc(live);
+      while (held >= 16) drain(16);
+    }
   }
-  best = group_max<32>(best);
-  if (lane == 0) emit_move(A, par, u, from, best);
+  if (held > 0) drain(held);
+  finish_item<false, 32, 2>(A, par, it, from, g);
+}
+
+// Class-0 nodes for k > 32, before gain_groups: no gain of u exceeds
+//   w(nets where u is the only pin of its block) - w(nets inside its block)
+// (a net outside every other block counts against every target), so only the
+// nodes where that is positive are kept, in the block's list.  Eight lanes per
+// node and LP_BOUND nodes per group in flight; the sums for 64 targets, most of
+// a node's work, are left to the nodes that remain (18 % of the nodes of the
+// finest level of a 4e6-node large-net V-cycle, 4 % on its coarse levels).
+// Measured (GB300, that finest level, 250,000 nodes and 2.4M incidences per
+// sub-round): best moves 81 -> 46 us.  For k <= 32 the sums cost less than a
+// second walk (63 to 99 % of the nodes of a 21,000-node V-cycle at k = 32 remain).
+constexpr int LP_BOUND = 2;
+constexpr int LP_KEPT = 2048;  // nodes kept by a block at a time
+constexpr int LP_QUEUE = 48;   // records queued by a warp: 15 left over and 32 new ones
+
+__device__ __forceinline__ void bound_groups(const LpArgs& A, const int4 (&it)[LP_BOUND], int sub,
+                                             int4* kept, int* nkept) {
+  unsigned long long own[LP_BOUND];
+  int32_t bound[LP_BOUND];
+  int32_t most = 0;
+#pragma unroll
+  for (int y = 0; y < LP_BOUND; ++y) {
+    own[y] = it[y].z > it[y].y ? 1ull << __ldcg(A.part + it[y].x) : 0;
+    bound[y] = 0;
+    most = max(most, it[y].z - it[y].y);
+  }
+  most = __reduce_max_sync(FULL, most);
+  for (int32_t x = sub; x - sub < most; x += 2 * SUB_G) {
+    int32_t e[LP_BOUND][2];
+#pragma unroll
+    for (int y = 0; y < LP_BOUND; ++y)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        const int32_t j = it[y].y + x + z * SUB_G;
+        e[y][z] = j < it[y].z ? __ldg(A.inets + j) : -1;
+      }
+    WideRec r[LP_BOUND][2];
+#pragma unroll
+    for (int y = 0; y < LP_BOUND; ++y)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        r[y][z] = WideRec{0, 0, 0};
+        if (e[y][z] >= 0) r[y][z] = load_wide(A.rec, e[y][z]);
+      }
+#pragma unroll
+    for (int y = 0; y < LP_BOUND; ++y)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        if (r[y][z].ones & own[y]) bound[y] += r[y][z].w;
+        if (r[y][z].lam == own[y]) bound[y] -= r[y][z].w;
+      }
+  }
+#pragma unroll
+  for (int y = 0; y < LP_BOUND; ++y) {
+    const int32_t sum = group_sum<SUB_G>(bound[y]);
+    if (sub == 0 && sum > 0) kept[atomicAdd(nkept, 1)] = it[y];
+  }
 }
 
 // ------------------------------------------------- pair selection (a12)
@@ -727,7 +864,7 @@ __global__ void __launch_bounds__(LP_THREADS, 2) k_lp_run(const __grid_constant_
   __shared__ int32_t s_hist[2 * MAX_SUBROUNDS], s_base[2 * MAX_SUBROUNDS];
   __shared__ long long s_bw[HG_MAX_K], s_slack[HG_MAX_K];
   __shared__ uint16_t s_big[MAX_PAIRS];
-  __shared__ int s_nbig;
+  __shared__ int s_nbig, s_kept;
   __shared__ int64_t s_obj[32];
   const int lane = lane_id(), wv = warp_in_block();
   // consecutive work items go to different blocks: few items spread over the chip
@@ -761,12 +898,42 @@ __global__ void __launch_bounds__(LP_THREADS, 2) k_lp_run(const __grid_constant_
       for (int i = blockIdx.x * LP_THREADS + threadIdx.x; i < kk; i += gridDim.x * LP_THREADS)
         A.dcnt[(par ^ 1) * kk + i] = 0;
       if (blockIdx.x == 0 && threadIdx.x < SW_WORDS) A.words[(par ^ 1) * SW_WORDS + threadIdx.x] = 0;
-      for (int32_t i = s_off[2 * s + 1] + gw; i < s_off[2 * s + 2]; i += NW)
-        gain_item<GRAPH, K, H>(A, par, __ldcg(A.items + i));
-      for (int32_t i0 = s_off[2 * s] + (NW - 1 - gw); i0 < s_off[2 * s + 1]; i0 += NG * NW) {
-        const int32_t i = i0 + grp * NW;
-        gain_groups<GRAPH, K, H>(
-            A, par, i < s_off[2 * s + 1] ? __ldcg(A.items + i) : make_int4(0, 0, 0, -1), sub);
+      if constexpr (!GRAPH && H == 2) {
+        int4* kept = reinterpret_cast<int4*>(smem);
+        int4* queue = kept + LP_KEPT + wv * LP_QUEUE;
+        for (int32_t i = s_off[2 * s + 1] + gw; i < s_off[2 * s + 2]; i += NW)
+          gain_item_wide(A, par, __ldcg(A.items + i), queue);
+        // in chunks of at most LP_KEPT nodes per block
+        constexpr int ROUNDS = LP_KEPT / (LP_WARPS * NG);
+        const int32_t hi = s_off[2 * s + 1];
+        for (int64_t c0 = s_off[2 * s]; c0 < hi; c0 += (int64_t)ROUNDS * NG * NW) {
+          __syncthreads();
+          if (threadIdx.x == 0) s_kept = 0;
+          __syncthreads();
+          for (int r = 0; r < ROUNDS; r += LP_BOUND) {
+            int64_t i = c0 + (int64_t)r * NG * NW + (NW - 1 - gw);
+            if (i >= hi) break;  // uniform in the warp
+            i += grp * NW;
+            int4 it[LP_BOUND];
+#pragma unroll
+            for (int y = 0; y < LP_BOUND; ++y, i += (int64_t)NG * NW)
+              it[y] = i < hi ? __ldcg(A.items + i) : make_int4(0, 0, 0, -1);
+            bound_groups(A, it, sub, kept, &s_kept);
+          }
+          __syncthreads();
+          for (int x = wv * NG; x < s_kept; x += LP_WARPS * NG)
+            gain_groups<GRAPH, K, H>(
+                A, par, x + grp < s_kept ? kept[x + grp] : make_int4(0, 0, 0, -1), sub);
+        }
+        __syncthreads();
+      } else {
+        for (int32_t i = s_off[2 * s + 1] + gw; i < s_off[2 * s + 2]; i += NW)
+          gain_item<GRAPH, K, H>(A, par, __ldcg(A.items + i));
+        for (int32_t i0 = s_off[2 * s] + (NW - 1 - gw); i0 < s_off[2 * s + 1]; i0 += NG * NW) {
+          const int32_t i = i0 + grp * NW;
+          gain_groups<GRAPH, K, H>(
+              A, par, i < s_off[2 * s + 1] ? __ldcg(A.items + i) : make_int4(0, 0, 0, -1), sub);
+        }
       }
       __syncwarp();
       if (!lp_sync(A, gen)) return;
@@ -880,6 +1047,8 @@ LpKernel lp_kernel(bool graph, int k) {
 // Moves per direction sorted in shared memory (more go through global
 // memory): pairs hold fewer moves as k grows, and two blocks share an SM.
 int sel_cap_for(int k) { return k <= 8 ? 4096 : 2048; }
+static_assert((LP_KEPT + LP_WARPS * LP_QUEUE) * sizeof(int4) <= select_bytes(2048),
+              "the lists of the best moves take the selection's buffers");
 static_assert(2 * RANK_MAX <= 2048, "the ranked keys take the upper half of the key buffers");
 
 size_t lp_smem_bytes(int k) { return select_bytes(sel_cap_for(k)); }
