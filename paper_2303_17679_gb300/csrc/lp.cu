@@ -17,9 +17,9 @@
 // wait per pass.  Blocks that stay resident pay a barrier instead: 0.35-0.4 us
 // in one thread-block cluster of up to 16 blocks (small levels), 1.4 us over
 // the whole chip (cooperative launch), and no host interaction at all.
-// Measured (GB300, whole call, before -> after): n = 10,000, k = 2 1.47 ->
-// 0.76 ms; n = 500,009 Zipf, k = 16 2.83 -> 1.96 ms; all levels of the 1e6 Zipf
-// V-cycle, k = 8 24.4 -> 19.1 ms; of the 4e6 large-net V-cycle, k = 64 87 -> 44 ms.
+// Measured (GB300, whole call, before -> after): n = 10,000, k = 2 1.45 ->
+// 0.69 ms; n = 500,009 Zipf, k = 16 2.79 -> 1.82 ms; all levels of the 1e6 Zipf
+// V-cycle, k = 8 24.4 -> 17.9 ms; of the 4e6 large-net V-cycle, k = 64 87 -> 44 ms.
 //
 // State that changes during the kernel (Pi, Phi, records, lists, counters) is
 // read with ld.cg or atomics, never through L1; the structure (ioff, inets,
@@ -1171,28 +1171,34 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
 
   static std::once_flag once;
   std::call_once(once, lp_attributes_once);
-  // Blocks: a lane group per node and about eight incidences per thread of a
-  // sub-round, and a warp per eight block pairs.  Up to 16 blocks run as one
-  // cluster (its barrier is three times faster than the grid's, and a small
-  // level leaves the other SMs to other streams); above that the kernel
-  // spreads over the chip, two blocks per SM when there is work for them.
+  // Blocks.  Small levels run as one cluster (its barrier is three times faster
+  // than the grid's): those with at most a lane group per node and two
+  // incidences per thread in 16 blocks; with more (eight per thread) the cluster
+  // takes 14 us for the best moves of 58,000 incidences, the grid 6.  Of the
+  // cluster sizes the largest that has work for every block is best: a sub-round
+  // of 92 nodes takes 7.5 us in one block, 6 us in 16.  Larger levels spread over
+  // the chip, two blocks per SM when there is work for them.  A handle that
+  // shares the GPU with others (it sleeps while it waits) takes no more blocks
+  // than its work fills, a lane group per node and eight incidences per thread.
   const LpKernel kernel = lp_kernel(L.graph, k);
   const size_t bytes = lp_smem_bytes(k);
-  const int64_t need = std::max<int64_t>(
-      {nodes_sr / (LP_WARPS * NG) + 1, inc_sr / (LP_THREADS * 8) + 1, (int64_t)k * (k - 1) / 256 + 1});
+  const bool shared = cx.sync_event != nullptr;
+  auto blocks_for = [&](int64_t nodes, int64_t inc) {
+    return std::max<int64_t>({nodes_sr / nodes + 1, inc_sr / inc + 1, (int64_t)k * (k - 1) / 256 + 1});
+  };
+  const int64_t need = blocks_for(LP_WARPS * NG, LP_THREADS * 8);
   int blocks = 1;
-  A.cluster = need <= CLUSTER_MAX;
+  A.cluster = (shared ? need : blocks_for(LP_WARPS * NG, LP_THREADS * 2)) <= CLUSTER_MAX;
   if (A.cluster) {
-    while (blocks < need) blocks <<= 1;
+    const int64_t want = shared ? need : blocks_for(LP_WARPS * NG / 8, LP_THREADS / 4);
+    while (blocks < want && blocks < CLUSTER_MAX) blocks <<= 1;
   } else {
     int per_sm = 0;
     HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
         &per_sm, reinterpret_cast<const void*>(kernel), LP_THREADS, bytes));
     if (per_sm < 1) throw HgError(HG_ERR_CUDA, "label propagation does not fit an SM");
-    // a handle that shares the GPU with others (it sleeps while it waits) takes
-    // no more blocks than its work fills
     const int64_t most = (int64_t)cx.num_sms * std::min(per_sm, 2);
-    blocks = (int)(cx.sync_event ? std::min(need, most) : need <= cx.num_sms ? cx.num_sms : most);
+    blocks = (int)(shared ? std::min(need, most) : need <= cx.num_sms ? cx.num_sms : most);
   }
   launch_persistent(cx, kernel, blocks, LP_THREADS, bytes, A.cluster, A);
   unsigned long long hres[LR_WORDS];
