@@ -241,6 +241,13 @@ __device__ __forceinline__ unsigned long long group_max(unsigned long long x) {
   return x;
 }
 
+// Edges j and j + share of a node whose edges end at `end` ({-1, 0} past it).
+__device__ __forceinline__ void edge_pair(const LpArgs& A, int32_t j, int32_t share, int32_t end,
+                                          int2& a0, int2& a1) {
+  a0 = j < end ? __ldg(A.adj + j) : make_int2(-1, 0);
+  a1 = j + share < end ? __ldg(A.adj + j + share) : make_int2(-1, 0);
+}
+
 // Class-0 nodes by groups of SUB_G lanes, one node (or none: an empty item) per
 // group: NG nodes' load chains per warp in flight (nodes of a few nets leave
 // most lanes of a warp idle and cost it a full chain of dependent loads each).
@@ -256,17 +263,20 @@ __device__ __forceinline__ void gain_groups(const LpArgs& A, int par, const int4
   const int from = on ? __ldcg(A.part + u) : 0, from_h = from - 32 * lane.half;
   Gain<GRAPH, K, H> g;
   g.init();
-  // two incidences per lane in flight
+  // two incidences per lane in flight, on graph levels the edges of the next
+  // step loaded ahead
   const int32_t steps = __reduce_max_sync(FULL, it.z - it.y);
+  int2 a0 = make_int2(-1, 0), a1 = a0;
+  if (GRAPH) edge_pair(A, it.y + lane.i, L::SHARE, it.z, a0, a1);
   for (int32_t x = lane.i; x - lane.i < steps; x += 2 * L::SHARE) {
     const int32_t j0 = it.y + x, j1 = j0 + L::SHARE;
     const bool v0 = j0 < it.z, v1 = j1 < it.z;
     if (GRAPH) {
-      const int2 a0 = v0 ? __ldg(A.adj + j0) : make_int2(-1, 0);
-      const int2 a1 = v1 ? __ldg(A.adj + j1) : make_int2(-1, 0);
       const int t0 = v0 ? __ldcg(A.part + a0.x) : 0, t1 = v1 ? __ldcg(A.part + a1.x) : 0;
-      g.add_edge(a0.y, t0 - 32 * lane.half, from_h);
-      g.add_edge(a1.y, t1 - 32 * lane.half, from_h);
+      const int32_t w0 = a0.y, w1 = a1.y;
+      edge_pair(A, j1 + L::SHARE, L::SHARE, it.z, a0, a1);
+      g.add_edge(w0, t0 - 32 * lane.half, from_h);
+      g.add_edge(w1, t1 - 32 * lane.half, from_h);
     } else {
       const int32_t e0 = v0 ? __ldg(A.inets + j0) : 0, e1 = v1 ? __ldg(A.inets + j1) : 0;
       NetRec r0{0, 0, 0}, r1{0, 0, 0};
@@ -344,12 +354,14 @@ __device__ __forceinline__ void gain_item(const LpArgs& A, int par, const int4 i
   Gain<GRAPH, K, H> g;
   g.init();
   if (GRAPH) {
+    int2 a0, a1;
+    edge_pair(A, beg + tl.i, L::SHARE, end, a0, a1);
     for (int32_t j = beg + tl.i; j < end; j += 2 * L::SHARE) {
-      const int32_t j1 = j + L::SHARE;
-      const int2 a0 = __ldg(A.adj + j), a1 = j1 < end ? __ldg(A.adj + j1) : make_int2(a0.x, 0);
-      const int t0 = __ldcg(A.part + a0.x), t1 = __ldcg(A.part + a1.x);
-      g.add_edge(a0.y, t0 - 32 * tl.half, from_h);
-      g.add_edge(a1.y, t1 - 32 * tl.half, from_h);
+      const int t0 = __ldcg(A.part + a0.x), t1 = a1.x >= 0 ? __ldcg(A.part + a1.x) : 0;
+      const int32_t w0 = a0.y, w1 = a1.y;
+      edge_pair(A, j + 2 * L::SHARE, L::SHARE, end, a0, a1);
+      g.add_edge(w0, t0 - 32 * tl.half, from_h);
+      g.add_edge(w1, t1 - 32 * tl.half, from_h);
     }
   } else {
     // chunks start at a multiple of 4; positions outside [beg, end) are skipped
