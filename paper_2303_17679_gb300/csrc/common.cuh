@@ -398,13 +398,15 @@ struct RefineCounters {
 struct PinState {
   DBuf<int32_t> phi;
   DBuf<unsigned long long> lam;
+  DBuf<int4> rec;
   DBuf<long long> bw;
-  DBuf<int32_t> tiles;
 };
 
-// counts == false (graph levels in label propagation): block weights only.
+// What goes with the pin counts: nothing and no counts either (graph levels in
+// label propagation), Lambda, or the packed records of gain.cuh.
+enum class PinMasks { none, lambda, records };
 void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, PinState& st,
-                     bool counts);
+                     PinMasks masks);
 
 // Seeded initial partition of a level into k blocks (initial.cu).
 void initial_partition(const Ctx& cx, const Level& L, int k, uint64_t seed, int32_t* part);

@@ -52,24 +52,6 @@ constexpr int MAX_PAIRS = HG_MAX_K * (HG_MAX_K - 1) / 2;
 // 1 <-> 2 toggles ones); the flips commute, so the records equal their
 // definition whatever the order of the moves.
 
-// Records from Phi, Lambda and w (one thread per net).
-__global__ void k_net_records(const int32_t* __restrict__ phi,
-                              const unsigned long long* __restrict__ lam,
-                              const int32_t* __restrict__ w, int32_t m, int k,
-                              int4* __restrict__ rec) {
-  const int H = k > 32 ? 2 : 1;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    unsigned long long ones = 0;
-    for (int i = 0; i < k; ++i)
-      if (phi[e * k + i] == 1) ones |= 1ull << i;
-    const unsigned long long l = lam[e];
-    for (int h = 0; h < H; ++h)
-      rec[H * e + h] = make_int4(w[e], (int32_t)(uint32_t)(ones >> (32 * h)),
-                                 (int32_t)(uint32_t)(l >> (32 * h)), 0);
-  }
-}
-
 // ------------------------------------------------------------- arguments
 
 // Counters of one sub-round (two sets, used in turn).
@@ -1084,20 +1066,9 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
                          int lp_block_deg, int32_t* part, RefineCounters& rc) {
   LPResult res;
   PinState st;
-  DBuf<int4> rec;
   {
     EventTimer tm(cx, &rc.ms_phi);
-    build_pin_state(cx, L, k, part, st, !L.graph);
-    if (!L.graph) {
-      rec.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1) * (k > 32 ? 2 : 1));
-      if (L.m > 0) {
-        k_net_records<<<grid_for(L.m, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
-            st.phi.p, st.lam.p, L.w.p, L.m, k, rec.p);
-        check_launch("net_records");
-        if (cx.launches) *cx.launches += 1;
-      }
-      st.lam.release();
-    }
+    build_pin_state(cx, L, k, part, st, L.graph ? PinMasks::none : PinMasks::records);
   }
   const int64_t per_block = (total_node_weight + k - 1) / k;
   const int kk = k * k;
@@ -1149,7 +1120,7 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
   A.m = L.m;
   A.part = part;
   A.phi = st.phi.p;
-  A.rec = rec.p;
+  A.rec = st.rec.p;
   A.bw = st.bw.p;
   A.k = k;
   A.S = S;
