@@ -837,12 +837,13 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lv_run, LV_THREADS, smem));
   if (per_sm < 1) throw HgError(HG_ERR_CUDA, "local moving does not fit an SM");
   // a block per 16 vertices or 256 edges of a sub-round (coarse levels: heavy
-  // vertices take a block each); four times that when the handle shares the GPU
-  // with others (it sleeps while it waits)
+  // vertices take a block each); four times that, and at most half the chip, when
+  // the handle shares the GPU with others (it sleeps while it waits)
   const int64_t share = cx.sync_event ? 4 : 1;
   const int64_t need =
       std::max<int64_t>(V / (S * 16 * share), g.E / (S * 256 * share)) + 1;
-  const int blocks = (int)std::min<int64_t>(need, (int64_t)cx.num_sms * std::min(per_sm, 2));
+  const int blocks =
+      (int)std::min<int64_t>(need, (int64_t)cx.num_sms * std::min(per_sm, share == 1 ? 2 : 1));
   launch_persistent(cx, k_lv_run, blocks, LV_THREADS, smem, false, A);
   lc.launches += 1;
   unsigned long long hres[LR_LV_WORDS];

@@ -1162,7 +1162,8 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
   // of 92 nodes takes 7.5 us in one block, 6 us in 16.  Larger levels spread over
   // the chip, two blocks per SM when there is work for them.  A handle that
   // shares the GPU with others (it sleeps while it waits) takes no more blocks
-  // than its work fills, a lane group per node and eight incidences per thread.
+  // than its work fills, a lane group per node and eight incidences per thread,
+  // and at most half the chip (see run_subrounds in cluster.cu).
   const LpKernel kernel = lp_kernel(L.graph, k);
   const size_t bytes = lp_smem_bytes(k);
   const bool shared = cx.sync_event != nullptr;
@@ -1180,7 +1181,7 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
     HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
         &per_sm, reinterpret_cast<const void*>(kernel), LP_THREADS, bytes));
     if (per_sm < 1) throw HgError(HG_ERR_CUDA, "label propagation does not fit an SM");
-    const int64_t most = (int64_t)cx.num_sms * std::min(per_sm, 2);
+    const int64_t most = (int64_t)cx.num_sms * std::min(per_sm, shared ? 1 : 2);
     blocks = (int)(shared ? std::min(need, most) : need <= cx.num_sms ? cx.num_sms : most);
   }
   launch_persistent(cx, kernel, blocks, LP_THREADS, bytes, A.cluster, A);
