@@ -38,17 +38,18 @@ WORKLOAD = ("hypergraph n=m=1,000,000: Zipf(2.2) net sizes in [2,1024], preferen
             "5 LP passes per level, full V-cycle")
 L2_FLUSH_BYTES = 512 << 20
 
-# DRAM traffic per launch of a kernel family (dram__bytes_read.sum +
-# dram__bytes_write.sum from one ncu capture, averaged per launch), reported
+# DRAM traffic per launch of the kernel that holds a family's phases
+# (dram__bytes_read.sum + dram__bytes_write.sum from one ncu capture, averaged
+# per launch; the whole kernel, with the other phases), reported
 # only while the source the counters were taken from is unchanged; the
 # captures are summarised under profiles/.
 TRAFFIC = {
-    "rating": {"source": "paper_2303_17679_gb300/csrc/coarsen.cu",
-               "source_sha256": "e791612ac7ac4700d2b822fa47e78481781f9cf5a71578e9c4b1bce5f331d485",
-               "bytes_per_launch": 21268333},
-    "lp_gain": {"source": "paper_2303_17679_gb300/csrc/refine.cu",
-                "source_sha256": "c51f75595d69410e0552f2464010ee93326afdafa9c1137fd140d2ace5ac64d2",
-                "bytes_per_launch": 7014247},
+    "rating": {"source": "paper_2303_17679_gb300/csrc/cluster.cu",
+               "source_sha256": "2dd0adddbf3beb5917e983fb3d2cf8eb01395633e07433ca2ddc95af920140b6",
+               "bytes_per_launch": 1274101280},
+    "lp_gain": {"source": "paper_2303_17679_gb300/csrc/lp.cu",
+                "source_sha256": "953be944311cf53dce6f2313c288fc8603943253ca93e07da0677483cacfda75",
+                "bytes_per_launch": 59933056},
 }
 
 
@@ -500,14 +501,13 @@ def family_rooflines(agg, steps, bm, peak):
     """Per-kernel-family achieved GB/s from the byte model and the families'
     event-timed durations inside the timed steps."""
     fam = {}
-    spec = [("rating", "k_rate_* (heavy-edge rating, a3)", "ms_rating_kernels", bm["rating"],
-             agg["rating_launches"]),
-            ("lp_gain", "k_lp_gain_* (LP best moves, a11; both branches of a sub-round, "
-                        "so a 'launch' here is one sub-round of two kernels)",
-             "ms_lp_gain_kernels", bm["lp_gain"], agg["lp_gain_launches"] // 2),
-            ("lp_select", "k_lp_select / k_lp_bucket (a12)", "ms_lp_select_kernels", None, None),
-            ("lp_apply", "k_lp_apply (a13)", "ms_lp_apply_kernels", bm["lp_apply"],
-             agg["lp_gain_launches"] // 2)]
+    spec = [("rating", "k_cluster_run (its rating phases, a3; one launch per level)",
+             "ms_rating_kernels", bm["rating"], agg["rating_launches"]),
+            ("lp_gain", "k_lp_run (its best-move phases, a11; one launch per level)",
+             "ms_lp_gain_kernels", bm["lp_gain"], agg["lp_gain_launches"]),
+            ("lp_select", "k_lp_run (selection phases, a12)", "ms_lp_select_kernels", None, None),
+            ("lp_apply", "k_lp_run (application phases, a13)", "ms_lp_apply_kernels",
+             bm["lp_apply"], agg["lp_gain_launches"])]
     for key, name, ms_key, nbytes, launches in spec:
         ms = agg.get(ms_key, 0.0) / steps
         rec = {"kernel": name, "ms_per_step": ms}
@@ -523,11 +523,8 @@ def family_rooflines(agg, steps, bm, peak):
 def timed_vcycle(hg, torch, hgr, k, opt, stream, steps, warmup, flush, instrumented=3):
     """create (device CSR) + hg_partition + destroy, per-step CUDA events on
     the library's stream, L2 flushed between steps.  The timed steps run
-    without per-kernel events; `instrumented` further steps with the kernel-
-    family events on (event pairs around every rating launch, event nodes
-    around every phase of the captured LP pass) give the family durations:
-    those events lengthen a step by about a tenth, so they stay out of the
-    headline steps."""
+    without phase timing; `instrumented` further steps, in which the persistent
+    kernels add up the times of their phases, give the family durations."""
     import numpy as np
     t = lambda a: torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda()
     d = (t(hgr.offsets), t(hgr.pins), t(hgr.net_w), t(hgr.node_w))
@@ -789,9 +786,9 @@ def run_ours(args, world, rank, local):
                      "peak": peak, "unit": "GB/s", "frac": d.get("frac", 0.0), "traffic": traffic,
                      "peak_kind": peak_kind + " (hbm_gbs, copy burst)",
                      "bytes_model": "per-phase algorithmic byte formulas (rating, approval, contraction, pin counts, LP gain and apply, objective) from per-level statistics",
-                     "durations": f"CUDA events on the library's stream over {ni} instrumented "
-                                  "steps run right after the timed steps (the per-kernel events "
-                                  "stay out of the headline steps)",
+                     "durations": f"phase times that the persistent kernels read from the GPU's "
+                                  f"nanosecond clock over {ni} instrumented steps run right after "
+                                  "the timed steps (the clock reads stay out of the headline steps)",
                      "instrumented_ms_per_step": iagg["instrumented_ms_per_step"],
                      "launches_per_step": d.get("launches_per_step"),
                      "algorithmic_bytes_per_launch":

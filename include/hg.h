@@ -102,8 +102,9 @@ typedef struct {
   int32_t lp_block_min_deg;
   /* 1: wait for the device by sleeping on a blocking-sync event instead of
    * spinning (frees the host core while waiting, at a few microseconds of
-   * wake-up latency per wait; the executor sets it for its jobs).  0 (default):
-   * spin. */
+   * wake-up latency per wait; the executor sets it for its jobs).  Such a
+   * handle is taken to share the GPU with others: the kernels that run a whole
+   * level use at most half the SMs.  0 (default): spin. */
   int32_t blocking_sync;
   /* Graph path (Sec. 10): 0 (default) = a level whose nets all have exactly
    * two pins is kept as a graph with one adjacency array (the other endpoint

@@ -12,10 +12,10 @@
 // that runs out of heavy nodes goes on to lighter ones), nodes are handed out
 // by tickets, and movers are published 32 at a time: three dependent atomics
 // per mover cost a warp about 2 us per node.
-// Measured (GB300, clustering and contraction of all levels, before -> after,
-// with the cluster words kept by passes over the nets): 1e6 Zipf, k = 8 70.6 ->
-// 52 ms; 4e6 large nets, k = 64 142 -> 107 ms; one level of 500,009 nodes 10.8 ->
-// 7.2 ms; of 1471 nodes 1.67 -> 1.2 ms.
+// Measured (GB300, clustering and contraction of all levels, as graphs -> when
+// this form and the passes over the nets came in -> now): 1e6 Zipf, k = 8 70.6 ->
+// 52 -> 45.6 ms; 4e6 large nets, k = 64 142 -> 107 -> 85.5 ms; one level of
+// 500,009 nodes 10.8 -> 7.2 -> 6.5 ms; of 1471 nodes 1.67 -> 1.2 -> 1.09 ms.
 #include <algorithm>
 #include <climits>
 #include <mutex>
