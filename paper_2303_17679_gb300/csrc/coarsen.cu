@@ -247,7 +247,10 @@ __device__ __forceinline__ void group_sort(int32_t b, int32_t sz, const int32_t*
 }
 
 // One warp per net: gpins = the grouped pin order, gkey = group key per
-// position.  Unrated nets and nets of more than GROUP_NET pins keep their order.
+// position.  Rated nets of more than GROUP_NET pins keep their order.  Of unrated
+// nets nothing but the pins' communities is ever read: without communities they
+// are left out (on large-net inputs they hold most pins, and one warp each copied
+// them: 1.2 ms per level of 31M pins, 0.9 ms without).
 __global__ void __launch_bounds__(GROUP_WARPS * 32)
 k_group_nets(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins, int32_t m, int T,
              const int32_t* __restrict__ c, const int32_t* __restrict__ comm, int64_t p,
@@ -257,7 +260,9 @@ k_group_nets(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
   for (int64_t e = (int64_t)blockIdx.x * GROUP_WARPS + warp_in_block(); e < m;
        e += (int64_t)gridDim.x * GROUP_WARPS) {
     const int32_t b = eoff[e], sz = eoff[e + 1] - b;
-    if (sz < 2 || sz > T || sz > GROUP_NET) {
+    const bool rated = sz >= 2 && sz <= T;
+    if (!rated && !comm) continue;
+    if (!rated || sz > GROUP_NET) {
       for (int32_t q = b + lane_id(); q < b + sz; q += 32) gpins[q] = pins[q];
     } else if (sz <= 32) {
       group_sort<1>(b, sz, pins, c, comm, gpins, gkey, nmeta + e);
