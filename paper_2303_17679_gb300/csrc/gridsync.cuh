@@ -18,9 +18,11 @@ constexpr int SPIN_LIMIT = 1 << 24;  // polls of one grid barrier (seconds)
 __device__ __forceinline__ bool grid_sync(bool cluster, unsigned* counter, int32_t* status,
                                           unsigned& gen) {
   if (cluster) {
+    // not the .aligned form: callers come from loops that lanes leave at
+    // different times, and nothing makes the compiler rejoin them first
     asm volatile(
-        "barrier.cluster.arrive.release.aligned;\n"
-        "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        "barrier.cluster.arrive.release;\n"
+        "barrier.cluster.wait.acquire;" ::: "memory");
     return true;
   }
   ++gen;

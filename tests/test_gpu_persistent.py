@@ -1,0 +1,46 @@
+"""The persistent kernels on the GPU: barriers behind loops that the lanes of a
+warp leave at different times, and what the launch rules decide.  All results are
+integers and compared exactly with the oracle."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2303_17679_gb300 import hg  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def create(hgr, seed, S=16, factor=160, **options):
+    o = hg.hg_default_options()
+    o.seed, o.subrounds, o.contraction_limit_factor = seed, S, factor
+    for name, value in options.items():
+        setattr(o, name, value)
+    return hg.hg_create(hgr.n, hgr.m, hgr.offsets, hgr.pins, hgr.net_w, hgr.node_w,
+                        hg.HG_MEM_HOST, o, torch.cuda.current_stream())
+
+
+# 2 S list counters that are no multiple of a warp, node counts that are none of a
+# block: small levels, whose blocks meet at the barrier of one cluster
+@pytest.mark.parametrize("n,S,k", [(333, 1, 2), (1471, 3, 5), (2999, 7, 33), (4001, 33, 8)])
+def test_ragged_small_levels(oracle_mod, n, S, k):
+    hgr = synth.zipf_preferential(n, n, n, name="ragged")
+    vc = oracle_mod.multilevel(hgr, k, 30000, S=S, factor=10, seed=n, max_passes=3)
+    h = create(hgr, n, S, 10)
+    try:
+        part = torch.empty(n, dtype=torch.int32, device="cuda")
+        obj = hg.hg_partition(h, k, 30000, 3, part)
+        assert hg.hg_num_levels(h) == len(vc.levels)
+        assert np.array_equal(part.cpu().numpy(), vc.parts[0]) and obj == vc.objectives[0]
+    finally:
+        hg.hg_destroy(h)
