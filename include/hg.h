@@ -80,7 +80,9 @@ typedef struct {
    * Both NULL: stream-ordered allocations (cudaMallocFromPoolAsync /
    * cudaFreeAsync) from the library's own memory pool of the device, which
    * keeps freed blocks for later handles (hg_trim_memory returns them to the
-   * driver); the device's default pool is not touched. */
+   * driver); the device's default pool is not touched.  A hook's blocks may have
+   * any alignment: the library asks for 31 bytes more than it needs and starts on
+   * a 32-byte boundary inside the block. */
   void* (*dev_alloc)(size_t bytes, void* ctx);
   void (*dev_free)(void* ptr, void* ctx);
   void* alloc_ctx;

@@ -22,6 +22,7 @@ struct hg_t {
   int sticky = 0;            // HG_ERR_CUDA once a CUDA error was seen
   int64_t launches = 0;
   hg_stats stats{};
+  DBuf<int32_t> status;      // cx.d_status
   std::vector<std::unique_ptr<Level>> levels;
 };
 
@@ -228,7 +229,8 @@ int hg_create(int32_t n, int32_t m, const int32_t* net_offsets, const int32_t* p
     h->cx.alloc.stream = h->cx.stream;
     h->cx.launches = &h->launches;
     if (!o.dev_alloc) h->cx.alloc.pool = hgk::library_pool(h->device);
-    h->cx.d_status = static_cast<int32_t*>(h->cx.alloc.get(sizeof(int32_t) * 4));
+    h->status.alloc(&h->cx.alloc, 4);
+    h->cx.d_status = h->status.p;
     HG_CUDA(cudaMemsetAsync(h->cx.d_status, 0, sizeof(int32_t) * 4, h->cx.stream));
     if (mem == HG_MEM_DEVICE) {
       int32_t ends[2] = {0, 0};
@@ -649,7 +651,7 @@ int hg_destroy(hg_t* h) {
   if (!h) return HG_OK;
   cudaSetDevice(h->device);
   h->levels.clear();
-  if (h->cx.d_status) h->cx.alloc.put(h->cx.d_status);
+  h->status.release();
   h->cx.d_status = nullptr;
   cudaStreamSynchronize(h->cx.stream);
   if (h->cx.sync_event) cudaEventDestroy(h->cx.sync_event);

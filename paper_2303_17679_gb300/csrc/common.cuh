@@ -204,11 +204,18 @@ struct Alloc {
 // The library's private stream-ordered memory pool of a device (prim.cu).
 cudaMemPool_t library_pool(int device);
 
+// Kernels read the buffers in units of up to 32 bytes (the net records of
+// gain.cuh), so every buffer starts on a 32-byte boundary.  The library's pool
+// returns blocks aligned to 256 bytes; a caller's hook may align less, so its
+// blocks are that much larger and the buffer starts inside.
+constexpr size_t BUF_ALIGN = 32;
+
 template <typename T>
 struct DBuf {
   T* p = nullptr;
   size_t n = 0;
   const Alloc* a = nullptr;
+  void* block = nullptr;  // what the allocator returned
   DBuf() = default;
   DBuf(const DBuf&) = delete;
   DBuf& operator=(const DBuf&) = delete;
@@ -216,22 +223,26 @@ struct DBuf {
   DBuf& operator=(DBuf&& o) noexcept {
     if (this != &o) {
       release();
-      p = o.p; n = o.n; a = o.a;
-      o.p = nullptr; o.n = 0;
+      p = o.p; n = o.n; a = o.a; block = o.block;
+      o.p = nullptr; o.n = 0; o.block = nullptr;
     }
     return *this;
   }
   ~DBuf() { release(); }
   void alloc(const Alloc* al, size_t count) {
     release();
+    if (count == 0) return;
     a = al;
+    block = al->get(count * sizeof(T) + (al->fn_alloc ? BUF_ALIGN - 1 : 0));
+    p = reinterpret_cast<T*>((reinterpret_cast<uintptr_t>(block) + BUF_ALIGN - 1) &
+                             ~(uintptr_t)(BUF_ALIGN - 1));
     n = count;
-    p = count ? static_cast<T*>(al->get(count * sizeof(T))) : nullptr;
   }
   void release() {
-    if (p && a) a->put(p);
+    if (block && a) a->put(block);
     p = nullptr;
     n = 0;
+    block = nullptr;
   }
   size_t bytes() const { return n * sizeof(T); }
 };

@@ -31,7 +31,8 @@ struct WideRec {
   unsigned long long ones, lam;
 };
 
-// One 32-byte load: a gather is bound by its requests, a line each.
+// One 32-byte load: a gather is bound by its requests, a line each.  The records
+// start on a 32-byte boundary (BUF_ALIGN).
 __device__ __forceinline__ WideRec load_wide(const int4* rec, int32_t e) {
   unsigned w, o0, l0, x0, x1, o1, l1, x2;
   asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"

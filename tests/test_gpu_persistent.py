@@ -1,6 +1,8 @@
 """The persistent kernels on the GPU: barriers behind loops that the lanes of a
 warp leave at different times, and what the launch rules decide.  All results are
 integers and compared exactly with the oracle."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -44,3 +46,44 @@ def test_ragged_small_levels(oracle_mod, n, S, k):
         assert np.array_equal(part.cpu().numpy(), vc.parts[0]) and obj == vc.objectives[0]
     finally:
         hg.hg_destroy(h)
+
+
+class Hooks:
+    """A caller's allocator whose blocks start `shift` bytes into torch's."""
+
+    def __init__(self, shift):
+        self.shift, self.live = shift, {}
+        self.alloc, self.free = hg.ALLOC_FN(self.get), hg.FREE_FN(self.put)
+
+    def get(self, size, ctx):
+        t = torch.empty(size + self.shift, dtype=torch.uint8, device="cuda")
+        self.live[t.data_ptr() + self.shift] = t
+        return t.data_ptr() + self.shift
+
+    def put(self, ptr, ctx):
+        del self.live[ptr]
+
+    def options(self):
+        return dict(dev_alloc=self.alloc, dev_free=self.free)
+
+
+# k = 64: net records of 32 bytes; nets of two pins: pins read in pairs
+@pytest.mark.parametrize("shift", [0, 4, 8, 16])
+@pytest.mark.parametrize("graph,k", [(False, 64), (False, 8), (True, 64)])
+def test_hook_blocks_of_any_alignment(oracle_mod, shift, graph, k):
+    hgr = synth.graph_preferential(3, 4000, 20_000) if graph else synth.zipf_preferential(3, 4000, 4000)
+    vc = oracle_mod.multilevel(hgr, k, 30000, S=16, factor=10, seed=3, max_passes=3)
+    hooks = Hooks(shift)
+    h = create(hgr, 3, factor=10, **hooks.options())
+    try:
+        part = torch.empty(hgr.n, dtype=torch.int32, device="cuda")
+        obj = hg.hg_partition(h, k, 30000, 3, part)
+        assert np.array_equal(part.cpu().numpy(), vc.parts[0]) and obj == vc.objectives[0]
+        b = torch.zeros(hgr.n, dtype=torch.int64, device="cuda")
+        p = torch.zeros((hgr.n, k), dtype=torch.int64, device="cuda")
+        hg.hg_gain_table(h, 0, k, part, b, p)
+        wb, wp = oracle_mod.gain_table(hgr, k, vc.parts[0])
+        assert np.array_equal(b.cpu().numpy(), wb) and np.array_equal(p.cpu().numpy(), wp)
+    finally:
+        hg.hg_destroy(h)
+    assert not hooks.live

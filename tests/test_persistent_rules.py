@@ -1,7 +1,9 @@
-"""Rules of the persistent kernels that can be checked without a GPU."""
+"""Rules of the kernels' launch code that can be checked without a GPU."""
 import glob
 import os
 import re
+
+from tests import hostcc
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_2303_17679_gb300", "csrc")
@@ -19,3 +21,38 @@ def test_cluster_barrier_takes_diverged_warps():
         for ins in re.findall(r'"(barrier\.cluster\.[a-z.]+)', open(path).read()):
             assert ".aligned" not in ins, (os.path.basename(path), ins)
     assert "barrier.cluster.wait.acquire" in source("gridsync.cuh")
+
+
+def test_buffers_of_a_hook_start_on_a_32_byte_boundary(tmp_path):
+    """Whatever alignment the hook's blocks have: the records of k > 32 are read 32
+    bytes at a time.  The block itself goes back to the hook."""
+    hostcc.run(tmp_path, ["common.cuh"], """
+    using namespace hgk;
+    void* Alloc::get(size_t bytes) const { return fn_alloc(bytes, ctx); }
+    void Alloc::put(void* p) const { fn_free(p, ctx); }
+    struct Hook { unsigned char* at; size_t asked; void* freed; };
+    int main() {
+      std::vector<unsigned char> room(4096);
+      for (int shift = 0; shift < 64; ++shift) {
+        Hook k{room.data() + shift, 0, nullptr};
+        Alloc a;
+        a.fn_alloc = [](size_t bytes, void* c) -> void* {
+          static_cast<Hook*>(c)->asked = bytes;
+          return static_cast<Hook*>(c)->at;
+        };
+        a.fn_free = [](void* p, void* c) { static_cast<Hook*>(c)->freed = p; };
+        a.ctx = &k;
+        {
+          DBuf<int4> b;
+          b.alloc(&a, 10);
+          CHECK((uintptr_t)b.p % 32 == 0);
+          CHECK((unsigned char*)b.p >= k.at);
+          CHECK((unsigned char*)(b.p + 10) <= k.at + k.asked);
+          DBuf<int4> c = std::move(b);
+          CHECK(!b.p && !k.freed);
+        }
+        CHECK(k.freed == k.at);
+      }
+      return 0;
+    }
+    """)
