@@ -30,8 +30,10 @@
 // eight lanes (a warp) that holds one edge per lane and sums the edges of a
 // cluster by exchanging them; up to LV_SMALL edges by one warp with a shared
 // table of the neighbouring clusters, up to LV_BLOCK by the block with all the
-// tables as one; larger vertices are split into parts by a hash of the cluster,
-// a block each, whose bests are compared after one more barrier.  Aggregation
+// tables as one; up to LV_HUGE in parts by a hash of the cluster, a block each,
+// whose bests are compared after one more barrier; larger vertices by chunks of
+// their edges, a block each, which sum a chunk in shared memory and add it to the
+// vertex's table in global memory, read in pieces after a barrier.  Aggregation
 // adds the edges to global tables, one per coarse vertex.
 // What bounds it: some 25 rounds of 16 dependent sub-rounds, each a chain of
 // gathers; as four or five launches per sub-round, with a host wait and the
@@ -41,24 +43,21 @@
 #include <mutex>
 
 #include "gridsync.cuh"
+#include "louvain.cuh"
 #include "pintile.cuh"
 
 namespace hgk {
 
 namespace {
 
-constexpr int LV_ROUNDS = 5;
 constexpr int LV_LEVELS = 32;
-constexpr int LV_CLASSES = 5;
-constexpr int LV_GROUP = 8;             // class 0: degree <= 8, eight lanes per vertex
-constexpr int LV_LANES = 32;            // class 1: degree <= 32, a warp per vertex
-constexpr int LV_SMALL = 256;           // class 2: degree <= 256, a warp and a shared table
-constexpr int LV_BLOCK = 4096;          // class 3: degree <= 4096, a block
-constexpr int LV_PART = 2048;           // class 4: neighbouring clusters per part
 constexpr int LV_THREADS = 512;
 constexpr int LV_WARPS = LV_THREADS / 32;
 constexpr int LV_SLOTS = 2 * LV_SMALL;  // slots per warp (load <= 1/2)
 constexpr int LV_BLOCK_SLOTS = LV_SLOTS * LV_WARPS;
+constexpr int LV_CHUNK_SLOTS = 2 * LV_CHUNK;
+static_assert(2 * LV_BLOCK <= LV_BLOCK_SLOTS && LV_CHUNK_SLOTS <= LV_BLOCK_SLOTS,
+              "the block's table is at most half full");
 constexpr int32_t LV_EMPTY = -1;
 
 using i128 = __int128;
@@ -117,10 +116,15 @@ __global__ void k_lv_offsets(const int32_t* __restrict__ ioff, const int32_t* __
     off[i] = i <= n ? (long long)ioff[i] : (long long)(p + eoff[i - n]);
 }
 
+// What k_lv_degrees adds up: the degrees, the table slots that the class 5
+// vertices of one sub-round take at most, and those slots per round and sub-round.
+enum { LD_TOTAL = 0, LD_MOST = 1, LD_SLOTS = 2 };
+
 // k_i = 2 self_i + sum of i's edge weights (a warp per vertex); W2 = sum k_i.
 __global__ void k_lv_degrees(const long long* __restrict__ off, const long long* __restrict__ aw,
-                             const long long* __restrict__ self, int64_t V,
-                             long long* __restrict__ k, unsigned long long* __restrict__ total) {
+                             const long long* __restrict__ self, int64_t V, uint64_t seed,
+                             int level, int S, long long* __restrict__ k,
+                             unsigned long long* __restrict__ sums) {
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   long long acc = 0;
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < V; i += nw) {
@@ -130,8 +134,16 @@ __global__ void k_lv_degrees(const long long* __restrict__ off, const long long*
     s += 2 * self[i];
     if (lane_id() == 0) k[i] = s;
     acc += s;
+    const long long deg = off[i + 1] - off[i];
+    if (deg > LV_HUGE && lane_id() < LV_ROUNDS) {
+      const int r = lane_id();
+      const unsigned long long slots = lv_slots(deg);
+      const unsigned long long before =
+          atomicAdd(&sums[LD_SLOTS + r * S + subround_louvain(seed, level, r, i, S)], slots);
+      atomicMax(&sums[LD_MOST], before + slots);
+    }
   }
-  if (lane_id() == 0 && acc) atomicAdd(total, (unsigned long long)acc);
+  if (lane_id() == 0 && acc) atomicAdd(&sums[LD_TOTAL], (unsigned long long)acc);
 }
 
 __global__ void k_lv_init(int64_t V, const long long* __restrict__ k, int32_t* __restrict__ cl,
@@ -202,6 +214,12 @@ struct PartBest {
   int32_t c, pad;
 };
 
+// A class 5 vertex of the round: its list entries and its table.
+struct HugeVertex {
+  int32_t i, entries;
+  unsigned long long tab, slots;
+};
+
 struct LvArgs {
   const long long* off;
   const int32_t* adj;
@@ -213,8 +231,13 @@ struct LvArgs {
   int64_t V;
   uint64_t seed;
   int level, S;
-  int2* list;       // {vertex, part | parts << 16} by (sub-round, class)
+  int2* list;       // {vertex, part} by (sub-round, class); class 5 {index in huge, chunk}
   int32_t *cnt, *fill;  // LV_CLASSES S each
+  HugeVertex* huge;
+  int32_t* nhuge;
+  unsigned long long* tabfill;  // S: table slots given out
+  int32_t* tkey;                // tables of the class 5 vertices of a sub-round
+  long long* tval;
   int2* mv;         // {vertex, cluster}
   int32_t* words;
   PartBest* parts;
@@ -222,19 +245,6 @@ struct LvArgs {
   unsigned* barrier;
   int32_t* status;
 };
-
-// Class and list entries of a vertex of degree deg (0: no neighbouring cluster,
-// never moves).
-__device__ __forceinline__ int lv_class(const LvArgs& A, long long deg, int32_t& entries) {
-  entries = 1;
-  if (deg <= LV_GROUP) return 0;
-  if (deg <= LV_LANES) return 1;
-  if (deg <= LV_SMALL) return 2;
-  if (deg <= LV_BLOCK) return 3;
-  const long long D = deg < A.V ? deg : A.V;  // bound on the neighbouring clusters
-  entries = (int32_t)((D + LV_PART - 1) / LV_PART);
-  return 4;
-}
 
 // Counts (scatter == false) or writes the list entries of the block's tiles of
 // vertices; one global claim per tile and key.
@@ -246,12 +256,13 @@ __device__ __forceinline__ void lv_list(const LvArgs& A, int round, bool scatter
   const int64_t stride = (int64_t)gridDim.x * LV_THREADS;
   for (int64_t i0 = (int64_t)blockIdx.x * LV_THREADS; i0 < A.V; i0 += stride) {
     const int64_t i = i0 + threadIdx.x;
-    int key = -1, slot = 0;
+    int key = -1, slot = 0, cls = 0;
     int32_t entries = 0;
+    long long deg = 0;
     if (i < A.V) {
-      const long long deg = A.off[i + 1] - A.off[i];
-      if (deg > 0) {
-        const int cls = lv_class(A, deg, entries);
+      deg = A.off[i + 1] - A.off[i];
+      if (deg > 0) {  // a vertex without neighbours never moves
+        cls = lv_class(deg, entries);
         key = subround_louvain(A.seed, A.level, round, i, A.S) * LV_CLASSES + cls;
         slot = atomicAdd(&s_hist[key], entries);
       }
@@ -265,7 +276,14 @@ __device__ __forceinline__ void lv_list(const LvArgs& A, int round, bool scatter
     __syncthreads();
     if (key >= 0) {
       int2* out = A.list + s_off[key] + s_base[key] + slot;
-      for (int32_t x = 0; x < entries; ++x) out[x] = make_int2((int32_t)i, x | (entries << 16));
+      int32_t name = (int32_t)i;
+      if (cls == 5) {
+        name = atomicAdd(A.nhuge, 1);
+        const unsigned long long slots = lv_slots(deg);
+        A.huge[name] = HugeVertex{(int32_t)i, entries,
+                                  atomicAdd(&A.tabfill[key / LV_CLASSES], slots), slots};
+      }
+      for (int32_t x = 0; x < entries; ++x) out[x] = make_int2(name, x);
     }
     __syncthreads();
   }
@@ -356,22 +374,41 @@ __device__ __forceinline__ void lv_lanes(const LvArgs& A, int32_t* words, int32_
 }
 
 // The best other candidate and the own cluster's entry among slots first,
-// first + step, ... of a table, which are cleared.
+// first + step, ... of a table, which are cleared.  Four slots at a time: the
+// volumes are gathers, whose latencies would follow one another (V-cycle with
+// communities on 250,007 nodes and 1.35M pins: 38.1 -> 37.1 ms; eight at a time
+// is slower again).
 __device__ __forceinline__ void lv_take(const LvArgs& A, int32_t i, int32_t* keys,
                                         long long* vals, int slots, int first, int step,
                                         Cand& best, long long& kia) {
+  constexpr int AT_ONCE = 4;
   const int32_t own = A.cl[i];
   const long long ki = A.k[i];
   best = Cand{0, -1};
   kia = 0;
-  for (int s = first; s < slots; s += step) {
-    const int32_t C = keys[s];
-    if (C == LV_EMPTY) continue;
-    const long long kic = vals[s];
-    keys[s] = LV_EMPTY;
-    vals[s] = 0;
-    if (C == own) kia = kic;
-    else cand_better(best, Cand{(i128)A.W2 * kic - (i128)ki * A.vol[C], C});
+  for (int s0 = first; s0 < slots; s0 += AT_ONCE * step) {
+    int32_t C[AT_ONCE];
+    long long kic[AT_ONCE], vol[AT_ONCE];
+#pragma unroll
+    for (int x = 0; x < AT_ONCE; ++x) {
+      const int s = s0 + x * step;
+      C[x] = s < slots ? keys[s] : LV_EMPTY;
+    }
+#pragma unroll
+    for (int x = 0; x < AT_ONCE; ++x) {
+      const int s = s0 + x * step;
+      kic[x] = vol[x] = 0;
+      if (C[x] == LV_EMPTY) continue;
+      kic[x] = vals[s];
+      vol[x] = A.vol[C[x]];
+      keys[s] = LV_EMPTY;
+      vals[s] = 0;
+    }
+#pragma unroll
+    for (int x = 0; x < AT_ONCE; ++x) {
+      if (C[x] == own) kia = kic[x];
+      else if (C[x] != LV_EMPTY) cand_better(best, Cand{(i128)A.W2 * kic[x] - (i128)ki * vol[x], C[x]});
+    }
   }
   warp_best(best);
   kia = warp_sum(kia);
@@ -383,27 +420,13 @@ __device__ __forceinline__ int lv_part(int32_t C, int parts) {
                32);
 }
 
-// Classes 3 and 4: the block rates vertex i over all its edges, keeping the
-// clusters of one part.
-__device__ __forceinline__ void lv_block(const LvArgs& A, int32_t* words, int32_t x,
-                                         int32_t* keys, long long* vals) {
+// The best of the block's candidates and the sum of its kia, in warp 0.
+__device__ __forceinline__ void lv_block_best(Cand& best, long long& kia) {
   __shared__ unsigned long long s_lo[LV_WARPS];
   __shared__ long long s_hi[LV_WARPS], s_kia[LV_WARPS];
   __shared__ int32_t s_c[LV_WARPS];
-  const int2 nd = A.list[x];
-  const int32_t i = nd.x;
-  const int part = nd.y & 0xffff, parts = nd.y >> 16;
-  const long long b = A.off[i], e = A.off[i + 1];
-  for (long long q = b + threadIdx.x; q < e; q += LV_THREADS) {
-    const int32_t C = A.cl[A.adj[q]];
-    if (parts > 1 && lv_part(C, parts) != part) continue;
-    if (!table_add(keys, vals, LV_BLOCK_SLOTS - 1, C, A.aw[q])) dev_fail(A.status, DEV_HASH_FULL);
-  }
-  __syncthreads();
-  Cand best;
-  long long kia;
-  lv_take(A, i, keys, vals, LV_BLOCK_SLOTS, threadIdx.x, LV_THREADS, best, kia);
-  if (lane_id() == 0) {
+  const int l = lane_id();
+  if (l == 0) {
     s_lo[warp_in_block()] = (unsigned long long)best.s;
     s_hi[warp_in_block()] = (long long)(best.s >> 64);
     s_c[warp_in_block()] = best.c;
@@ -411,7 +434,6 @@ __device__ __forceinline__ void lv_block(const LvArgs& A, int32_t* words, int32_
   }
   __syncthreads();
   if (warp_in_block() == 0) {
-    const int l = lane_id();
     best = Cand{0, -1};
     kia = 0;
     if (l < LV_WARPS) {
@@ -420,15 +442,97 @@ __device__ __forceinline__ void lv_block(const LvArgs& A, int32_t* words, int32_
     }
     warp_best(best);
     kia = warp_sum(kia);
-    if (parts == 1) {
-      lv_emit(A, words, l == 0 && lv_moves(A, i, kia, best), i, best.c);
-    } else if (l == 0) {
-      A.parts[x] = PartBest{(unsigned long long)best.s, (long long)(best.s >> 64), kia, best.c, 0};
-    }
+  }
+}
+
+__device__ __forceinline__ void lv_write_part(const LvArgs& A, int32_t x, const Cand& best,
+                                              long long kia) {
+  A.parts[x] = PartBest{(unsigned long long)best.s, (long long)(best.s >> 64), kia, best.c, 0};
+}
+
+// Classes 3 and 4: the block rates the entry's vertex over all its edges,
+// keeping the clusters of one part.
+__device__ __forceinline__ void lv_block(const LvArgs& A, int32_t* words, int32_t x,
+                                         int32_t* keys, long long* vals) {
+  const int2 nd = A.list[x];
+  const int32_t i = nd.x;
+  const long long b = A.off[i], e = A.off[i + 1];
+  int32_t parts;
+  lv_class(e - b, parts);
+  for (long long q = b + threadIdx.x; q < e; q += LV_THREADS) {
+    const int32_t C = A.cl[A.adj[q]];
+    if (parts > 1 && lv_part(C, parts) != nd.y) continue;
+    if (!table_add(keys, vals, LV_BLOCK_SLOTS - 1, C, A.aw[q])) dev_fail(A.status, DEV_HASH_FULL);
+  }
+  __syncthreads();
+  Cand best;
+  long long kia;
+  lv_take(A, i, keys, vals, LV_BLOCK_SLOTS, threadIdx.x, LV_THREADS, best, kia);
+  lv_block_best(best, kia);
+  if (warp_in_block() == 0) {
+    if (parts == 1)
+      lv_emit(A, words, lane_id() == 0 && lv_moves(A, i, kia, best), i, best.c);
+    else if (lane_id() == 0)
+      lv_write_part(A, x, best, kia);
   }
   __syncthreads();
 }
 
+// Class 5: the entry's chunk of edges, summed per cluster in the block's table,
+// then added to the vertex's.  (Edge by edge, the atomics of a hub whose
+// neighbours have joined few clusters would meet at those slots.)
+__device__ __forceinline__ void lv_insert_chunk(const LvArgs& A, int32_t x, int32_t* keys,
+                                                long long* vals) {
+  const int2 nd = A.list[x];
+  const HugeVertex h = A.huge[nd.x];
+  const long long b = A.off[h.i] + (long long)nd.y * LV_CHUNK;
+  const long long e = min(b + LV_CHUNK, A.off[h.i + 1]);
+  for (long long q = b + threadIdx.x; q < e; q += LV_THREADS)
+    if (!table_add(keys, vals, LV_CHUNK_SLOTS - 1, A.cl[A.adj[q]], A.aw[q]))
+      dev_fail(A.status, DEV_HASH_FULL);
+  __syncthreads();
+  for (int s = threadIdx.x; s < LV_CHUNK_SLOTS; s += LV_THREADS) {
+    const int32_t C = keys[s];
+    if (C == LV_EMPTY) continue;
+    if (!table_add(A.tkey + h.tab, A.tval + h.tab, (uint32_t)(h.slots - 1), C, vals[s]))
+      dev_fail(A.status, DEV_HASH_FULL);
+    keys[s] = LV_EMPTY;
+    vals[s] = 0;
+  }
+  __syncthreads();
+}
+
+// Class 5, after a barrier: the best of the entry's piece of the table, which is
+// cleared for the next sub-round.
+__device__ __forceinline__ void lv_scan_piece(const LvArgs& A, int32_t x) {
+  const int2 nd = A.list[x];
+  const HugeVertex h = A.huge[nd.x];
+  const unsigned long long lo = h.slots * (unsigned)nd.y / (unsigned)h.entries;
+  const unsigned long long hi = h.slots * (unsigned)(nd.y + 1) / (unsigned)h.entries;
+  const int32_t own = A.cl[h.i];
+  const long long ki = A.k[h.i];
+  Cand best{0, -1};
+  long long kia = 0;
+  for (unsigned long long s = h.tab + lo + threadIdx.x; s < h.tab + hi; s += LV_THREADS) {
+    const int32_t C = __ldcg(A.tkey + s);
+    if (C == LV_EMPTY) continue;
+    const long long kic = __ldcg(A.tval + s);
+    __stcg(A.tkey + s, LV_EMPTY);
+    __stcg(A.tval + s, 0ll);
+    if (C == own) kia = kic;
+    else cand_better(best, Cand{(i128)A.W2 * kic - (i128)ki * A.vol[C], C});
+  }
+  warp_best(best);
+  kia = warp_sum(kia);
+  lv_block_best(best, kia);
+  if (threadIdx.x == 0) lv_write_part(A, x, best, kia);
+  __syncthreads();
+}
+
+// HUGE: the level has class 5 vertices.  Their code stays out of the kernel of the
+// other levels, which its presence alone slows (V-cycle with communities on
+// 250,007 nodes and 1.35M pins: 37.1 ms, 39.9 with one kernel for all levels).
+template <bool HUGE>
 __global__ void __launch_bounds__(LV_THREADS, 2) k_lv_run(const __grid_constant__ LvArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   long long* vals = reinterpret_cast<long long*>(smem);
@@ -464,12 +568,16 @@ __global__ void __launch_bounds__(LV_THREADS, 2) k_lv_run(const __grid_constant_
         for (int x = blockIdx.x * LV_THREADS + threadIdx.x; x < nkeys; x += gridDim.x * LV_THREADS) {
           A.cnt[x] = 0;
           A.fill[x] = 0;
+          if (x < A.S) A.tabfill[x] = 0;
+          if (x == 0) *A.nhuge = 0;
         }
       const int32_t* at = s_off + LV_CLASSES * s;
       // ---- decisions from the state at the start of the sub-round
-      for (int32_t x = at[4] + (int32_t)blockIdx.x; x < at[5]; x += gridDim.x)
-        lv_block(A, words, x, keys, vals);
-      for (int32_t x = at[3] + (int32_t)blockIdx.x; x < at[4]; x += gridDim.x)
+      if constexpr (HUGE)
+        for (int32_t x = at[5] + (int32_t)blockIdx.x; x < at[6]; x += gridDim.x)
+          lv_insert_chunk(A, x, keys, vals);
+      // classes 4 and 3
+      for (int32_t x = at[5] - 1 - (int32_t)blockIdx.x; x >= at[3]; x -= gridDim.x)
         lv_block(A, words, x, keys, vals);
       for (int64_t x = at[2] + gw; x < at[3]; x += NW) {
         const int32_t i = A.list[x].x;
@@ -488,11 +596,24 @@ __global__ void __launch_bounds__(LV_THREADS, 2) k_lv_run(const __grid_constant_
       lv_lanes<LV_GROUP>(A, words, at[0], at[1], NW - 1 - gw, NW);
       __syncwarp();
       if (!sync()) return;
-      if (at[5] > at[4]) {
-        for (int64_t x = at[4] + gw; x < at[5]; x += NW) {
+      if constexpr (HUGE) {
+        if (at[6] > at[5]) {
+          for (int32_t x = at[5] + (int32_t)blockIdx.x; x < at[6]; x += gridDim.x)
+            lv_scan_piece(A, x);
+          if (!sync()) return;
+        }
+      }
+      if (at[6] > at[4]) {
+        for (int64_t x = at[4] + gw; x < at[6]; x += NW) {
           const int2 nd = A.list[x];
-          if ((nd.y & 0xffff) != 0) continue;  // the first part's entry combines
-          const int parts = nd.y >> 16;
+          if (nd.y != 0) continue;  // the first entry of a vertex combines
+          int32_t i = nd.x, parts;
+          if (!HUGE || x < at[5]) {
+            lv_class(A.off[i + 1] - A.off[i], parts);
+          } else {
+            parts = A.huge[nd.x].entries;
+            i = A.huge[nd.x].i;
+          }
           Cand best{0, -1};
           long long kia = 0;
           for (int t = lane; t < parts; t += 32) {
@@ -502,7 +623,7 @@ __global__ void __launch_bounds__(LV_THREADS, 2) k_lv_run(const __grid_constant_
           }
           warp_best(best);
           kia = warp_sum(kia);
-          lv_emit(A, words, lane == 0 && lv_moves(A, nd.x, kia, best), nd.x, best.c);
+          lv_emit(A, words, lane == 0 && lv_moves(A, i, kia, best), i, best.c);
         }
         if (!sync()) return;
       }
@@ -526,6 +647,8 @@ __global__ void __launch_bounds__(LV_THREADS, 2) k_lv_run(const __grid_constant_
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) A.res[LR_ROUNDS] = (unsigned long long)rounds;
 }
+
+using LvKernel = void (*)(LvArgs);
 
 size_t lv_smem(int S) {
   return (size_t)LV_BLOCK_SLOTS * 12 + (3 * (size_t)LV_CLASSES * S + 1) * sizeof(int32_t);
@@ -694,19 +817,23 @@ __global__ void k_lv_mark(const int32_t* __restrict__ comm, int32_t n, int32_t* 
 
 struct LvGraph {
   int64_t V = 0, E = 0;
+  int64_t slots = 0;  // of the class 5 tables of a sub-round
   DBuf<long long> off, aw, self, k;
   DBuf<int32_t> adj;
 };
 
-void lv_degrees(const Ctx& cx, LvGraph& g, long long* W2) {
+void lv_degrees(const Ctx& cx, LvGraph& g, uint64_t seed, int level, int S, long long* W2) {
   g.k.alloc(&cx.alloc, (size_t)std::max<int64_t>(g.V, 1));
-  DBuf<unsigned long long> tot;
-  tot.alloc(&cx.alloc, 1);
-  HG_CUDA(cudaMemsetAsync(tot.p, 0, sizeof(unsigned long long), cx.stream));
-  k_lv_degrees<<<grid_for(g.V, 8, cx.num_sms, 16), 256, 0, cx.stream>>>(g.off.p, g.aw.p, g.self.p,
-                                                                      g.V, g.k.p, tot.p);
+  DBuf<unsigned long long> sums;
+  sums.alloc(&cx.alloc, LD_SLOTS + (size_t)LV_ROUNDS * S);
+  HG_CUDA(cudaMemsetAsync(sums.p, 0, sums.bytes(), cx.stream));
+  k_lv_degrees<<<grid_for(g.V, 8, cx.num_sms, 16), 256, 0, cx.stream>>>(
+      g.off.p, g.aw.p, g.self.p, g.V, seed, level, S, g.k.p, sums.p);
   check_launch("lv_degrees");
-  *W2 = read_i64(cx, reinterpret_cast<const int64_t*>(tot.p));
+  unsigned long long h[LD_SLOTS];
+  read_back(cx, h, sums.p, sizeof(h));
+  *W2 = (long long)h[LD_TOTAL];
+  g.slots = (int64_t)h[LD_MOST];
 }
 
 // Aggregates the clustering cl of g into the next level's graph; cv[i] =
@@ -795,17 +922,27 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   k_lv_init<<<gV, 256, 0, cx.stream>>>(V, g.k.p, cl.p, vol.p);
   check_launch("lv_init");
   const size_t nkeys = (size_t)LV_CLASSES * S;
-  // a list entry per vertex, and one per further part of a large vertex
-  const size_t entries = (size_t)V + (size_t)(g.E / LV_PART) + 1;
+  // a list entry per vertex, and one per further part or chunk of a large vertex
+  const size_t entries = (size_t)V + (size_t)(g.E / std::min(LV_PART, LV_CHUNK)) + 1;
+  DBuf<HugeVertex> huge;
+  DBuf<int32_t> tkey;
+  DBuf<long long> tval;
+  huge.alloc(&cx.alloc, g.slots ? (size_t)(g.E / LV_HUGE) + 1 : 0);
+  tkey.alloc(&cx.alloc, (size_t)g.slots);
+  tval.alloc(&cx.alloc, (size_t)g.slots);
+  if (g.slots) {
+    HG_CUDA(cudaMemsetAsync(tkey.p, 0xff, tkey.bytes(), cx.stream));
+    HG_CUDA(cudaMemsetAsync(tval.p, 0, tval.bytes(), cx.stream));
+  }
   DBuf<int2> list, mv;
   DBuf<PartBest> parts;
-  DBuf<unsigned long long> zero;  // results, then 32-bit counters
+  DBuf<unsigned long long> zero;  // results, table slots given out, then 32-bit counters
   list.alloc(&cx.alloc, entries);
   mv.alloc(&cx.alloc, (size_t)V + 1);
   parts.alloc(&cx.alloc, entries);
-  zero.alloc(&cx.alloc, LR_LV_WORDS + nkeys + LV_WORDS + 1);
+  zero.alloc(&cx.alloc, LR_LV_WORDS + (size_t)S + nkeys + LV_WORDS + 1);
   HG_CUDA(cudaMemsetAsync(zero.p, 0, zero.bytes(), cx.stream));
-  int32_t* z = reinterpret_cast<int32_t*>(zero.p + LR_LV_WORDS);
+  int32_t* z = reinterpret_cast<int32_t*>(zero.p + LR_LV_WORDS + S);
   LvArgs A{};
   A.off = g.off.p;
   A.adj = g.adj.p;
@@ -823,18 +960,25 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   A.fill = z + nkeys;
   A.words = z + 2 * nkeys;
   A.barrier = reinterpret_cast<unsigned*>(z + 2 * nkeys + 2 * LV_WORDS);
+  A.nhuge = z + 2 * nkeys + 2 * LV_WORDS + 1;
+  A.tabfill = zero.p + LR_LV_WORDS;
+  A.huge = huge.p;
+  A.tkey = tkey.p;
+  A.tval = tval.p;
   A.mv = mv.p;
   A.parts = parts.p;
   A.res = zero.p;
   A.status = cx.d_status;
   static std::once_flag once;
   std::call_once(once, [] {
-    HG_CUDA(cudaFuncSetAttribute(k_lv_run, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)lv_smem(256)));
+    for (LvKernel f : {k_lv_run<false>, k_lv_run<true>})
+      HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)lv_smem(256)));
   });
+  const LvKernel kernel = g.slots ? k_lv_run<true> : k_lv_run<false>;
   const size_t smem = lv_smem(S);
   int per_sm = 0;
-  HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lv_run, LV_THREADS, smem));
+  HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, LV_THREADS, smem));
   if (per_sm < 1) throw HgError(HG_ERR_CUDA, "local moving does not fit an SM");
   // a block per 16 vertices or 256 edges of a sub-round (coarse levels: heavy
   // vertices take a block each); four times that, and at most half the chip, when
@@ -844,7 +988,7 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
       std::max<int64_t>(V / (S * 16 * share), g.E / (S * 256 * share)) + 1;
   const int blocks =
       (int)std::min<int64_t>(need, (int64_t)cx.num_sms * std::min(per_sm, share == 1 ? 2 : 1));
-  launch_persistent(cx, k_lv_run, blocks, LV_THREADS, smem, false, A);
+  launch_persistent(cx, kernel, blocks, LV_THREADS, smem, false, A);
   lc.launches += 1;
   unsigned long long hres[LR_LV_WORDS];
   read_back(cx, hres, A.res, sizeof(hres));
@@ -885,7 +1029,7 @@ int32_t detect_communities(const Ctx& cx, const Level& L, int S, uint64_t seed,
     check_launch("lv_net_edges");
   }
   long long W2 = 0;
-  lv_degrees(cx, g, &W2);
+  lv_degrees(cx, g, seed, 0, S, &W2);
   for (int level = 0; level < LV_LEVELS; ++level) {
     DBuf<int32_t> cl;
     const int64_t moves = lv_local_moving(cx, g, W2, S, seed, level, cl, lc);
@@ -899,7 +1043,7 @@ int32_t detect_communities(const Ctx& cx, const Level& L, int S, uint64_t seed,
     check_launch("lv_vmap");
     const bool shrank = next.V < g.V;
     long long W2n = 0;
-    lv_degrees(cx, next, &W2n);
+    lv_degrees(cx, next, seed, level + 1, S, &W2n);
     g = std::move(next);
     if (!shrank) break;
   }

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 
 import synth
+from tests.tiny import from_nets
 
 pytestmark = pytest.mark.gpu
 
@@ -87,3 +88,25 @@ def test_hook_blocks_of_any_alignment(oracle_mod, shift, graph, k):
     finally:
         hg.hg_destroy(h)
     assert not hooks.live
+
+
+@pytest.mark.parametrize("S", [1, 16])
+def test_louvain_hubs(oracle_mod, S):
+    """Net vertices around the degrees where a vertex is split into parts and into
+    chunks of its edges, and a node vertex above both."""
+    n = 60_000
+    rng = np.random.default_rng(S)
+    sizes = [4096, 4097, 32_767, 32_768, 32_769, 33_792, 33_793, 50_000]
+    nets = [rng.choice(n, size=s, replace=False).tolist() for s in sizes]
+    nets += [[7, int(v)] for v in rng.choice(np.arange(8, n), size=40_000, replace=False)]
+    nets += rng.integers(0, n // 2, size=(20_000, 1)).repeat(2, 1).__add__([0, n // 2]).tolist()
+    hgr = from_nets(n, nets, rng.integers(1, 9, size=len(nets)), None)
+    want, levels, moves = oracle_mod.communities(hgr, S=S, seed=2)
+    h = create(hgr, 2, S)
+    try:
+        hg.hg_detect_communities(h)
+        assert np.array_equal(hg.hg_get_communities(h, 0), want)
+        st = hg.hg_get_stats(h)
+        assert st["louvain_levels"] == levels and st["louvain_moves"] == moves
+    finally:
+        hg.hg_destroy(h)

@@ -56,3 +56,32 @@ def test_buffers_of_a_hook_start_on_a_32_byte_boundary(tmp_path):
       return 0;
     }
     """)
+
+
+def test_louvain_vertices_of_any_degree(tmp_path):
+    """Every edge of a vertex is covered by its list entries, read at most sixteen
+    times, and the entries' numbers stay positive up to the largest degree."""
+    hostcc.run(tmp_path, ["louvain.cuh"], """
+    using namespace hgk;
+    int main() {
+      std::vector<long long> degs = {1, 8, 9, 32, 33, 256, 257, 1 << 20, 1 << 26, (1 << 26) + 1,
+                                     100000000, (1ll << 31) - 1};
+      for (long long d : {4096ll, 32768ll, 33792ll})
+        for (long long x = -1; x <= 1; ++x) degs.push_back(d + x);
+      int last = 0;
+      std::sort(degs.begin(), degs.end());
+      for (long long d : degs) {
+        int32_t entries = 0;
+        const int cls = lv_class(d, entries);
+        CHECK(cls >= last && cls < LV_CLASSES && entries >= 1);
+        last = cls;
+        if (cls < 4) CHECK(entries == 1);
+        if (cls == 4) CHECK((long long)entries * LV_PART >= d && entries <= 16);
+        if (cls == 5) {
+          CHECK((long long)entries * LV_CHUNK >= d && (long long)(entries - 1) * LV_CHUNK < d);
+          CHECK(lv_slots(d) >= 2ull * d + 2 && (lv_slots(d) & (lv_slots(d) - 1)) == 0);
+        }
+      }
+      return 0;
+    }
+    """)
