@@ -596,6 +596,7 @@ __device__ void approve_contested(const ClusterArgs& A, int32_t* words, unsigned
     const int32_t cnt = R.gcnt[C];
     const int32_t off = A.slot_off[sl];
     const long long cap = (long long)R.c_max - R.cst[C].x;
+    if (threadIdx.x == 0) beat(A.barrier);
     long long added = 0;
     int32_t acc = 0;
     if (cnt <= GROUP_SMEM_CAP) {
@@ -644,6 +645,7 @@ __device__ void approve_contested(const ClusterArgs& A, int32_t* words, unsigned
       // large group: binary search for the first excluded key x, the largest
       // x with (sum of c over keys < x) <= cap; all keys < x are accepted
       unsigned long long lo = 0, hi = (1ull << 63);
+      BeatLoop work(A.barrier);
       while (hi - lo > 1) {
         const unsigned long long mid = lo + ((hi - lo) >> 1);
         long long f = 0;
@@ -651,6 +653,7 @@ __device__ void approve_contested(const ClusterArgs& A, int32_t* words, unsigned
           const int32_t u = A.glist[off + i];
           const unsigned long long kk = ((unsigned long long)(uint32_t)A.c[u] << 32) | (uint32_t)u;
           if (kk < mid) f += A.c[u];
+          work.trip();
         }
         f = block_sum(f, s_red);
         if (f <= cap) lo = mid; else hi = mid;
@@ -858,6 +861,7 @@ __device__ void refresh_huge(const ClusterArgs& A, const int2* list, int32_t cou
   const int32_t step = min((int32_t)gridDim.x, A.nets.bitmap_blocks);
   for (int32_t i = blockIdx.x; i < count; i += step) {
     const int2 net = list[i];
+    if (threadIdx.x == 0) beat(A.barrier);
     for (int turn = 0; turn < 2; ++turn) {
       for (int32_t q = threadIdx.x; q < net.y; q += RUN_THREADS) {
         const int2 r = A.rinfo[net.x + q];

@@ -794,7 +794,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   words.alloc(&cx.alloc, (size_t)S * CW_WORDS);
   clusters.alloc(&cx.alloc, 1);
   max_r.alloc(&cx.alloc, 3);  // largest possible rating, incidences of heavy nodes, total W
-  stats.alloc(&cx.alloc, (size_t)ST_TOTAL + 1);
+  stats.alloc(&cx.alloc, (size_t)ST_TOTAL + 1);  // then the barrier's two words
   rinfo.alloc(&cx.alloc, L.graph ? 1 : (size_t)std::max<int64_t>(L.p, 1));
   HG_CUDA(cudaMemsetAsync(gw.p, 0, gw.bytes(), cx.stream));
   HG_CUDA(cudaMemsetAsync(gcnt.p, 0, gcnt.bytes(), cx.stream));

@@ -242,7 +242,7 @@ struct LvArgs {
   int32_t* words;
   PartBest* parts;
   unsigned long long* res;
-  unsigned* barrier;
+  unsigned* barrier;  // two words (grid_sync)
   int32_t* status;
 };
 
@@ -940,7 +940,7 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   list.alloc(&cx.alloc, entries);
   mv.alloc(&cx.alloc, (size_t)V + 1);
   parts.alloc(&cx.alloc, entries);
-  zero.alloc(&cx.alloc, LR_LV_WORDS + (size_t)S + nkeys + LV_WORDS + 1);
+  zero.alloc(&cx.alloc, LR_LV_WORDS + (size_t)S + nkeys + LV_WORDS + 2);
   HG_CUDA(cudaMemsetAsync(zero.p, 0, zero.bytes(), cx.stream));
   int32_t* z = reinterpret_cast<int32_t*>(zero.p + LR_LV_WORDS + S);
   LvArgs A{};
@@ -960,7 +960,7 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   A.fill = z + nkeys;
   A.words = z + 2 * nkeys;
   A.barrier = reinterpret_cast<unsigned*>(z + 2 * nkeys + 2 * LV_WORDS);
-  A.nhuge = z + 2 * nkeys + 2 * LV_WORDS + 1;
+  A.nhuge = z + 2 * nkeys + 2 * LV_WORDS + 2;
   A.tabfill = zero.p + LR_LV_WORDS;
   A.huge = huge.p;
   A.tkey = tkey.p;

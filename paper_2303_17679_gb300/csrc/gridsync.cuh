@@ -5,18 +5,56 @@
 
 namespace hgk {
 
-constexpr int SPIN_LIMIT = 1 << 24;  // polls of one grid barrier (seconds)
+// Polls of a grid barrier without progress of the blocks it waits for (some ten
+// seconds).
+constexpr int SPIN_LIMIT = 1 << 24;
+
+// The polls a wait may still spend: `limit` since the progress word last changed.
+// The word counts units of work done by blocks that others may wait for long (a
+// sort of millions of moves, a group of as many movers), so such a wait lasts as
+// long as they work, and ends when nothing moves.
+struct WaitBudget {
+  int limit, polls = 0;
+  unsigned seen = 0;
+  __host__ __device__ explicit WaitBudget(int l) : limit(l) {}
+  template <typename Progress>
+  __host__ __device__ bool again(Progress&& progress) {
+    if (++polls < limit) return true;
+    const unsigned now = progress();
+    if (now == seen) return false;
+    seen = now;
+    polls = 0;
+    return true;
+  }
+};
+
+// One thread of a block reports that the block got on with a long phase.
+__device__ __forceinline__ void beat(unsigned* barrier) {
+  asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(barrier + 1) : "memory");
+}
+
+// Reports every 256th trip of a block's loop (a few hundred microseconds of
+// dependent accesses).
+struct BeatLoop {
+  unsigned* barrier;
+  int trips = 0;
+  __device__ __forceinline__ explicit BeatLoop(unsigned* b) : barrier(b) {}
+  __device__ __forceinline__ void trip() {
+    if ((++trips & 255) == 0 && threadIdx.x == 0) beat(barrier);
+  }
+};
 
 // cluster: the blocks are one thread-block cluster (hardware barrier, 0.35 to
-// 0.5 us); else they were launched cooperatively and count arrivals in
-// `counter` (zero at the launch; 1.4 us over 152 blocks).  `gen` counts the
-// barriers passed.  Returns false when a grid barrier gave up: the status
-// word is set and every thread of the block returns from the kernel.  The
+// 0.5 us, which waits until they arrive); else they were launched cooperatively
+// and count arrivals in barrier[0], with the progress word in barrier[1] (both
+// zero at the launch; 1.4 us over 152 blocks).  `gen` counts the barriers passed.
+// Returns false when a grid barrier gave up: the status word is set and every
+// thread of the block returns from the kernel.  The
 // release and acquire of the barrier itself order everything the block has
 // written and read; a fence of the device in front of them cost 4 ms of the 52 ms
 // coarsening of 1e6 Zipf nodes.
-__device__ __forceinline__ bool grid_sync(bool cluster, unsigned* counter, int32_t* status,
-                                          unsigned& gen) {
+__device__ __forceinline__ bool grid_sync(bool cluster, unsigned* barrier, int32_t* status,
+                                          unsigned& gen, int limit = SPIN_LIMIT) {
   if (cluster) {
     // not the .aligned form: callers come from loops that lanes leave at
     // different times, and nothing makes the compiler rejoin them first
@@ -30,12 +68,17 @@ __device__ __forceinline__ bool grid_sync(bool cluster, unsigned* counter, int32
   bool ok = true;
   if (threadIdx.x == 0) {
     const unsigned target = gen * gridDim.x;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
-    int polls = 0;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(barrier) : "memory");
+    WaitBudget budget(limit);
+    auto progress = [&]() {
+      unsigned p;
+      asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(p) : "l"(barrier + 1) : "memory");
+      return p;
+    };
     unsigned v;
     do {
-      asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-    } while ((int)(v - target) < 0 && ++polls < SPIN_LIMIT);
+      asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(barrier) : "memory");
+    } while ((int)(v - target) < 0 && budget.again(progress));
     ok = (int)(v - target) >= 0;
     if (!ok) dev_fail(status, DEV_TIMEOUT);
   }

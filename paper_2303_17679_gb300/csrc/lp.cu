@@ -97,7 +97,7 @@ struct LpArgs {
   int sel_cap;
   unsigned long long* gkeys;
   int32_t* gpre;
-  unsigned* barrier;
+  unsigned* barrier;       // two words (grid_sync)
   unsigned long long* res;
   int32_t* status;
 };
@@ -648,14 +648,16 @@ __device__ __forceinline__ void rank_sort2(const unsigned long long* a, int na,
 
 // Bitonic sorts of the two directions of a pair (Pa and Pb powers of two) by
 // the block, stage by stage together.
-__device__ void bitonic_sort2(unsigned long long* a, int Pa, unsigned long long* b, int Pb) {
+__device__ void bitonic_sort2(unsigned long long* a, int Pa, unsigned long long* b, int Pb,
+                              BeatLoop& work) {
   const int P = Pa > Pb ? Pa : Pb;
   for (int kk = 2; kk <= P; kk <<= 1) {
     for (int j = kk >> 1; j > 0; j >>= 1) {
-      for (int x = threadIdx.x; x < Pa + Pb; x += LP_THREADS) {
-        unsigned long long* buf = x < Pa ? a : b;
-        const int i = x < Pa ? x : x - Pa;
-        const int n = x < Pa ? Pa : Pb;
+      for (int64_t y = threadIdx.x; y < (int64_t)Pa + Pb; y += LP_THREADS) {
+        work.trip();
+        unsigned long long* buf = y < Pa ? a : b;
+        const int i = (int)(y < Pa ? y : y - Pa);
+        const int n = y < Pa ? Pa : Pb;
         if (kk > n) continue;
         const int ixj = i ^ j;
         if (ixj > i) {
@@ -676,7 +678,8 @@ __device__ void bitonic_sort2(unsigned long long* a, int Pa, unsigned long long*
 // concatenation of their sorted moves: A[x] = weight of the first x moves
 // a -> b (x = 0..na), B[x] likewise for b -> a.
 __device__ void weight_prefix2(const unsigned long long* ka, int na, const unsigned long long* kb,
-                               int nb, const int32_t* __restrict__ c, int32_t* A, int32_t* B) {
+                               int nb, const int32_t* __restrict__ c, int32_t* A, int32_t* B,
+                               BeatLoop& work) {
   __shared__ int32_t s_sum[LP_WARPS];
   __shared__ int32_t s_total_a;
   const int cnt = na + nb;
@@ -688,6 +691,7 @@ __device__ void weight_prefix2(const unsigned long long* ka, int na, const unsig
   }
   __syncthreads();
   for (int base = 0; base < cnt; base += LP_THREADS) {
+    work.trip();
     const int x = base + threadIdx.x;
     int32_t v = 0;
     if (x < na) v = __ldg(c + (int32_t)(uint32_t)ka[x]);
@@ -717,6 +721,7 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
                              const long long* s_slack, unsigned char* smem) {
   __shared__ int s_red[2];
   const int cap = P.sel_cap, k = P.k;
+  BeatLoop work(P.barrier);
   const int dab = a * k + b, dba = b * k + a;
   unsigned long long* s_keys0 = reinterpret_cast<unsigned long long*>(smem);
   unsigned long long* s_keys1 = s_keys0 + cap;
@@ -768,6 +773,7 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
   if (na > la || nb > lb) {
     const int32_t no = __ldcg(P.words + par * SW_WORDS + SW_OVERFLOW);
     for (int32_t i = threadIdx.x; i < no; i += LP_THREADS) {
+      work.trip();
       const int32_t d = __ldcg(P.ovf_dir + i);
       if (d == dab) ka[la + atomicAdd(&s_red[0], 1)] = __ldcg(P.ovf_key + i);
       else if (d == dba) kb[lb + atomicAdd(&s_red[1], 1)] = __ldcg(P.ovf_key + i);
@@ -782,9 +788,9 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
     for (int i = na + threadIdx.x; i < Pa; i += LP_THREADS) ka[i] = ~0ull;
     for (int i = nb + threadIdx.x; i < Pb; i += LP_THREADS) kb[i] = ~0ull;
     __syncthreads();
-    bitonic_sort2(ka, Pa, kb, Pb);
+    bitonic_sort2(ka, Pa, kb, Pb, work);
   }
-  weight_prefix2(ka, na, kb, nb, P.c, A, B);
+  weight_prefix2(ka, na, kb, nb, P.c, A, B, work);
   if (threadIdx.x == 0) s_red[0] = 0;
   __syncthreads();
   // diagonal r: i(r) = number of A steps among the first r
@@ -800,6 +806,7 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
   const long long lo = -s_slack[a], hi = s_slack[b];
   int best = 0;
   for (int r = threadIdx.x; r <= na + nb; r += LP_THREADS) {
+    work.trip();
     const int i = steps(r);
     const long long x = (long long)A[i] - B[r - i];
     if (lo <= x && x <= hi) best = r > best ? r : best;
@@ -811,6 +818,7 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
   const int ta = steps(r), tb = r - ta;
   int32_t incid = 0;
   for (int i0 = 32 * warp_in_block(); i0 < ta + tb; i0 += LP_THREADS) {
+    work.trip();
     const int i = i0 + lane_id();
     const bool from_a = i < ta;
     int32_t u = 0;

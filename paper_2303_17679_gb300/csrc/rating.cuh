@@ -576,7 +576,7 @@ struct ClusterArgs {
   int2* rinfo;
   int64_t p;
   NetLists nets;
-  unsigned* barrier;
+  unsigned* barrier;  // two words (grid_sync)
 };
 
 // Runs the S sub-rounds of a level (cluster.cu).  `listed` nodes, `heavy` of

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 
 import synth
+from tests import hostcc
 from tests.tiny import from_nets
 
 pytestmark = pytest.mark.gpu
@@ -110,3 +111,36 @@ def test_louvain_hubs(oracle_mod, S):
         assert st["louvain_levels"] == levels and st["louvain_moves"] == moves
     finally:
         hg.hg_destroy(h)
+
+
+# A barrier of two blocks with a short limit.  late: block 1 arrives after about
+# 50 ms, reporting its progress or not; never: it leaves without arriving.
+@pytest.mark.parametrize("late,beats,passes", [(0, 0, 1), (1, 1, 1), (1, 0, 0), (2, 0, 0)])
+def test_barrier_gives_up_on_lack_of_progress(tmp_path, late, beats, passes):
+    hostcc.run(tmp_path, ["gridsync.cuh"], f"""
+    using namespace hgk;
+    __global__ void k_wait(unsigned* barrier, int32_t* status, int32_t* passed) {{
+      unsigned gen = 0;
+      if (blockIdx.x == 1) {{
+        if ({late} == 2) return;
+        const unsigned long long t0 = now_ns();
+        for (int i = 0; {late} == 1 && i < 1 << 20 && now_ns() - t0 < 50000000ull; ++i) {{
+          __nanosleep(1000);
+          if ({beats} && threadIdx.x == 0) beat(barrier);
+        }}
+      }}
+      if (!grid_sync(false, barrier, status, gen, 1 << 12)) return;
+      if (blockIdx.x == 0 && threadIdx.x == 0) *passed = 1;
+    }}
+    int main() {{
+      int32_t* d = nullptr;
+      CHECK(cudaMalloc(&d, 16) == cudaSuccess && cudaMemset(d, 0, 16) == cudaSuccess);
+      Ctx cx;
+      launch_persistent(cx, k_wait, 2, 64, 0, false, (unsigned*)d, d + 2, d + 3);
+      int32_t h[4];
+      CHECK(cudaMemcpy(h, d, 16, cudaMemcpyDeviceToHost) == cudaSuccess);
+      CHECK(h[3] == {passes});
+      CHECK(h[2] == ({passes} ? DEV_OK : DEV_TIMEOUT));
+      return 0;
+    }}
+    """)

@@ -85,3 +85,27 @@ def test_louvain_vertices_of_any_degree(tmp_path):
       return 0;
     }
     """)
+
+
+def test_a_wait_lasts_while_the_others_get_on(tmp_path):
+    """Blocks may wait for one that sorts tens of millions of moves, so a barrier
+    gives up on lack of progress, not after a number of polls."""
+    hostcc.run(tmp_path, ["gridsync.cuh"], """
+    using namespace hgk;
+    int main() {
+      WaitBudget still(100);
+      int polls = 1;
+      while (still.again([] { return 0u; })) ++polls;
+      CHECK(polls == 100);
+      WaitBudget busy(100);
+      unsigned done = 0;
+      polls = 0;
+      while (polls < 100000 && busy.again([&] { return done; }))
+        if (++polls % 90 == 0) ++done;
+      CHECK(polls == 100000);
+      polls = 0;  // and then it stops
+      while (busy.again([&] { return done; })) ++polls;
+      CHECK(polls < 200);
+      return 0;
+    }
+    """)
