@@ -22,7 +22,9 @@
  *  - Streams: all work is issued on the stream given to hg_create, in
  *    stream order.  Entry points that return host scalars synchronize that
  *    stream before returning.  One handle must not be used from two host
- *    threads at once.
+ *    threads at once.  Calls of several handles that run at the same time on one
+ *    device overlap there: while there are others, a call's kernels take at most
+ *    half the SMs.
  *  - Errors: HG_ERR_INVALID for malformed arguments (nothing is changed),
  *    HG_ERR_UNSUPPORTED for sizes outside the supported range, HG_ERR_OOM
  *    when device memory runs out, HG_ERR_CUDA for a CUDA error (sticky: the
@@ -104,9 +106,8 @@ typedef struct {
   int32_t lp_block_min_deg;
   /* 1: wait for the device by sleeping on a blocking-sync event instead of
    * spinning (frees the host core while waiting, at a few microseconds of
-   * wake-up latency per wait; the executor sets it for its jobs).  Such a
-   * handle is taken to share the GPU with others: the kernels that run a whole
-   * level use at most half the SMs.  0 (default): spin. */
+   * wake-up latency per wait; the executor sets it for its jobs).  0 (default):
+   * spin. */
   int32_t blocking_sync;
   /* Graph path (Sec. 10): 0 (default) = a level whose nets all have exactly
    * two pins is kept as a graph with one adjacency array (the other endpoint

@@ -17,6 +17,7 @@ struct hg_t {
   hgk::Ctx cx;
   hg_options opt;
   int device = 0;
+  int depth = 0;             // of the calls at work (CallScope)
   int64_t W0 = 0;            // total node weight c(V), invariant under contraction
   bool finished = false;     // the last coarsening step shrank by < 1 %
   int sticky = 0;            // HG_ERR_CUDA once a CUDA error was seen
@@ -32,7 +33,9 @@ template <typename F>
 int guarded(hg_t* h, F&& body) {
   if (h && h->sticky) return h->sticky;
   try {
-    if (h) cudaSetDevice(h->device);
+    if (!h) return body();
+    cudaSetDevice(h->device);
+    const hgk::CallScope scope(h->device, h->depth);
     return body();
   } catch (const HgError& e) {
     if (h && (e.code == HG_ERR_CUDA)) h->sticky = HG_ERR_CUDA;
@@ -216,6 +219,8 @@ int hg_create(int32_t n, int32_t m, const int32_t* net_offsets, const int32_t* p
   h->opt = o;
   const int rc = guarded(nullptr, [&]() -> int {
     HG_CUDA(cudaGetDevice(&h->device));
+    const hgk::CallScope scope(h->device, h->depth);
+    h->cx.device = h->device;
     int sms = 0;
     HG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     h->cx.num_sms = sms;
@@ -524,6 +529,7 @@ int hg_partition(hg_t* h, int32_t k, int32_t eps_ppm, int32_t max_passes, int32_
   if (!h || !part) return HG_ERR_INVALID;
   if (k < 2 || k > HG_MAX_K || eps_ppm < 0 || max_passes < 0) return HG_ERR_INVALID;
   if (h->sticky) return h->sticky;
+  const hgk::CallScope scope(h->device, h->depth);
   int rc;
   if (h->opt.community_detection && h->levels.size() == 1 && !h->levels[0]->comm.p) {
     rc = hg_detect_communities(h, nullptr);

@@ -1011,15 +1011,15 @@ void run_subrounds(const Ctx& cx, ClusterArgs A, bool narrow, bool graph, size_t
   });
   // Blocks of a sub-round's work: one light node per warp, four heavy ones per
   // block, 256 visits per warp, 16 records per thread.  Up to 16 blocks run as
-  // one cluster, above that one block per SM.  A handle that shares the GPU
-  // with others (it sleeps while it waits) takes a quarter of that and at most
-  // half the SMs, so that several levels are resident at once: a block fills an
-  // SM, and a cooperative kernel for the whole chip waits until every other one
-  // has left it.  Serving 200 requests per second of 1e4 to 2e6 pins on 16
-  // streams: p50 / p99 664 / 1420 ms without the limit, 25 / 105 ms with it, 21 /
-  // 83 ms with a quarter of the SMs; but a request alone then takes 148 instead of
-  // 97 ms (1e6 Zipf nodes).  As separate launches: 56 / 230 ms, 109 ms alone.
-  const int64_t S = A.S, share = cx.sync_event ? 4 : 1;
+  // one cluster, above that one block per SM.  A call that shares the GPU with
+  // others (inflight.cuh) takes a quarter of that and at most half the SMs, so that
+  // several levels are resident at once.  Serving 200 requests per second of 1e4
+  // to 2e6 pins on 16 streams: p50 / p99 664 / 1420 ms without the limit, 25 / 112
+  // ms with it, 21 / 83 ms with a quarter of the SMs, which a large request on two
+  // streams pays for; as separate launches 56 / 230 ms.  Eight host threads with
+  // plain handles (20,000 nodes, k = 32): 224 -> 459 partitions per second with
+  // the limit (319 as separate launches), one thread 113.
+  const int64_t S = A.S, share = cx.shares_gpu() ? 4 : 1;
   const int64_t need =
       std::max<int64_t>({(listed - heavy) / (S * RUN_WARPS), heavy / (S * 4),
                          total_visits / (S * RUN_WARPS * 256), A.p / (RUN_THREADS * 16)}) /

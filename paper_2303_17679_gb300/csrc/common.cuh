@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/hg.h"
+#include "inflight.cuh"
 
 namespace hgk {
 
@@ -251,6 +252,7 @@ struct DBuf {
 
 struct Ctx {
   Alloc alloc;
+  int device = 0;
   cudaStream_t stream = nullptr;
   int32_t* d_status = nullptr;   // device status word (DevStatus)
   int num_sms = 0;
@@ -258,6 +260,10 @@ struct Ctx {
   bool timing = false;           // per-phase event timing (synchronizes at phase ends)
   bool kernel_timing = false;    // event pair around every rating / gain launch (no sync)
   cudaEvent_t sync_event = nullptr;  // blocking-sync event: waits sleep instead of spinning
+  // Another call is at work on the device (inflight.cuh).
+  bool shares_gpu() const {
+    return calls_in_flight(device).load(std::memory_order_relaxed) > 1;
+  }
 };
 
 // Grid size helper: enough blocks for `work` items of `per_block` each,

@@ -982,8 +982,8 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   if (per_sm < 1) throw HgError(HG_ERR_CUDA, "local moving does not fit an SM");
   // a block per 16 vertices or 256 edges of a sub-round (coarse levels: heavy
   // vertices take a block each); four times that, and at most half the chip, when
-  // the handle shares the GPU with others (it sleeps while it waits)
-  const int64_t share = cx.sync_event ? 4 : 1;
+  // the call shares the GPU with others (inflight.cuh)
+  const int64_t share = cx.shares_gpu() ? 4 : 1;
   const int64_t need =
       std::max<int64_t>(V / (S * 16 * share), g.E / (S * 256 * share)) + 1;
   const int blocks =

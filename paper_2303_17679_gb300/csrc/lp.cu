@@ -1168,13 +1168,13 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
   // takes 14 us for the best moves of 58,000 incidences, the grid 6.  Of the
   // cluster sizes the largest that has work for every block is best: a sub-round
   // of 92 nodes takes 7.5 us in one block, 6 us in 16.  Larger levels spread over
-  // the chip, two blocks per SM when there is work for them.  A handle that
-  // shares the GPU with others (it sleeps while it waits) takes no more blocks
-  // than its work fills, a lane group per node and eight incidences per thread,
+  // the chip, two blocks per SM when there is work for them.  A call that
+  // shares the GPU with others (inflight.cuh) takes no more blocks than its work
+  // fills, a lane group per node and eight incidences per thread,
   // and at most half the chip (see run_subrounds in cluster.cu).
   const LpKernel kernel = lp_kernel(L.graph, k);
   const size_t bytes = lp_smem_bytes(k);
-  const bool shared = cx.sync_event != nullptr;
+  const bool shared = cx.shares_gpu();
   auto blocks_for = [&](int64_t nodes, int64_t inc) {
     return std::max<int64_t>({nodes_sr / nodes + 1, inc_sr / inc + 1, (int64_t)k * (k - 1) / 256 + 1});
   };

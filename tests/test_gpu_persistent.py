@@ -1,7 +1,7 @@
 """The persistent kernels on the GPU: barriers behind loops that the lanes of a
 warp leave at different times, and what the launch rules decide.  All results are
 integers and compared exactly with the oracle."""
-import ctypes
+import threading
 
 import numpy as np
 import pytest
@@ -144,3 +144,36 @@ def test_barrier_gives_up_on_lack_of_progress(tmp_path, late, beats, passes):
       return 0;
     }}
     """)
+
+
+def test_plain_handles_at_once(oracle_mod):
+    """Levels of every launch form from several host threads, each result that of
+    the call alone."""
+    jobs = [(synth.zipf_preferential(i, n, n), k) for i, (n, k) in
+            enumerate([(1500, 2), (9000, 40), (30_000, 8), (60_000, 4)])]
+    want = [oracle_mod.multilevel(g, k, 30000, S=16, factor=20, seed=5, max_passes=2)
+            for g, k in jobs]
+    got = [None] * len(jobs)
+
+    def work(i):
+        g, k = jobs[i]
+        o = hg.hg_default_options()
+        o.seed, o.contraction_limit_factor, o.blocking_sync = 5, 20, i % 2
+        st = torch.cuda.Stream()
+        for _ in range(6):
+            part = torch.empty(g.n, dtype=torch.int32, device="cuda")
+            st.wait_stream(torch.cuda.default_stream())
+            h = hg.hg_create(g.n, g.m, g.offsets, g.pins, g.net_w, g.node_w, hg.HG_MEM_HOST, o, st)
+            try:
+                obj = hg.hg_partition(h, k, 30000, 2, part)
+            finally:
+                hg.hg_destroy(h)
+            same = np.array_equal(part.cpu().numpy(), want[i].parts[0])
+            got[i] = (obj, same) if got[i] in (None, (obj, same)) else "differs"
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert got == [(w.objectives[0], True) for w in want]

@@ -109,3 +109,40 @@ def test_a_wait_lasts_while_the_others_get_on(tmp_path):
       return 0;
     }
     """)
+
+
+def test_calls_in_flight(tmp_path):
+    """Every call counts once, whatever it calls in turn, on its own device."""
+    hostcc.run(tmp_path, ["inflight.cuh"], """
+    using namespace hgk;
+    int main() {
+      int a = 0, b = 0, c = 0;
+      {
+        CallScope outer(0, a);
+        CallScope inner(0, a);
+        CHECK(calls_in_flight(0) == 1);
+        CallScope other(0, b), elsewhere(1, c);
+        CHECK(calls_in_flight(0) == 2 && calls_in_flight(1) == 1);
+      }
+      CHECK(calls_in_flight(0) == 0 && calls_in_flight(1) == 0 && a == 0);
+      std::vector<std::thread> t;
+      for (int i = 0; i < 8; ++i)
+        t.emplace_back([] {
+          int depth = 0;
+          for (int x = 0; x < 10000; ++x) {
+            CallScope s(0, depth);
+            if (calls_in_flight(0) < 1) std::abort();
+          }
+        });
+      for (auto& x : t) x.join();
+      CHECK(calls_in_flight(0) == 0);
+      return 0;
+    }
+    """)
+
+
+def test_kernels_of_a_level_are_sized_by_the_calls_in_flight():
+    """Not by how a handle waits: plain handles that run at once share the GPU too,
+    and one that sleeps alone has all of it."""
+    for name in ("cluster.cu", "lp.cu", "community.cu"):
+        assert "shares_gpu()" in source(name) and "sync_event" not in source(name), name
