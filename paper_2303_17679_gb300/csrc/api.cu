@@ -18,6 +18,7 @@ struct hg_t {
   hg_options opt;
   int device = 0;
   int depth = 0;             // of the calls at work (CallScope)
+  hgk::PreparedKernels prepared;
   int64_t W0 = 0;            // total node weight c(V), invariant under contraction
   bool finished = false;     // the last coarsening step shrank by < 1 %
   int sticky = 0;            // HG_ERR_CUDA once a CUDA error was seen
@@ -221,6 +222,7 @@ int hg_create(int32_t n, int32_t m, const int32_t* net_offsets, const int32_t* p
     HG_CUDA(cudaGetDevice(&h->device));
     const hgk::CallScope scope(h->device, h->depth);
     h->cx.device = h->device;
+    h->cx.prepared = &h->prepared;
     int sms = 0;
     HG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     h->cx.num_sms = sms;

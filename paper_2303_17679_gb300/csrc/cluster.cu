@@ -18,7 +18,6 @@
 // 500,009 nodes 10.8 -> 7.2 -> 6.5 ms; of 1471 nodes 1.67 -> 1.2 -> 1.09 ms.
 #include <algorithm>
 #include <climits>
-#include <mutex>
 #include <type_traits>
 
 #include "gridsync.cuh"
@@ -986,12 +985,12 @@ k_cluster_run(const __grid_constant__ ClusterArgs A) {
 }
 
 template <typename VT, bool GRAPH>
-void run_attributes() {
-  const void* f = reinterpret_cast<const void*>(&k_cluster_run<VT, GRAPH>);
-  HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)std::max({part_bytes<VT>(), TEAM_SMEM<VT>, DENSE_SMEM + 64,
-                                              sizeof(JoinSet) * RUN_WARPS})));
-  HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+void launch_run(const Ctx& cx, const ClusterArgs& A, int blocks, size_t smem) {
+  prepare_kernel(cx, &k_cluster_run<VT, GRAPH>,
+                 std::max({part_bytes<VT>(), TEAM_SMEM<VT>, DENSE_SMEM + 64,
+                           sizeof(JoinSet) * RUN_WARPS}),
+                 true);
+  launch_persistent(cx, k_cluster_run<VT, GRAPH>, blocks, RUN_THREADS, smem, A.cluster, A);
 }
 
 constexpr int CLUSTER_MAX = 16;
@@ -1000,15 +999,6 @@ constexpr int CLUSTER_MAX = 16;
 
 void run_subrounds(const Ctx& cx, ClusterArgs A, bool narrow, bool graph, size_t smem,
                    int64_t listed, int64_t heavy, int64_t total_visits) {
-  // Attributes belong to the functions: set once per process, also when
-  // several handles rate concurrently from different host threads.
-  static std::once_flag once;
-  std::call_once(once, [] {
-    run_attributes<uint32_t, false>();
-    run_attributes<uint32_t, true>();
-    run_attributes<unsigned long long, false>();
-    run_attributes<unsigned long long, true>();
-  });
   // Blocks of a sub-round's work: one light node per warp, four heavy ones per
   // block, 256 visits per warp, 16 records per thread.  Up to 16 blocks run as
   // one cluster, above that one block per SM.  A call that shares the GPU with
@@ -1032,20 +1022,10 @@ void run_subrounds(const Ctx& cx, ClusterArgs A, bool narrow, bool graph, size_t
     blocks = 1;
     while (blocks < need) blocks <<= 1;
   }
-  if (graph) {
-    if (narrow)
-      launch_persistent(cx, k_cluster_run<uint32_t, true>, blocks, RUN_THREADS, smem, A.cluster, A);
-    else
-      launch_persistent(cx, k_cluster_run<unsigned long long, true>, blocks, RUN_THREADS, smem,
-                        A.cluster, A);
-  } else {
-    if (narrow)
-      launch_persistent(cx, k_cluster_run<uint32_t, false>, blocks, RUN_THREADS, smem, A.cluster,
-                        A);
-    else
-      launch_persistent(cx, k_cluster_run<unsigned long long, false>, blocks, RUN_THREADS, smem,
-                        A.cluster, A);
-  }
+  if (graph && narrow) launch_run<uint32_t, true>(cx, A, blocks, smem);
+  else if (graph) launch_run<unsigned long long, true>(cx, A, blocks, smem);
+  else if (narrow) launch_run<uint32_t, false>(cx, A, blocks, smem);
+  else launch_run<unsigned long long, false>(cx, A, blocks, smem);
 }
 
 }  // namespace hgk

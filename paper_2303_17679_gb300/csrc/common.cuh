@@ -250,9 +250,27 @@ struct DBuf {
 
 // ------------------------------------------------------------- context
 
+// Attributes of a function belong to the device (and its context), so every handle
+// sets those of the kernels it launches, each once (a few microseconds); nothing
+// about them is kept per process.
+class PreparedKernels {
+ public:
+  template <typename Set>
+  void once(const void* kernel, Set&& set) {
+    for (const void* k : done_)
+      if (k == kernel) return;
+    set();
+    done_.push_back(kernel);
+  }
+
+ private:
+  std::vector<const void*> done_;
+};
+
 struct Ctx {
   Alloc alloc;
   int device = 0;
+  PreparedKernels* prepared = nullptr;  // of the handle
   cudaStream_t stream = nullptr;
   int32_t* d_status = nullptr;   // device status word (DevStatus)
   int num_sms = 0;
@@ -280,6 +298,18 @@ inline void check_launch(const char* what) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)
     throw HgError(HG_ERR_CUDA, std::string("launch ") + what + ": " + cudaGetErrorString(e));
+}
+
+// Before a launch with up to max_smem bytes of dynamic shared memory (and, when
+// wide_cluster is set, up to 16 blocks per cluster).
+template <typename K>
+void prepare_kernel(const Ctx& cx, K* kernel, size_t max_smem, bool wide_cluster = false) {
+  const void* f = reinterpret_cast<const void*>(kernel);
+  cx.prepared->once(f, [&] {
+    HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem));
+    if (wide_cluster)
+      HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  });
 }
 
 // ------------------------------------------------------------- levels

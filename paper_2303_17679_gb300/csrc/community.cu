@@ -40,7 +40,6 @@
 // copy of all table offsets per round, the detection on 250,007 nodes and
 // 1.35M pins took 30.1 ms, now 16.1 ms.
 #include <algorithm>
-#include <mutex>
 
 #include "gridsync.cuh"
 #include "louvain.cuh"
@@ -969,14 +968,9 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   A.parts = parts.p;
   A.res = zero.p;
   A.status = cx.d_status;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    for (LvKernel f : {k_lv_run<false>, k_lv_run<true>})
-      HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)lv_smem(256)));
-  });
   const LvKernel kernel = g.slots ? k_lv_run<true> : k_lv_run<false>;
   const size_t smem = lv_smem(S);
+  prepare_kernel(cx, kernel, lv_smem(256));
   int per_sm = 0;
   HG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, LV_THREADS, smem));
   if (per_sm < 1) throw HgError(HG_ERR_CUDA, "local moving does not fit an SM");

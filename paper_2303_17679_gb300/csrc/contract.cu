@@ -14,7 +14,6 @@
 //       sums over a keep flag and the kept sizes, then the incidence lists.
 #include <algorithm>
 #include <climits>
-#include <mutex>
 
 #include "common.cuh"
 
@@ -861,12 +860,7 @@ void contract_level(const Ctx& cx, Level& L, const int32_t* cw, Level& out, int 
   if (n2 <= BLOCK_BITMAP_N) {
     const size_t bytes = ((size_t)words + words / 32 + 1) * sizeof(unsigned);
     const int per_sm = std::max(1, std::min(4, (int)(200 * 1024 / bytes)));
-    static std::once_flag once;
-    std::call_once(once, [] {
-      HG_CUDA(cudaFuncSetAttribute(k_remap_block_bitmap,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (BLOCK_BITMAP_N / 32 + BLOCK_BITMAP_N / 1024 + 1) * 4));
-    });
+    prepare_kernel(cx, k_remap_block_bitmap, (BLOCK_BITMAP_N / 32 + BLOCK_BITMAP_N / 1024 + 1) * 4);
     for (int c = 2; c < NCLS; ++c)
       if (hc[c])
         k_remap_block_bitmap<<<grid_for(hc[c], 1, cx.num_sms, per_sm), BIG_THREADS, bytes,

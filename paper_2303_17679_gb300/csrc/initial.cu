@@ -11,7 +11,6 @@
 // sort and a scan of k weights per node: 26 ms at n = 262,725, k = 64 (device:
 // 7.2 ms), 0.33 ms at n = 4445, k = 32 (0.16 ms).
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 
@@ -184,11 +183,7 @@ void initial_partition(const Ctx& cx, const Level& L, int k, uint64_t seed, int3
   const int32_t n = L.n;
   if (n <= 0) return;
   if (n <= INIT_SMALL) {
-    static std::once_flag once;
-    std::call_once(once, [] {
-      HG_CUDA(cudaFuncSetAttribute(k_init_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)INIT_SMEM));
-    });
+    prepare_kernel(cx, k_init_small, INIT_SMEM);
     k_init_small<<<1, INIT_THREADS, INIT_SMEM, cx.stream>>>(L.c.p, n, seed, k, part);
     check_launch("init_small");
     if (cx.launches) *cx.launches += 1;

@@ -26,7 +26,6 @@
 // adj, node weights) is constant and read through the read-only path.
 #include <algorithm>
 #include <climits>
-#include <mutex>
 
 #include "gain.cuh"
 #include "gridsync.cuh"
@@ -1057,16 +1056,6 @@ size_t lp_smem_bytes(int k) { return select_bytes(sel_cap_for(k)); }
 
 constexpr int CLUSTER_MAX = 16;
 
-void lp_attributes_once() {
-  for (bool graph : {false, true})
-    for (int k : {8, 16, 32, 64}) {
-      const void* f = reinterpret_cast<const void*>(lp_kernel(graph, k));
-      HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)lp_smem_bytes(k)));
-      HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    }
-}
-
 }  // namespace
 
 LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, int eps_ppm,
@@ -1160,8 +1149,6 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
   A.gpre = gpre.p;
   A.status = cx.d_status;
 
-  static std::once_flag once;
-  std::call_once(once, lp_attributes_once);
   // Blocks.  Small levels run as one cluster (its barrier is three times faster
   // than the grid's): those with at most a lane group per node and two
   // incidences per thread in 16 blocks; with more (eight per thread) the cluster
@@ -1174,6 +1161,7 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
   // and at most half the chip (see run_subrounds in cluster.cu).
   const LpKernel kernel = lp_kernel(L.graph, k);
   const size_t bytes = lp_smem_bytes(k);
+  prepare_kernel(cx, kernel, bytes, true);
   const bool shared = cx.shares_gpu();
   auto blocks_for = [&](int64_t nodes, int64_t inc) {
     return std::max<int64_t>({nodes_sr / nodes + 1, inc_sr / inc + 1, (int64_t)k * (k - 1) / 256 + 1});

@@ -3,7 +3,6 @@
 // Algorithm"), the single adjacency array of graph levels (Sec. 10, "Graph
 // Data Structure"), and validation of caller-provided device arrays.
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "pintile.cuh"
@@ -121,15 +120,10 @@ k_scatter_edges_local(const int2* __restrict__ pins, const int32_t* __restrict__
   }
 }
 
-void local_attributes() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    for (const void* f : {reinterpret_cast<const void*>(k_degrees_local),
-                          reinterpret_cast<const void*>(k_scatter_incidence_local),
-                          reinterpret_cast<const void*>(k_scatter_edges_local)})
-      HG_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   LOCAL_N * (int)sizeof(int32_t)));
-  });
+// Before a launch of one of the local forms.
+template <typename K>
+void prepare_local(const Ctx& cx, K* kernel) {
+  prepare_kernel(cx, kernel, LOCAL_N * sizeof(int32_t));
 }
 
 // Scatter every pin (e, v) into I(v) at a slot taken from v's cursor.
@@ -409,7 +403,7 @@ void build_incidence(const Ctx& cx, Level& L) {
   const int local = L.p > 0 ? local_blocks(cx, L.n, L.p, num_pin_tiles(L.p)) : 0;
   const size_t smem = (size_t)L.n * sizeof(int32_t);
   if (local) {
-    local_attributes();
+    prepare_local(cx, k_degrees_local);
     k_degrees_local<<<local, LOCAL_THREADS, smem, cx.stream>>>(L.pins.p, L.p, L.n, L.ioff.p);
     check_launch("degrees_local");
   } else if (L.p > 0) {
@@ -424,22 +418,26 @@ void build_incidence(const Ctx& cx, Level& L) {
                             cudaMemcpyDeviceToDevice, cx.stream));
     if (L.graph) {
       const int2* edges = reinterpret_cast<const int2*>(L.pins.p);
-      if (local)
+      if (local) {
+        prepare_local(cx, k_scatter_edges_local);
         k_scatter_edges_local<<<local, LOCAL_THREADS, smem, cx.stream>>>(
             edges, L.w.p, L.m, L.n, cursor.p, L.inets.p, L.adj.p);
-      else
+      } else {
         k_scatter_edges<<<grid_for(L.m, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(
             edges, L.w.p, L.m, cursor.p, L.inets.p, L.adj.p);
+      }
     } else {
       tiles.alloc(&cx.alloc, (size_t)num_pin_tiles(L.p) + 1);
       build_tile_index(cx, L.eoff.p, L.m, L.p, tiles.p);
-      if (local)
+      if (local) {
+        prepare_local(cx, k_scatter_incidence_local);
         k_scatter_incidence_local<<<local, LOCAL_THREADS, smem, cx.stream>>>(
             L.eoff.p, L.pins.p, tiles.p, L.m, L.p, L.n, cursor.p, L.inets.p);
-      else
+      } else {
         k_scatter_incidence<<<grid_for(num_pin_tiles(L.p), 1, cx.num_sms, 8), PIN_TILE_THREADS, 0,
                               cx.stream>>>(L.eoff.p, L.pins.p, tiles.p, L.m, L.p, cursor.p,
                                            L.inets.p);
+      }
     }
     check_launch("scatter_incidence");
     if (cx.launches) *cx.launches += 2;

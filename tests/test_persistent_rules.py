@@ -146,3 +146,32 @@ def test_kernels_of_a_level_are_sized_by_the_calls_in_flight():
     and one that sleeps alone has all of it."""
     for name in ("cluster.cu", "lp.cu", "community.cu"):
         assert "shares_gpu()" in source(name) and "sync_event" not in source(name), name
+
+
+def test_kernel_attributes_are_set_by_every_handle(tmp_path):
+    """CUDA keeps them per device; a process may hold handles on several."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        text = open(path).read()
+        assert "once_flag" not in text, os.path.basename(path)
+        if os.path.basename(path) != "common.cuh":
+            assert "cudaFuncSetAttribute" not in text, os.path.basename(path)
+    hostcc.run(tmp_path, ["common.cuh"], """
+    using namespace hgk;
+    int main() {
+      PreparedKernels one, two;
+      int a = 0, b = 0, sets = 0;
+      for (int i = 0; i < 3; ++i) {
+        one.once(&a, [&] { ++sets; });
+        one.once(&b, [&] { ++sets; });
+        two.once(&a, [&] { ++sets; });
+      }
+      CHECK(sets == 3);
+      try {
+        two.once(&b, [&] { throw 1; });
+      } catch (int) {
+      }
+      two.once(&b, [&] { ++sets; });  // set again after a failure
+      CHECK(sets == 4);
+      return 0;
+    }
+    """)
