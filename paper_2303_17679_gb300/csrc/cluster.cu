@@ -644,7 +644,6 @@ __device__ void approve_contested(const ClusterArgs& A, int32_t* words, unsigned
       // large group: binary search for the first excluded key x, the largest
       // x with (sum of c over keys < x) <= cap; all keys < x are accepted
       unsigned long long lo = 0, hi = (1ull << 63);
-      BeatLoop work(A.barrier);
       while (hi - lo > 1) {
         const unsigned long long mid = lo + ((hi - lo) >> 1);
         long long f = 0;
@@ -652,7 +651,7 @@ __device__ void approve_contested(const ClusterArgs& A, int32_t* words, unsigned
           const int32_t u = A.glist[off + i];
           const unsigned long long kk = ((unsigned long long)(uint32_t)A.c[u] << 32) | (uint32_t)u;
           if (kk < mid) f += A.c[u];
-          work.trip();
+          beat_along(A.barrier, i);
         }
         f = block_sum(f, s_red);
         if (f <= cap) lo = mid; else hi = mid;

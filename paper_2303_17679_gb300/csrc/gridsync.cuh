@@ -33,16 +33,11 @@ __device__ __forceinline__ void beat(unsigned* barrier) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(barrier + 1) : "memory");
 }
 
-// Reports every 256th trip of a block's loop (a few hundred microseconds of
-// dependent accesses).
-struct BeatLoop {
-  unsigned* barrier;
-  int trips = 0;
-  __device__ __forceinline__ explicit BeatLoop(unsigned* b) : barrier(b) {}
-  __device__ __forceinline__ void trip() {
-    if ((++trips & 255) == 0 && threadIdx.x == 0) beat(barrier);
-  }
-};
+// The same from a loop of a block over i = threadIdx.x, + blockDim.x, ... (a power
+// of two): every 131072 entries, a few hundred microseconds of dependent accesses.
+__device__ __forceinline__ void beat_along(unsigned* barrier, int64_t i) {
+  if (i > 0 && (i & 0x1ffff) == 0) beat(barrier);  // thread 0's entries
+}
 
 // cluster: the blocks are one thread-block cluster (hardware barrier, 0.35 to
 // 0.5 us, which waits until they arrive); else they were launched cooperatively

@@ -648,12 +648,12 @@ __device__ __forceinline__ void rank_sort2(const unsigned long long* a, int na,
 // Bitonic sorts of the two directions of a pair (Pa and Pb powers of two) by
 // the block, stage by stage together.
 __device__ void bitonic_sort2(unsigned long long* a, int Pa, unsigned long long* b, int Pb,
-                              BeatLoop& work) {
+                              unsigned* barrier) {
   const int P = Pa > Pb ? Pa : Pb;
   for (int kk = 2; kk <= P; kk <<= 1) {
     for (int j = kk >> 1; j > 0; j >>= 1) {
       for (int64_t y = threadIdx.x; y < (int64_t)Pa + Pb; y += LP_THREADS) {
-        work.trip();
+        beat_along(barrier, y);
         unsigned long long* buf = y < Pa ? a : b;
         const int i = (int)(y < Pa ? y : y - Pa);
         const int n = y < Pa ? Pa : Pb;
@@ -678,7 +678,7 @@ __device__ void bitonic_sort2(unsigned long long* a, int Pa, unsigned long long*
 // a -> b (x = 0..na), B[x] likewise for b -> a.
 __device__ void weight_prefix2(const unsigned long long* ka, int na, const unsigned long long* kb,
                                int nb, const int32_t* __restrict__ c, int32_t* A, int32_t* B,
-                               BeatLoop& work) {
+                               unsigned* barrier) {
   __shared__ int32_t s_sum[LP_WARPS];
   __shared__ int32_t s_total_a;
   const int cnt = na + nb;
@@ -690,8 +690,8 @@ __device__ void weight_prefix2(const unsigned long long* ka, int na, const unsig
   }
   __syncthreads();
   for (int base = 0; base < cnt; base += LP_THREADS) {
-    work.trip();
     const int x = base + threadIdx.x;
+    beat_along(barrier, x);
     int32_t v = 0;
     if (x < na) v = __ldg(c + (int32_t)(uint32_t)ka[x]);
     else if (x < cnt) v = __ldg(c + (int32_t)(uint32_t)kb[x - na]);
@@ -720,7 +720,6 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
                              const long long* s_slack, unsigned char* smem) {
   __shared__ int s_red[2];
   const int cap = P.sel_cap, k = P.k;
-  BeatLoop work(P.barrier);
   const int dab = a * k + b, dba = b * k + a;
   unsigned long long* s_keys0 = reinterpret_cast<unsigned long long*>(smem);
   unsigned long long* s_keys1 = s_keys0 + cap;
@@ -772,7 +771,7 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
   if (na > la || nb > lb) {
     const int32_t no = __ldcg(P.words + par * SW_WORDS + SW_OVERFLOW);
     for (int32_t i = threadIdx.x; i < no; i += LP_THREADS) {
-      work.trip();
+      beat_along(P.barrier, i);
       const int32_t d = __ldcg(P.ovf_dir + i);
       if (d == dab) ka[la + atomicAdd(&s_red[0], 1)] = __ldcg(P.ovf_key + i);
       else if (d == dba) kb[lb + atomicAdd(&s_red[1], 1)] = __ldcg(P.ovf_key + i);
@@ -787,9 +786,9 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
     for (int i = na + threadIdx.x; i < Pa; i += LP_THREADS) ka[i] = ~0ull;
     for (int i = nb + threadIdx.x; i < Pb; i += LP_THREADS) kb[i] = ~0ull;
     __syncthreads();
-    bitonic_sort2(ka, Pa, kb, Pb, work);
+    bitonic_sort2(ka, Pa, kb, Pb, P.barrier);
   }
-  weight_prefix2(ka, na, kb, nb, P.c, A, B, work);
+  weight_prefix2(ka, na, kb, nb, P.c, A, B, P.barrier);
   if (threadIdx.x == 0) s_red[0] = 0;
   __syncthreads();
   // diagonal r: i(r) = number of A steps among the first r
@@ -805,7 +804,7 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
   const long long lo = -s_slack[a], hi = s_slack[b];
   int best = 0;
   for (int r = threadIdx.x; r <= na + nb; r += LP_THREADS) {
-    work.trip();
+    beat_along(P.barrier, r);
     const int i = steps(r);
     const long long x = (long long)A[i] - B[r - i];
     if (lo <= x && x <= hi) best = r > best ? r : best;
@@ -817,8 +816,8 @@ __device__ void select_block(const LpArgs& P, int par, int a, int b, int na, int
   const int ta = steps(r), tb = r - ta;
   int32_t incid = 0;
   for (int i0 = 32 * warp_in_block(); i0 < ta + tb; i0 += LP_THREADS) {
-    work.trip();
     const int i = i0 + lane_id();
+    beat_along(P.barrier, i);
     const bool from_a = i < ta;
     int32_t u = 0;
     if (i < ta + tb) u = (int32_t)(uint32_t)(from_a ? ka[i] : kb[i - ta]);
