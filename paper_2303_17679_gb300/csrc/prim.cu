@@ -1,8 +1,10 @@
 // Data-parallel primitives: exclusive prefix sums, fills, scalar readback.
 // The prefix sums are the "parallel prefix sum operations" the contraction
 // algorithm relies on (Sec. 4.2), written here without CUB.
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "common.cuh"
@@ -218,27 +220,33 @@ void wait_stream(const Ctx& cx) {
 
 namespace {
 
-// Page-locked words of the calling thread that readbacks go through: copies to
-// them are queued behind the kernels like any other work, so a readback costs
-// one wait (a copy to pageable memory waits for the stream by itself, and one
-// more for the status word).  Freed when the thread ends.
-constexpr size_t STAGE_BYTES = 4096;
+// Words of the calling thread that readbacks go through.  They are the library's
+// own memory, page-locked for CUDA: copies to them are queued behind the kernels
+// like any other work, so a readback costs one wait (a copy to pageable memory
+// waits for the stream by itself, and one more for the status word).  After a
+// cudaDeviceReset, which ends the page lock but not the memory, the copies are
+// those to pageable memory and as correct.  A page is the lock's unit, up to 64 KB
+// on Arm hosts.  Freed when the thread ends.
+constexpr size_t STAGE_BYTES = 4096, STAGE_PAGE = 1 << 16;
 
 struct Stage {
-  unsigned char* p = nullptr;
+  void* p = nullptr;
+  bool locked = false;
   ~Stage() {
-    if (p) cudaFreeHost(p);
+    if (locked && cudaHostUnregister(p) != cudaSuccess) cudaGetLastError();
+    std::free(p);
   }
 };
 
 unsigned char* stage() {
   thread_local Stage s;
   if (!s.p) {
-    void* q = nullptr;
-    HG_CUDA(cudaHostAlloc(&q, STAGE_BYTES, cudaHostAllocPortable));
-    s.p = static_cast<unsigned char*>(q);
+    s.p = std::aligned_alloc(STAGE_PAGE, STAGE_PAGE);
+    if (!s.p) throw std::bad_alloc();
+    s.locked = cudaHostRegister(s.p, STAGE_PAGE, cudaHostRegisterPortable) == cudaSuccess;
+    if (!s.locked) cudaGetLastError();
   }
-  return s.p;
+  return static_cast<unsigned char*>(s.p);
 }
 
 void throw_status(const Ctx& cx, int32_t st) {

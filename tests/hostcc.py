@@ -19,13 +19,13 @@ PROLOGUE = """
 """
 
 
-def run(tmp_path, includes, body):
-    """Runs `body` (statements of main) after including the headers in `includes`."""
+def run(tmp_path, includes, body, link=()):
+    """Compiles and runs `body` (with its main) after the headers in `includes`."""
     src, exe = tmp_path / "host.cu", tmp_path / "host"
     text = PROLOGUE + "".join(f'#include "{name}"\n' for name in includes)
     src.write_text(text + textwrap.dedent(body))
     r = subprocess.run([build.nvcc(), *build.ARCH, "-O1", "-std=c++17", "--expt-relaxed-constexpr",
-                        "-I", build.CSRC, "-I", build.INCLUDE, str(src), "-o", str(exe)],
+                        "-I", build.CSRC, "-I", build.INCLUDE, str(src), *link, "-o", str(exe)],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)

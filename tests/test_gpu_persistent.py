@@ -16,7 +16,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():  # pragma: no cover
     pytest.skip("no CUDA device", allow_module_level=True)
 
-from paper_2303_17679_gb300 import hg  # noqa: E402
+from paper_2303_17679_gb300 import build, hg  # noqa: E402
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -177,3 +177,56 @@ def test_plain_handles_at_once(oracle_mod):
     for t in threads:
         t.join()
     assert got == [(w.objectives[0], True) for w in want]
+
+
+def test_handles_after_a_device_reset(tmp_path):
+    """The same thread and the same kernels, with the caller's own allocator: what
+    the library keeps beyond a handle must not outlive the context."""
+    out = hostcc.run(tmp_path, ["hg.h"], """
+    void* get(size_t bytes, void*) {
+      void* p = nullptr;
+      return cudaMalloc(&p, bytes) == cudaSuccess ? p : nullptr;
+    }
+    void put(void* p, void*) { cudaFree(p); }
+    uint64_t partition() {
+      const int n = 12000, m = 12000;  // levels with the wide shared-memory forms
+      std::vector<int32_t> off{0}, pins;
+      uint32_t x = 1;
+      for (int e = 0; e < m; ++e) {
+        const int size = 2 + e % 5 + (e % 500 == 0 ? 1500 : 0);
+        const int at = (x = x * 1664525u + 1013904223u) % n;
+        for (int i = 0; i < size; ++i) pins.push_back((at + i * 7) % n);
+        off.push_back((int32_t)pins.size());
+      }
+      hg_options o;
+      hg_default_options(&o);
+      o.dev_alloc = get;
+      o.dev_free = put;
+      o.contraction_limit_factor = 20;
+      o.community_detection = 1;
+      hg_t* h = nullptr;
+      CHECK(hg_create(n, m, off.data(), pins.data(), nullptr, nullptr, HG_MEM_HOST, &o, nullptr,
+                      &h) == HG_OK);
+      int32_t* part = nullptr;
+      CHECK(cudaMalloc(&part, 4 * n) == cudaSuccess);
+      int64_t f = 0;
+      CHECK(hg_partition(h, 4, 30000, 3, part, &f) == HG_OK);
+      std::vector<int32_t> got(n);
+      CHECK(cudaMemcpy(got.data(), part, 4 * n, cudaMemcpyDeviceToHost) == cudaSuccess);
+      hg_destroy(h);
+      cudaFree(part);
+      uint64_t sum = (uint64_t)f;
+      for (int32_t b : got) sum = sum * 31 + (uint64_t)b;
+      return sum;
+    }
+    int main() {
+      const uint64_t before = partition();
+      for (int i = 0; i < 2; ++i) {
+        CHECK(cudaDeviceReset() == cudaSuccess);
+        CHECK(partition() == before);
+      }
+      std::printf("same %llu", (unsigned long long)before);
+      return 0;
+    }
+    """, link=[build.LIB, "-cudart", "shared", "-Xlinker", "-rpath", "-Xlinker", build.HERE])
+    assert out.startswith("same")

@@ -175,3 +175,12 @@ def test_kernel_attributes_are_set_by_every_handle(tmp_path):
       return 0;
     }
     """)
+
+
+def test_readbacks_go_through_memory_that_no_reset_frees():
+    """cudaDeviceReset frees what CUDA allocated on the host; the words of a thread
+    outlive handles."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        text = open(path).read()
+        assert "cudaHostAlloc" not in text and "cudaMallocHost" not in text, path
+    assert "cudaHostRegister" in source("prim.cu")
