@@ -338,9 +338,10 @@ __device__ void rate_items(const RateArgs& A, int s, const SubPlan& P, RunShared
 // cluster id (part_of).  Every block walks all of the node's visits (the pin
 // clusters are read P times, from L2 at the levels where this happens) and
 // accumulates the candidates of its part in a shared table (PartCfg);
-// P = ceil(min(W, n) / PartCfg::D) keeps every table at most 60 % full, so no
-// insertion can fail.  A node of one part publishes its argmax directly;
-// otherwise each part leaves its best (rating, cluster) for the per-node
+// P = ceil(min(W, n) / PartCfg::D) makes every table 60 % full at most where the ids
+// spread evenly over the parts; a part whose table is full all the same fails the
+// run, which cluster_level repeats without parts.  A node of one part publishes its
+// argmax directly; otherwise each part leaves its best (rating, cluster) for the per-node
 // combine in rate_split_best.  All warps of the block walk the node's groups of
 // 32 records, sharing the chunks in turn.
 template <typename VT, bool GRAPH>
@@ -373,7 +374,9 @@ __device__ void rate_parts(const RateArgs& A, int s, int32_t* words, const SubPl
     // this one
     int32_t* nused = &sh.nused[0][it & 1];
     const int32_t cmu = A.comm ? A.comm[u] : -1;
+    bool full = false;  // nothing more is added: every probe would walk the table
     auto visit = [&](const int32_t(&q)[PART_ILP], const VT(&rr)[PART_ILP]) HG_INLINE {
+      if (full) return;
       int2 ri[PART_ILP];
       resolve_batch<GRAPH, PART_ILP>(A, s, q, ri, cmu);
 #pragma unroll
@@ -388,6 +391,7 @@ __device__ void rate_parts(const RateArgs& A, int s, int32_t* words, const SubPl
           if (y < (int32_t)CAP) used[y] = sl;
         } else if (sl == ADD_FULL) {
           dev_fail(A.status_word, DEV_HASH_FULL);
+          full = true;
         }
       }
     };

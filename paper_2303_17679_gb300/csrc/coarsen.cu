@@ -641,12 +641,13 @@ k_node_scatter(const int32_t* __restrict__ key_of, int32_t n, int nkeys,
 //   direct-indexed global table (n entries) when n <= min(2 W(u), 65536), so
 //   the table costs no more than the accumulation: groups of 32 nets over
 //   the grid (items);
-//   else P = ceil(D / part_d) shared-memory parts when P <= PART_MAX (no
+//   else P = ceil(D / part_d) shared-memory parts when P <= part_max (no
 //   global table);
 //   else a global hash table of a power of two >= 2 D + 2 slots, with items.
 __global__ void k_split_sizes(const int4* __restrict__ lsplit, int32_t nsplit,
                               const int32_t* __restrict__ wof,
-                              int32_t n, int32_t part_d, int32_t* __restrict__ items,
+                              int32_t n, int32_t part_d, int32_t part_max,
+                              int32_t* __restrict__ items,
                               int32_t* __restrict__ parts, int32_t* __restrict__ cap,
                               int8_t* __restrict__ dense) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nsplit; i += gridDim.x * blockDim.x) {
@@ -655,7 +656,7 @@ __global__ void k_split_sizes(const int4* __restrict__ lsplit, int32_t nsplit,
     const bool d = n <= SPLIT_DENSE_MAX && (int64_t)n <= 2 * (int64_t)wof[u];
     const int32_t D = min(wof[u], n);
     const int32_t P = d ? 0 : (D + part_d - 1) / part_d;
-    const bool part = !d && P <= PART_MAX;
+    const bool part = !d && P <= part_max;
     items[i] = part ? 0 : (deg + 31) / 32;
     parts[i] = part ? P : 0;
     dense[i] = d ? 1 : 0;
@@ -760,10 +761,10 @@ __global__ void k_init_cluster(const int32_t* __restrict__ c, int32_t n, uint64_
 
 // ---------------------------------------------------------- host side
 
-}  // namespace
-
-void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCounters& cc,
-                   DBuf<int32_t>& cw_out) {
+// The clustering of a level with split nodes of at most part_max parts.  Returns
+// false (and nothing of use) when a part's table was full.
+bool cluster_with_parts(const Ctx& cx, Level& L, const CoarsenParams& P, int32_t part_max,
+                        CoarsenCounters& cc, DBuf<int32_t>& cw_out) {
   const int32_t n = L.n;
   const int S = P.S;
   const int nkeys = S * NCLASS;
@@ -936,7 +937,7 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
     const int gs = grid_for(nsplit, 256, cx.num_sms, 4);
     k_split_sizes<<<gs, 256, 0, cx.stream>>>(
         lnode.p + split_base, nsplit, wof.p, n, narrow ? PartCfg<uint32_t>::D : PartCfg<unsigned long long>::D,
-        items.p, parts.p, cap32.p, tab_dense.p);
+        part_max, items.p, parts.p, cap32.p, tab_dense.p);
     check_launch("split_sizes");
     scan_exclusive_i32(cx, items.p, item_off.p, nsplit, item_off.p + nsplit);
     scan_exclusive_i32(cx, parts.p, part_off.p, nsplit, part_off.p + nsplit);
@@ -1103,7 +1104,12 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
   HG_CUDA(cudaMemcpy2DAsync(cw_out.p, sizeof(int32_t), cst.p, sizeof(int2), sizeof(int32_t),
                             (size_t)n, cudaMemcpyDeviceToDevice, cx.stream));
   unsigned long long hs[ST_TOTAL];
-  read_back(cx, hs, stats.p, sizeof(hs));
+  const int32_t status = read_status(cx, hs, stats.p, sizeof(hs));
+  if (status == DEV_HASH_FULL && any_parts) {
+    HG_CUDA(cudaMemsetAsync(cx.d_status, 0, sizeof(int32_t), cx.stream));
+    return false;
+  }
+  throw_status(cx, status);
   for (int c = 0; c < NCLASS; ++c) {
     const unsigned long long* h = hs + c * ST_WORDS;
     cc.rating_pin_visits += (int64_t)h[ST_PINS];
@@ -1121,6 +1127,19 @@ void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCount
     cc.ms_approve += hs[ST_NS_APPROVE] * 1e-6;
     cc.ms_refresh += hs[ST_NS_REFRESH] * 1e-6;
   }
+  return true;
+}
+
+}  // namespace
+
+// The parts of a node hold its candidates by a fixed hash of their ids, so ids
+// chosen to meet in one part overfill its table, which then drops candidates and
+// says so.  Such a level is clustered once more with tables in global memory
+// instead, which have a slot for every candidate.
+void cluster_level(const Ctx& cx, Level& L, const CoarsenParams& P, CoarsenCounters& cc,
+                   DBuf<int32_t>& cw_out) {
+  if (!cluster_with_parts(cx, L, P, PART_MAX, cc, cw_out))
+    cluster_with_parts(cx, L, P, 0, cc, cw_out);
 }
 
 }  // namespace hgk

@@ -354,6 +354,8 @@ void scan_exclusive_i64(const Ctx& cx, const int64_t* in, int64_t* out, int64_t 
 // returns the status instead.
 void read_back(const Ctx& cx, void* dst, const void* src, size_t bytes);
 int32_t read_status(const Ctx& cx, void* dst, const void* src, size_t bytes);
+// Clears the status word and throws the error of a status other than DEV_OK.
+void throw_status(const Ctx& cx, int32_t st);
 int32_t read_i32(const Ctx& cx, const int32_t* d);
 int64_t read_i64(const Ctx& cx, const int64_t* d);
 void check_status(const Ctx& cx);

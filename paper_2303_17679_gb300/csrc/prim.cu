@@ -249,6 +249,8 @@ unsigned char* stage() {
   return static_cast<unsigned char*>(s.p);
 }
 
+}  // namespace
+
 void throw_status(const Ctx& cx, int32_t st) {
   if (st == DEV_OK) return;
   int32_t zero = 0;
@@ -260,8 +262,6 @@ void throw_status(const Ctx& cx, int32_t st) {
     default: throw HgError(HG_ERR_CUDA, "internal: device capacity exceeded");
   }
 }
-
-}  // namespace
 
 int32_t read_status(const Ctx& cx, void* dst, const void* src, size_t bytes) {
   unsigned char* st = stage();

@@ -230,3 +230,43 @@ def test_handles_after_a_device_reset(tmp_path):
     }
     """, link=[build.LIB, "-cudart", "shared", "-Xlinker", "-rpath", "-Xlinker", build.HERE])
     assert out.startswith("same")
+
+
+def part_of(ids, parts):
+    """The part of a candidate (rating.cuh)."""
+    h = (ids.astype(np.uint64) * np.uint64(0x85EBCA77)) & np.uint64(0xffffffff)
+    return (h * np.uint64(parts)) >> np.uint64(32)
+
+
+# A node rated in the first sub-round, before anything has joined, with candidates
+# that all lie in one part of the table: 2-pin nets (64-bit ratings, 16384 slots) on
+# the hypergraph and the graph path, nets of 750 pins (32-bit, 22528 slots).
+@pytest.mark.parametrize("form,count,parts", [("nets", 24_000, 5), ("graph", 24_000, 3),
+                                              ("wide nets", 30_000, 3)])
+def test_candidates_that_meet_in_one_part(oracle_mod, form, count, parts):
+    n, seed = 200_000, 1
+    ids = np.arange(n, dtype=np.uint64)
+    x = (ids ^ np.uint64(seed)) + np.uint64(0x9E3779B97F4A7C15)
+    x = (x ^ (x >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+    x = (x ^ (x >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+    x ^= x >> np.uint64(31)
+    hub = int(np.flatnonzero(x % np.uint64(16) == 0)[0])
+    cand = np.flatnonzero(part_of(ids, parts) == 0)
+    cand = cand[cand != hub][:count]
+    assert len(cand) == count and count * 15 // 16 > (22_528 if form == "wide nets" else 16_384)
+    if form == "wide nets":
+        nets = [[hub, *c.tolist()] for c in cand.reshape(-1, 750)]
+    else:
+        nets = [[hub, int(v)] for v in cand]
+    if form == "nets":
+        nets.append([n - 3, n - 2, n - 1])
+    rng = np.random.default_rng(2)
+    hgr = from_nets(n, nets, rng.integers(1, 100, size=len(nets)), None)
+    ref = oracle_mod.multilevel(hgr, 2, 30000, S=16, factor=160, seed=seed, max_passes=0)
+    h = create(hgr, seed)
+    try:
+        assert hg.hg_level_is_graph(h, 0) == (form == "graph")
+        assert hg.hg_coarsen_level(h, 2)[0] == hg.HG_OK
+        assert np.array_equal(hg.hg_get_level(h, 0, with_map=True)["map"], ref.maps[0])
+    finally:
+        hg.hg_destroy(h)
