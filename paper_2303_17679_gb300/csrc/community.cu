@@ -122,7 +122,7 @@ enum { LD_TOTAL = 0, LD_MOST = 1, LD_SLOTS = 2 };
 // k_i = 2 self_i + sum of i's edge weights (a warp per vertex); W2 = sum k_i.
 __global__ void k_lv_degrees(const long long* __restrict__ off, const long long* __restrict__ aw,
                              const long long* __restrict__ self, int64_t V, uint64_t seed,
-                             int level, int S, long long* __restrict__ k,
+                             int level, int S, int huge, long long* __restrict__ k,
                              unsigned long long* __restrict__ sums) {
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   long long acc = 0;
@@ -134,7 +134,7 @@ __global__ void k_lv_degrees(const long long* __restrict__ off, const long long*
     if (lane_id() == 0) k[i] = s;
     acc += s;
     const long long deg = off[i + 1] - off[i];
-    if (deg > LV_HUGE && lane_id() < LV_ROUNDS) {
+    if (deg > huge && lane_id() < LV_ROUNDS) {
       const int r = lane_id();
       const unsigned long long slots = lv_slots(deg);
       const unsigned long long before =
@@ -230,6 +230,7 @@ struct LvArgs {
   int64_t V;
   uint64_t seed;
   int level, S;
+  int huge_deg;     // class 5 above this degree
   int2* list;       // {vertex, part} by (sub-round, class); class 5 {index in huge, chunk}
   int32_t *cnt, *fill;  // LV_CLASSES S each
   HugeVertex* huge;
@@ -261,7 +262,7 @@ __device__ __forceinline__ void lv_list(const LvArgs& A, int round, bool scatter
     if (i < A.V) {
       deg = A.off[i + 1] - A.off[i];
       if (deg > 0) {  // a vertex without neighbours never moves
-        cls = lv_class(deg, entries);
+        cls = lv_class(deg, A.huge_deg, entries);
         key = subround_louvain(A.seed, A.level, round, i, A.S) * LV_CLASSES + cls;
         slot = atomicAdd(&s_hist[key], entries);
       }
@@ -457,7 +458,7 @@ __device__ __forceinline__ void lv_block(const LvArgs& A, int32_t* words, int32_
   const int32_t i = nd.x;
   const long long b = A.off[i], e = A.off[i + 1];
   int32_t parts;
-  lv_class(e - b, parts);
+  lv_class(e - b, A.huge_deg, parts);
   for (long long q = b + threadIdx.x; q < e; q += LV_THREADS) {
     const int32_t C = A.cl[A.adj[q]];
     if (parts > 1 && lv_part(C, parts) != nd.y) continue;
@@ -608,7 +609,7 @@ __global__ void __launch_bounds__(LV_THREADS, 2) k_lv_run(const __grid_constant_
           if (nd.y != 0) continue;  // the first entry of a vertex combines
           int32_t i = nd.x, parts;
           if (!HUGE || x < at[5]) {
-            lv_class(A.off[i + 1] - A.off[i], parts);
+            lv_class(A.off[i + 1] - A.off[i], A.huge_deg, parts);
           } else {
             parts = A.huge[nd.x].entries;
             i = A.huge[nd.x].i;
@@ -816,7 +817,8 @@ __global__ void k_lv_mark(const int32_t* __restrict__ comm, int32_t n, int32_t* 
 
 struct LvGraph {
   int64_t V = 0, E = 0;
-  int64_t slots = 0;  // of the class 5 tables of a sub-round
+  int huge = LV_HUGE;  // class 5 above this degree
+  int64_t slots = 0;   // of the class 5 tables of a sub-round
   DBuf<long long> off, aw, self, k;
   DBuf<int32_t> adj;
 };
@@ -827,7 +829,7 @@ void lv_degrees(const Ctx& cx, LvGraph& g, uint64_t seed, int level, int S, long
   sums.alloc(&cx.alloc, LD_SLOTS + (size_t)LV_ROUNDS * S);
   HG_CUDA(cudaMemsetAsync(sums.p, 0, sums.bytes(), cx.stream));
   k_lv_degrees<<<grid_for(g.V, 8, cx.num_sms, 16), 256, 0, cx.stream>>>(
-      g.off.p, g.aw.p, g.self.p, g.V, seed, level, S, g.k.p, sums.p);
+      g.off.p, g.aw.p, g.self.p, g.V, seed, level, S, g.huge, g.k.p, sums.p);
   check_launch("lv_degrees");
   unsigned long long h[LD_SLOTS];
   read_back(cx, h, sums.p, sizeof(h));
@@ -910,7 +912,8 @@ void lv_aggregate(const Ctx& cx, const LvGraph& g, const int32_t* cl, LvGraph& o
   if (cx.launches) *cx.launches += 14;
 }
 
-// One Louvain level on g (clusters start as singletons).  Returns the moves.
+// One Louvain level on g (clusters start as singletons).  Returns the moves, or -1
+// when the table of a part was full.
 int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, uint64_t seed,
                         int level, DBuf<int32_t>& cl, LouvainCounters& lc) {
   const int64_t V = g.V;
@@ -926,7 +929,7 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   DBuf<HugeVertex> huge;
   DBuf<int32_t> tkey;
   DBuf<long long> tval;
-  huge.alloc(&cx.alloc, g.slots ? (size_t)(g.E / LV_HUGE) + 1 : 0);
+  huge.alloc(&cx.alloc, g.slots ? (size_t)(g.E / g.huge) + 1 : 0);
   tkey.alloc(&cx.alloc, (size_t)g.slots);
   tval.alloc(&cx.alloc, (size_t)g.slots);
   if (g.slots) {
@@ -954,6 +957,7 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   A.seed = seed;
   A.level = level;
   A.S = S;
+  A.huge_deg = g.huge;
   A.list = list.p;
   A.cnt = z;
   A.fill = z + nkeys;
@@ -985,7 +989,12 @@ int64_t lv_local_moving(const Ctx& cx, const LvGraph& g, long long W2, int S, ui
   launch_persistent(cx, kernel, blocks, LV_THREADS, smem, false, A);
   lc.launches += 1;
   unsigned long long hres[LR_LV_WORDS];
-  read_back(cx, hres, A.res, sizeof(hres));
+  const int32_t status = read_status(cx, hres, A.res, sizeof(hres));
+  if (status == DEV_HASH_FULL && g.huge > LV_BLOCK) {
+    HG_CUDA(cudaMemsetAsync(cx.d_status, 0, sizeof(int32_t), cx.stream));
+    return -1;
+  }
+  throw_status(cx, status);
   lc.rounds += (int64_t)hres[LR_ROUNDS];
   return (int64_t)hres[LR_MOVED];
 }
@@ -1026,7 +1035,13 @@ int32_t detect_communities(const Ctx& cx, const Level& L, int S, uint64_t seed,
   lv_degrees(cx, g, seed, 0, S, &W2);
   for (int level = 0; level < LV_LEVELS; ++level) {
     DBuf<int32_t> cl;
-    const int64_t moves = lv_local_moving(cx, g, W2, S, seed, level, cl, lc);
+    int64_t moves = lv_local_moving(cx, g, W2, S, seed, level, cl, lc);
+    if (moves < 0) {  // once more with a table for every vertex above LV_BLOCK
+      g.huge = LV_BLOCK;
+      long long same = 0;
+      lv_degrees(cx, g, seed, level, S, &same);
+      moves = lv_local_moving(cx, g, W2, S, seed, level, cl, lc);
+    }
     lc.moves += moves;
     if (moves == 0) break;
     lc.levels = level + 1;

@@ -23,13 +23,15 @@ constexpr int LV_CHUNK = 1024;    // class 5: a block per chunk of the edges
 // 22.9 and 26.7 ms, with this limit 22.3, 19.3, 16.0 and 17.8 ms; one net of 1e6
 // pins 55.8 -> 18.4 ms.  (Half the limit: 4 nets of 30,000 pins 5 % slower, 60 nets
 // of 20,000 pins 5 % faster.)
-__host__ __device__ inline int lv_class(long long deg, int32_t& entries) {
+// (The parts hold clusters by a hash of their ids; `huge` = LV_BLOCK leaves class 4
+// out for ids that meet in one part.)
+__host__ __device__ inline int lv_class(long long deg, int huge, int32_t& entries) {
   entries = 1;
   if (deg <= LV_GROUP) return 0;
   if (deg <= LV_LANES) return 1;
   if (deg <= LV_SMALL) return 2;
   if (deg <= LV_BLOCK) return 3;
-  if (deg <= LV_HUGE) {
+  if (deg <= huge) {
     entries = (int32_t)((deg + LV_PART - 1) / LV_PART);
     return 4;
   }

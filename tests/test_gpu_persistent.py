@@ -150,7 +150,7 @@ def test_plain_handles_at_once(oracle_mod):
     """Levels of every launch form from several host threads, each result that of
     the call alone."""
     jobs = [(synth.zipf_preferential(i, n, n), k) for i, (n, k) in
-            enumerate([(1500, 2), (9000, 40), (30_000, 8), (60_000, 4)])]
+            enumerate([(1500, 2), (5000, 40), (12_000, 8), (20_000, 4)])]
     want = [oracle_mod.multilevel(g, k, 30000, S=16, factor=20, seed=5, max_passes=2)
             for g, k in jobs]
     got = [None] * len(jobs)
@@ -232,6 +232,14 @@ def test_handles_after_a_device_reset(tmp_path):
     assert out.startswith("same")
 
 
+def mix64(x):
+    """SplitMix64's output function on a uint64 array."""
+    x = x + np.uint64(0x9E3779B97F4A7C15)
+    x = (x ^ (x >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+    x = (x ^ (x >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+    return x ^ (x >> np.uint64(31))
+
+
 def part_of(ids, parts):
     """The part of a candidate (rating.cuh)."""
     h = (ids.astype(np.uint64) * np.uint64(0x85EBCA77)) & np.uint64(0xffffffff)
@@ -246,11 +254,7 @@ def part_of(ids, parts):
 def test_candidates_that_meet_in_one_part(oracle_mod, form, count, parts):
     n, seed = 200_000, 1
     ids = np.arange(n, dtype=np.uint64)
-    x = (ids ^ np.uint64(seed)) + np.uint64(0x9E3779B97F4A7C15)
-    x = (x ^ (x >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
-    x = (x ^ (x >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
-    x ^= x >> np.uint64(31)
-    hub = int(np.flatnonzero(x % np.uint64(16) == 0)[0])
+    hub = int(np.flatnonzero(mix64(ids ^ np.uint64(seed)) % np.uint64(16) == 0)[0])
     cand = np.flatnonzero(part_of(ids, parts) == 0)
     cand = cand[cand != hub][:count]
     assert len(cand) == count and count * 15 // 16 > (22_528 if form == "wide nets" else 16_384)
@@ -268,5 +272,26 @@ def test_candidates_that_meet_in_one_part(oracle_mod, form, count, parts):
         assert hg.hg_level_is_graph(h, 0) == (form == "graph")
         assert hg.hg_coarsen_level(h, 2)[0] == hg.HG_OK
         assert np.array_equal(hg.hg_get_level(h, 0, with_map=True)["map"], ref.maps[0])
+    finally:
+        hg.hg_destroy(h)
+
+
+def test_louvain_clusters_that_meet_in_one_part(oracle_mod):
+    """A net vertex of 32,768 neighbours, sixteen parts, whose clusters all belong to
+    one of them."""
+    n, size, seed = 700_000, 32_768, 4
+    ids = np.arange(n, dtype=np.uint64)
+    part = ((mix64(ids ^ np.uint64(0xA5A5A5A500000000)) >> np.uint64(32)) * np.uint64(16)) >> np.uint64(32)
+    pins = np.flatnonzero(part == 3)[:size]
+    key = seed ^ (1 << 62) ^ (1 << 48) ^ n  # the net's vertex in the first round
+    assert len(pins) == size and mix64(np.array([key], np.uint64))[0] % np.uint64(16) < 11
+    hgr = from_nets(n, [pins.tolist(), [0, 1], [1, 2, 3]], [100, 1, 1], None)
+    want, levels, moves = oracle_mod.communities(hgr, S=16, seed=seed)
+    h = create(hgr, seed)
+    try:
+        hg.hg_detect_communities(h)
+        assert np.array_equal(hg.hg_get_communities(h, 0), want)
+        st = hg.hg_get_stats(h)
+        assert st["louvain_levels"] == levels and st["louvain_moves"] == moves
     finally:
         hg.hg_destroy(h)

@@ -72,7 +72,8 @@ def test_louvain_vertices_of_any_degree(tmp_path):
       std::sort(degs.begin(), degs.end());
       for (long long d : degs) {
         int32_t entries = 0;
-        const int cls = lv_class(d, entries);
+        if (d > LV_BLOCK) CHECK(lv_class(d, LV_BLOCK, entries) == 5);
+        const int cls = lv_class(d, LV_HUGE, entries);
         CHECK(cls >= last && cls < LV_CLASSES && entries >= 1);
         last = cls;
         if (cls < 4) CHECK(entries == 1);
