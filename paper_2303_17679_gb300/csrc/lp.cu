@@ -58,7 +58,7 @@ enum SubroundWord { SW_OVERFLOW = 0, SW_ITEMS = 1, SW_WORDS = 4 };
 // Results and totals of a call.
 enum LpResultWord {
   LR_MOVES = 0, LR_MOVED_INCID = 1, LR_OBJECTIVE = 2, LR_PASSES = 3,
-  LR_NS_GAIN = 4, LR_NS_SELECT = 5, LR_NS_APPLY = 6, LR_WORDS = 8
+  LR_NS_GAIN = 4, LR_NS_SELECT = 5, LR_NS_APPLY = 6, LR_NS_OBJECTIVE = 7, LR_WORDS = 8
 };
 
 struct LpArgs {
@@ -1005,6 +1005,7 @@ __global__ void __launch_bounds__(LP_THREADS, 2) k_lp_run(const __grid_constant_
     moves_before = moves;
   }
   // ---- objective (a14)
+  if (clock) t0 = now_ns();
   int64_t f = 0;
   const int64_t stride = (int64_t)gridDim.x * LP_THREADS;
   for (int64_t e = (int64_t)blockIdx.x * LP_THREADS + threadIdx.x; e < A.m; e += stride) {
@@ -1026,6 +1027,7 @@ __global__ void __launch_bounds__(LP_THREADS, 2) k_lp_run(const __grid_constant_
     A.res[LR_NS_GAIN] = t_gain;
     A.res[LR_NS_SELECT] = t_select;
     A.res[LR_NS_APPLY] = t_apply;
+    if (clock) A.res[LR_NS_OBJECTIVE] = now_ns() - t0;
   }
 }
 
@@ -1196,6 +1198,7 @@ LPResult lp_refine_level(const Ctx& cx, const Level& L, int level_index, int k, 
     rc.ms_gain += g;
     rc.ms_select += s;
     rc.ms_apply += a;
+    rc.ms_objective += hres[LR_NS_OBJECTIVE] * 1e-6;
   }
   if (cx.kernel_timing) {
     rc.ms_gain_kernels += g;

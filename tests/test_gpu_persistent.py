@@ -295,3 +295,18 @@ def test_louvain_clusters_that_meet_in_one_part(oracle_mod):
         assert st["louvain_levels"] == levels and st["louvain_moves"] == moves
     finally:
         hg.hg_destroy(h)
+
+
+def test_phase_times_of_label_propagation():
+    hgr = synth.zipf_preferential(1, 200_000, 200_000)
+    h = create(hgr, 1)
+    try:
+        part = torch.empty(hgr.n, dtype=torch.int32, device="cuda")
+        hg.hg_initial_partition(h, 0, 4, part)
+        hg.hg_enable_timing(h, 1)
+        hg.hg_lp_refine(h, 0, 4, 30000, 2, part)
+        st = hg.hg_get_stats(h)
+        for name in ("ms_phi", "ms_lp_gain", "ms_lp_select", "ms_lp_apply", "ms_objective"):
+            assert st[name] > 0, name
+    finally:
+        hg.hg_destroy(h)
