@@ -1096,10 +1096,11 @@ bool cluster_with_parts(const Ctx& cx, Level& L, const CoarsenParams& P, int32_t
   size_t smem = narrow ? TEAM_SMEM<uint32_t> : TEAM_SMEM<unsigned long long>;
   if (dense_block) smem = std::max(smem, dense_bytes * (size_t)(RUN_WARPS / R.dense_tw));
   if (any_parts) smem = std::max(smem, narrow ? part_bytes<uint32_t>() : part_bytes<unsigned long long>());
-  cc.rating_launches += 1;
-  if (hoff[nkeys] > 0)
+  if (hoff[nkeys] > 0) {
+    cc.rating_launches += 1;
     run_subrounds(cx, A, narrow, L.graph, smem, hoff[nkeys], hoff[nkeys] - hoff[S],
                   (int64_t)hmax[2]);
+  }
   // cluster weights for the contraction (valid at representatives)
   HG_CUDA(cudaMemcpy2DAsync(cw_out.p, sizeof(int32_t), cst.p, sizeof(int2), sizeof(int32_t),
                             (size_t)n, cudaMemcpyDeviceToDevice, cx.stream));

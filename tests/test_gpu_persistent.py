@@ -310,3 +310,16 @@ def test_phase_times_of_label_propagation():
             assert st[name] > 0, name
     finally:
         hg.hg_destroy(h)
+
+
+@pytest.mark.parametrize("size,launches", [(20, 0), (4, 1)])
+def test_rating_launches_counts_launches(size, launches):
+    """Levels without a rated net launch no rating kernel."""
+    n = 2000
+    hgr = from_nets(n, np.arange(n).reshape(-1, size).tolist())
+    h = create(hgr, 1, factor=10, rating_max_net_size=10)
+    try:
+        hg.hg_coarsen_level(h, 2)
+        assert hg.hg_get_stats(h)["rating_launches"] == launches
+    finally:
+        hg.hg_destroy(h)
