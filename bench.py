@@ -815,7 +815,6 @@ def run_ours(args, world, rank, local):
                      "lp_gain_kernels": iagg["ms_lp_gain_kernels"] / ni,
                      "lp_select_kernels": iagg["ms_lp_select_kernels"] / ni,
                      "lp_apply_kernels": iagg["ms_lp_apply_kernels"] / ni,
-                     "timing_failures": int(iagg["timing_failures"]),
                      "from": f"{ni} instrumented steps"},
         "work_per_step": {key: int(agg[key] // args.steps) for key in (
             "rating_nodes", "rating_incidences", "rating_pin_visits", "lp_nodes", "lp_incidences",

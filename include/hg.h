@@ -122,9 +122,13 @@ typedef struct {
   int32_t community_detection;
 } hg_options;
 
-/* Per-phase device time (milliseconds, from CUDA events) and work counters,
- * accumulated since hg_create or the last hg_reset_stats.  Phases are only
- * timed when hg_enable_timing(h, 1) was called. */
+/* Per-phase device time (milliseconds) and work counters, accumulated since
+ * hg_create or the last hg_reset_stats.  Phases are only timed when
+ * hg_enable_timing(h, 1) was called: those that are launches of their own
+ * (transpose, contract, project, phi, initial, communities) with CUDA events on
+ * the handle's stream, those inside a kernel that runs a whole level (rating,
+ * approve, refresh, label propagation and its objective) by the kernel itself,
+ * from the GPU's nanosecond clock read by one block. */
 typedef struct {
   double ms_transpose;  /* incidence build (a1) */
   double ms_rating;     /* heavy-edge rating of all sub-rounds (a3) */
@@ -155,7 +159,7 @@ typedef struct {
   double ms_lp_apply_kernels;  /* move application phases (timing flag 2) */
   int64_t lp_moved_incidences; /* incident nets of the moved nodes */
   int64_t lp_passes;           /* label-propagation passes run */
-  int64_t timing_failures;     /* kernel-timing event pairs that could not be read */
+  int64_t timing_failures;     /* 0 (the phases of the kernels are timed on the device) */
   double ms_communities;       /* community detection (timing flag 1) */
   int64_t louvain_levels;      /* Louvain levels aggregated */
   int64_t louvain_rounds;      /* local-moving rounds */

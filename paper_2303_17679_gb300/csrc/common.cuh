@@ -276,7 +276,7 @@ struct Ctx {
   int num_sms = 0;
   int64_t* launches = nullptr;   // host counter
   bool timing = false;           // per-phase event timing (synchronizes at phase ends)
-  bool kernel_timing = false;    // event pair around every rating / gain launch (no sync)
+  bool kernel_timing = false;    // phase times inside the persistent kernels only
   cudaEvent_t sync_event = nullptr;  // blocking-sync event: waits sleep instead of spinning
   // Another call is at work on the device (inflight.cuh).
   bool shares_gpu() const {
@@ -438,7 +438,7 @@ int32_t detect_communities(const Ctx& cx, const Level& L, int S, uint64_t seed,
 
 struct RefineCounters {
   int64_t lp_incidences = 0, lp_nodes = 0, lp_gain_launches = 0, lp_moved_incidences = 0,
-          lp_passes = 0, timing_failures = 0;
+          lp_passes = 0;
   double ms_phi = 0, ms_gain = 0, ms_select = 0, ms_apply = 0, ms_objective = 0,
          ms_gain_kernels = 0, ms_select_kernels = 0, ms_apply_kernels = 0;
 };
@@ -524,40 +524,6 @@ struct EventTimer {
     }
   }
   ~EventTimer() { stop(); }
-};
-
-// Accumulates the summed duration of a set of kernel launches (each launch
-// bracketed by its own event pair) when timing is on; resolved by flush().
-struct KernelTimer {
-  const Ctx* cx;
-  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev;
-  explicit KernelTimer(const Ctx& c) : cx(&c) {}
-  void begin() {
-    if (!cx->kernel_timing) return;
-    cudaEvent_t a, b;
-    cudaEventCreate(&a);
-    cudaEventCreate(&b);
-    cudaEventRecord(a, cx->stream);
-    ev.push_back({a, b});
-  }
-  void end() {
-    if (!cx->kernel_timing || ev.empty()) return;
-    cudaEventRecord(ev.back().second, cx->stream);
-  }
-  double flush() {
-    double total = 0;
-    for (auto& p : ev) {
-      cudaEventSynchronize(p.second);
-      float ms = 0;
-      cudaEventElapsedTime(&ms, p.first, p.second);
-      total += ms;
-      cudaEventDestroy(p.first);
-      cudaEventDestroy(p.second);
-    }
-    ev.clear();
-    return total;
-  }
-  ~KernelTimer() { flush(); }
 };
 
 }  // namespace hgk

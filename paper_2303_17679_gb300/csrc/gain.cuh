@@ -34,13 +34,14 @@ struct WideRec {
 // One 32-byte load: a gather is bound by its requests, a line each.  The records
 // start on a 32-byte boundary (BUF_ALIGN).
 __device__ __forceinline__ WideRec load_wide(const int4* rec, int32_t e) {
-  unsigned w, o0, l0, x0, x1, o1, l1, x2;
+  unsigned r[8];  // w, ones, lam, 0 of either half
   asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(w), "=r"(o0), "=r"(l0), "=r"(x0), "=r"(x1), "=r"(o1), "=r"(l1), "=r"(x2)
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
                : "l"(rec + 2 * (int64_t)e)
                : "memory");
-  return WideRec{(int32_t)w, (unsigned long long)o0 | (unsigned long long)o1 << 32,
-                 (unsigned long long)l0 | (unsigned long long)l1 << 32};
+  return WideRec{(int32_t)r[0], (unsigned long long)r[1] | (unsigned long long)r[5] << 32,
+                 (unsigned long long)r[2] | (unsigned long long)r[6] << 32};
 }
 
 // Sum over the W lanes of the caller's group (W a power of two); the whole warp

@@ -115,9 +115,9 @@ struct PackedHash {
     val[i] = 0;
   }
   // the slot index when C was inserted by this call, else ADD_EXISTING / ADD_FULL
-  __device__ __forceinline__ int32_t add(int32_t C, uint32_t r, uint32_t max_probe = 0xFFFFFFFFu) {
+  __device__ __forceinline__ int32_t add(int32_t C, uint32_t r) {
     uint32_t h = slot_hash(C) & mask;
-    for (uint32_t probe = 0; probe <= mask && probe < max_probe; ++probe) {
+    for (uint32_t probe = 0; probe <= mask; ++probe) {
       int32_t k = key[h];
       bool fresh = false;
       if (k == EMPTY_KEY) {
@@ -152,10 +152,9 @@ struct WideHash {
     key[i] = EMPTY_KEY;
     val[i] = 0;
   }
-  __device__ __forceinline__ int32_t add(int32_t C, unsigned long long r,
-                                         uint32_t max_probe = 0xFFFFFFFFu) {
+  __device__ __forceinline__ int32_t add(int32_t C, unsigned long long r) {
     uint32_t h = slot_hash(C) & mask;
-    for (uint32_t probe = 0; probe <= mask && probe < max_probe; ++probe) {
+    for (uint32_t probe = 0; probe <= mask; ++probe) {
       int32_t k = key[h];
       bool fresh = false;
       if (k == EMPTY_KEY) {
@@ -277,7 +276,7 @@ __device__ __forceinline__ EachVisit<VT, ILP, F> each_visit(F f) {
 template <bool GRAPH, int ILP>
 __device__ __forceinline__ void resolve_batch(const RateArgs& A, int s, const int32_t (&q)[ILP],
                                               int2 (&ri)[ILP], int32_t cmu) {
-  if (!GRAPH) {
+  if constexpr (!GRAPH) {
 #pragma unroll
     for (int k = 0; k < ILP; ++k) ri[k] = q[k] >= 0 ? A.rinfo[q[k]] : make_int2(-1, 0);
     if (cmu >= 0) {
@@ -285,16 +284,16 @@ __device__ __forceinline__ void resolve_batch(const RateArgs& A, int s, const in
       for (int k = 0; k < ILP; ++k)
         if (ri[k].x >= 0 && A.pcomm[q[k]] != cmu) ri[k].x = -1;
     }
-    return;
-  }
-  int32_t C[ILP];
+  } else {
+    int32_t C[ILP];
 #pragma unroll
-  for (int k = 0; k < ILP; ++k)
-    C[k] = q[k] >= 0 && (cmu < 0 || A.comm[q[k]] == cmu) ? A.rep[q[k]] : -1;
+    for (int k = 0; k < ILP; ++k)
+      C[k] = q[k] >= 0 && (cmu < 0 || A.comm[q[k]] == cmu) ? A.rep[q[k]] : -1;
 #pragma unroll
-  for (int k = 0; k < ILP; ++k) {
-    const int2 cs = C[k] >= 0 ? A.cst[C[k]] : make_int2(0, 0);
-    ri[k] = make_int2(C[k], cs.y == s ? 0x7fffffff : cs.x);
+    for (int k = 0; k < ILP; ++k) {
+      const int2 cs = C[k] >= 0 ? A.cst[C[k]] : make_int2(0, 0);
+      ri[k] = make_int2(C[k], cs.y == s ? 0x7fffffff : cs.x);
+    }
   }
 }
 
@@ -435,37 +434,38 @@ __device__ __forceinline__ TeamWalk team_walk(int32_t beg, int32_t end, int wt, 
 template <bool GRAPH, typename VT, int ILP, typename Visit>
 __device__ __forceinline__ int32_t rate_group_raw(const RateArgs& A, int32_t g0, int32_t end,
                                                   int wt, int TW, int32_t& run, Visit& visit_batch) {
-  if (GRAPH) return graph_walk<VT, ILP>(A, g0, min(g0 + 32, end), wt, TW, visit_batch);
-  const int32_t j = g0 + lane_id();
-  return walk_group<VT, ILP>(inc_meta<VT>(A, j < end ? j : -1), wt, TW, run, visit_batch);
+  if constexpr (GRAPH) {
+    return graph_walk<VT, ILP>(A, g0, min(g0 + 32, end), wt, TW, visit_batch);
+  } else {
+    const int32_t j = g0 + lane_id();
+    return walk_group<VT, ILP>(inc_meta<VT>(A, j < end ? j : -1), wt, TW, run, visit_batch);
+  }
 }
 
 // The groups g0 = first, first + step, ... (< end) of I(u), walked as by
 // rate_group_raw with the load of the next group's net metadata issued
-// before the current group is walked.
+// before the current group is walked (graph levels: one walk over all of it).
 template <bool GRAPH, typename VT, int ILP, typename Visit>
 __device__ __forceinline__ int64_t rate_groups_raw(const RateArgs& A, int32_t first, int32_t end,
                                                    int32_t step, int wt, int TW, int32_t& run,
                                                    Visit& visit_batch) {
-  const int lane = lane_id();
-  int64_t visits = 0;
   if (first >= end) return 0;
-  if (GRAPH) {
-    if (step == 32) return graph_walk<VT, ILP>(A, first, end, wt, TW, visit_batch);
-    for (int32_t g = first; g < end; g += step)
-      visits += graph_walk<VT, ILP>(A, g, min(g + 32, end), wt, TW, visit_batch);
+  if constexpr (GRAPH) {
+    return graph_walk<VT, ILP>(A, first, end, wt, TW, visit_batch);
+  } else {
+    const int lane = lane_id();
+    int64_t visits = 0;
+    int32_t g = first;
+    NetMeta<VT> m = inc_meta<VT>(A, g + lane < end ? g + lane : -1);
+    while (g < end) {
+      const int32_t gn = g + step;
+      const NetMeta<VT> mn = inc_meta<VT>(A, gn + lane < end ? gn + lane : -1);
+      visits += walk_group<VT, ILP>(m, wt, TW, run, visit_batch);
+      m = mn;
+      g = gn;
+    }
     return visits;
   }
-  int32_t g = first;
-  NetMeta<VT> m = inc_meta<VT>(A, g + lane < end ? g + lane : -1);
-  while (g < end) {
-    const int32_t gn = g + step;
-    const NetMeta<VT> mn = inc_meta<VT>(A, gn + lane < end ? gn + lane : -1);
-    visits += walk_group<VT, ILP>(m, wt, TW, run, visit_batch);
-    m = mn;
-    g = gn;
-  }
-  return visits;
 }
 
 // rate_group_raw / rate_groups_raw with the admissibility filter of
