@@ -99,7 +99,10 @@ struct TeamLane {
 // (Shared-memory counters with one atomic per block of Lambda(e), which k > 16
 // used before, serialise on coarse levels, whose nets touch the same blocks:
 // 37 us per sub-round at k = 64 and 31M pins, 60 us with lane groups.)
-// All sums are below 2^31 (the total net weight).
+// Every sum is over distinct nets with one sign (bw subtracts them, and in the k > 32
+// form adds others), so it lies between -W and W, W the total net weight: hg_create
+// refuses W >= 2^31, and contraction keeps or drops nets but never adds weight.  So
+// 32 bits hold them on every level, the atomics of a split node included.
 template <bool GRAPH, int K, int H>
 struct Gain {
   int32_t acc[K];

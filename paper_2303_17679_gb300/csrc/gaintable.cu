@@ -183,7 +183,7 @@ __device__ __forceinline__ void gt_row(const int32_t* __restrict__ inets,
   const int from = on ? part[u] : 0, from_h = from - 32 * lane.half;
   Gain<GRAPH, K, H> g;
   g.init();
-  int32_t wsum = 0;
+  int32_t wsum = 0;  // of distinct nets: below 2^31, as the sums of gain.cuh
   const int32_t steps = __reduce_max_sync(FULL, end - beg);
   for (int32_t x = lane.i; x - lane.i < steps; x += 2 * L::SHARE) {
     const int32_t j0 = beg + x, j1 = j0 + L::SHARE;

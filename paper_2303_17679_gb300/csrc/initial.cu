@@ -71,7 +71,8 @@ constexpr int32_t PACK_MAX_C = 1 << 20;
 __device__ __forceinline__ void assign_in_order(const int2* __restrict__ order, int32_t n, int k,
                                                 bool packed, int32_t* __restrict__ part) {
   const int lane = lane_id();
-  // weight << 6 | block, or the weight alone; all ones for no block
+  // weight << 6 | block, or the weight alone; all ones for no block.  Unpacked, a
+  // block's weight is at most c(V) < 2^31 (hg_create).
   unsigned w0 = lane < k ? (packed ? (unsigned)lane : 0u) : ~0u;
   unsigned w1 = lane + 32 < k ? (packed ? (unsigned)lane + 32u : 0u) : ~0u;
   int2 next = lane < n ? order[lane] : make_int2(0, 0);

@@ -443,7 +443,8 @@ __device__ __forceinline__ void gain_item_wide(const LpArgs& A, int par, const i
   finish_item<false, 32, 2>(A, par, it, from, g);
 }
 
-// Class-0 nodes for k > 32, before gain_groups: no gain of u exceeds
+// Class-0 nodes for k > 32, before gain_groups (32-bit sums: gain.cuh): no gain of
+// u exceeds
 //   w(nets where u is the only pin of its block) - w(nets inside its block)
 // (a net outside every other block counts against every target), so only the
 // nodes where that is positive are kept, in the block's list.  Eight lanes per
@@ -675,7 +676,9 @@ __device__ void bitonic_sort2(unsigned long long* a, int Pa, unsigned long long*
 
 // Weight prefixes of both directions from one block-wide scan over the
 // concatenation of their sorted moves: A[x] = weight of the first x moves
-// a -> b (x = 0..na), B[x] likewise for b -> a.
+// a -> b (x = 0..na), B[x] likewise for b -> a.  A node is in one direction at most,
+// so all of them together weigh c(V) < 2^31 at most (hg_create) and 32 bits do;
+// their differences against the slack are taken in 64.
 __device__ void weight_prefix2(const unsigned long long* ka, int na, const unsigned long long* kb,
                                int nb, const int32_t* __restrict__ c, int32_t* A, int32_t* B,
                                unsigned* barrier) {

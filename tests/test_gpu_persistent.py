@@ -323,3 +323,42 @@ def test_rating_launches_counts_launches(size, launches):
         assert hg.hg_get_stats(h)["rating_launches"] == launches
     finally:
         hg.hg_destroy(h)
+
+
+# hg_create refuses total net or node weights of 2^31 and more, which is what makes
+# 32-bit sums enough; a node in every net, many nets (one item per 128 to 1024 of
+# them) and few
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("m,k", [(7, 2), (3000, 8), (3000, 40), (40, 33)])
+def test_largest_total_weights(oracle_mod, m, k, graph):
+    n, top = 4000, (1 << 31) - 1
+    rng = np.random.default_rng(m + k)
+    size = 2 if graph else 4
+    nets = [[0, *rng.choice(np.arange(1, n), size=size - 1, replace=False).tolist()]
+            for _ in range(m)]
+
+    def spread(count):
+        w = np.full(count, top // count, np.int64)
+        w[-1] += top - w.sum()
+        return w.astype(np.int32)
+
+    hgr = from_nets(n, nets, spread(m), spread(n))
+    assert hgr.net_w.sum(dtype=np.int64) == top == hgr.node_w.sum(dtype=np.int64)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda()  # noqa: E731
+    for part0 in (rng.integers(0, k, size=n).astype(np.int32),
+                  np.where(np.arange(n) == 0, 1, 0).astype(np.int32)):
+        ref = oracle_mod.lp_refine(hgr, k, part0, 10**9, 16, 3, 0, 3)
+        h = create(hgr, 3, lp_block_min_deg=64)
+        try:
+            d = dev(part0)
+            assert hg.hg_lp_refine(h, 0, k, 10**9, 3, d) == (ref["objective"], ref["moves"])
+            assert np.array_equal(d.cpu().numpy(), ref["part"])
+            b = torch.zeros(n, dtype=torch.int64, device="cuda")
+            p = torch.zeros((n, k), dtype=torch.int64, device="cuda")
+            hg.hg_gain_table(h, 0, k, dev(part0), b, p)
+            wb, wp = oracle_mod.gain_table(hgr, k, part0)
+            assert np.array_equal(b.cpu().numpy(), wb) and np.array_equal(p.cpu().numpy(), wp)
+            hg.hg_initial_partition(h, 0, k, d)
+            assert np.array_equal(d.cpu().numpy(), oracle_mod.initial_partition(hgr.node_w, k, 3))
+        finally:
+            hg.hg_destroy(h)
