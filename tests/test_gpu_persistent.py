@@ -362,3 +362,24 @@ def test_largest_total_weights(oracle_mod, m, k, graph):
             assert np.array_equal(d.cpu().numpy(), oracle_mod.initial_partition(hgr.node_w, k, 3))
         finally:
             hg.hg_destroy(h)
+
+
+@pytest.mark.parametrize("k", [9, 32])
+def test_directions_longer_than_the_shared_buffers(oracle_mod, k):
+    """For k > 8 the selection sorts up to 2048 moves of a direction in shared memory.
+    More come from the direction's key list and the overflow list into global keys at
+    twice the direction's offset, with their weight prefixes.  All moves are between
+    blocks 0 and 1."""
+    n, seed, eps = 400_000, 7, 2_000_000_000
+    hgr = synth.random_uniform(61 + k, n, n)
+    part0 = synth.uniform_ints(n + k, n, 0, 1)
+    _, mv = oracle_mod.lp_subround(hgr, k, part0, eps, 16, seed, 0, 0, 0)
+    assert np.bincount(mv["src"] * k + mv["dst"], minlength=k * k).max() > 2048
+    ref = oracle_mod.lp_refine(hgr, k, part0, eps, 16, seed, 0, 1)
+    h = create(hgr, seed)
+    try:
+        d = torch.from_numpy(np.ascontiguousarray(part0, np.int32)).cuda()
+        assert hg.hg_lp_refine(h, 0, k, eps, 1, d) == (ref["objective"], ref["moves"])
+        assert np.array_equal(d.cpu().numpy(), ref["part"])
+    finally:
+        hg.hg_destroy(h)
