@@ -452,8 +452,9 @@ struct PinState {
 };
 
 // What goes with the pin counts: nothing and no counts either (graph levels in
-// label propagation), Lambda, or the packed records of gain.cuh.
-enum class PinMasks { none, lambda, records };
+// label propagation), Lambda with or without the counts, or the packed records of
+// gain.cuh.
+enum class PinMasks { none, lambda_only, lambda, records };
 void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, PinState& st,
                      PinMasks masks);
 

@@ -26,7 +26,8 @@ __global__ void k_project(const int32_t* __restrict__ map, const int32_t* __rest
 // Phi, and Lambda or the packed records (gain.cuh), of every net: a net's pins
 // are counted per block in shared memory by eight lanes (up to COUNT_SMALL
 // pins), a warp (up to COUNT_WARP) or the block, which then write the net's row
-// of Phi and its masks once.  Bound by the row writes on levels of small nets (m
+// of Phi and its masks once; nets of more than COUNT_HUGE pins by chunks over the
+// grid, added to the row (as one block's, a net of 20M pins took 24 ms).  Bound by the row writes on levels of small nets (m
 // k words), by the pins' block ids on the others.  (A thread per pin that found
 // equal (net, block) pairs by a match over the warp and added them with atomics to
 // a cleared table, and a second pass for the records, took 0.53 + 0.23 ms per
@@ -36,20 +37,25 @@ constexpr int COUNT_NETS = 32 / COUNT_LANES;
 constexpr int32_t COUNT_SMALL = 64, COUNT_WARP = 2048;
 constexpr int COUNT_STRIDE = HG_MAX_K + 1;  // a warp's sets start in different banks
 constexpr int COUNT_BIG = 64;               // nets a block keeps for later
+constexpr int32_t COUNT_HUGE = 32768, COUNT_CHUNK = 8192;
 
 struct CountArgs {
   const int32_t *eoff, *pins, *part, *w;
   int32_t m;
   int k;
-  int32_t* phi;
+  int32_t* phi;             // when asked for
   unsigned long long* lam;  // or
   int4* rec;
+  // chunks of the nets above COUNT_HUGE: {net, its first chunk}, their number, and
+  // the chunks done per net (at its first chunk)
+  int2* chunks;
+  int32_t *nchunks, *done;
 };
 
 // Writes the row of net e from `sets` sets of counters `stride` apart and clears
 // them; the lanes l = 0 .. W-1 of the caller share the blocks.  The masks of
 // their blocks are returned.
-template <int W>
+template <int W, bool PHI>
 __device__ __forceinline__ void write_row(const CountArgs& A, int32_t e, int32_t* cnt, int sets,
                                           int l, unsigned long long& ones,
                                           unsigned long long& lam) {
@@ -60,7 +66,7 @@ __device__ __forceinline__ void write_row(const CountArgs& A, int32_t e, int32_t
       c += cnt[x * COUNT_STRIDE + t];
       cnt[x * COUNT_STRIDE + t] = 0;
     }
-    A.phi[(int64_t)e * A.k + t] = c;
+    if (PHI) A.phi[(int64_t)e * A.k + t] = c;
     if (c == 1) ones |= 1ull << t;
     if (c > 0) lam |= 1ull << t;
   }
@@ -103,7 +109,9 @@ __device__ __forceinline__ void count_pins(const CountArgs& A, int32_t b, int32_
   }
 }
 
-__global__ void __launch_bounds__(COUNT_WARPS * 32) k_pin_counts(CountArgs A) {
+// PHI: the counts themselves, else only Lambda.
+template <bool PHI>
+__global__ void __launch_bounds__(COUNT_WARPS * 32, 8) k_pin_counts(CountArgs A) {
   __shared__ int32_t s_cnt[COUNT_WARPS * COUNT_NETS * COUNT_STRIDE];
   __shared__ int32_t s_big[COUNT_BIG];
   __shared__ int s_nbig;
@@ -119,7 +127,7 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32) k_pin_counts(CountArgs A) {
     count_pins(A, b, sz, lane, 32, mine);
     __syncwarp();
     unsigned long long ones, lam;
-    write_row<32>(A, e, sets, COUNT_NETS, lane, ones, lam);
+    write_row<32, PHI>(A, e, sets, COUNT_NETS, lane, ones, lam);
     ones = or_lanes<32>(ones);
     lam = or_lanes<32>(lam);
     if (lane == 0) write_masks(A, e, ones, lam);
@@ -134,7 +142,7 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32) k_pin_counts(CountArgs A) {
     if (sz <= COUNT_SMALL) count_pins(A, b, sz, sub, COUNT_LANES, mine);
     __syncwarp();
     unsigned long long ones = 0, lam = 0;
-    if (on && sz <= COUNT_SMALL) write_row<COUNT_LANES>(A, (int32_t)e, mine, 1, sub, ones, lam);
+    if (on && sz <= COUNT_SMALL) write_row<COUNT_LANES, PHI>(A, (int32_t)e, mine, 1, sub, ones, lam);
     __syncwarp();
     ones = or_lanes<COUNT_LANES>(ones);
     lam = or_lanes<COUNT_LANES>(lam);
@@ -145,6 +153,18 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32) k_pin_counts(CountArgs A) {
       const int32_t we = (int32_t)(e0 + l / COUNT_LANES);
       const int32_t wb = __shfl_sync(FULL, b, l), wsz = __shfl_sync(FULL, sz, l);
       int slot = COUNT_BIG;
+      if (wsz > COUNT_HUGE) {
+        const int32_t count = (wsz + COUNT_CHUNK - 1) / COUNT_CHUNK;
+        int32_t first = 0;
+        if (lane == 0) first = atomicAdd(A.nchunks, count);
+        first = __shfl_sync(FULL, first, 0);
+        for (int32_t c = lane; c < count; c += 32) A.chunks[first + c] = make_int2(we, first);
+        if (PHI)
+          for (int t = lane; t < A.k; t += 32) A.phi[(int64_t)we * A.k + t] = 0;
+        else if (lane == 0)
+          A.lam[we] = 0;
+        continue;
+      }
       if (wsz > COUNT_WARP) {
         if (lane == 0) slot = atomicAdd(&s_nbig, 1);
         slot = __shfl_sync(FULL, slot, 0);
@@ -161,11 +181,60 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32) k_pin_counts(CountArgs A) {
     if (threadIdx.x == 0) s_ones = s_lam = 0;
     __syncthreads();
     unsigned long long ones, lam;
-    write_row<COUNT_WARPS * 32>(A, e, s_cnt, COUNT_WARPS * COUNT_NETS, threadIdx.x, ones, lam);
+    write_row<COUNT_WARPS * 32, PHI>(A, e, s_cnt, COUNT_WARPS * COUNT_NETS, threadIdx.x, ones, lam);
     if (ones) atomicOr(&s_ones, ones);
     if (lam) atomicOr(&s_lam, lam);
     __syncthreads();
     if (threadIdx.x == 0) write_masks(A, e, s_ones, s_lam);
+    __syncthreads();
+  }
+}
+
+// The chunks listed by k_pin_counts: a block counts one in shared memory and adds it
+// to the net's row; the last chunk of a net writes its masks.
+template <bool PHI>
+__global__ void __launch_bounds__(COUNT_WARPS * 32) k_pin_counts_huge(CountArgs A) {
+  __shared__ int32_t s_cnt[COUNT_WARPS * COUNT_STRIDE];
+  __shared__ unsigned long long s_ones, s_lam;
+  __shared__ int s_last;
+  for (int i = threadIdx.x; i < COUNT_WARPS * COUNT_STRIDE; i += blockDim.x) s_cnt[i] = 0;
+  __syncthreads();
+  int32_t* mine = s_cnt + warp_in_block() * COUNT_STRIDE;
+  const int32_t n = *A.nchunks;
+  const int t = threadIdx.x;
+  for (int32_t x = blockIdx.x; x < n; x += gridDim.x) {
+    const int2 it = A.chunks[x];
+    const int32_t e = it.x, b = A.eoff[e], sz = A.eoff[e + 1] - b;
+    const int32_t at = (x - it.y) * COUNT_CHUNK, left = min(COUNT_CHUNK, sz - at);
+    count_pins(A, b + at, left, t, COUNT_WARPS * 32, mine);
+    if (t == 0) s_ones = s_lam = 0;
+    __syncthreads();
+    int32_t c = 0;
+    if (t < A.k)
+      for (int w = 0; w < COUNT_WARPS; ++w) {
+        c += s_cnt[w * COUNT_STRIDE + t];
+        s_cnt[w * COUNT_STRIDE + t] = 0;
+      }
+    if (!PHI) {
+      if (c) atomicOr(&A.lam[e], 1ull << t);
+      __syncthreads();
+      continue;
+    }
+    if (c) atomicAdd(&A.phi[(int64_t)e * A.k + t], c);
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_last = atomicAdd(&A.done[it.y], 1) == (sz + COUNT_CHUNK - 1) / COUNT_CHUNK - 1;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      if (t < A.k) {
+        const int32_t all = __ldcg(&A.phi[(int64_t)e * A.k + t]);
+        if (all == 1) atomicOr(&s_ones, 1ull << t);
+        if (all > 0) atomicOr(&s_lam, 1ull << t);
+      }
+      __syncthreads();
+      if (t == 0) write_masks(A, e, s_ones, s_lam);
+    }
     __syncthreads();
   }
 }
@@ -219,15 +288,34 @@ void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, 
   st.bw.alloc(&cx.alloc, (size_t)k);
   HG_CUDA(cudaMemsetAsync(st.bw.p, 0, st.bw.bytes(), cx.stream));
   if (masks != PinMasks::none) {
-    st.phi.alloc(&cx.alloc, (size_t)L.m * k + 1);
-    if (masks == PinMasks::lambda) st.lam.alloc(&cx.alloc, (size_t)L.m + 1);
+    if (masks != PinMasks::lambda_only) st.phi.alloc(&cx.alloc, (size_t)L.m * k + 1);
+    if (masks != PinMasks::records) st.lam.alloc(&cx.alloc, (size_t)L.m + 1);
     else st.rec.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1) * (k > 32 ? 2 : 1));
     if (L.m > 0) {
-      const CountArgs A{L.eoff.p, L.pins.p, part, L.w.p, L.m, k, st.phi.p, st.lam.p, st.rec.p};
-      k_pin_counts<<<grid_for(L.m, COUNT_WARPS * COUNT_NETS, cx.num_sms, 8), COUNT_WARPS * 32, 0,
-                     cx.stream>>>(A);
+      CountArgs A{L.eoff.p, L.pins.p, part,     L.w.p,   L.m,    k,
+                  st.phi.p, st.lam.p, st.rec.p, nullptr, nullptr, nullptr};
+      DBuf<int2> chunks;
+      DBuf<int32_t> done;  // and the number of chunks
+      if (L.p > COUNT_HUGE) {
+        const size_t cap = (size_t)(L.p / COUNT_CHUNK + L.p / COUNT_HUGE) + 1;
+        chunks.alloc(&cx.alloc, cap);
+        done.alloc(&cx.alloc, cap + 1);
+        HG_CUDA(cudaMemsetAsync(done.p, 0, done.bytes(), cx.stream));
+        A.chunks = chunks.p;
+        A.nchunks = done.p + cap;
+        A.done = done.p;
+      }
+      const bool phi = st.phi.p != nullptr;
+      (phi ? k_pin_counts<true> : k_pin_counts<false>)<<<
+          grid_for(L.m, COUNT_WARPS * COUNT_NETS, cx.num_sms, 8), COUNT_WARPS * 32, 0,
+          cx.stream>>>(A);
       check_launch("pin_counts");
-      if (cx.launches) *cx.launches += 1;
+      if (L.p > COUNT_HUGE) {
+        (phi ? k_pin_counts_huge<true> : k_pin_counts_huge<false>)<<<
+            grid_for(L.p, COUNT_CHUNK, cx.num_sms, 4), COUNT_WARPS * 32, 0, cx.stream>>>(A);
+        check_launch("pin_counts_huge");
+      }
+      if (cx.launches) *cx.launches += 1 + (L.p > COUNT_HUGE);
     }
   }
   k_block_weights<<<grid_for(L.n, 256, cx.num_sms, 4), 256, 0, cx.stream>>>(part, L.c.p, L.n, k,
@@ -254,7 +342,7 @@ int64_t objective_from_lambda(const Ctx& cx, const Level& L, const unsigned long
 
 int64_t objective_of(const Ctx& cx, const Level& L, int k, const int32_t* part) {
   PinState st;
-  build_pin_state(cx, L, k, part, st, PinMasks::lambda);
+  build_pin_state(cx, L, k, part, st, PinMasks::lambda_only);
   return objective_from_lambda(cx, L, st.lam.p);
 }
 

@@ -383,3 +383,36 @@ def test_directions_longer_than_the_shared_buffers(oracle_mod, k):
         assert np.array_equal(d.cpu().numpy(), ref["part"])
     finally:
         hg.hg_destroy(h)
+
+
+def nets_around(n, sizes, seed, rest=3000):
+    """A net of each size and `rest` nets of three pins."""
+    rng = np.random.default_rng(seed)
+    nets = [rng.choice(n, size=s, replace=False).tolist() for s in sizes]
+    nets += [rng.choice(n, size=3, replace=False).tolist() for _ in range(rest)]
+    order = rng.permutation(len(nets))
+    return from_nets(n, [nets[i] for i in order], rng.integers(1, 9, size=len(nets)),
+                     rng.integers(1, 4, size=n))
+
+
+# nets around the size above which chunks of a net are counted by different blocks
+@pytest.mark.parametrize("k", [1, 5, 64])
+def test_pin_counts_of_huge_nets(oracle_mod, k):
+    n = 60_000
+    hgr = nets_around(n, [2048, 2049, 32_767, 32_768, 32_769, 40_960, 40_961, 60_000], k)
+    part = np.random.default_rng(k).integers(0, max(1, k - 1), size=n).astype(np.int32)
+    part[:3] = k - 1  # a block of few pins
+    h = create(hgr, 1)
+    try:
+        d = torch.from_numpy(part).cuda()
+        phi, lam = oracle_mod.pin_counts(hgr, k, part)
+        got = hg.hg_pin_counts(h, 0, k, d)
+        assert np.array_equal(got[0], phi) and np.array_equal(got[1], lam)
+        assert np.array_equal(got[2], oracle_mod.block_weights(hgr, k, part))
+        assert hg.hg_objective(h, 0, k, d) == oracle_mod.objective(hgr, k, part)
+        if k > 1:
+            ref = oracle_mod.lp_refine(hgr, k, part, 50000, 16, 1, 0, 2)
+            assert hg.hg_lp_refine(h, 0, k, 50000, 2, d) == (ref["objective"], ref["moves"])
+            assert np.array_equal(d.cpu().numpy(), ref["part"])
+    finally:
+        hg.hg_destroy(h)
