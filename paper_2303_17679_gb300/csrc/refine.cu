@@ -25,8 +25,8 @@ __global__ void k_project(const int32_t* __restrict__ map, const int32_t* __rest
 
 // Phi, and Lambda or the packed records (gain.cuh), of every net: a net's pins
 // are counted per block in shared memory by eight lanes (up to COUNT_SMALL
-// pins), a warp (up to COUNT_WARP) or the block, which then write the net's row
-// of Phi and its masks once; nets of more than COUNT_HUGE pins by chunks over the
+// pins) or a warp (up to COUNT_WARP), which then write the net's row of Phi and its
+// masks once; those of larger nets by chunks over the
 // grid, added to the row (as one block's, a net of 20M pins took 24 ms).  Bound by the row writes on levels of small nets (m
 // k words), by the pins' block ids on the others.  (A thread per pin that found
 // equal (net, block) pairs by a match over the warp and added them with atomics to
@@ -36,8 +36,7 @@ constexpr int COUNT_WARPS = 8, COUNT_LANES = 8;
 constexpr int COUNT_NETS = 32 / COUNT_LANES;
 constexpr int32_t COUNT_SMALL = 64, COUNT_WARP = 2048;
 constexpr int COUNT_STRIDE = HG_MAX_K + 1;  // a warp's sets start in different banks
-constexpr int COUNT_BIG = 64;               // nets a block keeps for later
-constexpr int32_t COUNT_HUGE = 32768, COUNT_CHUNK = 8192;
+constexpr int32_t COUNT_CHUNK = 4096;
 
 struct CountArgs {
   const int32_t *eoff, *pins, *part, *w;
@@ -46,7 +45,7 @@ struct CountArgs {
   int32_t* phi;             // when asked for
   unsigned long long* lam;  // or
   int4* rec;
-  // chunks of the nets above COUNT_HUGE: {net, its first chunk}, their number, and
+  // chunks of the nets above COUNT_WARP: {net, its first chunk}, their number, and
   // the chunks done per net (at its first chunk)
   int2* chunks;
   int32_t *nchunks, *done;
@@ -113,15 +112,11 @@ __device__ __forceinline__ void count_pins(const CountArgs& A, int32_t b, int32_
 template <bool PHI>
 __global__ void __launch_bounds__(COUNT_WARPS * 32, 8) k_pin_counts(CountArgs A) {
   __shared__ int32_t s_cnt[COUNT_WARPS * COUNT_NETS * COUNT_STRIDE];
-  __shared__ int32_t s_big[COUNT_BIG];
-  __shared__ int s_nbig;
-  __shared__ unsigned long long s_ones, s_lam;
   const int lane = lane_id(), sub = lane % COUNT_LANES, grp = lane / COUNT_LANES;
   int32_t* sets = s_cnt + warp_in_block() * COUNT_NETS * COUNT_STRIDE;
   int32_t* mine = sets + grp * COUNT_STRIDE;
   for (int i = threadIdx.x; i < COUNT_WARPS * COUNT_NETS * COUNT_STRIDE; i += blockDim.x)
     s_cnt[i] = 0;
-  if (threadIdx.x == 0) s_nbig = 0;
   __syncthreads();
   auto by_warp = [&](int32_t e, int32_t b, int32_t sz) {
     count_pins(A, b, sz, lane, 32, mine);
@@ -152,8 +147,7 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 8) k_pin_counts(CountArgs A)
       const int l = __ffs(rest) - 1;
       const int32_t we = (int32_t)(e0 + l / COUNT_LANES);
       const int32_t wb = __shfl_sync(FULL, b, l), wsz = __shfl_sync(FULL, sz, l);
-      int slot = COUNT_BIG;
-      if (wsz > COUNT_HUGE) {
+      if (wsz > COUNT_WARP) {
         const int32_t count = (wsz + COUNT_CHUNK - 1) / COUNT_CHUNK;
         int32_t first = 0;
         if (lane == 0) first = atomicAdd(A.nchunks, count);
@@ -165,28 +159,8 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 8) k_pin_counts(CountArgs A)
           A.lam[we] = 0;
         continue;
       }
-      if (wsz > COUNT_WARP) {
-        if (lane == 0) slot = atomicAdd(&s_nbig, 1);
-        slot = __shfl_sync(FULL, slot, 0);
-        if (slot < COUNT_BIG && lane == 0) s_big[slot] = we;
-      }
-      if (slot >= COUNT_BIG) by_warp(we, wb, wsz);
+      by_warp(we, wb, wsz);
     }
-  }
-  __syncthreads();
-  const int big = min(s_nbig, COUNT_BIG);
-  for (int x = 0; x < big; ++x) {
-    const int32_t e = s_big[x], b = A.eoff[e], sz = A.eoff[e + 1] - b;
-    count_pins(A, b, sz, threadIdx.x, COUNT_WARPS * 32, mine);
-    if (threadIdx.x == 0) s_ones = s_lam = 0;
-    __syncthreads();
-    unsigned long long ones, lam;
-    write_row<COUNT_WARPS * 32, PHI>(A, e, s_cnt, COUNT_WARPS * COUNT_NETS, threadIdx.x, ones, lam);
-    if (ones) atomicOr(&s_ones, ones);
-    if (lam) atomicOr(&s_lam, lam);
-    __syncthreads();
-    if (threadIdx.x == 0) write_masks(A, e, s_ones, s_lam);
-    __syncthreads();
   }
 }
 
@@ -296,8 +270,8 @@ void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, 
                   st.phi.p, st.lam.p, st.rec.p, nullptr, nullptr, nullptr};
       DBuf<int2> chunks;
       DBuf<int32_t> done;  // and the number of chunks
-      if (L.p > COUNT_HUGE) {
-        const size_t cap = (size_t)(L.p / COUNT_CHUNK + L.p / COUNT_HUGE) + 1;
+      if (L.p > COUNT_WARP) {
+        const size_t cap = (size_t)(L.p / COUNT_CHUNK + L.p / COUNT_WARP) + 1;
         chunks.alloc(&cx.alloc, cap);
         done.alloc(&cx.alloc, cap + 1);
         HG_CUDA(cudaMemsetAsync(done.p, 0, done.bytes(), cx.stream));
@@ -310,12 +284,12 @@ void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, 
           grid_for(L.m, COUNT_WARPS * COUNT_NETS, cx.num_sms, 8), COUNT_WARPS * 32, 0,
           cx.stream>>>(A);
       check_launch("pin_counts");
-      if (L.p > COUNT_HUGE) {
+      if (L.p > COUNT_WARP) {
         (phi ? k_pin_counts_huge<true> : k_pin_counts_huge<false>)<<<
             grid_for(L.p, COUNT_CHUNK, cx.num_sms, 4), COUNT_WARPS * 32, 0, cx.stream>>>(A);
         check_launch("pin_counts_huge");
       }
-      if (cx.launches) *cx.launches += 1 + (L.p > COUNT_HUGE);
+      if (cx.launches) *cx.launches += 1 + (L.p > COUNT_WARP);
     }
   }
   k_block_weights<<<grid_for(L.n, 256, cx.num_sms, 4), 256, 0, cx.stream>>>(part, L.c.p, L.n, k,

@@ -399,7 +399,7 @@ def nets_around(n, sizes, seed, rest=3000):
 @pytest.mark.parametrize("k", [1, 5, 64])
 def test_pin_counts_of_huge_nets(oracle_mod, k):
     n = 60_000
-    hgr = nets_around(n, [2048, 2049, 32_767, 32_768, 32_769, 40_960, 40_961, 60_000], k)
+    hgr = nets_around(n, [2048, 2049, 4096, 4097, 8192, 8193, 40_960, 60_000], k)
     part = np.random.default_rng(k).integers(0, max(1, k - 1), size=n).astype(np.int32)
     part[:3] = k - 1  # a block of few pins
     h = create(hgr, 1)
