@@ -74,12 +74,23 @@ __device__ __forceinline__ void write_rec(int4* rec, int64_t e, int k, int32_t w
                                (int32_t)(uint32_t)(x.s >> (32 * h)), 0);
 }
 
-// Records of the nets of up to GT_BIG_NET pins; larger ones are listed.  The
-// partition has been checked.
+// Lists the chunks of GT_BIG_NET pins of a larger net, {net, first of its chunks}
+// each (one thread).
+__device__ __forceinline__ void list_chunks(int32_t e, int32_t sz, int2* chunks, int32_t* nchunks) {
+  const int32_t count = (sz + GT_BIG_NET - 1) / GT_BIG_NET;
+  const int32_t first = atomicAdd(nchunks, count);
+  for (int32_t c = 0; c < count; ++c) chunks[first + c] = make_int2(e, first);
+}
+
+// At most that many chunks on a level of p pins.
+size_t chunk_cap(int64_t p) { return 2 * (size_t)(p / GT_BIG_NET) + 1; }
+
+// Records of the nets of up to GT_BIG_NET pins; the chunks of larger ones are
+// listed.  The partition has been checked.
 __global__ void __launch_bounds__(GT_WARPS * 32)
 k_gt_records(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
              const int32_t* __restrict__ w, const int32_t* __restrict__ part, int32_t m, int k,
-             int4* __restrict__ rec, int32_t* __restrict__ big, int32_t* __restrict__ nbig) {
+             int4* __restrict__ rec, int2* __restrict__ chunks, int32_t* __restrict__ nchunks) {
   const int lane = lane_id(), sub = lane % SUB_G;
   const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
   for (int64_t e0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; e0 < m; e0 += stride) {
@@ -104,7 +115,7 @@ k_gt_records(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
       const int64_t we = e0 + l / SUB_G;
       const int32_t wb = __shfl_sync(FULL, b, l), ws = __shfl_sync(FULL, sz, l);
       if (ws > GT_BIG_NET) {
-        if (lane == 0) big[atomicAdd(nbig, 1)] = (int32_t)we;
+        if (lane == 0) list_chunks((int32_t)we, ws, chunks, nchunks);
         continue;
       }
       Seen y;
@@ -136,35 +147,35 @@ __device__ __forceinline__ Seen block_seen(Seen x) {
   return y;
 }
 
-// Records of the listed larger nets: chunks of GT_BIG_NET pins over the grid,
-// joined in acc (two words per net, then a count of finished chunks).
+// Records of the larger nets, a block per listed chunk (whole nets one after the
+// other, their chunks over the grid, left two blocks at work on nets of two chunks:
+// 54 ms for 5000 of them, 0.5 now), joined in three words per net at its first
+// chunk: seen, seen twice and the chunks done.
 __global__ void __launch_bounds__(GT_BIG_THREADS)
 k_gt_records_big(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
                  const int32_t* __restrict__ w, const int32_t* __restrict__ part, int k,
-                 int4* __restrict__ rec, const int32_t* __restrict__ big,
-                 const int32_t* __restrict__ nbig, Mask* __restrict__ acc) {
-  const int32_t cnt = *nbig;
-  for (int32_t i = 0; i < cnt; ++i) {
-    const int32_t e = big[i];
-    const int32_t b = eoff[e], sz = eoff[e + 1] - b;
-    const int32_t chunks = (sz + GT_BIG_NET - 1) / GT_BIG_NET;
-    for (int32_t c = blockIdx.x; c < chunks; c += gridDim.x) {
-      Seen x;
-      for (int64_t q = (int64_t)c * GT_BIG_NET + threadIdx.x;
-           q < sz && q < (int64_t)(c + 1) * GT_BIG_NET; q += blockDim.x)
-        x.add(part[pins[b + q]]);
-      x = block_seen(x);
-      if (threadIdx.x == 0) {
-        const Mask before = atomicOr(&acc[3 * (int64_t)i], x.s);
-        atomicOr(&acc[3 * (int64_t)i + 1], x.t | (before & x.s));
+                 int4* __restrict__ rec, const int2* __restrict__ chunks,
+                 const int32_t* __restrict__ nchunks, Mask* __restrict__ words) {
+  const int32_t cnt = *nchunks;
+  for (int32_t c = blockIdx.x; c < cnt; c += gridDim.x) {
+    const int2 it = chunks[c];
+    const int32_t e = it.x, b = eoff[e], sz = eoff[e + 1] - b;
+    const int32_t lo = (c - it.y) * GT_BIG_NET, hi = min(sz - lo, GT_BIG_NET) + lo;
+    Seen x;
+    for (int32_t q = lo + threadIdx.x; q < hi; q += GT_BIG_THREADS) x.add(part[pins[b + q]]);
+    __syncwarp();
+    x = block_seen(x);
+    if (threadIdx.x == 0) {
+      Mask* acc = words + 3 * (int64_t)it.y;
+      const Mask before = atomicOr(&acc[0], x.s);
+      atomicOr(&acc[1], x.t | (before & x.s));
+      __threadfence();
+      if (atomicAdd(&acc[2], 1ull) == (Mask)((sz + GT_BIG_NET - 1) / GT_BIG_NET - 1)) {
         __threadfence();
-        if (atomicAdd(&acc[3 * (int64_t)i + 2], 1ull) == (Mask)chunks - 1) {
-          __threadfence();
-          Seen y;
-          y.s = atomicOr(&acc[3 * (int64_t)i], 0ull);
-          y.t = atomicOr(&acc[3 * (int64_t)i + 1], 0ull);
-          write_rec(rec, e, k, w[e], y);
-        }
+        Seen y;
+        y.s = atomicOr(&acc[0], 0ull);
+        y.t = atomicOr(&acc[1], 0ull);
+        write_rec(rec, e, k, w[e], y);
       }
     }
   }
@@ -405,23 +416,23 @@ void gain_table_build(const Ctx& cx, const Level& L, int k, const int32_t* part,
   validate_partition(cx, part, L.n, k);
   DBuf<int4> rec;
   if (!L.graph && L.m > 0) {
-    const int64_t cap = L.p / GT_BIG_NET + 1;  // nets above GT_BIG_NET pins
-    DBuf<int32_t> big;
-    DBuf<Mask> acc;
+    const size_t cap = chunk_cap(L.p);
+    DBuf<int2> chunks;
+    DBuf<Mask> words;  // three per net, then the number of chunks
     rec.alloc(&cx.alloc, (size_t)L.m * (k > 32 ? 2 : 1));
-    big.alloc(&cx.alloc, (size_t)cap + 1);
-    acc.alloc(&cx.alloc, 3 * (size_t)cap);
-    HG_CUDA(cudaMemsetAsync(big.p + cap, 0, sizeof(int32_t), cx.stream));
-    HG_CUDA(cudaMemsetAsync(acc.p, 0, acc.bytes(), cx.stream));
+    chunks.alloc(&cx.alloc, cap);
+    words.alloc(&cx.alloc, 3 * cap + 1);
+    HG_CUDA(cudaMemsetAsync(words.p, 0, words.bytes(), cx.stream));
+    int32_t* nchunks = reinterpret_cast<int32_t*>(words.p + 3 * cap);
     k_gt_records<<<grid_for(L.m, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0, cx.stream>>>(
-        L.eoff.p, L.pins.p, L.w.p, part, L.m, k, rec.p, big.p, big.p + cap);
+        L.eoff.p, L.pins.p, L.w.p, part, L.m, k, rec.p, chunks.p, nchunks);
     check_launch("gt_records");
     if (L.p > GT_BIG_NET) {
-      k_gt_records_big<<<cx.num_sms, GT_BIG_THREADS, 0, cx.stream>>>(
-          L.eoff.p, L.pins.p, L.w.p, part, k, rec.p, big.p, big.p + cap, acc.p);
+      k_gt_records_big<<<grid_for(L.p, GT_BIG_NET, cx.num_sms, 8), GT_BIG_THREADS, 0, cx.stream>>>(
+          L.eoff.p, L.pins.p, L.w.p, part, k, rec.p, chunks.p, nchunks, words.p);
       check_launch("gt_records_big");
     }
-    if (cx.launches) *cx.launches += 2;
+    if (cx.launches) *cx.launches += 1 + (L.p > GT_BIG_NET);
   }
   build_kernel(L.graph, k)<<<grid_for(L.n, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0,
                              cx.stream>>>(L.ioff.p, L.inets.p, L.adj.p, rec.p, part, L.n, k,

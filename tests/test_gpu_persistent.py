@@ -416,3 +416,36 @@ def test_pin_counts_of_huge_nets(oracle_mod, k):
             assert np.array_equal(d.cpu().numpy(), ref["part"])
     finally:
         hg.hg_destroy(h)
+
+
+# nets around the size above which chunks of a net go to different blocks
+@pytest.mark.parametrize("k", [2, 33])
+def test_gain_tools_of_huge_nets(oracle_mod, k):
+    n = 30_000
+    hgr = nets_around(n, [64, 65, 4095, 4096, 4097, 8192, 8193, 30_000], k)
+    rng = np.random.default_rng(k)
+    part = rng.integers(0, max(1, k - 1), size=n).astype(np.int32)
+    part[:2] = k - 1  # blocks of one or two pins, in different chunks
+    nodes = np.concatenate([[0], rng.permutation(np.arange(1, n))[:3000]]).astype(np.int32)
+    targets = ((part[nodes] + 1 + rng.integers(0, k - 1, size=len(nodes))) % k).astype(np.int32)
+    moved = part.copy()
+    moved[nodes] = targets
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda()  # noqa: E731
+    h = create(hgr, 1)
+    try:
+        d = dev(part)
+        gains = torch.zeros(len(nodes), dtype=torch.int64, device="cuda")
+        hg.hg_recalculate_gains(h, 0, k, d, dev(nodes), dev(targets), gains)
+        assert np.array_equal(gains.cpu().numpy(),
+                              oracle_mod.recalculate_gains(hgr, k, part, nodes, targets))
+        b = torch.zeros(n, dtype=torch.int64, device="cuda")
+        p = torch.zeros((n, k), dtype=torch.int64, device="cuda")
+        hg.hg_gain_table(h, 0, k, d, b, p)
+        wb, wp = oracle_mod.gain_table(hgr, k, part)
+        assert np.array_equal(b.cpu().numpy(), wb) and np.array_equal(p.cpu().numpy(), wp)
+        hg.hg_gain_table_move(h, 0, k, d, dev(nodes), dev(targets), b, p)
+        wb, wp = oracle_mod.gain_table(hgr, k, moved)
+        assert np.array_equal(b.cpu().numpy(), wb) and np.array_equal(p.cpu().numpy(), wp)
+        assert np.array_equal(d.cpu().numpy(), moved)
+    finally:
+        hg.hg_destroy(h)
