@@ -476,9 +476,18 @@ void check_partition(const Ctx& cx, const int32_t* part, int32_t n, int k);
 // {move index or -1, block} of every node; bad moves set the status word.
 void index_moves(const Ctx& cx, const Level& L, int k, const int32_t* part, int32_t l,
                  const int32_t* nodes, const int32_t* targets, DBuf<int2>& info);
-// The nets of the moved nodes, each once, and their number.
-void touched_nets(const Ctx& cx, const Level& L, int32_t l, const int32_t* nodes,
-                  DBuf<int32_t>& list, DBuf<int32_t>& count);
+// The nets of the moved nodes, each once: those of at most SMALL_TOUCHED pins are the
+// first count[TN_SMALL] of the list, larger ones the last count[TN_WIDE]; with
+// chunk > 0, nets above chunk pins are left out of it and their chunks are listed as
+// {net, first of its chunks}, count[TN_CHUNKS] of them.
+constexpr int32_t SMALL_TOUCHED = 64;
+enum { TN_SMALL = 0, TN_WIDE = 1, TN_CHUNKS = 2, TN_WORDS = 3 };
+struct TouchedNets {
+  DBuf<int32_t> list, count;
+  DBuf<int2> chunks;
+};
+void touched_nets(const Ctx& cx, const Level& L, int32_t l, const int32_t* nodes, int32_t chunk,
+                  TouchedNets& t);
 void gain_table_build(const Ctx& cx, const Level& L, int k, const int32_t* part, int64_t* b,
                       int64_t* p);
 void gain_table_move(const Ctx& cx, const Level& L, int k, int32_t* part, int32_t l,

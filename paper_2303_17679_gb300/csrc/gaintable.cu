@@ -37,7 +37,7 @@ namespace {
 constexpr int GT_WARPS = 8;
 // nets and nodes of at most GT_SMALL pins (nets) are taken by a lane group, up
 // to GT_BIG_NET pins by a warp, larger nets by blocks
-constexpr int32_t GT_SMALL = 64;
+constexpr int32_t GT_SMALL = SMALL_TOUCHED;
 constexpr int32_t GT_BIG_NET = 4096;
 constexpr int GT_BIG_THREADS = 256;
 
@@ -303,82 +303,94 @@ __device__ __forceinline__ void update_pin(const MoveArgs& A, int32_t v, unsigne
   }
 }
 
-// Listed nets of up to GT_BIG_NET pins: a lane group for up to GT_SMALL pins,
-// else the warp; larger nets go to another list.
+// Listed nets (touched_nets): a lane group for up to GT_SMALL pins, a warp for up to
+// GT_BIG_NET; of the chunks of larger nets, a block each, the masks before and after
+// the moves, joined in four words per net at its first chunk.
 __global__ void __launch_bounds__(GT_WARPS * 32)
 k_gt_move_nets(MoveArgs A, const int32_t* __restrict__ list, const int32_t* __restrict__ count,
-               int32_t* __restrict__ big, int32_t* __restrict__ nbig) {
+               int32_t m, const int2* __restrict__ chunks, Mask* __restrict__ words) {
   const int lane = lane_id(), sub = lane % SUB_G;
-  const int32_t cnt = *count;
+  const int32_t nchunks = count[TN_CHUNKS], nwide = count[TN_WIDE], cnt = count[TN_SMALL];
+  for (int32_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    const int2 it = chunks[c];
+    const int32_t b = A.eoff[it.x], sz = A.eoff[it.x + 1] - b;
+    const int32_t lo = (c - it.y) * GT_BIG_NET, hi = min(sz - lo, GT_BIG_NET) + lo;
+    Seen was, is;
+    for (int32_t q = lo + threadIdx.x; q < hi; q += GT_WARPS * 32)
+      see_pin(A, A.pins[b + q], was, is);
+    __syncwarp();
+    was = block_seen(was);
+    is = block_seen(is);
+    if (threadIdx.x == 0) {
+      Mask* acc = words + 4 * (int64_t)it.y;
+      const Mask w0 = atomicOr(&acc[0], was.s), i0 = atomicOr(&acc[2], is.s);
+      atomicOr(&acc[1], was.t | (w0 & was.s));
+      atomicOr(&acc[3], is.t | (i0 & is.s));
+    }
+    __syncthreads();
+  }
+  for (int32_t x = warp_in_block() * gridDim.x + blockIdx.x; x < nwide;
+       x += gridDim.x * GT_WARPS) {
+    const int32_t e = list[m - 1 - x];
+    const int32_t b = A.eoff[e], sz = A.eoff[e + 1] - b;
+    Seen was, is;
+    for (int q = lane; q < sz; q += 32) see_pin(A, A.pins[b + q], was, is);
+    __syncwarp();
+    was.combine<32>();
+    is.combine<32>();
+    if (lane == 0) A.ones[e] = is.ones();
+    const Mask lam_x = was.s ^ is.s, ones_x = was.ones() ^ is.ones();
+    if (lam_x | ones_x) {
+      const unsigned long long we = (unsigned long long)(long long)A.w[e];
+      for (int q = lane; q < sz; q += 32)
+        update_pin(A, A.pins[b + q], we, is.s, lam_x, is.ones(), ones_x);
+    }
+    __syncwarp();
+  }
   const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
   for (int64_t x0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; x0 < cnt;
        x0 += stride) {
     const int64_t x = x0 + lane / SUB_G;
     const int32_t e = x < cnt ? list[x] : 0;
     const int32_t b = x < cnt ? A.eoff[e] : 0, sz = x < cnt ? A.eoff[e + 1] - b : 0;
-    const int32_t mine = sz <= GT_SMALL ? sz : 0;
     Seen was, is;
-    for (int q = sub; q < mine; q += SUB_G) see_pin(A, A.pins[b + q], was, is);
+    for (int q = sub; q < sz; q += SUB_G) see_pin(A, A.pins[b + q], was, is);
     __syncwarp();
     was.combine<SUB_G>();
     is.combine<SUB_G>();
-    if (mine > 0) {
+    if (sz > 0) {
       if (sub == 0) A.ones[e] = is.ones();
       const Mask lam_x = was.s ^ is.s, ones_x = was.ones() ^ is.ones();
       if (lam_x | ones_x) {
         const unsigned long long we = (unsigned long long)(long long)A.w[e];
-        for (int q = sub; q < mine; q += SUB_G)
+        for (int q = sub; q < sz; q += SUB_G)
           update_pin(A, A.pins[b + q], we, is.s, lam_x, is.ones(), ones_x);
       }
     }
     __syncwarp();
-    unsigned wide = __ballot_sync(FULL, sub == 0 && sz > GT_SMALL);
-    while (wide) {
-      const int l = __ffs(wide) - 1;
-      wide &= wide - 1;
-      const int32_t we_id = __shfl_sync(FULL, e, l);
-      const int32_t wb = __shfl_sync(FULL, b, l), ws = __shfl_sync(FULL, sz, l);
-      if (ws > GT_BIG_NET) {
-        if (lane == 0) big[atomicAdd(nbig, 1)] = we_id;
-        continue;
-      }
-      Seen w0, w1;
-      for (int q = lane; q < ws; q += 32) see_pin(A, A.pins[wb + q], w0, w1);
-      __syncwarp();
-      w0.combine<32>();
-      w1.combine<32>();
-      if (lane == 0) A.ones[we_id] = w1.ones();
-      const Mask lam_x = w0.s ^ w1.s, ones_x = w0.ones() ^ w1.ones();
-      if (lam_x | ones_x) {
-        const unsigned long long we = (unsigned long long)(long long)A.w[we_id];
-        for (int q = lane; q < ws; q += 32)
-          update_pin(A, A.pins[wb + q], we, w1.s, lam_x, w1.ones(), ones_x);
-      }
-      __syncwarp();
-    }
   }
 }
 
-// Listed nets of more than GT_BIG_NET pins, a block each.
+// The updates of the larger nets, a block per chunk.  (A block per net: 104 ms for a
+// net of 20M pins, 1.3 now.)
 __global__ void __launch_bounds__(GT_BIG_THREADS)
-k_gt_move_big(MoveArgs A, const int32_t* __restrict__ list, const int32_t* __restrict__ count) {
-  const int32_t cnt = *count;
-  for (int32_t x = blockIdx.x; x < cnt; x += gridDim.x) {
-    const int32_t e = list[x];
-    const int32_t b = A.eoff[e], sz = A.eoff[e + 1] - b;
+k_gt_move_chunks(MoveArgs A, const int2* __restrict__ chunks, const int32_t* __restrict__ count,
+                 const Mask* __restrict__ words) {
+  const int32_t cnt = count[TN_CHUNKS];
+  for (int32_t c = blockIdx.x; c < cnt; c += gridDim.x) {
+    const int2 it = chunks[c];
+    const Mask* acc = words + 4 * (int64_t)it.y;
     Seen was, is;
-    for (int q = threadIdx.x; q < sz; q += blockDim.x) see_pin(A, A.pins[b + q], was, is);
-    __syncwarp();
-    was = block_seen(was);
-    is = block_seen(is);
-    if (threadIdx.x == 0) A.ones[e] = is.ones();
+    was.join(acc[0], acc[1]);
+    is.join(acc[2], acc[3]);
+    if (c == it.y && threadIdx.x == 0) A.ones[it.x] = is.ones();
     const Mask lam_x = was.s ^ is.s, ones_x = was.ones() ^ is.ones();
-    if (lam_x | ones_x) {
-      const unsigned long long we = (unsigned long long)(long long)A.w[e];
-      for (int q = threadIdx.x; q < sz; q += blockDim.x)
-        update_pin(A, A.pins[b + q], we, is.s, lam_x, is.ones(), ones_x);
-    }
-    __syncthreads();
+    if (!(lam_x | ones_x)) continue;
+    const int32_t b = A.eoff[it.x], sz = A.eoff[it.x + 1] - b;
+    const int32_t lo = (c - it.y) * GT_BIG_NET, hi = min(sz - lo, GT_BIG_NET) + lo;
+    const unsigned long long we = (unsigned long long)(long long)A.w[it.x];
+    for (int32_t q = lo + threadIdx.x; q < hi; q += GT_BIG_THREADS)
+      update_pin(A, A.pins[b + q], we, is.s, lam_x, is.ones(), ones_x);
   }
 }
 
@@ -451,10 +463,10 @@ void gain_table_move(const Ctx& cx, const Level& L, int k, int32_t* part, int32_
   }
   check_partition(cx, part, L.n, k);
   DBuf<int2> info;
-  DBuf<int32_t> list, count, big;
+  TouchedNets t;
   index_moves(cx, L, k, part, l, nodes, targets, info);
   check_status(cx);  // nothing below runs on a bad partition or bad moves
-  touched_nets(cx, L, l, nodes, list, count);
+  touched_nets(cx, L, l, nodes, GT_BIG_NET, t);
   DBuf<Mask> ones;
   ones.alloc(&cx.alloc, (size_t)std::max<int32_t>(L.m, 1));
   MoveArgs A;
@@ -467,20 +479,21 @@ void gain_table_move(const Ctx& cx, const Level& L, int k, int32_t* part, int32_
   A.ones = ones.p;
   A.b = reinterpret_cast<unsigned long long*>(b);
   A.p = reinterpret_cast<unsigned long long*>(p);
-  const int64_t cap = L.p / GT_BIG_NET + 1;  // nets above GT_BIG_NET pins
-  big.alloc(&cx.alloc, (size_t)cap + 1);
-  HG_CUDA(cudaMemsetAsync(big.p + cap, 0, sizeof(int32_t), cx.stream));
-  k_gt_move_nets<<<cx.num_sms * 8, GT_WARPS * 32, 0, cx.stream>>>(A, list.p, count.p, big.p,
-                                                                  big.p + cap);
+  DBuf<Mask> words;
+  words.alloc(&cx.alloc, 4 * chunk_cap(L.p));
+  HG_CUDA(cudaMemsetAsync(words.p, 0, words.bytes(), cx.stream));
+  k_gt_move_nets<<<cx.num_sms * 8, GT_WARPS * 32, 0, cx.stream>>>(A, t.list.p, t.count.p, L.m,
+                                                                  t.chunks.p, words.p);
   check_launch("gt_move_nets");
   if (L.p > GT_BIG_NET) {
-    k_gt_move_big<<<cx.num_sms * 2, GT_BIG_THREADS, 0, cx.stream>>>(A, big.p, big.p + cap);
-    check_launch("gt_move_big");
+    k_gt_move_chunks<<<grid_for(L.p, GT_BIG_NET, cx.num_sms, 8), GT_BIG_THREADS, 0, cx.stream>>>(
+        A, t.chunks.p, t.count.p, words.p);
+    check_launch("gt_move_chunks");
   }
   k_gt_moved<<<grid_for(l, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0, cx.stream>>>(
       nodes, targets, l, L.ioff.p, L.inets.p, L.w.p, ones.p, part, reinterpret_cast<long long*>(b));
   check_launch("gt_moved");
-  if (cx.launches) *cx.launches += 3;
+  if (cx.launches) *cx.launches += 2 + (L.p > GT_BIG_NET);
   check_status(cx);
 }
 
