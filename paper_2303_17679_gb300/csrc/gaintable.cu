@@ -182,8 +182,12 @@ k_gt_records_big(const int32_t* __restrict__ eoff, const int32_t* __restrict__ p
 }
 
 // Table rows of the nodes: a lane group per node of at most GT_SMALL incident
-// nets, else the warp.
-template <bool GRAPH, int K, int H, int W>
+// nets, a warp for up to GT_HUB; items of GT_ITEM incident nets of larger nodes are
+// listed for a warp each, which add to the row (ADD).  One warp for a node of 5M
+// nets took 434 ms at k = 64, whatever the rest of the chip did.
+constexpr int32_t GT_HUB = 4096, GT_ITEM = 1024;
+
+template <bool GRAPH, int K, int H, int W, bool ADD = false>
 __device__ __forceinline__ void gt_row(const int32_t* __restrict__ inets,
                                        const int2* __restrict__ adj, const int4* __restrict__ rec,
                                        const int32_t* __restrict__ part, bool on, int64_t u,
@@ -221,12 +225,18 @@ __device__ __forceinline__ void gt_row(const int32_t* __restrict__ inets,
   constexpr int OWN = K / L::SHARE > 0 ? K / L::SHARE : 1;
   constexpr int SAME = L::SHARE / K > 1 ? L::SHARE / K : 1;
   if (on) {
-    if (l == 0) b[u] = wsum + bw;
+    if (l == 0) {
+      if (ADD) atomic_add_i64(&b[u], wsum + bw);
+      else b[u] = wsum + bw;
+    }
     if (lane.i % SAME == 0) {
 #pragma unroll
       for (int i = 0; i < OWN; ++i)
-        if (b0 + i < k)
-          p[u * k + b0 + i] = GRAPH && b0 + i == from ? 0 : wsum - g.acc[i];
+        if (b0 + i < k) {
+          const int32_t x = GRAPH && b0 + i == from ? 0 : wsum - g.acc[i];
+          if (!ADD) p[u * k + b0 + i] = x;
+          else if (x) atomic_add_i64(&p[u * k + b0 + i], x);
+        }
     }
   }
 }
@@ -236,12 +246,18 @@ __global__ void __launch_bounds__(GT_WARPS * 32)
 k_gt_build(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
            const int2* __restrict__ adj, const int4* __restrict__ rec,
            const int32_t* __restrict__ part, int32_t n, int k, long long* __restrict__ b,
-           long long* __restrict__ p) {
+           long long* __restrict__ p, int2* __restrict__ items, int32_t* __restrict__ nitems) {
   const int lane = lane_id();
   const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
   for (int64_t u0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; u0 < n; u0 += stride) {
     const int64_t u = u0 + lane / SUB_G;
     const int32_t beg = u < n ? ioff[u] : 0, end = u < n ? ioff[u + 1] : 0;
+    if (!__any_sync(FULL, end > beg)) {  // nodes without nets: whole rows of zeros
+      const int64_t stop = (u0 + NG < n ? u0 + NG : n) * k;
+      for (int64_t x = u0 * k + lane; x < stop; x += 32) p[x] = 0;
+      if (u < n && lane % SUB_G == 0) b[u] = 0;
+      continue;
+    }
     const bool small = end - beg <= GT_SMALL;
     gt_row<GRAPH, K, H, SUB_G>(inets, adj, rec, part, u < n && small, u, beg, small ? end : beg,
                                lane % SUB_G, k, b, p);
@@ -249,26 +265,79 @@ k_gt_build(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
     while (wide) {
       const int l = __ffs(wide) - 1;
       wide &= wide - 1;
-      gt_row<GRAPH, K, H, 32>(inets, adj, rec, part, true, u0 + l / SUB_G,
-                              __shfl_sync(FULL, beg, l), __shfl_sync(FULL, end, l), lane, k, b, p);
+      const int64_t wu = u0 + l / SUB_G;
+      const int32_t wb = __shfl_sync(FULL, beg, l), we = __shfl_sync(FULL, end, l);
+      if (we - wb > GT_HUB) {
+        const int32_t count = (we - wb + GT_ITEM - 1) / GT_ITEM;
+        int32_t first = 0;
+        if (lane == 0) {
+          first = atomicAdd(nitems, count);
+          b[wu] = 0;
+        }
+        first = __shfl_sync(FULL, first, 0);
+        for (int32_t i = lane; i < count; i += 32) items[first + i] = make_int2((int)wu, i);
+        for (int t = lane; t < k; t += 32) p[wu * k + t] = 0;
+        continue;
+      }
+      gt_row<GRAPH, K, H, 32>(inets, adj, rec, part, true, wu, wb, we, lane, k, b, p);
     }
   }
 }
 
-using BuildKernel = void (*)(const int32_t*, const int32_t*, const int2*, const int4*,
-                             const int32_t*, int32_t, int, long long*, long long*);
-
-BuildKernel build_kernel(bool graph, int k) {
-  if (graph) {
-    if (k <= 8) return k_gt_build<true, 8, 1>;
-    if (k <= 16) return k_gt_build<true, 16, 1>;
-    if (k <= 32) return k_gt_build<true, 32, 1>;
-    return k_gt_build<true, 32, 2>;
+template <bool GRAPH, int K, int H>
+__global__ void __launch_bounds__(GT_WARPS * 32)
+k_gt_build_hubs(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
+                const int2* __restrict__ adj, const int4* __restrict__ rec,
+                const int32_t* __restrict__ part, int k, long long* __restrict__ b,
+                long long* __restrict__ p, const int2* __restrict__ items,
+                const int32_t* __restrict__ nitems) {
+  const int32_t cnt = *nitems;
+  for (int32_t x = warp_in_block() * gridDim.x + blockIdx.x; x < cnt; x += gridDim.x * GT_WARPS) {
+    const int2 it = items[x];
+    const int32_t beg = ioff[it.x] + it.y * GT_ITEM;
+    const int32_t end = beg + min(GT_ITEM, ioff[it.x + 1] - beg);
+    gt_row<GRAPH, K, H, 32, true>(inets, adj, rec, part, true, it.x, beg, end, lane_id(), k, b, p);
   }
-  if (k <= 8) return k_gt_build<false, 8, 1>;
-  if (k <= 16) return k_gt_build<false, 16, 1>;
-  if (k <= 32) return k_gt_build<false, 32, 1>;
-  return k_gt_build<false, 32, 2>;
+}
+
+template <bool GRAPH, int K, int H>
+void build_rows(const Ctx& cx, const Level& L, int k, const int4* rec, const int32_t* part,
+                long long* b, long long* p) {
+  DBuf<int2> items;
+  DBuf<int32_t> nitems;
+  const bool hubs = L.p > GT_HUB;
+  if (hubs) {
+    items.alloc(&cx.alloc, (size_t)(L.p / GT_ITEM + L.p / GT_HUB) + 1);
+    nitems.alloc(&cx.alloc, 1);
+    HG_CUDA(cudaMemsetAsync(nitems.p, 0, sizeof(int32_t), cx.stream));
+  }
+  k_gt_build<GRAPH, K, H><<<grid_for(L.n, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0,
+                            cx.stream>>>(L.ioff.p, L.inets.p, L.adj.p, rec, part, L.n, k, b, p,
+                                         items.p, nitems.p);
+  check_launch("gt_build");
+  if (hubs) {
+    k_gt_build_hubs<GRAPH, K, H><<<grid_for(L.p, GT_ITEM * GT_WARPS, cx.num_sms, 8),
+                                   GT_WARPS * 32, 0, cx.stream>>>(
+        L.ioff.p, L.inets.p, L.adj.p, rec, part, k, b, p, items.p, nitems.p);
+    check_launch("gt_build_hubs");
+  }
+  if (cx.launches) *cx.launches += 1 + hubs;
+}
+
+using BuildRows = void (*)(const Ctx&, const Level&, int, const int4*, const int32_t*, long long*,
+                           long long*);
+
+BuildRows build_rows_for(bool graph, int k) {
+  if (graph) {
+    if (k <= 8) return build_rows<true, 8, 1>;
+    if (k <= 16) return build_rows<true, 16, 1>;
+    if (k <= 32) return build_rows<true, 32, 1>;
+    return build_rows<true, 32, 2>;
+  }
+  if (k <= 8) return build_rows<false, 8, 1>;
+  if (k <= 16) return build_rows<false, 16, 1>;
+  if (k <= 32) return build_rows<false, 32, 1>;
+  return build_rows<false, 32, 2>;
 }
 
 // ------------------------------------------------------------ moves
@@ -446,12 +515,8 @@ void gain_table_build(const Ctx& cx, const Level& L, int k, const int32_t* part,
     }
     if (cx.launches) *cx.launches += 1 + (L.p > GT_BIG_NET);
   }
-  build_kernel(L.graph, k)<<<grid_for(L.n, GT_WARPS * NG, cx.num_sms, 8), GT_WARPS * 32, 0,
-                             cx.stream>>>(L.ioff.p, L.inets.p, L.adj.p, rec.p, part, L.n, k,
-                                          reinterpret_cast<long long*>(b),
-                                          reinterpret_cast<long long*>(p));
-  check_launch("gt_build");
-  if (cx.launches) *cx.launches += 1;
+  build_rows_for(L.graph, k)(cx, L, k, rec.p, part, reinterpret_cast<long long*>(b),
+                             reinterpret_cast<long long*>(p));
   check_status(cx);
 }
 

@@ -449,3 +449,27 @@ def test_gain_tools_of_huge_nets(oracle_mod, k):
         assert np.array_equal(d.cpu().numpy(), moved)
     finally:
         hg.hg_destroy(h)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("k", [3, 16, 30, 64])
+def test_gain_table_of_hubs(oracle_mod, graph, k):
+    """Nodes around the number of nets above which a row is summed by several warps."""
+    n, degs = 9000, [4095, 4096, 4097, 5120, 5121, 8000]
+    rng = np.random.default_rng(k)
+    nets = [[u, int(v)] for u, d in enumerate(degs)
+            for v in rng.choice(np.arange(100, n), size=d, replace=False)]
+    if not graph:
+        nets += [rng.choice(n, size=5, replace=False).tolist() for _ in range(500)]
+    hgr = from_nets(n, nets, rng.integers(1, 90_000, size=len(nets)), None)
+    part = rng.integers(0, k, size=n).astype(np.int32)
+    h = create(hgr, 1)
+    try:
+        assert hg.hg_level_is_graph(h, 0) == graph
+        b = torch.full((n,), 7, dtype=torch.int64, device="cuda")
+        p = torch.full((n, k), 7, dtype=torch.int64, device="cuda")
+        hg.hg_gain_table(h, 0, k, torch.from_numpy(part).cuda(), b, p)
+        wb, wp = oracle_mod.gain_table(hgr, k, part)
+        assert np.array_equal(b.cpu().numpy(), wb) and np.array_equal(p.cpu().numpy(), wp)
+    finally:
+        hg.hg_destroy(h)
