@@ -52,7 +52,7 @@
 //            indexed by cluster id when n <= min(2 W, 65536), filled by items
 //            of 32 incident nets spread over the grid (the table padded to a
 //            multiple of 4 entries); else P = ceil(D / 13516) parts (64-bit
-//            ratings: ceil(D / 9830); P <= 8), a block each, owning the
+//            ratings: ceil(D / 9830); P <= 12), a block each, owning the
 //            candidates of one hash part in a 22528-slot (16384) shared table
 //            with a list of its inserted slots; else a global hash table filled
 //            by items.  A second step takes the argmax per node (or the best of

@@ -17,8 +17,11 @@ constexpr int32_t TEAM_W = 65536;        // largest W of a node rated by one eig
 constexpr int32_t DENSE_W = 32768;       // largest W of a direct-indexed block node
 constexpr int32_t TEAM_RECORDS = 4096;   // most records of a node rated by one team or block
 constexpr int32_t SPLIT_DENSE_MAX = 65536;
-// part blocks: see PartCfg (table slots and distinct candidates per part)
-constexpr int32_t PART_MAX = 8;          // more parts: the node uses a global hash table
+// Part blocks: see PartCfg (table slots and distinct candidates per part).  A node of
+// more parts uses a global hash table, whose random sectors cost about fifteen times
+// a visit that is only read.  Level of 118,445 nodes with 400 nets of 5000 pins, nine
+// parts per node: 240 ms with global tables (a limit of 8), 95 ms in parts.
+constexpr int32_t PART_MAX = 12;
 constexpr int32_t EMPTY_KEY = -1;
 
 constexpr int RUN_THREADS = 1024;        // the sub-round kernel: one block per SM

@@ -473,3 +473,24 @@ def test_gain_table_of_hubs(oracle_mod, graph, k):
         assert np.array_equal(b.cpu().numpy(), wb) and np.array_equal(p.cpu().numpy(), wp)
     finally:
         hg.hg_destroy(h)
+
+
+# candidates on both sides of the twelve parts that a node may have (32-bit ratings:
+# nets of 900 pins; 64-bit: of two), above it a table in global memory
+@pytest.mark.parametrize("size,count", [(900, 162_000), (900, 163_000), (2, 58_900), (2, 59_200)])
+def test_parts_of_a_heavy_node(oracle_mod, size, count):
+    n, seed = 200_000, 1
+    ids = np.arange(n, dtype=np.uint64)
+    hub = int(np.flatnonzero(mix64(ids ^ np.uint64(seed)) % np.uint64(16) == 0)[0])
+    rng = np.random.default_rng(size)
+    cand = rng.permutation(np.delete(np.arange(n), hub))[:count]
+    nets = [[hub, *c.tolist()] for c in np.array_split(cand, -(-count // (size - 1)))]
+    nets += [[n - 3, n - 2, n - 1]]
+    hgr = from_nets(n, nets, rng.integers(1, 5, size=len(nets)), None)
+    ref = oracle_mod.multilevel(hgr, 2, 30000, S=16, factor=160, seed=seed, max_passes=0)
+    h = create(hgr, seed)
+    try:
+        hg.hg_coarsen_level(h, 2)
+        assert np.array_equal(hg.hg_get_level(h, 0, with_map=True)["map"], ref.maps[0])
+    finally:
+        hg.hg_destroy(h)
