@@ -198,17 +198,16 @@ __global__ void k_validate_nodes(const int32_t* __restrict__ c, int32_t n, int32
 }
 
 // No node twice in a net.  A warp takes up to 32 nets (fewer when there is a
-// warp for each): those of at most
-// DISTINCT_LANE pins a lane each, comparing all pairs in registers; those of at
-// most 32 pins by the warp, every lane against half of the others; those of at
-// most DISTINCT_SMALL pins into a per-warp hash set in shared memory (a pin
-// found already present is a repeat).  (A warp per net with a match over its
-// lanes was bound by the match, a step per distinct pin: 1.27 ms at 4e6 edges,
-// 0.04 ms
-// now.)  Larger nets are listed for k_distinct_big (a block
-// that looks for them among all nets waits on two offsets per net: 5 of 6 ms at
-// 2e6 nets).  Runs only on offsets and pins already checked, so every read
-// stays in bounds.
+// warp for each): those of at most DISTINCT_LANE pins a lane each, comparing all
+// pairs in registers; those of at most 32 pins by the warp, every lane against half
+// of the others.  (A warp per net with a match over its lanes was bound by the match,
+// a step per distinct pin: 1.27 ms at 4e6 edges, 0.04 ms now.)  Larger nets are
+// listed by size: up to DISTINCT_SMALL pins for k_distinct_mid (a warp and a hash set
+// in shared memory each; by the warp that found them, neighbouring nets of 900 pins
+// queued up: hg_create with 3000 of them 0.44 -> 0.73 ms), larger ones for
+// k_distinct_big (a block that looks for them among all nets waits on two offsets per
+// net: 5 of 6 ms at 2e6 nets).  Runs only on offsets and pins already checked, so
+// every read stays in bounds.
 constexpr int DISTINCT_WARPS = 4;
 constexpr int DISTINCT_SMALL = 1024;
 constexpr int DISTINCT_LANE = 8;
@@ -240,21 +239,22 @@ __device__ __forceinline__ void set_erase(int32_t* set, uint32_t mask, int32_t v
   }
 }
 
+// The lists of nets of more than 32 pins and their lengths.
+struct DistinctLists {
+  int32_t *mid, *big, *count;  // count[0]: mid, [1]: big
+};
+
 __global__ void __launch_bounds__(DISTINCT_WARPS * 32)
 k_distinct_small(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins, int32_t m,
-                 int per, int32_t* __restrict__ big, int32_t* __restrict__ nbig, int32_t* status) {
-  __shared__ int32_t s_set[DISTINCT_WARPS][DISTINCT_SET];
+                 int per, DistinctLists D, int32_t* status) {
   const int wv = warp_in_block(), lane = lane_id();
-  int32_t* set = s_set[wv];
-  for (int i = lane; i < DISTINCT_SET; i += 32) set[i] = -1;
-  __syncwarp();
   const int64_t stride = (int64_t)gridDim.x * DISTINCT_WARPS * per;
   for (int64_t e0 = ((int64_t)blockIdx.x * DISTINCT_WARPS + wv) * per; e0 < m; e0 += stride) {
     const int64_t e = e0 + lane;
     const bool on = lane < per && e < m;
     const int32_t b = on ? eoff[e] : 0, sz = on ? eoff[e + 1] - b : 0;
     bool dup = false;
-    if (sz > DISTINCT_SMALL) big[atomicAdd(nbig, 1)] = (int32_t)e;
+    if (sz > DISTINCT_SMALL) D.big[atomicAdd(&D.count[1], 1)] = (int32_t)e;
     if (sz <= DISTINCT_LANE) {
       int32_t v[DISTINCT_LANE];
 #pragma unroll
@@ -265,23 +265,46 @@ k_distinct_small(const int32_t* __restrict__ eoff, const int32_t* __restrict__ p
         for (int j = 0; j < i; ++j) dup |= v[i] == v[j];
     }
     __syncwarp();
-    unsigned todo = __ballot_sync(FULL, sz > DISTINCT_LANE && sz <= DISTINCT_SMALL);
+    const bool mid = sz > 32 && sz <= DISTINCT_SMALL;
+    const unsigned mids = __ballot_sync(FULL, mid);
+    if (mids) {
+      int32_t at = 0;
+      if (lane == 0) at = atomicAdd(&D.count[0], __popc(mids));
+      at = __shfl_sync(FULL, at, 0) + __popc(mids & ((1u << lane) - 1u));
+      if (mid) D.mid[at] = (int32_t)e;
+    }
+    unsigned todo = __ballot_sync(FULL, sz > DISTINCT_LANE && sz <= 32);
     while (todo) {
       const int l = __ffs(todo) - 1;
       todo &= todo - 1;
       const int32_t wb = __shfl_sync(FULL, b, l), wsz = __shfl_sync(FULL, sz, l);
-      if (wsz <= 32) {
-        const int32_t v = lane < wsz ? pins[wb + lane] : -1 - lane;
+      const int32_t v = lane < wsz ? pins[wb + lane] : -1 - lane;
 #pragma unroll
-        for (int d = 1; d <= 16; ++d) dup |= __shfl_sync(FULL, v, (lane + d) & 31) == v;
-      } else {
-        for (int32_t q = lane; q < wsz; q += 32)
-          dup |= !set_insert_new(set, DISTINCT_SET - 1, pins[wb + q]);
-        __syncwarp();
-        for (int32_t q = lane; q < wsz; q += 32) set_erase(set, DISTINCT_SET - 1, pins[wb + q]);
-        __syncwarp();
-      }
+      for (int d = 1; d <= 16; ++d) dup |= __shfl_sync(FULL, v, (lane + d) & 31) == v;
     }
+    if (__any_sync(FULL, dup) && lane == 0) dev_fail(status, DEV_BAD_INPUT);
+  }
+}
+
+__global__ void __launch_bounds__(DISTINCT_WARPS * 32)
+k_distinct_mid(const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
+               DistinctLists D, int32_t* status) {
+  __shared__ int32_t s_set[DISTINCT_WARPS][DISTINCT_SET];
+  const int wv = warp_in_block(), lane = lane_id();
+  int32_t* set = s_set[wv];
+  const int32_t cnt = D.count[0];
+  int32_t x = wv * gridDim.x + blockIdx.x;
+  if (x >= cnt) return;
+  for (int i = lane; i < DISTINCT_SET; i += 32) set[i] = -1;
+  __syncwarp();
+  for (; x < cnt; x += gridDim.x * DISTINCT_WARPS) {
+    const int32_t e = D.mid[x], b = eoff[e], sz = eoff[e + 1] - b;
+    bool dup = false;
+    for (int32_t q = lane; q < sz; q += 32)
+      dup |= !set_insert_new(set, DISTINCT_SET - 1, pins[b + q]);
+    __syncwarp();
+    for (int32_t q = lane; q < sz; q += 32) set_erase(set, DISTINCT_SET - 1, pins[b + q]);
+    __syncwarp();
     if (__any_sync(FULL, dup) && lane == 0) dev_fail(status, DEV_BAD_INPUT);
   }
 }
@@ -455,16 +478,20 @@ bool distinct_pins(const Ctx& cx, const Level& L) {
   HG_CUDA(cudaMemsetAsync(mx.p, 0, sizeof(int32_t), cx.stream));
   k_max_net_size<<<grid_for(L.m, 256, cx.num_sms, 8), 256, 0, cx.stream>>>(L.eoff.p, L.m, mx.p);
   check_launch("max_net_size");
-  DBuf<int32_t> big;  // nets above DISTINCT_SMALL pins, then their number
-  const size_t nb = (size_t)(L.p / (DISTINCT_SMALL + 1)) + 1;
-  big.alloc(&cx.alloc, nb + 1);
-  int32_t* nbig = big.p + nb;
-  HG_CUDA(cudaMemsetAsync(nbig, 0, sizeof(int32_t), cx.stream));
+  DBuf<int32_t> lists;  // nets of 33 pins and more, of more than DISTINCT_SMALL, lengths
+  const size_t nmid = (size_t)(L.p / 33) + 1, nb = (size_t)(L.p / (DISTINCT_SMALL + 1)) + 1;
+  lists.alloc(&cx.alloc, nmid + nb + 2);
+  const DistinctLists D{lists.p, lists.p + nmid, lists.p + nmid + nb};
+  const int32_t *big = D.big, *nbig = D.count + 1;
+  HG_CUDA(cudaMemsetAsync(D.count, 0, 2 * sizeof(int32_t), cx.stream));
   const int64_t warps = (int64_t)cx.num_sms * 6 * DISTINCT_WARPS;
   const int per = (int)std::min<int64_t>(32, (L.m + warps - 1) / warps);
   k_distinct_small<<<grid_for(L.m, DISTINCT_WARPS * per, cx.num_sms, 6), DISTINCT_WARPS * 32, 0,
-                     cx.stream>>>(L.eoff.p, L.pins.p, L.m, per, big.p, nbig, cx.d_status);
+                     cx.stream>>>(L.eoff.p, L.pins.p, L.m, per, D, cx.d_status);
   check_launch("distinct_small");
+  k_distinct_mid<<<grid_for(L.p, 33 * DISTINCT_WARPS, cx.num_sms, 6), DISTINCT_WARPS * 32, 0,
+                   cx.stream>>>(L.eoff.p, L.pins.p, D, cx.d_status);
+  check_launch("distinct_mid");
   const int32_t biggest = read_i32(cx, mx.p);
   const int64_t words = ((int64_t)L.n + 31) / 32;
   if (biggest > DISTINCT_SMALL && (int64_t)cx.num_sms * words * 4 <= DISTINCT_BITMAP_BYTES) {
@@ -472,7 +499,7 @@ bool distinct_pins(const Ctx& cx, const Level& L) {
     DBuf<uint32_t> scratch;
     scratch.alloc(&cx.alloc, (size_t)blocks * (size_t)words);
     HG_CUDA(cudaMemsetAsync(scratch.p, 0, scratch.bytes(), cx.stream));
-    k_distinct_big_bitmap<<<blocks, 1024, 0, cx.stream>>>(L.eoff.p, L.pins.p, big.p, nbig,
+    k_distinct_big_bitmap<<<blocks, 1024, 0, cx.stream>>>(L.eoff.p, L.pins.p, big, nbig,
                                                           scratch.p, words, cx.d_status);
     check_launch("distinct_big_bitmap");
   } else if (biggest > DISTINCT_SMALL) {
@@ -482,7 +509,7 @@ bool distinct_pins(const Ctx& cx, const Level& L) {
     DBuf<int32_t> scratch;
     scratch.alloc(&cx.alloc, (size_t)blocks * cap);
     HG_CUDA(cudaMemsetAsync(scratch.p, 0xff, scratch.bytes(), cx.stream));
-    k_distinct_big<<<blocks, 1024, 0, cx.stream>>>(L.eoff.p, L.pins.p, big.p, nbig, scratch.p,
+    k_distinct_big<<<blocks, 1024, 0, cx.stream>>>(L.eoff.p, L.pins.p, big, nbig, scratch.p,
                                                    cap, cx.d_status);
     check_launch("distinct_big");
   }

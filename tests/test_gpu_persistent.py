@@ -494,3 +494,26 @@ def test_parts_of_a_heavy_node(oracle_mod, size, count):
         assert np.array_equal(hg.hg_get_level(h, 0, with_map=True)["map"], ref.maps[0])
     finally:
         hg.hg_destroy(h)
+
+
+# one repeated pin in one net: sizes around the classes of the check, many big nets
+# in a row
+@pytest.mark.parametrize("size", [2, 8, 9, 32, 33, 900, 1024, 1025])
+@pytest.mark.parametrize("bad", [None, 0, 299])
+def test_repeated_pin_by_net_size(size, bad):
+    n, m = 4000, 300
+    rng = np.random.default_rng(size)
+    pins = np.stack([rng.permutation(n)[:size] for _ in range(m)])
+    if bad is not None:
+        pins[bad, -1] = pins[bad, 0]
+    small = np.stack([rng.permutation(n)[:2] for _ in range(500)])
+    off = np.concatenate([[0], size * np.arange(1, m + 1), size * m + 2 * np.arange(1, 501)])
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda()  # noqa: E731
+    args = (n, m + 500, dev(off), dev(np.concatenate([pins.reshape(-1), small.reshape(-1)])), None,
+            None, hg.HG_MEM_DEVICE, None, torch.cuda.current_stream())
+    if bad is None:
+        hg.hg_destroy(hg.hg_create(*args))
+    else:
+        with pytest.raises(hg.HgError) as ei:
+            hg.hg_create(*args)
+        assert ei.value.status == hg.HG_ERR_INVALID
