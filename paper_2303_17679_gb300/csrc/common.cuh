@@ -448,7 +448,7 @@ struct PinState {
   DBuf<int32_t> phi;
   DBuf<unsigned long long> lam;
   DBuf<int4> rec;
-  DBuf<long long> bw;
+  DBuf<long long> bw;  // k block weights (then working lists of build_pin_state)
 };
 
 // What goes with the pin counts: nothing and no counts either (graph levels in

@@ -26,8 +26,10 @@ __global__ void k_project(const int32_t* __restrict__ map, const int32_t* __rest
 // Phi, and Lambda or the packed records (gain.cuh), of every net: a net's pins
 // are counted per block in shared memory by eight lanes (up to COUNT_SMALL
 // pins) or a warp (up to COUNT_WARP), which then write the net's row of Phi and its
-// masks once; those of larger nets by chunks over the
-// grid, added to the row (as one block's, a net of 20M pins took 24 ms).  Bound by the row writes on levels of small nets (m
+// masks once.  Larger nets: by chunks over the grid, added to the row (as one block's,
+// a net of 20M pins took 24 ms, 1.2 now); on levels of at most COUNT_LEVEL pins by
+// the block, after its other nets (the launch for the chunks costs 7 of 700 us of
+// label propagation at n = 10,000).  Bound by the row writes on levels of small nets (m
 // k words), by the pins' block ids on the others.  (A thread per pin that found
 // equal (net, block) pairs by a match over the warp and added them with atomics to
 // a cleared table, and a second pass for the records, took 0.53 + 0.23 ms per
@@ -37,6 +39,8 @@ constexpr int COUNT_NETS = 32 / COUNT_LANES;
 constexpr int32_t COUNT_SMALL = 64, COUNT_WARP = 2048;
 constexpr int COUNT_STRIDE = HG_MAX_K + 1;  // a warp's sets start in different banks
 constexpr int32_t COUNT_CHUNK = 4096;
+constexpr int64_t COUNT_LEVEL = 1 << 17;
+constexpr int COUNT_BIG = 64;               // nets a block keeps for later
 
 struct CountArgs {
   const int32_t *eoff, *pins, *part, *w;
@@ -46,7 +50,7 @@ struct CountArgs {
   unsigned long long* lam;  // or
   int4* rec;
   // chunks of the nets above COUNT_WARP: {net, its first chunk}, their number, and
-  // the chunks done per net (at its first chunk)
+  // the chunks done per net (at its first chunk); NULL on small levels
   int2* chunks;
   int32_t *nchunks, *done;
 };
@@ -112,11 +116,15 @@ __device__ __forceinline__ void count_pins(const CountArgs& A, int32_t b, int32_
 template <bool PHI>
 __global__ void __launch_bounds__(COUNT_WARPS * 32, 8) k_pin_counts(CountArgs A) {
   __shared__ int32_t s_cnt[COUNT_WARPS * COUNT_NETS * COUNT_STRIDE];
+  __shared__ int32_t s_big[COUNT_BIG];
+  __shared__ int s_nbig;
+  __shared__ unsigned long long s_ones, s_lam;
   const int lane = lane_id(), sub = lane % COUNT_LANES, grp = lane / COUNT_LANES;
   int32_t* sets = s_cnt + warp_in_block() * COUNT_NETS * COUNT_STRIDE;
   int32_t* mine = sets + grp * COUNT_STRIDE;
   for (int i = threadIdx.x; i < COUNT_WARPS * COUNT_NETS * COUNT_STRIDE; i += blockDim.x)
     s_cnt[i] = 0;
+  if (threadIdx.x == 0) s_nbig = 0;
   __syncthreads();
   auto by_warp = [&](int32_t e, int32_t b, int32_t sz) {
     count_pins(A, b, sz, lane, 32, mine);
@@ -147,7 +155,7 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 8) k_pin_counts(CountArgs A)
       const int l = __ffs(rest) - 1;
       const int32_t we = (int32_t)(e0 + l / COUNT_LANES);
       const int32_t wb = __shfl_sync(FULL, b, l), wsz = __shfl_sync(FULL, sz, l);
-      if (wsz > COUNT_WARP) {
+      if (wsz > COUNT_WARP && A.chunks) {
         const int32_t count = (wsz + COUNT_CHUNK - 1) / COUNT_CHUNK;
         int32_t first = 0;
         if (lane == 0) first = atomicAdd(A.nchunks, count);
@@ -159,8 +167,29 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, 8) k_pin_counts(CountArgs A)
           A.lam[we] = 0;
         continue;
       }
-      by_warp(we, wb, wsz);
+      int slot = COUNT_BIG;
+      if (wsz > COUNT_WARP) {
+        if (lane == 0) slot = atomicAdd(&s_nbig, 1);
+        slot = __shfl_sync(FULL, slot, 0);
+        if (slot < COUNT_BIG && lane == 0) s_big[slot] = we;
+      }
+      if (slot >= COUNT_BIG) by_warp(we, wb, wsz);
     }
+  }
+  __syncthreads();
+  const int big = min(s_nbig, COUNT_BIG);
+  for (int x = 0; x < big; ++x) {
+    const int32_t e = s_big[x], b = A.eoff[e], sz = A.eoff[e + 1] - b;
+    count_pins(A, b, sz, threadIdx.x, COUNT_WARPS * 32, mine);
+    if (threadIdx.x == 0) s_ones = s_lam = 0;
+    __syncthreads();
+    unsigned long long ones, lam;
+    write_row<COUNT_WARPS * 32, PHI>(A, e, s_cnt, COUNT_WARPS * COUNT_NETS, threadIdx.x, ones, lam);
+    if (ones) atomicOr(&s_ones, ones);
+    if (lam) atomicOr(&s_lam, lam);
+    __syncthreads();
+    if (threadIdx.x == 0) write_masks(A, e, s_ones, s_lam);
+    __syncthreads();
   }
 }
 
@@ -259,7 +288,11 @@ void project_partition(const Ctx& cx, const Level& fine, const int32_t* coarse_p
 // records.
 void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, PinState& st,
                      PinMasks masks) {
-  st.bw.alloc(&cx.alloc, (size_t)k);
+  // the block weights, then the chunk lists: one allocation and one memset for all
+  // that starts at zero
+  const size_t cap = masks != PinMasks::none && L.p > COUNT_LEVEL
+                         ? (size_t)(L.p / COUNT_CHUNK + L.p / COUNT_WARP) + 1 : 0;
+  st.bw.alloc(&cx.alloc, (size_t)k + cap + (cap + 2) / 2);
   HG_CUDA(cudaMemsetAsync(st.bw.p, 0, st.bw.bytes(), cx.stream));
   if (masks != PinMasks::none) {
     if (masks != PinMasks::lambda_only) st.phi.alloc(&cx.alloc, (size_t)L.m * k + 1);
@@ -268,28 +301,22 @@ void build_pin_state(const Ctx& cx, const Level& L, int k, const int32_t* part, 
     if (L.m > 0) {
       CountArgs A{L.eoff.p, L.pins.p, part,     L.w.p,   L.m,    k,
                   st.phi.p, st.lam.p, st.rec.p, nullptr, nullptr, nullptr};
-      DBuf<int2> chunks;
-      DBuf<int32_t> done;  // and the number of chunks
-      if (L.p > COUNT_WARP) {
-        const size_t cap = (size_t)(L.p / COUNT_CHUNK + L.p / COUNT_WARP) + 1;
-        chunks.alloc(&cx.alloc, cap);
-        done.alloc(&cx.alloc, cap + 1);
-        HG_CUDA(cudaMemsetAsync(done.p, 0, done.bytes(), cx.stream));
-        A.chunks = chunks.p;
-        A.nchunks = done.p + cap;
-        A.done = done.p;
+      if (cap) {
+        A.chunks = reinterpret_cast<int2*>(st.bw.p + k);
+        A.done = reinterpret_cast<int32_t*>(st.bw.p + k + cap);
+        A.nchunks = A.done + cap;
       }
       const bool phi = st.phi.p != nullptr;
       (phi ? k_pin_counts<true> : k_pin_counts<false>)<<<
           grid_for(L.m, COUNT_WARPS * COUNT_NETS, cx.num_sms, 8), COUNT_WARPS * 32, 0,
           cx.stream>>>(A);
       check_launch("pin_counts");
-      if (L.p > COUNT_WARP) {
+      if (cap) {
         (phi ? k_pin_counts_huge<true> : k_pin_counts_huge<false>)<<<
             grid_for(L.p, COUNT_CHUNK, cx.num_sms, 4), COUNT_WARPS * 32, 0, cx.stream>>>(A);
         check_launch("pin_counts_huge");
       }
-      if (cx.launches) *cx.launches += 1 + (L.p > COUNT_WARP);
+      if (cx.launches) *cx.launches += 1 + (cap > 0);
     }
   }
   k_block_weights<<<grid_for(L.n, 256, cx.num_sms, 4), 256, 0, cx.stream>>>(part, L.c.p, L.n, k,

@@ -395,11 +395,15 @@ def nets_around(n, sizes, seed, rest=3000):
                      rng.integers(1, 4, size=n))
 
 
-# nets around the size above which chunks of a net are counted by different blocks
+# nets around the size above which a block, or on levels of more than 131,072 pins the
+# grid by chunks, counts a net
+@pytest.mark.parametrize("sizes,rest", [([2048, 2049, 4096, 4097, 8192, 8193, 40_960, 60_000], 3000),
+                                        ([2049, 4097, 20_000, 95_000], 0),
+                                        ([2049, 4097, 20_000, 95_000], 3500)])
 @pytest.mark.parametrize("k", [1, 5, 64])
-def test_pin_counts_of_huge_nets(oracle_mod, k):
-    n = 60_000
-    hgr = nets_around(n, [2048, 2049, 4096, 4097, 8192, 8193, 40_960, 60_000], k)
+def test_pin_counts_of_huge_nets(oracle_mod, k, sizes, rest):
+    n = 100_000
+    hgr = nets_around(n, sizes, k, rest)
     part = np.random.default_rng(k).integers(0, max(1, k - 1), size=n).astype(np.int32)
     part[:3] = k - 1  # a block of few pins
     h = create(hgr, 1)
