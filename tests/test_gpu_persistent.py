@@ -414,6 +414,11 @@ def test_pin_counts_of_huge_nets(oracle_mod, k, sizes, rest):
         assert np.array_equal(got[0], phi) and np.array_equal(got[1], lam)
         assert np.array_equal(got[2], oracle_mod.block_weights(hgr, k, part))
         assert hg.hg_objective(h, 0, k, d) == oracle_mod.objective(hgr, k, part)
+        on = [torch.from_numpy(np.ascontiguousarray(a, np.int32)).cuda()
+              for a in (hgr.offsets, hgr.pins, hgr.net_w, hgr.node_w)]
+        assert hg.hg_objective_noalloc(hgr.n, hgr.m, hgr.p, *on, k, d,
+                                       torch.cuda.current_stream())[0] == \
+            oracle_mod.objective(hgr, k, part)
         if k > 1:
             ref = oracle_mod.lp_refine(hgr, k, part, 50000, 16, 1, 0, 2)
             assert hg.hg_lp_refine(h, 0, k, 50000, 2, d) == (ref["objective"], ref["moves"])
