@@ -20,7 +20,7 @@ namespace {
 
 constexpr int GR_WARPS = 8;
 constexpr int GR_LANES = 8;   // lanes per move or per net of at most GR_SMALL pins
-constexpr int32_t GR_SMALL = SMALL_TOUCHED;
+constexpr int32_t GR_SMALL = SMALL_TOUCHED, GR_BIG = 32768;
 
 // info[v] = {index of v's move or -1, Pi[v]}: a pin costs one 8-byte gather.
 __global__ void k_gr_info(const int32_t* __restrict__ part, int32_t n, int2* __restrict__ info) {
@@ -112,8 +112,14 @@ struct NetBlocks {
   }
 };
 
-// The two loops of Algorithm 4 over pins [b, end) by W threads (`at` of them),
-// with the net's arrays clear on entry and cleared again.
+// The two loops of Algorithm 4 over pins [b, end) by W threads (`at` of them; more
+// than a warp: the block), with the net's arrays clear on entry and cleared again.
+template <int W>
+__device__ __forceinline__ void net_sync() {
+  if (W <= 32) __syncwarp();
+  else __syncthreads();
+}
+
 template <int W>
 __device__ __forceinline__ void gr_net(const int32_t* __restrict__ pins,
                                        const int2* __restrict__ info,
@@ -140,7 +146,7 @@ __device__ __forceinline__ void gr_net(const int32_t* __restrict__ pins,
   for (int x = 0; x < 2; ++x)
     if (b + at + x * W < end) enter(keep[x]);
   for (int32_t q = b + at + 2 * W; q < end; q += W) enter(info[pins[q]]);
-  __syncwarp();
+  net_sync<W>();
   auto leave = [&](const int2& nd) {
     const int32_t i = nd.x;
     if (i < 0) return;
@@ -153,25 +159,33 @@ __device__ __forceinline__ void gr_net(const int32_t* __restrict__ pins,
 #pragma unroll
   for (int x = 0; x < 2; ++x) leave(keep[x]);
   for (int32_t q = b + at + 2 * W; q < end; q += W) leave(info[pins[q]]);
-  __syncwarp();
+  net_sync<W>();
   for (int x = at; x < k; x += W) N.clear(x);
-  __syncwarp();
+  net_sync<W>();
 }
 
 // Listed nets: eight lanes per net of at most GR_SMALL pins (most nets have a
-// handful; a warp per net left its lanes idle), a warp for the others.
+// handful; a warp per net left its lanes idle), a warp for the others, a block for
+// those above GR_BIG (listed with their first chunk; a net of 1M pins: 40 ms by a
+// warp).
 __global__ void __launch_bounds__(GR_WARPS * 32)
 k_gr_net(const int32_t* __restrict__ list, const int32_t* __restrict__ count, int32_t m,
          const int32_t* __restrict__ eoff, const int32_t* __restrict__ pins,
          const int32_t* __restrict__ w, const int2* __restrict__ info,
-         const int32_t* __restrict__ targets, int k,
+         const int32_t* __restrict__ targets, int k, const int2* __restrict__ chunks,
          unsigned long long* __restrict__ gains, int32_t* status) {
   constexpr int PER = 32 / GR_LANES;
   __shared__ NetBlocks s_blocks[GR_WARPS][PER];
   const int wv = warp_in_block(), lane = lane_id(), sub = lane % GR_LANES, grp = lane / GR_LANES;
   for (int x = sub; x < HG_MAX_K; x += GR_LANES) s_blocks[wv][grp].clear(x);
-  __syncwarp();
-  const int32_t nwide = count[TN_WIDE], cnt = count[TN_SMALL];
+  __syncthreads();
+  const int32_t nchunks = count[TN_CHUNKS], nwide = count[TN_WIDE], cnt = count[TN_SMALL];
+  for (int32_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    const int2 it = chunks[c];
+    if (it.y == c)
+      gr_net<GR_WARPS * 32>(pins, info, targets, k, eoff[it.x], eoff[it.x + 1], w[it.x],
+                            (int)threadIdx.x, s_blocks[0][0], gains, status);
+  }
   for (int32_t x = wv * gridDim.x + blockIdx.x; x < nwide; x += gridDim.x * GR_WARPS) {
     const int32_t e = list[m - 1 - x];
     gr_net<32>(pins, info, targets, k, eoff[e], eoff[e + 1], w[e], lane, s_blocks[wv][0], gains,
@@ -226,10 +240,10 @@ void recalculate_gains(const Ctx& cx, const Level& L, int k, const int32_t* part
   DBuf<int2> info;
   TouchedNets t;
   index_moves(cx, L, k, part, l, nodes, targets, info);
-  touched_nets(cx, L, l, nodes, 0, t);
+  touched_nets(cx, L, l, nodes, GR_BIG, t);
   k_gr_net<<<cx.num_sms * 8, GR_WARPS * 32, 0, cx.stream>>>(
       t.list.p, t.count.p, L.m, L.eoff.p, L.pins.p, L.w.p, info.p, targets, k,
-      reinterpret_cast<unsigned long long*>(gains), cx.d_status);
+      t.chunks.p, reinterpret_cast<unsigned long long*>(gains), cx.d_status);
   check_launch("gr_net");
   if (cx.launches) *cx.launches += 1;
   check_status(cx);

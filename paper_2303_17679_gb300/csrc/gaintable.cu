@@ -184,8 +184,10 @@ k_gt_records_big(const int32_t* __restrict__ eoff, const int32_t* __restrict__ p
 // Table rows of the nodes: a lane group per node of at most GT_SMALL incident
 // nets, a warp for up to GT_HUB; items of GT_ITEM incident nets of larger nodes are
 // listed for a warp each, which add to the row (ADD).  One warp for a node of 5M
-// nets took 434 ms at k = 64, whatever the rest of the chip did.
-constexpr int32_t GT_HUB = 4096, GT_ITEM = 1024;
+// nets took 434 ms at k = 64, whatever the rest of the chip did, and four neighbours
+// of 2000 nets in one warp 0.64 ms for a complete graph of 2000 nodes (0.17 now;
+// limits of 256 and 1024 are no different).
+constexpr int32_t GT_HUB = 512, GT_ITEM = 512;
 
 template <bool GRAPH, int K, int H, int W, bool ADD = false>
 __device__ __forceinline__ void gt_row(const int32_t* __restrict__ inets,

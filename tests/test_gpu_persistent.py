@@ -430,8 +430,8 @@ def test_pin_counts_of_huge_nets(oracle_mod, k, sizes, rest):
 # nets around the size above which chunks of a net go to different blocks
 @pytest.mark.parametrize("k", [2, 33])
 def test_gain_tools_of_huge_nets(oracle_mod, k):
-    n = 30_000
-    hgr = nets_around(n, [64, 65, 4095, 4096, 4097, 8192, 8193, 30_000], k)
+    n = 40_000
+    hgr = nets_around(n, [64, 65, 4095, 4096, 4097, 8192, 8193, 32_768, 32_769, 40_000], k)
     rng = np.random.default_rng(k)
     part = rng.integers(0, max(1, k - 1), size=n).astype(np.int32)
     part[:2] = k - 1  # blocks of one or two pins, in different chunks
@@ -464,7 +464,7 @@ def test_gain_tools_of_huge_nets(oracle_mod, k):
 @pytest.mark.parametrize("k", [3, 16, 30, 64])
 def test_gain_table_of_hubs(oracle_mod, graph, k):
     """Nodes around the number of nets above which a row is summed by several warps."""
-    n, degs = 9000, [4095, 4096, 4097, 5120, 5121, 8000]
+    n, degs = 9000, [511, 512, 513, 1024, 1025, 8000]
     rng = np.random.default_rng(k)
     nets = [[u, int(v)] for u, d in enumerate(degs)
             for v in rng.choice(np.arange(100, n), size=d, replace=False)]
