@@ -45,11 +45,11 @@ L2_FLUSH_BYTES = 512 << 20
 # captures are summarised under profiles/.
 TRAFFIC = {
     "rating": {"source": "paper_2303_17679_gb300/csrc/cluster.cu",
-               "source_sha256": "2dd0adddbf3beb5917e983fb3d2cf8eb01395633e07433ca2ddc95af920140b6",
-               "bytes_per_launch": 1274101280},
+               "source_sha256": "294644e365021572aa06700bd762feeae87e55a440f28daebcee26b3427dd3f1",
+               "bytes_per_launch": 1270702368},
     "lp_gain": {"source": "paper_2303_17679_gb300/csrc/lp.cu",
-                "source_sha256": "953be944311cf53dce6f2313c288fc8603943253ca93e07da0677483cacfda75",
-                "bytes_per_launch": 59933056},
+                "source_sha256": "5298a76d07251c269ca16e728e4cbb7f46686dd25a9ce56cb5a708664a20f484",
+                "bytes_per_launch": 60318566},
 }
 
 

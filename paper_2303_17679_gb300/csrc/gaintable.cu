@@ -19,7 +19,7 @@
 // (its lemma); the benefits of the moved nodes are recomputed from the masks
 // after the moves.
 // Measured (GB300, n = m = 1e6 Zipf, k = 8, 100,000 moves): build, moves and the
-// exact gains of the sequence (gainrecalc.cu) together 1.18 -> 0.65 ms.
+// exact gains of the sequence (gainrecalc.cu) together 1.18 -> 0.64 ms.
 //
 // Graph levels (Sec. 10, "The Gain Table"): the table of a graph is
 // w(u, V_i), the weight of u's edges into V_i; the benefit and penalties follow:
