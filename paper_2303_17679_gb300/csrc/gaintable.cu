@@ -185,7 +185,7 @@ k_gt_records_big(const int32_t* __restrict__ eoff, const int32_t* __restrict__ p
 // nets, a warp for up to GT_HUB; items of GT_ITEM incident nets of larger nodes are
 // listed for a warp each, which add to the row (ADD).  One warp for a node of 5M
 // nets took 434 ms at k = 64, whatever the rest of the chip did, and four neighbours
-// of 2000 nets in one warp 0.64 ms for a complete graph of 2000 nodes (0.17 now;
+// of 2000 nets in one warp 0.64 ms for a complete graph of 2000 nodes (0.07 now;
 // limits of 256 and 1024 are no different).
 constexpr int32_t GT_HUB = 512, GT_ITEM = 512;
 
@@ -243,13 +243,55 @@ __device__ __forceinline__ void gt_row(const int32_t* __restrict__ inets,
   }
 }
 
+// The same on graph levels for k > 16 with counters in shared memory (`cnt`, k words
+// that are zero before and after): an edge is one add there, in registers a comparison
+// with every block (n = 500,003, 2M edges, k = 64: 0.22 ms, 0.13 here).
+constexpr int GT_COUNTERS = HG_MAX_K + 8;  // of a lane group: 8 banks apart
+
+template <int W, bool ADD = false>
+__device__ __forceinline__ void gt_row_counted(const int2* __restrict__ adj,
+                                               const int32_t* __restrict__ part, bool on,
+                                               int64_t u, int32_t beg, int32_t end, int l, int k,
+                                               long long* __restrict__ b,
+                                               long long* __restrict__ p, int32_t* cnt) {
+  const int from = on ? part[u] : 0;
+  int32_t wsum = 0;
+  for (int32_t j = beg + l; j < end; j += 2 * W) {
+    const bool two = j + W < end;
+    const int2 a0 = adj[j], a1 = two ? adj[j + W] : make_int2(-1, 0);
+    const int t0 = part[a0.x], t1 = two ? part[a1.x] : 0;
+    atomicAdd(&cnt[t0], a0.y);
+    if (two) atomicAdd(&cnt[t1], a1.y);
+    wsum += a0.y + a1.y;
+  }
+  __syncwarp();
+  wsum = group_sum<W>(wsum);
+  for (int t = l; on && t < k; t += W) {
+    const int32_t x = t == from ? 0 : wsum - cnt[t];
+    if (t == from) {
+      if (ADD) atomic_add_i64(&b[u], wsum - cnt[t]);
+      else b[u] = wsum - cnt[t];
+    }
+    if (!ADD) p[u * k + t] = x;
+    else if (x) atomic_add_i64(&p[u * k + t], x);
+    cnt[t] = 0;
+  }
+  __syncwarp();
+}
+
 template <bool GRAPH, int K, int H>
 __global__ void __launch_bounds__(GT_WARPS * 32)
 k_gt_build(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
            const int2* __restrict__ adj, const int4* __restrict__ rec,
            const int32_t* __restrict__ part, int32_t n, int k, long long* __restrict__ b,
            long long* __restrict__ p, int2* __restrict__ items, int32_t* __restrict__ nitems) {
+  constexpr bool COUNTED = GRAPH && K == 32;
+  __shared__ int32_t s_cnt[COUNTED ? GT_WARPS : 1][NG][GT_COUNTERS];
   const int lane = lane_id();
+  if (COUNTED) {
+    for (int i = lane; i < NG * GT_COUNTERS; i += 32) (&s_cnt[warp_in_block()][0][0])[i] = 0;
+    __syncwarp();
+  }
   const int64_t stride = (int64_t)gridDim.x * GT_WARPS * NG;
   for (int64_t u0 = ((int64_t)blockIdx.x * GT_WARPS + warp_in_block()) * NG; u0 < n; u0 += stride) {
     const int64_t u = u0 + lane / SUB_G;
@@ -261,8 +303,12 @@ k_gt_build(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
       continue;
     }
     const bool small = end - beg <= GT_SMALL;
-    gt_row<GRAPH, K, H, SUB_G>(inets, adj, rec, part, u < n && small, u, beg, small ? end : beg,
-                               lane % SUB_G, k, b, p);
+    if constexpr (COUNTED)
+      gt_row_counted<SUB_G>(adj, part, u < n && small, u, beg, small ? end : beg, lane % SUB_G, k,
+                            b, p, s_cnt[warp_in_block()][lane / SUB_G]);
+    else
+      gt_row<GRAPH, K, H, SUB_G>(inets, adj, rec, part, u < n && small, u, beg, small ? end : beg,
+                                 lane % SUB_G, k, b, p);
     unsigned wide = __ballot_sync(FULL, lane % SUB_G == 0 && !small);
     while (wide) {
       const int l = __ffs(wide) - 1;
@@ -281,7 +327,10 @@ k_gt_build(const int32_t* __restrict__ ioff, const int32_t* __restrict__ inets,
         for (int t = lane; t < k; t += 32) p[wu * k + t] = 0;
         continue;
       }
-      gt_row<GRAPH, K, H, 32>(inets, adj, rec, part, true, wu, wb, we, lane, k, b, p);
+      if constexpr (COUNTED)
+        gt_row_counted<32>(adj, part, true, wu, wb, we, lane, k, b, p, s_cnt[warp_in_block()][0]);
+      else
+        gt_row<GRAPH, K, H, 32>(inets, adj, rec, part, true, wu, wb, we, lane, k, b, p);
     }
   }
 }
@@ -293,12 +342,23 @@ k_gt_build_hubs(const int32_t* __restrict__ ioff, const int32_t* __restrict__ in
                 const int32_t* __restrict__ part, int k, long long* __restrict__ b,
                 long long* __restrict__ p, const int2* __restrict__ items,
                 const int32_t* __restrict__ nitems) {
+  constexpr bool COUNTED = GRAPH && K == 32;
+  __shared__ int32_t s_cnt[COUNTED ? GT_WARPS : 1][GT_COUNTERS];
+  if (COUNTED) {
+    for (int i = lane_id(); i < GT_COUNTERS; i += 32) s_cnt[warp_in_block()][i] = 0;
+    __syncwarp();
+  }
   const int32_t cnt = *nitems;
   for (int32_t x = warp_in_block() * gridDim.x + blockIdx.x; x < cnt; x += gridDim.x * GT_WARPS) {
     const int2 it = items[x];
     const int32_t beg = ioff[it.x] + it.y * GT_ITEM;
     const int32_t end = beg + min(GT_ITEM, ioff[it.x + 1] - beg);
-    gt_row<GRAPH, K, H, 32, true>(inets, adj, rec, part, true, it.x, beg, end, lane_id(), k, b, p);
+    if constexpr (COUNTED)
+      gt_row_counted<32, true>(adj, part, true, it.x, beg, end, lane_id(), k, b, p,
+                               s_cnt[warp_in_block()]);
+    else
+      gt_row<GRAPH, K, H, 32, true>(inets, adj, rec, part, true, it.x, beg, end, lane_id(), k, b,
+                                    p);
   }
 }
 
@@ -333,8 +393,7 @@ BuildRows build_rows_for(bool graph, int k) {
   if (graph) {
     if (k <= 8) return build_rows<true, 8, 1>;
     if (k <= 16) return build_rows<true, 16, 1>;
-    if (k <= 32) return build_rows<true, 32, 1>;
-    return build_rows<true, 32, 2>;
+    return build_rows<true, 32, 1>;
   }
   if (k <= 8) return build_rows<false, 8, 1>;
   if (k <= 16) return build_rows<false, 16, 1>;
